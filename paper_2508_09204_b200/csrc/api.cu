@@ -73,10 +73,10 @@ int pick_kernel(int path, int M, const moqe_expert* const* ex, int E) {
     return 0;
 }
 
-// the arrival counters at the head of the workspace body (both split-K kernels keep theirs there)
+// the arrival counters at the head of the workspace body (all split-K kernels keep theirs there)
 size_t body_zero_bytes(int M, int Np) {
-    const size_t a = stream_zero_bytes(M, Np), b = decode_zero_bytes(M);
-    return a > b ? a : b;
+    const size_t a = stream_zero_bytes(M, Np), b = decode_zero_bytes(M), c = tc_zero_bytes();
+    return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
 
 }  // namespace
@@ -123,8 +123,7 @@ moqe_status run_sorted(int kernel, int path, const void* X, int M, const moqe_ex
     if (kernel == 2) return launch_qgemm_decode_multi(&X, M, 1, ex, E, &Y, perm, offsets, body, body_bytes, st);
     if (kernel == 1) return launch_qgemm_stream(X, M, N, K, ex, E, Y, perm, offsets, body, body_bytes, st);
     if (kernel == 3) return launch_qgemm_dense(X, M, N, K, ex, E, Y, perm, offsets, body, body_bytes, st);
-    tc_set_tile_tokens(path == 3 ? 128 : (path == 4 ? 256 : 0));
-    return launch_qgemm_tc(X, M, N, K, ex, E, Y, perm, offsets, body, body_bytes, st);
+    return launch_qgemm_tc(X, M, N, K, ex, E, Y, perm, offsets, body, body_bytes, path == 3 ? 128 : (path == 4 ? 256 : 0), st);
 }
 }  // namespace
 
@@ -140,7 +139,7 @@ extern "C" moqe_status moqe_routed_qgemm_path(const void* X_bf16, const int32_t*
     char* base = (char*)workspace;
     int32_t* perm = (int32_t*)(base + w.perm);
     int32_t* offsets = (int32_t*)(base + w.offsets);
-    const size_t zero_bytes = kernel != 0 ? body_zero_bytes(M, h_experts[0]->Np) : 0;
+    const size_t zero_bytes = kernel != 3 ? body_zero_bytes(M, h_experts[0]->Np) : 0;
     s = launch_sort(row_ids, M, E, perm, offsets, base + w.sort, w.body - w.sort, base + w.body, zero_bytes, Y_bf16,
                     h_experts[0]->N, st);
     if (s != MOQE_OK) return s;

@@ -106,11 +106,6 @@ size_t sort_workspace_bytes(int M, int E);
 moqe_status launch_gather(const void* X, const int32_t* perm, const int32_t* offsets_E, int M, int C, void* Xp,
                           cudaStream_t st);
 
-// 64-row boxes of the expert-sorted activations: copied to Xp only where the rows are not already consecutive in X
-size_t gather_boxes_bytes(int M, int E);
-moqe_status launch_gather_boxes(const void* X, const int32_t* perm, const int32_t* offsets, int M, int C, int E, void* Xp,
-                                int32_t* box_src, cudaStream_t st);
-
 // qgemm_stream.cu
 size_t stream_workspace_bytes(int M, int Np, int E);
 moqe_status launch_qgemm_stream(const void* X, int M, int N, int K, const moqe_expert* const* ex, int E, void* Y,
@@ -142,12 +137,12 @@ size_t dense_workspace_bytes(int M, int K, int E, int Np, int Kp);
 moqe_status launch_qgemm_dense(const void* X, int M, int N, int K, const moqe_expert* const* ex, int E, void* Y,
                                const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes, cudaStream_t st);
 
-// qgemm_tcgen05.cu
-void tc_set_tile_tokens(int tn);   // 0 = automatic, else 128 or 256 (testing / measurement)
+// qgemm_tcgen05.cu; tile_tokens: 0 = automatic (work split by k-blocks where that balances it), 128 / 256 = whole
+// tiles of that many tokens (testing / measurement)
+size_t tc_zero_bytes();
 size_t tc_workspace_bytes(int M, int K, int E, int Np);
 moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_expert* const* ex, int E, void* Y,
-                            const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes,
-                            cudaStream_t st);
+                            const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes, int tile_tokens, cudaStream_t st);
 
 __device__ __forceinline__ void latch_status(int* status, int code) {
     if (status) atomicCAS(status, 0, code);

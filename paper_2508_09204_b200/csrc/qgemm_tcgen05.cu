@@ -1,31 +1,34 @@
-// Routed dequant-GEMM for large batches (prefill shapes): a persistent,
-// warp-specialised grouped GEMM on the 5th-generation tensor cores.
+// Routed dequant-GEMM for batches beyond the decode kernel's: a persistent, warp-specialised grouped GEMM on the
+// 5th-generation tensor cores, two SMs to a tile (cta_group::2).
 //
-//   tile         : 128 output channels (UMMA M, the TMEM lanes) x TN tokens (UMMA N, TMEM columns)
-//   A operand    : the expert's weights.  Packed 128x128-code tiles arrive by bulk
-//                  async copy; four "dequant" warps unpack them in registers to the
-//                  exact integers (c - z) in bf16 and store them as a K-major,
-//                  128-byte-swizzled shared-memory operand (64 k per stage).
-//   B operand    : token rows, loaded by TMA (2-D tiled, 128-byte swizzle) from the
-//                  expert-sorted activation matrix.
-//   accumulation : tcgen05.mma (kind::f16, bf16 x bf16 -> fp32) into one of two TMEM
-//                  buffers per quantization group; eight "epilogue" warps drain the
-//                  finished buffer, multiply by the group's fp32 scale and add into
-//                  register accumulators while the MMA fills the other buffer:
+//   tile         : 256 output channels x up to 128 * NH tokens.  CTA r of the pair owns channels 128 r .. 128 r + 127
+//                  (its TMEM lanes) of every token of the tile.
+//   A operand    : the expert's weights, in TENSOR MEMORY.  Packed 128x128-code tiles arrive by bulk async copy; a
+//                  "dequant" thread owns one channel, unpacks its 128 codes of a k-block in registers to the exact
+//                  numbers (c - z) * 2^-13 in bf16 and stores them to its TMEM lane.  The unpacked weights never pass
+//                  through shared memory, whose bandwidth the token operand needs.
+//   B operand    : token rows, 64 per CTA and half tile (each SM of the pair reads its own half and they share it).
+//                  Sorted rows that are consecutive in X come as one TMA box; any others are gathered through `perm` by
+//                  two warps' 16-byte cp.async copies into the same swizzled layout (the fused permutation: no gathered
+//                  copy of X exists).
+//   accumulation : fp32 in three rotating TMEM buffers of 128 tokens.  Grouped experts finish a buffer per (half tile,
+//                  quantization group, at most 128 k); eight "epilogue" warps drain it, multiply by the group's fp32
+//                  scale and add into register accumulators while the tensor core fills the next one:
 //                      Y[m][n] = sum_G s[n][G] * (sum_{k in G} X[m][k] * (c[n][k] - z[n][G]))
-//                  so the tensor core only multiplies exactly representable numbers.
-//                  Per-channel experts need a single scale at the end of K.
-//   scheduling   : one CTA per SM walks the tile list (expert, token tile, channel
-//                  tile) derived on the device from the per-expert offset table;
-//                  rows are written straight to their original positions through
-//                  `perm` (fused un-permutation).
+//                  so the tensor core only multiplies exactly representable numbers.  Per-channel experts keep one
+//                  buffer per half tile for the whole of K.
+//   scheduling   : the tile list (expert, token tile, channel pair) is derived on the device from the per-expert offset
+//                  table.  Whole rounds of it go tile by tile to the clusters; the rest (everything, for a small
+//                  batch) is split by k-blocks ("stream-K": equal cost per cluster, whatever the routing).  A warp that
+//                  holds part of a tile parks its fp32 sums and bumps an arrival counter; the last arrival adds them up
+//                  in cluster order and stores.  Nobody waits for another cluster.  Rows go straight to their original
+//                  positions through `perm` (fused un-permutation).
 //
-// Every mbarrier wait is bounded (2 s of %globaltimer); on expiry the CTA sets
-// an abort flag, latches MOQE_ERR_TIMEOUT, lets copies in flight land, frees
-// its TMEM and returns.
+// Every mbarrier wait is bounded (2 s of %globaltimer); on expiry the CTA sets an abort flag, latches
+// MOQE_ERR_TIMEOUT, lets copies in flight land, frees its TMEM and returns.
 //
-// The operation is Section 3.1 of the paper (the selected quantization expert
-// runs the sample); the paper describes no kernel.
+// The operation is Section 3.1 of the paper (the selected quantization expert runs the sample); the paper describes
+// no kernel.
 #include <cuda.h>
 
 #include <type_traits>
@@ -37,375 +40,780 @@
 namespace moqe {
 namespace {
 
-constexpr int TC_THREADS = 512;
-constexpr int NS = 3;                 // operand stages (A tile + X tile, 64 k each)
-constexpr int NWS = 3;                // packed-weight stages (128 k each)
-constexpr int A_STAGE_BYTES = 128 * 128;          // 128 channels x 64 bf16
-constexpr int W_STAGE_BYTES = 128 * 128 + 4 * 512;   // largest packed tile (W8 codes) + largest per-tile meta
-constexpr int XBOX_ROWS = 64;
-constexpr int XBOX_BYTES = XBOX_ROWS * 128;
+constexpr int TC_MAX_CLUSTERS = 80;
+constexpr int TC_EPI = 8;                          // epilogue warps
+constexpr int TC_NW_MAX = 12;                      // packed-weight stages
+constexpr int TC_XHALF = 2 * 64 * 128;             // 64 token rows x 128 k bf16: two 64-k swizzled sub-tiles
+constexpr int TC_A_COLS = 64;                      // TMEM columns of one k-block of unpacked weights
+constexpr int TC_ACC_COLS = 128;                   // TMEM columns of one accumulator buffer
+constexpr int TC_NACC = 3;
+constexpr int TC_NSC = 8;                          // k-blocks of scales between the dequant warps and the epilogue
+constexpr int TC_A_BASE = TC_NACC * TC_ACC_COLS;   // two weight buffers behind the accumulators
+
+// NH: half tiles of 128 tokens.  2: few, large tiles (a k-block's 1024 tensor cycles hide one dequant warpgroup's
+// work); 1: small batches, where unpacking is the critical role and gets two warpgroups that take turns.
+template <int NH>
+struct TcCfg {
+    static constexpr int dq_warps = NH == 2 ? 4 : 8;
+    static constexpr int epi_warp0 = 4 + dq_warps;
+    static constexpr int threads = (epi_warp0 + TC_EPI) * 32;
+    static constexpr int nx = NH == 2 ? 4 : 6;                               // token stages: one k-block of the tile
+    static constexpr int xstage = NH * TC_XHALF;
+    // shared memory
+    static constexpr int x_off = 0;
+    static constexpr int bar_off = nx * xstage;
+    static constexpr int n_bars = 2 * TC_NW_MAX + 2 * nx + 2 + 2 * TC_NACC + TC_NSC;   // wfull wempty xfull done afull accfull accempty scfull
+    static constexpr int misc_off = bar_off + n_bars * 8;                    // tmem addr, abort flag, clusters of the split, T, Td
+    static constexpr int cost_off = (misc_off + 32 + 15) / 16 * 16;          // long long: base[32], total
+    static constexpr int sched_off = cost_off + 33 * 8;                      // ints: see TcSched
+    static constexpr int sched_ints = 34 + 33 + 5 * 32;
+    static constexpr int perm_off = sched_off + sched_ints * 4;
+    static constexpr int xrow_off = perm_off + TC_EPI * 64 * NH * 4;         // rows of X to gather, one list per gather warp
+    static constexpr int sc_off = (xrow_off + 2 * 64 * NH * 4 + 15) / 16 * 16;   // scales on their way to the epilogue
+    static constexpr int w_off = (sc_off + TC_NSC * 4 * 128 * 2 + 127) / 128 * 128;
+    static constexpr int total = 226 * 1024;
+    static constexpr int w_bytes = (total - w_off) / 128 * 128;
+    static constexpr int dyn_bytes = total + 1024;                           // slack for manual 1024-byte alignment
+};
+static_assert(TcCfg<2>::dyn_bytes <= 232448 && TcCfg<2>::w_bytes >= 3 * 18432, "shared memory budget");
 
 struct TcParams {
     ExpertDev ex[MOQE_MAX_EXPERTS];
     const int32_t* perm;
     const int32_t* offsets;
-    const int32_t* box_src;   // per 64-row box: first source row in X if its rows are consecutive there, else -1 (use Xp)
+    const uint16_t* X;
     uint16_t* Y;
+    float* partials;          // [cluster][2][rank][cols][128]
+    uint32_t* counters;       // [cluster][rank][warp]; zero on entry, left zero
     int* status;
-    int M, N, K, Np, KB, E, n_tiles;
+    int M, N, K, KB, E, NT1, NTP;    // NT1: 128-channel tiles, NTP: pairs of them
+    int cols;                 // token columns of a parked partial sum
+    int nw, wstage;           // packed-weight ring
+    int split;                // 0: whole tiles only
 };
 
-template <int TN>
-struct Smem {
-    static constexpr int a_off = 0;
-    static constexpr int x_off = a_off + NS * A_STAGE_BYTES;
-    static constexpr int w_off = x_off + NS * TN * 128;
-    static constexpr int bar_off = w_off + NWS * W_STAGE_BYTES;
-    // barriers: wfull[NWS] wempty[NWS] xfull[NS] afull[NS] empty[NS] accfull[2] accempty[2]
-    static constexpr int n_bars = 2 * NWS + 3 * NS + 4;
-    static constexpr int misc_off = bar_off + n_bars * 8;              // tmem addr, abort flag
-    static constexpr int off_off = misc_off + 16;                      // offsets[E+1]
-    static constexpr int perm_off = off_off + (MOQE_MAX_EXPERTS + 2) * 4;
-    static constexpr int total = perm_off + 8 * (TN / 2) * 4;          // per epilogue warp: its columns' target rows
-    static constexpr int dyn_bytes = total + 1024;                     // slack for manual 1024-byte alignment
-};
-
-// ---------------------------------------------------------------------------- TMA tile load
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
+// ---------------------------------------------------------------------------- PTX of the two-CTA forms
+__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+    uint32_t d;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
+    return d;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// (Arrivals on the other CTA's barriers order tensor-memory work and async copies only, so they need no cluster-scope
+// release; with one, 16384 rows of a per-channel expert took 9.1 ms a LLaMA block instead of 4.9.)
+__device__ __forceinline__ void remote_arrive(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ void remote_expect_tx_only(uint32_t cluster_addr, uint32_t bytes) {
+    asm volatile("mbarrier.expect_tx.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(cluster_addr), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void tma_box_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t cluster_bar) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar) : "memory");
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(cluster_bar) : "memory");
+}
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t smem_dst, uint32_t cols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t cols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
+}
+// D[256 x n] (+)= A[256 x 16] (TMEM of both CTAs) . B[n x 16]^T (n / 2 rows in each CTA's shared memory)
+__device__ __forceinline__ void umma_pair_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5, %5, %5, %5, %5}, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(0u) : "memory");
+}
+// arrives at the same barrier of both CTAs when every MMA issued so far is done
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+    const uint16_t both = 3;
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(both) : "memory");
+}
+// bf16 x bf16 -> fp32, both operands K-major, M = 256 over the pair, N = n
+__device__ __forceinline__ uint32_t umma_idesc_pair(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((256u >> 4) << 24);
 }
 
-// ---------------------------------------------------------------------------- tile list
-struct TileInfo { int e, nt, m0, rows; };
+// ---------------------------------------------------------------------------- schedule
+struct TcSched {
+    int* off;      // [E + 1] (34)
+    int* tile0;    // [E + 1] first tile of each expert (33)
+    int* rpt;      // rows per token tile
+    int* us;       // first unit (k-block of a tile, counted per expert) that is split
+    int* ub;       // this cluster's share of the split units
+    int* ue;
+    int* w;        // cost of a unit
+    long long* base;   // cost before each expert's split units; [32]: total
+    int* misc;     // {clusters of the split, T, Td}
+};
 
-template <int TN>
-__device__ __forceinline__ bool decode_tile(const int* s_off, int E, int n_tiles, int t, TileInfo& ti) {
-    for (int e = 0; e < E; ++e) {
-        int Me = s_off[e + 1] - s_off[e];
-        int cnt = ((Me + TN - 1) / TN) * n_tiles;
-        if (t < cnt) {
-            int mt = t / n_tiles;
-            ti.e = e;
-            ti.nt = t - mt * n_tiles;
-            ti.m0 = s_off[e] + mt * TN;
-            ti.rows = min(TN, Me - mt * TN);
-            return true;
+struct TcPiece { int e, ntp, m0, rows, kb0, kb1, tile; };   // tile: inside the expert
+
+// a walk over the pieces of work of one cluster: whole tiles first, then its share of the split
+struct TcWalk {
+    int t, e, u, ue;
+    __device__ __forceinline__ void start(int cluster) { t = cluster; e = -1; u = ue = 0; }
+    __device__ __forceinline__ bool next(const TcSched& s, const TcParams& p, int nclusters, TcPiece& pc) {
+        int tile;
+        if (t < s.misc[2]) {
+            int ee = 0;
+            while (t >= s.tile0[ee + 1]) ++ee;
+            pc.e = ee;
+            tile = t - s.tile0[ee];
+            pc.kb0 = 0;
+            pc.kb1 = p.KB;
+            t += nclusters;
+        } else {
+            while (u >= ue) {
+                if (++e >= p.E) return false;
+                u = s.ub[e];
+                ue = s.ue[e];
+            }
+            pc.e = e;
+            tile = u / p.KB;
+            pc.kb0 = u - tile * p.KB;
+            pc.kb1 = min(p.KB, pc.kb0 + (ue - u));
+            u += pc.kb1 - pc.kb0;
         }
-        t -= cnt;
+        const int mt = tile / p.NTP, rpt = s.rpt[pc.e], first = s.off[pc.e] + mt * rpt;
+        pc.tile = tile;
+        pc.ntp = tile - mt * p.NTP;
+        pc.m0 = first;
+        pc.rows = min(rpt, s.off[pc.e + 1] - first);
+        return true;
     }
-    return false;
-}
+};
+// MMA columns of half tile h of a tile with `rows` tokens
+__device__ __forceinline__ int half_cols(int rows, int h) { return (min(128, rows - 128 * h) + 31) & ~31; }
 
-// ---------------------------------------------------------------------------- dequant role
-// One k-block (128 k) of one tile: wait for the packed tile, pull this thread's four pieces into
-// registers, release the packed stage, then fill the two 64-k operand stages.
-template <int BITS>
-__device__ __forceinline__ bool dequant_kblock(const ExpertDev& ex, int nt, unsigned char* smem_w,
-                                               unsigned char* smem_a_base, uint32_t bar_wfull, uint32_t bar_wempty,
-                                               uint32_t wphase, uint32_t bar_empty0, uint32_t bar_afull0, Ring& ring,
-                                               volatile int* abort_flag, int* status) {
-    const int lane = threadIdx.x & 31, dw = (threadIdx.x >> 5) & 3;
-    const int q = lane >> 3, r = (lane & 7) ^ (2 * q);          // slot = lane holds piece (q, r)
-    constexpr int NWORDS = PieceWords<BITS>::n;
-    const float sym_z = (float)(1 << (BITS - 1));
-    // zero-points of the four pieces' channels, per chunk: per-channel experts read theirs from global memory
-    // before the wait, the others from the tile's own meta once it has landed
-    float z[4][4];
-    const bool tile_zeros = ex.has_zeros && ex.group != 0;
+// ---------------------------------------------------------------------------- unpacking
+__device__ __forceinline__ uint32_t fma_bf16x2(uint32_t a, uint32_t b, uint32_t c) {
+    const __nv_bfloat162 r = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b),
+                                     *reinterpret_cast<const __nv_bfloat162*>(&c));
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+// Chunk G of a piece as bf16 pairs (c - z) * 2^-13.  A code zero-extended to 16 bits IS the bf16 number c * 2^-133
+// (subnormal below 128; the encoding runs on linearly through the first normal binade, so a code may also sit up to
+// four, three or six bits higher as long as it stays below bit 8).  One fused multiply-add per PAIR of codes,
+// c * 2^(-133+s) * 2^(120-s) - z * 2^-13, is exact (|c - z| <= 255 has 8 significant bits); the scale takes the 2^13.
+// nz: -z * 2^-13 in both halves.
+template <int BITS, int G>
+__device__ __forceinline__ void unpack_scaled(const uint32_t (&w)[PieceWords<BITS>::n], uint32_t nz, uint32_t* out) {
+    constexpr uint32_t P120 = 0x7B807B80u, P118 = 0x7A807A80u, P117 = 0x7A007A00u, P116 = 0x79807980u, P114 = 0x78807880u;
+    if constexpr (BITS == 4) {
+        const uint32_t v = w[G], u = v >> 8;
+        out[0] = fma_bf16x2(v & 0x000F000Fu, P120, nz);
+        out[1] = fma_bf16x2(v & 0x00F000F0u, P116, nz);
+        out[2] = fma_bf16x2(u & 0x000F000Fu, P120, nz);
+        out[3] = fma_bf16x2(u & 0x00F000F0u, P116, nz);
+    } else if constexpr (BITS == 2) {
+        const uint32_t v = (G & 1) ? w[G >> 1] >> 8 : w[G >> 1];
+        out[0] = fma_bf16x2(v & 0x00030003u, P120, nz);
+        out[1] = fma_bf16x2(v & 0x000C000Cu, P118, nz);
+        out[2] = fma_bf16x2(v & 0x00300030u, P116, nz);
+        out[3] = fma_bf16x2(v & 0x00C000C0u, P114, nz);
+    } else if constexpr (BITS == 3) {
 #pragma unroll
-    for (int pi = 0; pi < 4; ++pi) {
-        const int n = nt * 128 + (2 * dw + (pi >> 1)) * 16 + (pi & 1) * 8 + r;
-        const float v = (ex.has_zeros && ex.group == 0) ? __bfloat162float(ex.zeros_pc[n]) : sym_z;
-#pragma unroll
-        for (int G = 0; G < 4; ++G) z[pi][G] = v;
-    }
-    if (!mbar_wait(bar_wfull, wphase, abort_flag, status)) return false;
-    uint32_t w[4][NWORDS];
-#pragma unroll
-    for (int pi = 0; pi < 4; ++pi)
-        load_piece_smem<BITS>(smem_w + (2 * dw + (pi >> 1)) * moqe_blob_bytes(BITS), pi & 1, lane, w[pi]);
-    if (tile_zeros) {
-        const int per_tile = moqe_groups_per_tile(ex.group);
-#pragma unroll
-        for (int pi = 0; pi < 4; ++pi) {
-            const int row = (2 * dw + (pi >> 1)) * 16 + (pi & 1) * 8 + r;
-#pragma unroll
-            for (int G = 0; G < 4; ++G) {
-                const int j = per_tile == 4 ? G : (per_tile == 2 ? (G >> 1) : 0);
-                z[pi][G] = __bfloat162float(moqe_tile_zeros(smem_w, BITS, j)[row]);
+        for (int i = 0; i < 4; ++i) {
+            const int p = 4 * G + i, f = p % 5;
+            if (p == 15) {
+                const uint32_t v = ((w[0] >> 15) & 0x00010001u) | ((w[1] >> 14) & 0x00020002u) | ((w[2] >> 13) & 0x00040004u);
+                out[i] = fma_bf16x2(v, P120, nz);
+            } else {
+                const uint32_t v = f < 2 ? w[p / 5] : (f < 4 ? w[p / 5] >> 6 : w[p / 5] >> 12);
+                out[i] = (f & 1) ? fma_bf16x2(v & 0x00380038u, P117, nz) : fma_bf16x2(v & 0x00070007u, P120, nz);
             }
         }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            out[i] = fma_bf16x2(__byte_perm(w[2 * G + (i >> 1)], 0u, (i & 1) ? 0x4342u : 0x4140u), P120, nz);
     }
-    mbar_arrive(bar_wempty);
+}
+__device__ __forceinline__ uint32_t neg_z(float z) { const float v = z * -0.0001220703125f; return pack_bf16x2(v, v); }
+
+// One k-block of one channel: its four pieces from the packed tile into registers, then to the lane's 64 TMEM columns.
+// scales: where the channel's scales go.  zpc: the channel's zero-point if it is not in the tile (per channel, or a
+// symmetric grid).  bar_free: the barrier whose phase fphase hands the operand buffer back (0: it has not been used
+// yet).  Returns false on abort.
+template <int BITS>
+__device__ __forceinline__ bool dequant_kblock(const ExpertDev& ex, const unsigned char* tile, int row, uint32_t zpc, bool tile_zeros,
+                                               __half* scales, uint32_t bar_scfull, uint32_t bar_wfull, uint32_t wphase, uint32_t bar_wempty,
+                                               uint32_t bar_free, uint32_t fphase, uint32_t a_tmem, volatile int* abort_flag, int* status) {
+    const int lane = threadIdx.x & 31;
+    const int half = (row >> 3) & 1, r = row & 7;
+    const unsigned char* blob = tile + (row >> 4) * moqe_blob_bytes(BITS);
+    bool ok = __all_sync(0xffffffffu, mbar_wait_short(bar_wfull, wphase, abort_flag, status));
+    uint32_t w[4][PieceWords<BITS>::n];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        if (!mbar_wait(bar_empty0 + 8 * ring.stage, ring.phase ^ 1u, abort_flag, status)) return false;
-        unsigned char* a_stage = smem_a_base + ring.stage * A_STAGE_BYTES;
-#pragma unroll
-        for (int pi = 0; pi < 4; ++pi) {
-            const int row = (2 * dw + (pi >> 1)) * 16 + (pi & 1) * 8 + r;
-            auto put = [&](auto Gc) {
-                constexpr int G = decltype(Gc)::value;
-                uint32_t out[4];
-                unpack_chunk<BITS, G>(w[pi], z[pi][G], out);
-                const int chunk = (G & 1) * 4 + q;
-                *reinterpret_cast<uint4*>(a_stage + row * 128 + ((chunk ^ (row & 7)) << 4)) =
-                    make_uint4(out[0], out[1], out[2], out[3]);
-            };
-            if (h == 0) { put(std::integral_constant<int, 0>{}); put(std::integral_constant<int, 1>{}); }
-            else        { put(std::integral_constant<int, 2>{}); put(std::integral_constant<int, 3>{}); }
+    for (int q = 0; q < 4; ++q) {
+        const int slot = q * 8 + (r ^ (2 * q));
+        if constexpr (BITS == 3) {
+            // both halves share the 16-byte slot: {A, B, C of half 0, A of half 1}
+            const uint4 v = *reinterpret_cast<const uint4*>(blob + slot * 16);
+            const uint2 u = *reinterpret_cast<const uint2*>(blob + 512 + slot * 8);
+            w[q][0] = half ? v.w : v.x;
+            w[q][1] = half ? u.x : v.y;
+            w[q][2] = half ? u.y : v.z;
+        } else {
+            load_piece_smem<BITS>(blob, half, slot, w[q]);
         }
-        fence_proxy_async();
-        mbar_arrive(bar_afull0 + 8 * ring.stage);
-        ring.advance(NS);
     }
-    return true;
+    const int per = moqe_groups_per_tile(ex.group);
+    uint32_t nz[4] = {zpc, zpc, zpc, zpc};
+    if (tile_zeros) {
+#pragma unroll
+        for (int G = 0; G < 4; ++G) {
+            const int j = per == 4 ? G : (per == 2 ? (G >> 1) : 0);
+            nz[G] = neg_z(__bfloat162float(moqe_tile_zeros(tile, BITS, j)[row]));
+        }
+    }
+    // the tile's scales travel on to the epilogue warps
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (j < per) scales[j * 128 + row] = moqe_tile_scales(tile, BITS, ex.has_zeros, j)[row];
+    __syncwarp();
+    if (lane == 0) { mbar_arrive(bar_wempty); mbar_arrive(bar_scfull); }
+    if (bar_free) ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_free, fphase, abort_flag, status));
+    tc_fence_after();
+    auto chunk = [&](auto Gc) {
+        constexpr int G = decltype(Gc)::value;
+        uint32_t o[16];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) unpack_scaled<BITS, G>(w[q], nz[G], o + 4 * q);
+        tmem_st16(a_tmem + 16 * G, o);
+    };
+    chunk(std::integral_constant<int, 0>{});
+    chunk(std::integral_constant<int, 1>{});
+    chunk(std::integral_constant<int, 2>{});
+    chunk(std::integral_constant<int, 3>{});
+    tmem_st_wait();
+    return ok;
+}
+
+// acc[0..31] += s * v
+// (Scalar: the packed two-column form needs aligned register pairs, and the moves that make them cost more than it saves.)
+__device__ __forceinline__ void fma_cols32(float* acc, const uint32_t (&v)[32], float s) {
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = fmaf(s, __uint_as_float(v[i]), acc[i]);
 }
 
 // ---------------------------------------------------------------------------- the kernel
-// W2: the instantiation that also takes 2-bit experts (kept apart: the extra unpack path costs the dequant warps of
-// the common instantiation 14 % through register allocation alone)
-template <int TN, bool REGSPLIT, bool W2>
-__global__ void __launch_bounds__(TC_THREADS, 1) qgemm_tc_kernel(const __grid_constant__ TcParams p,
-                                                                const __grid_constant__ CUtensorMap tmap,
-                                                                const __grid_constant__ CUtensorMap tmap_x) {
+template <int NH>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 1)
+    qgemm_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap tmap) {
+    using L = TcCfg<NH>;
+    constexpr int NX = L::nx;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    using L = Smem<TN>;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t rank = cluster_rank();
+    const int cluster = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
     const uint32_t sbase = smem_u32(smem);
-    const uint32_t bar0 = sbase + L::bar_off;
-    const uint32_t bar_wfull = bar0, bar_wempty = bar0 + 8 * NWS, bar_xfull = bar0 + 16 * NWS;
-    const uint32_t bar_afull = bar_xfull + 8 * NS, bar_empty = bar_afull + 8 * NS;
-    const uint32_t bar_accfull = bar_empty + 8 * NS, bar_accempty = bar_accfull + 16;
+    // done[stage]: every MMA of the k-block in that token stage has finished.  One commit per k-block hands back the token
+    // stage and the weight buffer and announces the accumulator buffer filled last (a commit costs the issuing warp about
+    // 200 cycles, three k16 steps of a half tile).
+    const uint32_t bar_wfull = sbase + L::bar_off, bar_wempty = bar_wfull + 8 * TC_NW_MAX;
+    const uint32_t bar_xfull = bar_wempty + 8 * TC_NW_MAX, bar_done = bar_xfull + 8 * NX;
+    const uint32_t bar_afull = bar_done + 8 * NX;
+    const uint32_t bar_accfull = bar_afull + 16, bar_accempty = bar_accfull + 8 * TC_NACC, bar_scfull = bar_accempty + 8 * TC_NACC;
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + L::misc_off);
     volatile int* s_abort = reinterpret_cast<volatile int*>(smem + L::misc_off + 4);
-    int* s_off = reinterpret_cast<int*>(smem + L::off_off);
+    TcSched sc;
+    sc.misc = reinterpret_cast<int*>(smem + L::misc_off + 8);
+    sc.base = reinterpret_cast<long long*>(smem + L::cost_off);
+    sc.off = reinterpret_cast<int*>(smem + L::sched_off);
+    sc.tile0 = sc.off + 34;
+    sc.rpt = sc.tile0 + 33;
+    sc.us = sc.rpt + 32;
+    sc.ub = sc.us + 32;
+    sc.ue = sc.ub + 32;
+    sc.w = sc.ue + 32;
     int* s_perm = reinterpret_cast<int*>(smem + L::perm_off);
+    __half* s_sc = reinterpret_cast<__half*>(smem + L::sc_off);
 
+    // ---- prologue: nothing here depends on the previous kernel in the stream
     if (tid == 0) {
-        for (int i = 0; i < NWS; ++i) { mbar_init(bar_wfull + 8 * i, 1); mbar_init(bar_wempty + 8 * i, 128); }
-        for (int i = 0; i < NS; ++i) { mbar_init(bar_xfull + 8 * i, 1); mbar_init(bar_afull + 8 * i, 128); mbar_init(bar_empty + 8 * i, 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(bar_accfull + 8 * i, 1); mbar_init(bar_accempty + 8 * i, 256); }
+        for (int i = 0; i < TC_NW_MAX; ++i) { mbar_init(bar_wfull + 8 * i, 1); mbar_init(bar_wempty + 8 * i, 4); }
+        for (int i = 0; i < NX; ++i) { mbar_init(bar_xfull + 8 * i, 4); mbar_init(bar_done + 8 * i, 1); }
+        for (int i = 0; i < 2; ++i) mbar_init(bar_afull + 8 * i, 8);
+        for (int i = 0; i < TC_NACC; ++i) { mbar_init(bar_accfull + 8 * i, 1); mbar_init(bar_accempty + 8 * i, 2 * TC_EPI); }
+        for (int i = 0; i < TC_NSC; ++i) mbar_init(bar_scfull + 8 * i, 4);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = tid; i <= p.E; i += TC_THREADS) s_off[i] = p.offsets[i];
-    if (warp == 1) tmem_alloc(sbase + L::misc_off, 2 * TN);
+    if (warp == 1) tmem_alloc_pair(sbase + L::misc_off, 512);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (warp == 0) {
+        // ---- the schedule: lane e works out expert e
+        const int e = lane;
+        const int o0 = e < p.E ? __ldcg(p.offsets + e) : 0, o1 = e < p.E ? __ldcg(p.offsets + e + 1) : 0;
+        const int R = o1 - o0, TN = 128 * NH;
+        const int mt = (R + TN - 1) / TN;
+        const int rpt = mt >= 4 ? TN : (mt > 0 ? ((R + mt - 1) / mt + 31) & ~31 : 32);
+        const int T_e = mt * p.NTP;
+        int incl = T_e;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += o;
+        }
+        const int T = __shfl_sync(0xffffffffu, incl, 31), tile0 = incl - T_e;
+        int Td = T;
+        if (p.split && T % nclusters != 0) Td = T >= 2 * nclusters ? (T / nclusters - 1) * nclusters : 0;
+        const int us = min(max(Td - tile0, 0), T_e) * p.KB;
+        const int cnt = T_e * p.KB - us;
+        // cost of a k-block: tensor cycles of its token columns, or what streaming and unpacking it takes
+        const int bits = e < p.E ? p.ex[e].bits : 4;
+        const int floor_cost = bits == 8 ? 700 : 450;
+        const int w = max(4 * min(rpt, TN), floor_cost);
+        const long long cost = (long long)cnt * w;
+        long long cincl = cost;
+        int wmax = cnt > 0 ? w : 1;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const long long o = __shfl_up_sync(0xffffffffu, cincl, d);
+            if (lane >= d) cincl += o;
+            wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, d));
+        }
+        const long long C = __shfl_sync(0xffffffffu, cincl, 31), base = cincl - cost;
+        // every cluster's share holds at least one unit's start
+        const int Gs = (int)min((long long)nclusters, C / wmax);
+        int ub = 0, ue = 0;
+        if (cnt > 0 && cluster < Gs) {
+            const long long den = (long long)w * Gs;
+            const long long n0 = (long long)cluster * C - base * Gs, n1 = (long long)(cluster + 1) * C - base * Gs;
+            const long long t0 = n0 <= 0 ? 0 : (n0 + den - 1) / den, t1 = n1 <= 0 ? 0 : (n1 + den - 1) / den;
+            ub = us + (int)min(t0, (long long)cnt);
+            ue = us + (int)min(t1, (long long)cnt);
+        }
+        if (e < p.E) { sc.off[e] = o0; sc.tile0[e] = tile0; }
+        if (e == p.E - 1) { sc.off[p.E] = o1; sc.tile0[p.E] = T; }
+        sc.rpt[e] = rpt; sc.us[e] = us; sc.ub[e] = ub; sc.ue[e] = ue; sc.w[e] = w; sc.base[e] = base;
+        if (lane == 0) { sc.misc[0] = Gs; sc.misc[1] = T; sc.misc[2] = Td; sc.base[32] = C; }
+    }
     tc_fence_before();
     __syncthreads();
+    cluster_sync();                                        // the pair's barriers are initialised, its TMEM allocated
     tc_fence_after();
     const uint32_t tmem_base = *s_tmem;
 
     if (warp < 4) {
-        if constexpr (REGSPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-        if (warp == 0 && lane == 0) {
-            // ---------------- X producer: TMA boxes of 64 token rows x 64 k ----------------
-            Ring ring;
-            TileInfo ti;
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        if (warp == 0 || warp == 3) {
+            // ---------------- X producers: this CTA's 64 token rows of every half tile, 128 k per stage ----------------
+            // Both warps walk the stages and arrive on the pair's xfull barrier; warp 0 also adds the byte count of the TMA
+            // boxes.  A warp gathers every other pair of rows; its arrival for a stage follows once its copies have landed,
+            // LAG stages later (at once where nothing is gathered).
+            constexpr int LAG = NX == 4 ? 3 : 4;
+            const int gw = warp == 0 ? 0 : 1;
+            int* s_xrow = reinterpret_cast<int*>(smem + L::xrow_off) + gw * 64 * NH;
+            const int hi = lane >> 4, c16 = lane & 15;
+            // byte offset of this lane's 16-byte chunk of row 4 i + 2 gw + hi: sub-tile, then the 128-byte swizzle
+            const uint32_t r0 = 2 * gw + hi;
+            const uint32_t sw0 = (c16 >> 3) * 8192 + r0 * 128 + (((c16 & 7) ^ r0) << 4), sw1 = (c16 >> 3) * 8192 + (r0 + 4) * 128 + (((c16 & 7) ^ (r0 + 4)) << 4);
+            Ring ring, aring;                              // aring: the stage whose arrival is due next
+            TcPiece pc;
+            TcWalk wk;
+            wk.start(cluster);
             bool ok = true;
-            for (int t = blockIdx.x; ok && decode_tile<TN>(s_off, p.E, p.n_tiles, t, ti); t += gridDim.x) {
-                const int nbox = (ti.rows + XBOX_ROWS - 1) / XBOX_ROWS;
-                // where each 64-row box of this tile comes from: straight from X when its rows are consecutive there
-                int box0 = (ti.m0 - s_off[ti.e]) / XBOX_ROWS;
-                for (int e2 = 0; e2 < ti.e; ++e2) box0 += (s_off[e2 + 1] - s_off[e2] + XBOX_ROWS - 1) / XBOX_ROWS;
-                int src_row[TN / XBOX_ROWS];
+            int pending = 0;
+            const uint32_t full0 = mapa(bar_xfull, 0);
+            auto arrive = [&]() {
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) remote_arrive(full0 + 8 * aring.stage);
+                aring.advance(NX);
+            };
+            while (ok && wk.next(sc, p, nclusters, pc)) {
+                const int nh = NH == 1 ? 1 : (pc.rows > 128 ? 2 : 1);
+                int src[NH], cnt[NH], bytes = 0;
+                bool gathers = false;
+                __syncwarp();
 #pragma unroll
-                for (int b = 0; b < TN / XBOX_ROWS; ++b) src_row[b] = b < nbox ? p.box_src[box0 + b] : -1;
-                for (int ks = 0; ks < 2 * p.KB; ++ks) {
-                    if (!(ok = mbar_wait(bar_empty + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status))) break;
-                    const uint32_t full = bar_xfull + 8 * ring.stage;
-                    mbar_expect_tx(full, nbox * XBOX_BYTES);
-                    const uint32_t dst = sbase + L::x_off + ring.stage * (TN * 128);
+                for (int h = 0; h < NH; ++h) {
+                    src[h] = -1; cnt[h] = 0;
+                    if (h < nh) {
+                        const int per_cta = half_cols(pc.rows, h) >> 1;
+                        const int first_row = h * 128 + (int)rank * per_cta;
+                        const int c = max(min(per_cta, pc.rows - first_row), 0);         // real rows of this CTA
+                        const int a = lane < c ? __ldcg(p.perm + pc.m0 + first_row + lane) : 0;
+                        const int b = lane + 32 < c ? __ldcg(p.perm + pc.m0 + first_row + lane + 32) : 0;
+                        const int first = __shfl_sync(0xffffffffu, a, 0);
+                        const bool run = __all_sync(0xffffffffu, (lane >= c || a == first + lane) && (lane + 32 >= c || b == first + lane + 32));
+                        s_xrow[h * 64 + lane] = a;
+                        s_xrow[h * 64 + lane + 32] = b;
+                        // (a box fetches 64 rows whatever it needs; operand rows beyond the real ones yield columns that are
+                        // never stored, so they may hold anything)
+                        src[h] = run && c >= 32 ? first : -1;
+                        cnt[h] = c;
+                        bytes += src[h] >= 0 ? TC_XHALF : 0;
+                        gathers |= src[h] < 0 && c > 0;
+                    }
+                }
+                __syncwarp();
+                for (int kb = pc.kb0; kb < pc.kb1; ++kb) {
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status)))) break;
+                    const uint32_t stage = sbase + L::x_off + ring.stage * L::xstage;
+                    if (gw == 0 && bytes > 0) {
+                        const uint32_t full = full0 + 8 * ring.stage;
+                        if (lane == 0) remote_expect_tx_only(full, bytes);
+                        __syncwarp();
 #pragma unroll
-                    for (int b = 0; b < TN / XBOX_ROWS; ++b) {
-                        if (b < nbox) {
-                            if (src_row[b] >= 0) tma_load_2d(dst + b * XBOX_BYTES, &tmap_x, ks * 64, src_row[b], full);
-                            else tma_load_2d(dst + b * XBOX_BYTES, &tmap, ks * 64, ti.m0 + b * XBOX_ROWS, full);
+                        for (int h = 0; h < NH; ++h)
+                            if (src[h] >= 0 && lane < 2) tma_box_pair(stage + h * TC_XHALF + lane * 8192, &tmap, kb * 128 + lane * 64, src[h], full);
+                        __syncwarp();
+                    }
+                    const int k = kb * 128 + c16 * 8;
+                    const int real = k < p.K ? 16 : 0;
+                    const char* xk = reinterpret_cast<const char*>(p.X) + (real ? (size_t)k * 2 : 0);
+#pragma unroll
+                    for (int h = 0; h < NH; ++h) {
+                        if (src[h] < 0) {
+                            const uint32_t dst = stage + h * TC_XHALF;
+#pragma unroll 4
+                            for (int i = 0; i < 16; ++i) {
+                                const int r = 4 * i + (int)r0;
+                                if (4 * i + 2 * gw >= cnt[h]) break;
+                                if (r < cnt[h])
+                                    cp_async16(dst + ((i & 1) ? sw1 : sw0) + (i >> 1) * 1024, xk + (size_t)s_xrow[h * 64 + r] * (size_t)(p.K * 2), real);
+                            }
                         }
                     }
-                    ring.advance(NS);
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                    ring.advance(NX);
+                    ++pending;
+                    if (!gathers) {
+                        asm volatile("cp.async.wait_group 0;" ::: "memory");
+                        for (; pending > 0; --pending) arrive();
+                    } else if (pending == LAG) {
+                        asm volatile("cp.async.wait_group %0;" ::"n"(LAG - 1) : "memory");
+                        arrive();
+                        --pending;
+                    }
                 }
             }
-        } else if (warp == 2 && lane == 0) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            for (; ok && pending > 0; --pending) arrive();
+            // every stage handed back (the commits come from the leading CTA) before this CTA may exit
+            for (int i = 0; ok && i < NX; ++i) {
+                ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status));
+                ring.advance(NX);
+            }
+        } else if (warp == 2) {
             // ---------------- W producer: one packed 128x128-code tile per k-block ----------------
-            Ring ring;
-            TileInfo ti;
-            bool ok = true;
-            for (int t = blockIdx.x; ok && decode_tile<TN>(s_off, p.E, p.n_tiles, t, ti); t += gridDim.x) {
-                const ExpertDev& ex = p.ex[ti.e];
-                const uint32_t bytes = (uint32_t)ex.tile_stride;          // codes + the tile's scales / zero-points
-                const uint8_t* src = ex.tiles + (size_t)ti.nt * p.KB * bytes;
-                for (int kb = 0; kb < p.KB; ++kb) {
-                    if (!(ok = mbar_wait(bar_wempty + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status))) break;
-                    const uint32_t full = bar_wfull + 8 * ring.stage;
-                    mbar_expect_tx(full, bytes);
-                    bulk_load(sbase + L::w_off + ring.stage * W_STAGE_BYTES, src + (size_t)kb * bytes, bytes, full);
-                    ring.advance(NWS);
+            if (lane == 0) {
+                Ring ring;
+                TcPiece pc;
+                TcWalk wk;
+                wk.start(cluster);
+                bool ok = true;
+                while (ok && wk.next(sc, p, nclusters, pc)) {
+                    const int nt = 2 * pc.ntp + (int)rank;
+                    if (nt >= p.NT1) continue;                              // the second half of the last, odd pair
+                    const ExpertDev& ex = p.ex[pc.e];
+                    const uint32_t bytes = (uint32_t)ex.tile_stride;        // codes + the tile's scales / zero-points
+                    const uint8_t* src = ex.tiles + ((size_t)nt * p.KB + pc.kb0) * bytes;
+                    for (int kb = pc.kb0; kb < pc.kb1; ++kb, src += bytes) {
+                        if (!(ok = mbar_wait(bar_wempty + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status))) break;
+                        const uint32_t full = bar_wfull + 8 * ring.stage;
+                        mbar_expect_tx(full, bytes);
+                        bulk_load(sbase + L::w_off + ring.stage * p.wstage, src, bytes, full);
+                        ring.advance(p.nw);
+                    }
                 }
             }
-        } else if (warp == 1) {
-            // ---------------- MMA issuer ----------------
+        } else if (warp == 1 && rank == 0) {
+            // ---------------- MMA issuer (the leading CTA's, for the pair) ----------------
             // (Its waits spin on the plain try_wait: they sit on the critical path and coming round a short spin is
             // faster than waking from the hinted sleep.)
-            // The WHOLE warp walks the tiles, so that control flow stays warp-uniform, and one elected lane issues
-            // straight-line MMAs whose operands were all computed beforehand.  Measured on B200: issued this way a
-            // 128x256x16 MMA costs its 128 tensor-pipe cycles (and a 16-column one 24); issued from a loop that
-            // only lane 0 runs (`if (lane == 0)`) and that builds descriptors between MMAs, every MMA costs ~250.
+            // The WHOLE warp walks the pieces, so that control flow stays warp-uniform, and one elected lane issues
+            // straight-line MMAs whose operands were all computed beforehand: issued from a loop that only lane 0
+            // runs, every MMA costs ~250 cycles.
             Ring ring;
-            TileInfo ti;
+            TcPiece pc;
+            TcWalk wk;
+            wk.start(cluster);
             bool ok = true;
-            uint32_t acc_use[2] = {0, 0};
+            uint32_t kcount = 0;                           // k-blocks so far (weight buffers alternate)
             int buf = 0;
-            for (int t = blockIdx.x; ok && decode_tile<TN>(s_off, p.E, p.n_tiles, t, ti); t += gridDim.x) {
-                const ExpertDev& ex = p.ex[ti.e];
-                const int n_eff = (ti.rows + 15) & ~15;
-                const uint32_t idesc = umma_idesc(n_eff);
-                const int group_k = ex.group == 0 ? p.KB * 128 : min(ex.group, 128);
-                int kcount = 0;
-                for (int ks = 0; ok && ks < 2 * p.KB; ++ks) {
-                    if (!(ok = __all_sync(0xffffffffu, mbar_wait_short(bar_xfull + 8 * ring.stage, ring.phase, s_abort, p.status)))) break;
-                    if (!(ok = __all_sync(0xffffffffu, mbar_wait_short(bar_afull + 8 * ring.stage, ring.phase, s_abort, p.status)))) break;
-                    const uint64_t adesc = umma_desc_sw128(sbase + L::a_off + ring.stage * A_STAGE_BYTES);
-                    const uint64_t bdesc = umma_desc_sw128(sbase + L::x_off + ring.stage * (TN * 128));
-                    const uint32_t empty_bar = bar_empty + 8 * ring.stage;
-                    if (group_k >= 64) {
-                        // the stage's four MMAs feed one accumulator buffer
-                        if (kcount == 0 &&
-                            !(ok = __all_sync(0xffffffffu, mbar_wait_short(bar_accempty + 8 * buf, (acc_use[buf] & 1u) ^ 1u, s_abort, p.status)))) break;
-                        tc_fence_after();
-                        const uint32_t d = tmem_base + buf * TN;
-                        const bool group_ends = kcount + 64 == group_k;
-                        if (elect_one()) {
-                            umma_bf16(d, adesc, bdesc, idesc, kcount > 0 ? 1u : 0u);
-                            umma_bf16(d, adesc + 2, bdesc + 2, idesc, 1u);
-                            umma_bf16(d, adesc + 4, bdesc + 4, idesc, 1u);
-                            umma_bf16(d, adesc + 6, bdesc + 6, idesc, 1u);
-                            if (group_ends) umma_commit(bar_accfull + 8 * buf);
-                            umma_commit(empty_bar);
-                        }
-                        __syncwarp();
-                        kcount += 64;
-                        if (group_ends) {
-                            acc_use[buf]++;
-                            buf ^= 1;
-                            kcount = 0;
-                        }
-                    } else {
-                        // groups of 32 k: two accumulator buffers per stage
-                        tc_fence_after();
-                        for (int j = 0; ok && j < 4; ++j) {
-                            if (kcount == 0) {
-                                if (!(ok = __all_sync(0xffffffffu, mbar_wait_short(bar_accempty + 8 * buf, (acc_use[buf] & 1u) ^ 1u, s_abort, p.status)))) break;
-                                tc_fence_after();
-                            }
-                            const bool group_ends = kcount + 16 == group_k;
+            uint32_t buf_phase = 1;                        // parity of "empty" for the buffers of this round
+            auto next_buf = [&]() { if (++buf == TC_NACC) { buf = 0; buf_phase ^= 1u; } };
+            while (ok && wk.next(sc, p, nclusters, pc)) {
+                const int nh = NH == 1 ? 1 : (pc.rows > 128 ? 2 : 1);
+                const int group = p.ex[pc.e].group;
+                // A per-channel expert's half tile h stays in buffer (buf + h) of the rotation for the whole piece.
+                const bool keep = group == 0;
+                const int steps = keep || group >= 128 ? 8 : group >> 4;         // MMAs into one accumulator buffer
+                for (int kb = pc.kb0; ok && kb < pc.kb1; ++kb, ++kcount) {
+                    const uint32_t ab = kcount & 1u;
+                    ok = __all_sync(0xffffffffu, mbar_wait_short(bar_xfull + 8 * ring.stage, ring.phase, s_abort, p.status));
+                    ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_afull + 8 * ab, (kcount >> 1) & 1u, s_abort, p.status));
+                    tc_fence_after();
+                    const uint32_t a_tmem = tmem_base + TC_A_BASE + ab * TC_A_COLS;
+                    const uint32_t done = bar_done + 8 * ring.stage;
+#pragma unroll 1
+                    for (int h = 0; h < nh; ++h) {
+                        const uint32_t idesc = umma_idesc_pair(half_cols(pc.rows, h));
+                        const uint64_t bdesc = umma_desc_sw128(sbase + L::x_off + ring.stage * L::xstage + h * TC_XHALF);
+                        const bool last_half = h + 1 == nh;
+                        if (steps == 8) {
+                            const int b2 = keep && h ? (buf + 1 == TC_NACC ? 0 : buf + 1) : buf;
+                            const uint32_t ph = keep && h && buf + 1 == TC_NACC ? buf_phase ^ 1u : buf_phase;
+                            const uint32_t add = keep && kb > pc.kb0 ? 1u : 0u;
+                            if (!add) ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_accempty + 8 * b2, ph, s_abort, p.status));
+                            tc_fence_after();
+                            const uint32_t d = tmem_base + b2 * TC_ACC_COLS;
                             if (elect_one()) {
-                                umma_bf16(tmem_base + buf * TN, adesc + 2 * j, bdesc + 2 * j, idesc, kcount > 0 ? 1u : 0u);
-                                if (group_ends) umma_commit(bar_accfull + 8 * buf);
-                                if (j == 3) umma_commit(empty_bar);
+#pragma unroll
+                                for (int i = 0; i < 8; ++i)
+                                    umma_pair_ts(d, a_tmem + 8 * i, bdesc + (i >> 2) * 512 + (i & 3) * 2, idesc, i > 0 ? 1u : add);
+                                if (keep) {
+                                    if (last_half) umma_commit_pair(done);
+                                    if (kb + 1 == pc.kb1) umma_commit_pair(bar_accfull + 8 * b2);
+                                } else {
+                                    umma_commit_pair(last_half ? done : bar_accfull + 8 * b2);
+                                }
                             }
                             __syncwarp();
-                            kcount += 16;
-                            if (group_ends) {
-                                acc_use[buf]++;
-                                buf ^= 1;
-                                kcount = 0;
+                            if (!keep) next_buf();
+                        } else {
+#pragma unroll 1
+                            for (int i0 = 0; i0 < 8; i0 += steps) {
+                                ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_accempty + 8 * buf, buf_phase, s_abort, p.status));
+                                tc_fence_after();
+                                const uint32_t d = tmem_base + buf * TC_ACC_COLS;
+                                const uint64_t bd = bdesc + (i0 >> 2) * 512 + (i0 & 3) * 2;
+                                if (elect_one()) {
+                                    umma_pair_ts(d, a_tmem + 8 * i0, bd, idesc, 0u);
+                                    umma_pair_ts(d, a_tmem + 8 * i0 + 8, bd + 2, idesc, 1u);
+                                    if (steps == 4) {
+                                        umma_pair_ts(d, a_tmem + 8 * i0 + 16, bd + 4, idesc, 1u);
+                                        umma_pair_ts(d, a_tmem + 8 * i0 + 24, bd + 6, idesc, 1u);
+                                    }
+                                    umma_commit_pair(last_half && i0 + steps == 8 ? done : bar_accfull + 8 * buf);
+                                }
+                                __syncwarp();
+                                next_buf();
                             }
                         }
-                        if (!ok) break;
                     }
-                    ring.advance(NS);
+                    ring.advance(NX);
                 }
+                if (keep) for (int h = 0; h < nh; ++h) next_buf();
             }
         }
-    } else if (warp < 8) {
-        if constexpr (REGSPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
-        // ---------------- dequant warps ----------------
-        Ring wring, ring;
-        TileInfo ti;
+    } else if (warp < L::epi_warp0) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+        // ---------------- dequant warps: thread = channel = TMEM lane ----------------
+        const int row = (warp & 3) * 32 + lane;
+        const uint32_t my_group = NH == 2 ? 0u : (uint32_t)((warp - 4) >> 2);
+        const uint32_t afull0 = mapa(bar_afull, 0);
+        const uint32_t lane_tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + TC_A_BASE;
+        Ring wring, dring;
+        TcPiece pc;
+        TcWalk wk;
+        wk.start(cluster);
         bool ok = true;
-        for (int t = blockIdx.x; ok && decode_tile<TN>(s_off, p.E, p.n_tiles, t, ti); t += gridDim.x) {
-            const ExpertDev& ex = p.ex[ti.e];
-            for (int kb = 0; ok && kb < p.KB; ++kb) {
-                unsigned char* sw = smem + L::w_off + wring.stage * W_STAGE_BYTES;
-                const uint32_t wf = bar_wfull + 8 * wring.stage, we = bar_wempty + 8 * wring.stage;
-                if (ex.bits == 4)
-                    ok = dequant_kblock<4>(ex, ti.nt, sw, smem + L::a_off, wf, we, wring.phase, bar_empty, bar_afull, ring, s_abort, p.status);
-                else if (ex.bits == 8)
-                    ok = dequant_kblock<8>(ex, ti.nt, sw, smem + L::a_off, wf, we, wring.phase, bar_empty, bar_afull, ring, s_abort, p.status);
-                else if (W2 && ex.bits == 2) {
-                    if constexpr (W2)
-                        ok = dequant_kblock<2>(ex, ti.nt, sw, smem + L::a_off, wf, we, wring.phase, bar_empty, bar_afull, ring, s_abort, p.status);
-                } else
-                    ok = dequant_kblock<3>(ex, ti.nt, sw, smem + L::a_off, wf, we, wring.phase, bar_empty, bar_afull, ring, s_abort, p.status);
-                wring.advance(NWS);
+        uint32_t kcount = 0;
+        while (ok && wk.next(sc, p, nclusters, pc)) {
+            const ExpertDev& ex = p.ex[pc.e];
+            const int nt = 2 * pc.ntp + (int)rank;
+            const bool active = nt < p.NT1;
+            const bool tile_zeros = ex.has_zeros && ex.group != 0;
+            float z = (float)(1 << (ex.bits - 1));
+            if (ex.has_zeros && ex.group == 0 && active) z = __bfloat162float(ex.zeros_pc[nt * 128 + row]);
+            const uint32_t zpc = neg_z(z);
+            for (int kb = pc.kb0; ok && kb < pc.kb1; ++kb, ++kcount) {
+                const uint32_t ab = kcount & 1u;
+                const bool mine = NH == 2 || ab == my_group;
+                // the buffer is free once the k-block before the last is done
+                const uint32_t free_bar = kcount >= 2 ? bar_done + 8 * dring.stage : 0u;
+                const uint32_t scfull = bar_scfull + 8 * (kcount & (TC_NSC - 1));
+                if (mine && active) {
+                    const unsigned char* tile = smem + L::w_off + wring.stage * p.wstage;
+                    __half* scales = s_sc + (kcount & (TC_NSC - 1)) * 512;
+                    const uint32_t wf = bar_wfull + 8 * wring.stage, we = bar_wempty + 8 * wring.stage, at = lane_tmem + ab * TC_A_COLS;
+                    switch (ex.bits) {
+                        case 4: ok = dequant_kblock<4>(ex, tile, row, zpc, tile_zeros, scales, scfull, wf, wring.phase, we, free_bar, dring.phase, at, s_abort, p.status); break;
+                        case 8: ok = dequant_kblock<8>(ex, tile, row, zpc, tile_zeros, scales, scfull, wf, wring.phase, we, free_bar, dring.phase, at, s_abort, p.status); break;
+                        case 3: ok = dequant_kblock<3>(ex, tile, row, zpc, tile_zeros, scales, scfull, wf, wring.phase, we, free_bar, dring.phase, at, s_abort, p.status); break;
+                        default: ok = dequant_kblock<2>(ex, tile, row, zpc, tile_zeros, scales, scfull, wf, wring.phase, we, free_bar, dring.phase, at, s_abort, p.status); break;
+                    }
+                } else if (mine) {
+                    // no channels here: the operand buffer keeps whatever it holds (those products are never read)
+                    if (lane == 0) mbar_arrive(scfull);
+                    if (free_bar) ok = __all_sync(0xffffffffu, mbar_wait_short(free_bar, dring.phase, s_abort, p.status));
+                }
+                if (mine) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) remote_arrive(afull0 + 8 * ab);
+                }
+                if (active) wring.advance(p.nw);
+                if (kcount >= 2) dring.advance(NX);
             }
         }
     } else {
-        if constexpr (REGSPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 184;");
+        if constexpr (NH == 2) asm volatile("setmaxnreg.inc.sync.aligned.u32 184;");
+        else asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
         // ---------------- epilogue warps: scale-and-accumulate, then store ----------------
-        constexpr int NCOL = TN / 2;                       // columns (tokens) per warp
-        const int ew = warp - 8, quarter = ew & 3, colhalf = ew >> 2;
-        const int col0 = colhalf * NCOL;
-        const int row = quarter * 32 + lane;               // channel inside the tile = TMEM lane
-        TileInfo ti;
+        const int ew = warp - L::epi_warp0, quarter = warp & 3, colhalf = ew >> 2;
+        const int row = quarter * 32 + lane;               // channel inside the 128-channel tile = TMEM lane
+        const int col0 = colhalf * 64;                     // this warp's columns of every half tile
+        const uint32_t accempty0 = mapa(bar_accempty, 0);
+        const uint32_t lane_tmem = tmem_base + ((uint32_t)(quarter * 32) << 16) + col0;
+        int* my_perm = s_perm + ew * 64 * NH;              // private to this warp: no cross-warp barrier
+        TcPiece pc;
+        TcWalk wk;
+        wk.start(cluster);
         bool ok = true;
-        uint32_t acc_use[2] = {0, 0};
         int buf = 0;
-        for (int t = blockIdx.x; ok && decode_tile<TN>(s_off, p.E, p.n_tiles, t, ti); t += gridDim.x) {
-            const ExpertDev& ex = p.ex[ti.e];
-            const int n = ti.nt * 128 + row;
-            const int n_eff = (ti.rows + 15) & ~15;
-            int* my_perm = s_perm + ew * NCOL;                     // private to this warp: no cross-warp barrier
+        uint32_t full_phase = 0;                           // bit b: parity of the next arrival on accfull[b]
+        uint32_t kcount = 0;
+        Ring dring;                                        // the k-block whose last accumulator is drained next
+        while (ok && wk.next(sc, p, nclusters, pc)) {
+            const ExpertDev& ex = p.ex[pc.e];
+            const int nt = 2 * pc.ntp + (int)rank, n = nt * 128 + row;
+            const bool active = nt < p.NT1;
+            const int nh = NH == 1 ? 1 : (pc.rows > 128 ? 2 : 1);
             __syncwarp();
-            for (int i = lane; i < NCOL; i += 32) my_perm[i] = (col0 + i < ti.rows) ? p.perm[ti.m0 + col0 + i] : -1;
+#pragma unroll
+            for (int i = 0; i < 2 * NH; ++i) {
+                const int col = (i >> 1) * 128 + col0 + (i & 1) * 32 + lane;
+                my_perm[i * 32 + lane] = col < pc.rows ? __ldcg(p.perm + pc.m0 + col) : -1;
+            }
             __syncwarp();
-            float acc[NCOL];
+            float acc[NH][64];
 #pragma unroll
-            for (int i = 0; i < NCOL; ++i) acc[i] = 0.f;
-            const int group_k = ex.group == 0 ? p.KB * 128 : min(ex.group, 128);
-            const int ngroups = p.KB * 128 / group_k;
-            for (int gi = 0; ok && gi < ngroups; ++gi) {
-                float s;
-                if (ex.group == 0) {
-                    s = __half2float(ex.scales_pc[n]);
-                } else {                                   // the scale sits in the meta of the tile the group lies in
-                    const int per_tile = moqe_groups_per_tile(ex.group);
-                    const unsigned char* tile = ex.tiles + ((size_t)ti.nt * p.KB + gi / per_tile) * (size_t)ex.tile_stride;
-                    s = __half2float(moqe_tile_scales(tile, ex.bits, ex.has_zeros, gi % per_tile)[row]);
-                }
-                if (ex.bits == 8) s *= W8_PRESCALE;          // 8-bit chunks are unpacked as (c - z) * 2^-13
-                if (!(ok = mbar_wait(bar_accfull + 8 * buf, acc_use[buf] & 1u, s_abort, p.status))) break;
-                tc_fence_after();
+            for (int h = 0; h < NH; ++h)
 #pragma unroll
-                for (int c = 0; c < NCOL / 32; ++c) {
-                    if (col0 + c * 32 < n_eff) {
-                        uint32_t v[32];
-                        tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * TN + col0 + c * 32, v);
-                        tmem_ld_wait();
-                        // acc += s * v, two columns per instruction (each half rounds as a scalar fma does)
+                for (int i = 0; i < 64; ++i) acc[h][i] = 0.f;
+            // One round per k-block (grouped: every group's buffer is drained, the last one of the k-block being announced by
+            // the k-block's own barrier) or one for the whole piece (per channel).  The loops are kept rolled: unrolled over
+            // the groups and the barriers' outcomes the kernel was 235 KB of code and spent a quarter of its warps' time
+            // fetching instructions.
+            const bool keep = ex.group == 0;
+            const int per = keep ? 1 : moqe_groups_per_tile(ex.group), rounds = keep ? 1 : pc.kb1 - pc.kb0;
+            const float s_pc = keep && active ? __half2float(ex.scales_pc[n]) * W8_PRESCALE : 0.f;   // (weights are unpacked as (c - z) * 2^-13)
+#pragma unroll 1
+            for (int it = 0; ok && it < rounds; ++it) {
+                const uint32_t slot = kcount & (TC_NSC - 1);
+                // (slot reuse: the dequant warps write k-block k after k - 2 is done, and three buffers bound how far the
+                // drains may be behind)
+                if (!keep) ok = __all_sync(0xffffffffu, mbar_wait_short(bar_scfull + 8 * slot, (kcount / TC_NSC) & 1u, s_abort, p.status));
 #pragma unroll
-                        for (int i = 0; i < 32; i += 2)
-                            asm("{\n\t.reg .b64 a, x, s2;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 x, {%3, %4};\n\tmov.b64 s2, {%2, %2};\n\t"
-                                "fma.rn.f32x2 a, s2, x, a;\n\tmov.b64 {%0, %1}, a;\n\t}"
-                                : "+f"(acc[c * 32 + i]), "+f"(acc[c * 32 + i + 1]) : "f"(s), "r"(v[i]), "r"(v[i + 1]));
+                for (int h = 0; h < NH; ++h) {
+                    if (h < nh) {
+                        const int cols = half_cols(pc.rows, h);
+#pragma unroll 1
+                        for (int j = 0; j < per; ++j) {
+                            const bool by_done = !keep && h + 1 == nh && j + 1 == per;
+                            const uint32_t bar = by_done ? bar_done + 8 * dring.stage : bar_accfull + 8 * buf;
+                            const uint32_t phase = by_done ? dring.phase : (full_phase >> buf) & 1u;
+                            const float s = keep ? s_pc : __half2float(s_sc[slot * 512 + j * 128 + row]) * W8_PRESCALE;
+                            ok &= __all_sync(0xffffffffu, mbar_wait_short(bar, phase, s_abort, p.status));
+                            if (!by_done) full_phase ^= 1u << buf;
+                            tc_fence_after();
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) {
+                                if (col0 + 32 * c < cols) {
+                                    uint32_t v[32];
+                                    tmem_ld32(lane_tmem + buf * TC_ACC_COLS + 32 * c, v);
+                                    tmem_ld_wait();
+                                    fma_cols32(acc[h] + 32 * c, v, s);
+                                }
+                            }
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) remote_arrive(accempty0 + 8 * buf);
+                            if (++buf == TC_NACC) buf = 0;
+                        }
                     }
                 }
-                tc_fence_before();
-                mbar_arrive(bar_accempty + 8 * buf);
-                acc_use[buf]++;
-                buf ^= 1;
+                if (!keep) { dring.advance(NX); ++kcount; }
             }
-            if (ok && n < p.N) {
+            if (keep) {
+                const int k = dring.stage + (pc.kb1 - pc.kb0);
+                dring.phase ^= (uint32_t)(k / NX) & 1u;
+                dring.stage = k % NX;
+                kcount += pc.kb1 - pc.kb0;
+            }
+            if (!ok) break;
+            if (!active) continue;
+            if (pc.kb0 != 0 || pc.kb1 != p.KB) {
+                // part of a tile: park this warp's sums, announce, and add everything up if this was the last arrival
+                const long long C = sc.base[32], first = sc.base[pc.e] + (long long)(pc.tile * p.KB - sc.us[pc.e]) * sc.w[pc.e];
+                const int Gs = sc.misc[0];
+                const int c_a = (int)(first * Gs / C), c_b = (int)((first + (long long)(p.KB - 1) * sc.w[pc.e]) * Gs / C);
+                const size_t slot = (size_t)p.cols * 128;
+                auto slot_of = [&](int c, int which) { return p.partials + ((size_t)(c * 2 + which) * 2 + rank) * slot + (size_t)col0 * 128 + row; };
+                {
+                    float* dst = slot_of(cluster, pc.kb0 == 0 ? 1 : 0);
 #pragma unroll
-                for (int i = 0; i < NCOL; ++i) {
-                    const int col = col0 + i;
-                    if (col < ti.rows) p.Y[(size_t)my_perm[i] * p.N + n] = __bfloat16_as_ushort(__float2bfloat16_rn(acc[i]));
+                    for (int h = 0; h < NH; ++h)
+#pragma unroll
+                        for (int i0 = 0; i0 < 64; i0 += 8)
+                            if (h * 128 + col0 + i0 < pc.rows) {
+#pragma unroll
+                                for (int i = i0; i < i0 + 8; ++i) __stcg(dst + (size_t)(h * 128 + i) * 128, acc[h][i]);
+                            }
                 }
+                __syncwarp();
+                unsigned* counter = p.counters + (c_a * 2 + (int)rank) * TC_EPI + ew;
+                unsigned arrived = 0;
+                // one acquire-release increment: the release side publishes the warp's parked sums (ordered before it by the
+                // warp barrier above), the acquire side lets the last arriver read everybody else's
+                if (lane == 0) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(counter) : "memory");
+                arrived = __shfl_sync(0xffffffffu, arrived, 0);
+                if (arrived != (unsigned)(c_b - c_a)) continue;
+                __syncwarp();
+#pragma unroll
+                for (int h = 0; h < NH; ++h)
+#pragma unroll
+                    for (int i = 0; i < 64; ++i) acc[h][i] = 0.f;
+#pragma unroll 1
+                for (int c = c_a; c <= c_b; ++c) {
+                    const float* src = slot_of(c, c == c_a ? 1 : 0);
+#pragma unroll
+                    for (int h = 0; h < NH; ++h)
+#pragma unroll
+                        for (int i0 = 0; i0 < 64; i0 += 8)
+                            if (h * 128 + col0 + i0 < pc.rows) {
+                                float v[8];
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) v[i] = __ldcg(src + (size_t)(h * 128 + i0 + i) * 128);
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) acc[h][i0 + i] += v[i];
+                            }
+                }
+                if (lane == 0) *counter = 0u;
             }
+            // Store: lanes hold neighbouring channels, registers tokens.  Neighbouring lanes swap one of every two tokens, so
+            // that a lane writes two channels of one token.
+            const int odd = lane & 1;
+            uint16_t* y = p.Y + (n & ~1);
+#pragma unroll
+            for (int h = 0; h < NH; ++h)
+#pragma unroll
+                for (int i0 = 0; i0 < 64; i0 += 8)
+                    if (h * 128 + col0 + i0 < pc.rows) {
+#pragma unroll
+                        for (int i = i0; i < i0 + 8; i += 2) {
+                            const uint32_t mine = pack_bf16x2(acc[h][i], acc[h][i + 1]);
+                            const uint32_t other = __shfl_xor_sync(0xffffffffu, mine, 1);
+                            const uint32_t pair = __byte_perm(mine, other, odd ? 0x3276u : 0x5410u);
+                            const int to = my_perm[h * 64 + i + odd];
+                            if (to >= 0 && n < p.N) *reinterpret_cast<uint32_t*>(y + (size_t)to * p.N) = pair;
+                        }
+                    }
         }
     }
 
@@ -416,12 +824,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) qgemm_tc_kernel(const __grid_co
         // let bulk copies that may still be in flight land before the shared memory is released
         unsigned long long t0 = global_ns();
         while (global_ns() - t0 < 200000ull) __nanosleep(1000);
-        __syncthreads();
     }
+    cluster_sync();                                        // the peer no longer touches this CTA's barriers or TMEM
     if (warp == 1) {
-        __syncwarp();
         tc_fence_after();
-        tmem_dealloc(tmem_base, 2 * TN);
+        tmem_dealloc_pair(tmem_base, 512);
     }
 }
 
@@ -430,85 +837,77 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const EncodeTiledFn fn = []() -> EncodeTiledFn {
         void* f = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)f;
-    }
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+            return (EncodeTiledFn)f;
+        return nullptr;
+    }();
     return fn;
 }
 
-int g_tile_tokens_override = 0;
+// columns of a parked partial sum: no tile has more tokens than the batch
+int tc_cols(int M) { return M >= 256 ? 256 : (M + 31) / 32 * 32; }
 
 }  // namespace
 
-void tc_set_tile_tokens(int tn) { g_tile_tokens_override = tn; }
+size_t tc_zero_bytes() { return (size_t)TC_MAX_CLUSTERS * 2 * TC_EPI * sizeof(uint32_t); }
 
 size_t tc_workspace_bytes(int M, int K, int E, int Np) {
-    (void)Np;
-    return ((size_t)M * K * 2 + 255) / 256 * 256 + gather_boxes_bytes(M, E);
+    (void)K; (void)E; (void)Np;
+    return (tc_zero_bytes() + 255) / 256 * 256 + (size_t)TC_MAX_CLUSTERS * 4 * tc_cols(M) * 128 * sizeof(float);
 }
 
 moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_expert* const* ex, int E, void* Y,
-                            const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes, cudaStream_t st) {
+                            const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes, int tile_tokens, cudaStream_t st) {
     if (M == 0) return MOQE_OK;
     if (!ws || ws_bytes < tc_workspace_bytes(M, K, E, ex[0]->Np)) return MOQE_ERR_WORKSPACE;
     EncodeTiledFn enc = encode_fn();
     if (!enc) return MOQE_ERR_CUDA;
-    // 1. expert-sorted copy of the activations (rows with an invalid id become zero rows at the end)
-    void* Xp = ws;
-    int32_t* box_src = (int32_t*)((char*)ws + ((size_t)M * K * 2 + 255) / 256 * 256);
-    moqe_status s = launch_gather_boxes(X, perm, offsets, M, K, E, Xp, box_src, st);
-    if (s != MOQE_OK) return s;
-    // 2. tensor map over Xp[M][K] bf16: boxes of 64 k x 64 rows, 128-byte swizzle, zero fill outside
+    // tensor map over X[M][K] bf16: boxes of 64 k x 64 rows, 128-byte swizzle, zero fill outside
     CUtensorMap tmap;
     cuuint64_t gdim[2] = {(cuuint64_t)K, (cuuint64_t)M};
     cuuint64_t gstride[1] = {(cuuint64_t)K * 2};
-    cuuint32_t box[2] = {64, (cuuint32_t)XBOX_ROWS};
-    cuuint32_t estr[2] = {1, 1};
-    if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Xp, gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return MOQE_ERR_CUDA;
-    CUtensorMap tmap_x;                                   // the same boxes over the caller's X (unsorted rows)
-    if (enc(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(X), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    cuuint32_t box[2] = {64, 64}, estr[2] = {1, 1};
+    if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(X), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return MOQE_ERR_CUDA;
     TcParams p;
+    int stride = 0;
     for (int e = 0; e < E; ++e) {
         p.ex[e] = ex[e]->dev();
+        stride = p.ex[e].tile_stride > stride ? p.ex[e].tile_stride : stride;
     }
-    p.box_src = box_src;
-    p.perm = perm; p.offsets = offsets; p.Y = (uint16_t*)Y; p.status = device_status_word();
-    p.M = M; p.N = N; p.K = K; p.Np = ex[0]->Np; p.KB = ex[0]->Kp / 128; p.E = E; p.n_tiles = p.Np / 128;
+    p.perm = perm; p.offsets = offsets; p.X = (const uint16_t*)X; p.Y = (uint16_t*)Y; p.status = device_status_word();
+    p.counters = (uint32_t*)ws;
+    p.partials = (float*)((char*)ws + (tc_zero_bytes() + 255) / 256 * 256);
+    p.M = M; p.N = N; p.K = K; p.KB = ex[0]->Kp / 128; p.E = E; p.NT1 = ex[0]->Np / 128; p.NTP = (p.NT1 + 1) / 2;
+    p.cols = tc_cols(M);
+    p.split = tile_tokens == 0 ? 1 : 0;
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int tn = g_tile_tokens_override ? g_tile_tokens_override : (M >= 2048 ? 256 : 128);
-    long long max_tiles = ((long long)(M + tn - 1) / tn + E) * p.n_tiles;
-    int grid = (int)(max_tiles < sms ? max_tiles : sms);
-    cudaError_t err;
-    bool any_w2 = false;
-    for (int e = 0; e < E; ++e) any_w2 = any_w2 || ex[e]->bits == 2;
-    // (the attribute is set at every launch: it belongs to the current device, and the call is cheap)
-    auto launch = [&](auto kernel, int smem) -> bool {
+    const int clusters = sms / 2 < TC_MAX_CLUSTERS ? sms / 2 : TC_MAX_CLUSTERS;
+    const int nh = tile_tokens ? tile_tokens / 128 : (M > 256 ? 2 : 1);
+    auto launch = [&](auto kernel, int threads, int smem, int w_bytes) -> bool {
+        p.wstage = (stride + 127) / 128 * 128;
+        p.nw = w_bytes / p.wstage < TC_NW_MAX ? w_bytes / p.wstage : TC_NW_MAX;
+        // (the attribute is set at every launch: it belongs to the current device, and the call is cheap)
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return false;
-        kernel<<<grid, TC_THREADS, smem, st>>>(p, tmap, tmap_x);
-        return true;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2 * clusters); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at; cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kernel, p, tmap) == cudaSuccess;
     };
-    bool launched;
-    if (tn == 256)
-        launched = any_w2 ? launch(qgemm_tc_kernel<256, true, true>, Smem<256>::dyn_bytes) : launch(qgemm_tc_kernel<256, true, false>, Smem<256>::dyn_bytes);
-    else
-        launched = any_w2 ? launch(qgemm_tc_kernel<128, false, true>, Smem<128>::dyn_bytes) : launch(qgemm_tc_kernel<128, false, false>, Smem<128>::dyn_bytes);
-    if (!launched) return MOQE_ERR_CUDA;
-    err = cudaGetLastError();
+    const bool launched = nh == 2 ? launch(qgemm_tc_kernel<2>, TcCfg<2>::threads, TcCfg<2>::dyn_bytes, TcCfg<2>::w_bytes)
+                                  : launch(qgemm_tc_kernel<1>, TcCfg<1>::threads, TcCfg<1>::dyn_bytes, TcCfg<1>::w_bytes);
+    if (!launched) { cudaGetLastError(); return MOQE_ERR_CUDA; }
     count_launch();
-    return cuda_ok(err);
+    return cuda_ok(cudaGetLastError());
 }
 
 }  // namespace moqe

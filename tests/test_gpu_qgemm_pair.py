@@ -1,0 +1,63 @@
+"""GPU parity of the two-SM grouped GEMM at the sizes where its tiling can go wrong: batches one row either side of a
+half tile and of a whole token tile, an odd number of 128-channel tiles, K below and just above a k-block, rows that are
+consecutive in X (read as boxes), scattered (gathered) and mixed, and the split by k-blocks against whole tiles.
+
+Tolerance: that of the routed product (bf16 output, fp32 sums), max relative error 1e-2, mean absolute error 2e-3.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import moqe_workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+FORMATS = [(8, 0, True), (4, 128, False), (3, 64, False), (2, 32, True), (4, 0, False)]
+
+
+def _ids(kind, M, E):
+    g = np.random.default_rng(M * 31 + E)
+    if kind == "scattered":
+        return g.integers(0, E, size=M).astype(np.int32)
+    if kind == "runs":                                       # long runs: whole boxes are consecutive rows of X
+        return np.sort(g.integers(0, E, size=M)).astype(np.int32)
+    return np.repeat(g.integers(0, E, size=(M + 44) // 45), 45)[:M].astype(np.int32)   # short runs: boxes straddle them
+
+
+def _run(X, ids, gpu, path):
+    import torch
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import dev, bf16_to_torch, torch_to_bits
+    Y = torch.full((X.shape[0], gpu[0].N), float("nan"), dtype=torch.bfloat16, device=dev())
+    moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), gpu, Y=Y, path=path)
+    assert moqe.moqe_async_status() == moqe.OK
+    return torch_to_bits(Y)
+
+
+@pytest.mark.parametrize("kind", ["scattered", "runs", "short runs"])
+@pytest.mark.parametrize("M,N,K", [(1, 8, 32), (127, 128, 64), (129, 136, 192), (257, 384, 1088), (640, 264, 640)])
+def test_pair_kernel_edges(M, N, K, kind):
+    from gpu_helpers import build_experts, assert_close
+    specs = [f for f in FORMATS if f[1] == 0 or K % f[1] == 0]
+    W = wl.weights_f32(f"pair/{N}/{K}", N, K)
+    X = wl.activations_bf16(f"pair/{M}/{K}", M, K)
+    gpu, What, _ = build_experts(W, specs)
+    ids = _ids(kind, M, len(specs))
+    ref = oracle.routed_gemm(X, ids, What)
+    for path in (2, 3, 4):                                   # split by k-blocks; whole tiles of 128 and of 256 tokens
+        assert_close(_run(X, ids, gpu, path), ref, f"path {path} {kind} M{M} N{N} K{K}")
+
+
+def test_pair_kernel_split_is_deterministic_and_clears_its_counters():
+    """One token tile of one expert, 40 k-blocks deep: every cluster holds a part of it; the parts are added in a fixed
+    order (same bits every time) and the arrival counters come back to zero (the second call still completes)."""
+    from gpu_helpers import build_experts, assert_close
+    M, N, K = 200, 256, 5120
+    W = wl.weights_f32("pair/split", N, K)
+    X = wl.activations_bf16("pair/split/X", M, K)
+    gpu, What, _ = build_experts(W, [(4, 128, False)])
+    ids = np.zeros(M, np.int32)
+    first = _run(X, ids, gpu, 2)
+    assert_close(first, oracle.routed_gemm(X, ids, What), "split")
+    for _ in range(3):
+        assert np.array_equal(_run(X, ids, gpu, 2), first)
