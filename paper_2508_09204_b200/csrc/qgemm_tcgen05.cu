@@ -1,17 +1,17 @@
 // Routed dequant-GEMM for batches beyond the decode kernel's: a persistent, warp-specialised grouped GEMM on the
 // 5th-generation tensor cores, two SMs to a tile (cta_group::2).
 //
-//   tile         : 256 output channels x up to 128 * NH tokens.  CTA r of the pair owns channels 128 r .. 128 r + 127
-//                  (its TMEM lanes) of every token of the tile.
+//   tile         : 256 output channels x up to TN = 256, 128 or 64 tokens, in NH half tiles of HC = TN / NH columns.  CTA r
+//                  of the pair owns channels 128 r .. 128 r + 127 (its TMEM lanes) of every token of the tile.
 //   A operand    : the expert's weights, in TENSOR MEMORY.  Packed 128x128-code tiles arrive by bulk async copy; a
 //                  "dequant" thread owns one channel, unpacks its 128 codes of a k-block in registers to the exact
 //                  numbers (c - z) * 2^-13 in bf16 and stores them to its TMEM lane.  The unpacked weights never pass
 //                  through shared memory, whose bandwidth the token operand needs.
-//   B operand    : token rows, 64 per CTA and half tile (each SM of the pair reads its own half and they share it).
+//   B operand    : token rows, HC / 2 per CTA and half tile (each SM of the pair reads its own half and they share it).
 //                  Sorted rows that are consecutive in X come as one TMA box; any others are gathered through `perm` by
 //                  two warps' 16-byte cp.async copies into the same swizzled layout (the fused permutation: no gathered
 //                  copy of X exists).
-//   accumulation : fp32 in three rotating TMEM buffers of 128 tokens.  Grouped experts finish a buffer per (half tile,
+//   accumulation : fp32 in three rotating TMEM buffers of HC tokens.  Grouped experts finish a buffer per (half tile,
 //                  quantization group, at most 128 k); eight "epilogue" warps drain it, multiply by the group's fp32
 //                  scale and add into register accumulators while the tensor core fills the next one:
 //                      Y[m][n] = sum_G s[n][G] * (sum_{k in G} X[m][k] * (c[n][k] - z[n][G]))
@@ -43,39 +43,48 @@ namespace {
 constexpr int TC_MAX_CLUSTERS = 80;
 constexpr int TC_EPI = 8;                          // epilogue warps
 constexpr int TC_NW_MAX = 12;                      // packed-weight stages
-constexpr int TC_XHALF = 2 * 64 * 128;             // 64 token rows x 128 k bf16: two 64-k swizzled sub-tiles
 constexpr int TC_A_COLS = 64;                      // TMEM columns of one k-block of unpacked weights
-constexpr int TC_ACC_COLS = 128;                   // TMEM columns of one accumulator buffer
 constexpr int TC_NACC = 3;
-constexpr int TC_NSC = 8;                          // k-blocks of scales between the dequant warps and the epilogue
-constexpr int TC_A_BASE = TC_NACC * TC_ACC_COLS;   // two weight buffers behind the accumulators
 
-// NH: half tiles of 128 tokens.  2: few, large tiles (a k-block's 1024 tensor cycles hide one dequant warpgroup's
-// work); 1: small batches, where unpacking is the critical role and gets two warpgroups that take turns.
-template <int NH>
+// TN: tokens of a tile.  256: the tensor core's 1024 cycles a k-block hide one dequant warpgroup's work; 128 and 64: small
+// batches, where unpacking is the critical role and gets two warpgroups that take turns (and, with 64, five weight buffers
+// instead of two, so that they do not wait for the round trip through the tensor core).
+template <int TN>
 struct TcCfg {
-    static constexpr int dq_warps = NH == 2 ? 4 : 8;
+    static constexpr int NH = TN == 256 ? 2 : 1;                             // half tiles
+    static constexpr int HC = TN / NH;                                       // columns of a half tile = of an accumulator buffer
+    static constexpr int XR = HC / 2;                                        // token rows a CTA fetches for a half tile
+    static constexpr int xhalf = 2 * XR * 128;                               // XR rows x 128 k bf16: two 64-k swizzled sub-tiles
+    static constexpr int a_base = TC_NACC * HC;                              // the weight buffers sit behind the accumulators
+    static constexpr int NA = (512 - a_base) / TC_A_COLS;
+    static constexpr int EC = TN / 2;                                        // columns of an epilogue warp
+    static constexpr int dq_warps = TN == 256 ? 4 : 8;
     static constexpr int epi_warp0 = 4 + dq_warps;
     static constexpr int threads = (epi_warp0 + TC_EPI) * 32;
-    static constexpr int nx = NH == 2 ? 4 : 6;                               // token stages: one k-block of the tile
-    static constexpr int xstage = NH * TC_XHALF;
+    static constexpr int nx = TN == 256 ? 4 : 6;                             // token stages: one k-block of the tile
+    static_assert(NA <= nx, "the dequant warps wait for the k-block NA ago on its token stage's barrier");
+    // k-blocks of scales between the dequant warps and the epilogue.  When the scales of k-block k are written, the k-block
+    // NA + 2 before it is done and at most three buffers are still to be drained: slot k - nsc must be older than that.
+    static constexpr int nsc = NA == 2 ? 8 : 16;
+    static_assert(nsc > NA + 2 + TC_NACC, "scale slots");
+    static constexpr int xstage = NH * xhalf;
     // shared memory
     static constexpr int x_off = 0;
     static constexpr int bar_off = nx * xstage;
-    static constexpr int n_bars = 2 * TC_NW_MAX + 2 * nx + 2 + 2 * TC_NACC + TC_NSC;   // wfull wempty xfull done afull accfull accempty scfull
+    static constexpr int n_bars = 2 * TC_NW_MAX + 2 * nx + NA + (NH + 1) * TC_NACC + nsc;   // wfull wempty xfull done afull accfull accempty scfull
     static constexpr int misc_off = bar_off + n_bars * 8;                    // tmem addr, abort flag, clusters of the split, T, Td
     static constexpr int cost_off = (misc_off + 32 + 15) / 16 * 16;          // long long: base[32], total
     static constexpr int sched_off = cost_off + 33 * 8;                      // ints: see TcSched
     static constexpr int sched_ints = 34 + 33 + 5 * 32;
     static constexpr int perm_off = sched_off + sched_ints * 4;
-    static constexpr int xrow_off = perm_off + TC_EPI * 64 * NH * 4;         // rows of X to gather, one list per gather warp
-    static constexpr int sc_off = (xrow_off + 2 * 64 * NH * 4 + 15) / 16 * 16;   // scales on their way to the epilogue
-    static constexpr int w_off = (sc_off + TC_NSC * 4 * 128 * 2 + 127) / 128 * 128;
+    static constexpr int xrow_off = perm_off + TC_EPI * EC * 4;              // rows of X to gather, one list per gather warp
+    static constexpr int sc_off = (xrow_off + 2 * NH * XR * 4 + 15) / 16 * 16;   // scales on their way to the epilogue
+    static constexpr int w_off = (sc_off + nsc * 4 * 128 * 2 + 127) / 128 * 128;
     static constexpr int total = 226 * 1024;
     static constexpr int w_bytes = (total - w_off) / 128 * 128;
     static constexpr int dyn_bytes = total + 1024;                           // slack for manual 1024-byte alignment
 };
-static_assert(TcCfg<2>::dyn_bytes <= 232448 && TcCfg<2>::w_bytes >= 3 * 18432, "shared memory budget");
+static_assert(TcCfg<256>::dyn_bytes <= 232448 && TcCfg<256>::w_bytes >= 3 * 18432, "shared memory budget");
 
 struct TcParams {
     ExpertDev ex[MOQE_MAX_EXPERTS];
@@ -104,8 +113,8 @@ __device__ __forceinline__ void cluster_sync() {
 }
 // (Arrivals on the other CTA's barriers order tensor-memory work and async copies only, so they need no cluster-scope
 // release; with one, 16384 rows of a per-channel expert took 9.1 ms a LLaMA block instead of 4.9.)
-__device__ __forceinline__ void remote_arrive(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+__device__ __forceinline__ void remote_arrive(uint32_t cluster_addr, uint32_t count = 1) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_addr), "r"(count) : "memory");
 }
 __device__ __forceinline__ void remote_expect_tx_only(uint32_t cluster_addr, uint32_t bytes) {
     asm volatile("mbarrier.expect_tx.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(cluster_addr), "r"(bytes) : "memory");
@@ -190,7 +199,8 @@ struct TcWalk {
     }
 };
 // MMA columns of half tile h of a tile with `rows` tokens
-__device__ __forceinline__ int half_cols(int rows, int h) { return (min(128, rows - 128 * h) + 31) & ~31; }
+template <int HC>
+__device__ __forceinline__ int half_cols(int rows, int h) { return (min(HC, rows - HC * h) + 31) & ~31; }
 
 // ---------------------------------------------------------------------------- unpacking
 __device__ __forceinline__ uint32_t fma_bf16x2(uint32_t a, uint32_t b, uint32_t c) {
@@ -305,11 +315,11 @@ __device__ __forceinline__ void fma_cols32(float* acc, const uint32_t (&v)[32], 
 }
 
 // ---------------------------------------------------------------------------- the kernel
-template <int NH>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 1)
+template <int TN>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 1)
     qgemm_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap tmap) {
-    using L = TcCfg<NH>;
-    constexpr int NX = L::nx;
+    using L = TcCfg<TN>;
+    constexpr int NH = L::NH, NX = L::nx, NA = L::NA, NSC = L::nsc;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -322,7 +332,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
     const uint32_t bar_wfull = sbase + L::bar_off, bar_wempty = bar_wfull + 8 * TC_NW_MAX;
     const uint32_t bar_xfull = bar_wempty + 8 * TC_NW_MAX, bar_done = bar_xfull + 8 * NX;
     const uint32_t bar_afull = bar_done + 8 * NX;
-    const uint32_t bar_accfull = bar_afull + 16, bar_accempty = bar_accfull + 8 * TC_NACC, bar_scfull = bar_accempty + 8 * TC_NACC;
+    const uint32_t bar_accfull = bar_afull + 8 * NA, bar_accempty = bar_accfull + 8 * NH * TC_NACC, bar_scfull = bar_accempty + 8 * TC_NACC;
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + L::misc_off);
     volatile int* s_abort = reinterpret_cast<volatile int*>(smem + L::misc_off + 4);
     TcSched sc;
@@ -342,9 +352,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
     if (tid == 0) {
         for (int i = 0; i < TC_NW_MAX; ++i) { mbar_init(bar_wfull + 8 * i, 1); mbar_init(bar_wempty + 8 * i, 4); }
         for (int i = 0; i < NX; ++i) { mbar_init(bar_xfull + 8 * i, 4); mbar_init(bar_done + 8 * i, 1); }
-        for (int i = 0; i < 2; ++i) mbar_init(bar_afull + 8 * i, 8);
-        for (int i = 0; i < TC_NACC; ++i) { mbar_init(bar_accfull + 8 * i, 1); mbar_init(bar_accempty + 8 * i, 2 * TC_EPI); }
-        for (int i = 0; i < TC_NSC; ++i) mbar_init(bar_scfull + 8 * i, 4);
+        for (int i = 0; i < NA; ++i) mbar_init(bar_afull + 8 * i, 8);
+        for (int i = 0; i < NH * TC_NACC; ++i) mbar_init(bar_accfull + 8 * i, 1);
+        for (int i = 0; i < TC_NACC; ++i) mbar_init(bar_accempty + 8 * i, 2 * TC_EPI);
+        for (int i = 0; i < NSC; ++i) mbar_init(bar_scfull + 8 * i, 4);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -355,7 +366,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
         // ---- the schedule: lane e works out expert e
         const int e = lane;
         const int o0 = e < p.E ? __ldcg(p.offsets + e) : 0, o1 = e < p.E ? __ldcg(p.offsets + e + 1) : 0;
-        const int R = o1 - o0, TN = 128 * NH;
+        const int R = o1 - o0;
         const int mt = (R + TN - 1) / TN;
         const int rpt = mt >= 4 ? TN : (mt > 0 ? ((R + mt - 1) / mt + 31) & ~31 : 32);
         const int T_e = mt * p.NTP;
@@ -406,19 +417,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
     const uint32_t tmem_base = *s_tmem;
 
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        if constexpr (TN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         if (warp == 0 || warp == 3) {
-            // ---------------- X producers: this CTA's 64 token rows of every half tile, 128 k per stage ----------------
+            // ---------------- X producers: this CTA's XR token rows of every half tile, 128 k per stage ----------------
             // Both warps walk the stages and arrive on the pair's xfull barrier; warp 0 also adds the byte count of the TMA
             // boxes.  A warp gathers every other pair of rows; its arrival for a stage follows once its copies have landed,
             // LAG stages later (at once where nothing is gathered).
             constexpr int LAG = NX == 4 ? 3 : 4;
             const int gw = warp == 0 ? 0 : 1;
-            int* s_xrow = reinterpret_cast<int*>(smem + L::xrow_off) + gw * 64 * NH;
+            int* s_xrow = reinterpret_cast<int*>(smem + L::xrow_off) + gw * NH * L::XR;
             const int hi = lane >> 4, c16 = lane & 15;
             // byte offset of this lane's 16-byte chunk of row 4 i + 2 gw + hi: sub-tile, then the 128-byte swizzle
             const uint32_t r0 = 2 * gw + hi;
-            const uint32_t sw0 = (c16 >> 3) * 8192 + r0 * 128 + (((c16 & 7) ^ r0) << 4), sw1 = (c16 >> 3) * 8192 + (r0 + 4) * 128 + (((c16 & 7) ^ (r0 + 4)) << 4);
+            const uint32_t sw0 = (c16 >> 3) * (L::XR * 128) + r0 * 128 + (((c16 & 7) ^ r0) << 4), sw1 = (c16 >> 3) * (L::XR * 128) + (r0 + 4) * 128 + (((c16 & 7) ^ (r0 + 4)) << 4);
             Ring ring, aring;                              // aring: the stage whose arrival is due next
             TcPiece pc;
             TcWalk wk;
@@ -433,7 +445,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
                 aring.advance(NX);
             };
             while (ok && wk.next(sc, p, nclusters, pc)) {
-                const int nh = NH == 1 ? 1 : (pc.rows > 128 ? 2 : 1);
+                const int nh = NH == 1 ? 1 : (pc.rows > L::HC ? 2 : 1);
                 int src[NH], cnt[NH], bytes = 0;
                 bool gathers = false;
                 __syncwarp();
@@ -441,20 +453,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
                 for (int h = 0; h < NH; ++h) {
                     src[h] = -1; cnt[h] = 0;
                     if (h < nh) {
-                        const int per_cta = half_cols(pc.rows, h) >> 1;
-                        const int first_row = h * 128 + (int)rank * per_cta;
+                        const int per_cta = half_cols<L::HC>(pc.rows, h) >> 1;
+                        const int first_row = h * L::HC + (int)rank * per_cta;
                         const int c = max(min(per_cta, pc.rows - first_row), 0);         // real rows of this CTA
                         const int a = lane < c ? __ldcg(p.perm + pc.m0 + first_row + lane) : 0;
                         const int b = lane + 32 < c ? __ldcg(p.perm + pc.m0 + first_row + lane + 32) : 0;
                         const int first = __shfl_sync(0xffffffffu, a, 0);
                         const bool run = __all_sync(0xffffffffu, (lane >= c || a == first + lane) && (lane + 32 >= c || b == first + lane + 32));
-                        s_xrow[h * 64 + lane] = a;
-                        s_xrow[h * 64 + lane + 32] = b;
-                        // (a box fetches 64 rows whatever it needs; operand rows beyond the real ones yield columns that are
+                        s_xrow[h * L::XR + lane] = a;
+                        if (L::XR > 32) s_xrow[h * L::XR + lane + 32] = b;
+                        // (a box fetches XR rows whatever it needs; operand rows beyond the real ones yield columns that are
                         // never stored, so they may hold anything)
-                        src[h] = run && c >= 32 ? first : -1;
+                        src[h] = run && 2 * c >= L::XR ? first : -1;
                         cnt[h] = c;
-                        bytes += src[h] >= 0 ? TC_XHALF : 0;
+                        bytes += src[h] >= 0 ? L::xhalf : 0;
                         gathers |= src[h] < 0 && c > 0;
                     }
                 }
@@ -468,7 +480,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
                         __syncwarp();
 #pragma unroll
                         for (int h = 0; h < NH; ++h)
-                            if (src[h] >= 0 && lane < 2) tma_box_pair(stage + h * TC_XHALF + lane * 8192, &tmap, kb * 128 + lane * 64, src[h], full);
+                            if (src[h] >= 0 && lane < 2) tma_box_pair(stage + h * L::xhalf + lane * (L::XR * 128), &tmap, kb * 128 + lane * 64, src[h], full);
                         __syncwarp();
                     }
                     const int k = kb * 128 + c16 * 8;
@@ -477,13 +489,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
 #pragma unroll
                     for (int h = 0; h < NH; ++h) {
                         if (src[h] < 0) {
-                            const uint32_t dst = stage + h * TC_XHALF;
+                            const uint32_t dst = stage + h * L::xhalf;
 #pragma unroll 4
-                            for (int i = 0; i < 16; ++i) {
+                            for (int i = 0; i < L::XR / 4; ++i) {
                                 const int r = 4 * i + (int)r0;
                                 if (4 * i + 2 * gw >= cnt[h]) break;
                                 if (r < cnt[h])
-                                    cp_async16(dst + ((i & 1) ? sw1 : sw0) + (i >> 1) * 1024, xk + (size_t)s_xrow[h * 64 + r] * (size_t)(p.K * 2), real);
+                                    cp_async16(dst + ((i & 1) ? sw1 : sw0) + (i >> 1) * 1024, xk + (size_t)s_xrow[h * L::XR + r] * (size_t)(p.K * 2), real);
                             }
                         }
                     }
@@ -542,27 +554,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
             TcWalk wk;
             wk.start(cluster);
             bool ok = true;
-            uint32_t kcount = 0;                           // k-blocks so far (weight buffers alternate)
+            Ring aring;                                    // weight buffers
             int buf = 0;
             uint32_t buf_phase = 1;                        // parity of "empty" for the buffers of this round
             auto next_buf = [&]() { if (++buf == TC_NACC) { buf = 0; buf_phase ^= 1u; } };
             while (ok && wk.next(sc, p, nclusters, pc)) {
-                const int nh = NH == 1 ? 1 : (pc.rows > 128 ? 2 : 1);
+                const int nh = NH == 1 ? 1 : (pc.rows > L::HC ? 2 : 1);
                 const int group = p.ex[pc.e].group;
                 // A per-channel expert's half tile h stays in buffer (buf + h) of the rotation for the whole piece.
                 const bool keep = group == 0;
                 const int steps = keep || group >= 128 ? 8 : group >> 4;         // MMAs into one accumulator buffer
-                for (int kb = pc.kb0; ok && kb < pc.kb1; ++kb, ++kcount) {
-                    const uint32_t ab = kcount & 1u;
+                for (int kb = pc.kb0; ok && kb < pc.kb1; ++kb) {
                     ok = __all_sync(0xffffffffu, mbar_wait_short(bar_xfull + 8 * ring.stage, ring.phase, s_abort, p.status));
-                    ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_afull + 8 * ab, (kcount >> 1) & 1u, s_abort, p.status));
+                    ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_afull + 8 * aring.stage, aring.phase, s_abort, p.status));
                     tc_fence_after();
-                    const uint32_t a_tmem = tmem_base + TC_A_BASE + ab * TC_A_COLS;
+                    const uint32_t a_tmem = tmem_base + L::a_base + aring.stage * TC_A_COLS;
                     const uint32_t done = bar_done + 8 * ring.stage;
 #pragma unroll 1
                     for (int h = 0; h < nh; ++h) {
-                        const uint32_t idesc = umma_idesc_pair(half_cols(pc.rows, h));
-                        const uint64_t bdesc = umma_desc_sw128(sbase + L::x_off + ring.stage * L::xstage + h * TC_XHALF);
+                        const uint32_t idesc = umma_idesc_pair(half_cols<L::HC>(pc.rows, h));
+                        const uint64_t bdesc = umma_desc_sw128(sbase + L::x_off + ring.stage * L::xstage + h * L::xhalf);
                         const bool last_half = h + 1 == nh;
                         if (steps == 8) {
                             const int b2 = keep && h ? (buf + 1 == TC_NACC ? 0 : buf + 1) : buf;
@@ -570,16 +581,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
                             const uint32_t add = keep && kb > pc.kb0 ? 1u : 0u;
                             if (!add) ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_accempty + 8 * b2, ph, s_abort, p.status));
                             tc_fence_after();
-                            const uint32_t d = tmem_base + b2 * TC_ACC_COLS;
+                            const uint32_t d = tmem_base + b2 * L::HC;
                             if (elect_one()) {
 #pragma unroll
                                 for (int i = 0; i < 8; ++i)
-                                    umma_pair_ts(d, a_tmem + 8 * i, bdesc + (i >> 2) * 512 + (i & 3) * 2, idesc, i > 0 ? 1u : add);
+                                    umma_pair_ts(d, a_tmem + 8 * i, bdesc + (i >> 2) * (L::XR * 8) + (i & 3) * 2, idesc, i > 0 ? 1u : add);
                                 if (keep) {
                                     if (last_half) umma_commit_pair(done);
-                                    if (kb + 1 == pc.kb1) umma_commit_pair(bar_accfull + 8 * b2);
+                                    if (kb + 1 == pc.kb1) umma_commit_pair(bar_accfull + 8 * (h * TC_NACC + b2));
                                 } else {
-                                    umma_commit_pair(last_half ? done : bar_accfull + 8 * b2);
+                                    umma_commit_pair(last_half ? done : bar_accfull + 8 * (h * TC_NACC + b2));
                                 }
                             }
                             __syncwarp();
@@ -589,8 +600,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
                             for (int i0 = 0; i0 < 8; i0 += steps) {
                                 ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_accempty + 8 * buf, buf_phase, s_abort, p.status));
                                 tc_fence_after();
-                                const uint32_t d = tmem_base + buf * TC_ACC_COLS;
-                                const uint64_t bd = bdesc + (i0 >> 2) * 512 + (i0 & 3) * 2;
+                                const uint32_t d = tmem_base + buf * L::HC;
+                                const uint64_t bd = bdesc + (i0 >> 2) * (L::XR * 8) + (i0 & 3) * 2;
                                 if (elect_one()) {
                                     umma_pair_ts(d, a_tmem + 8 * i0, bd, idesc, 0u);
                                     umma_pair_ts(d, a_tmem + 8 * i0 + 8, bd + 2, idesc, 1u);
@@ -598,7 +609,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
                                         umma_pair_ts(d, a_tmem + 8 * i0 + 16, bd + 4, idesc, 1u);
                                         umma_pair_ts(d, a_tmem + 8 * i0 + 24, bd + 6, idesc, 1u);
                                     }
-                                    umma_commit_pair(last_half && i0 + steps == 8 ? done : bar_accfull + 8 * buf);
+                                    umma_commit_pair(last_half && i0 + steps == 8 ? done : bar_accfull + 8 * (h * TC_NACC + buf));
                                 }
                                 __syncwarp();
                                 next_buf();
@@ -606,18 +617,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
                         }
                     }
                     ring.advance(NX);
+                    aring.advance(NA);
                 }
                 if (keep) for (int h = 0; h < nh; ++h) next_buf();
             }
         }
     } else if (warp < L::epi_warp0) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+        if constexpr (TN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
         // ---------------- dequant warps: thread = channel = TMEM lane ----------------
         const int row = (warp & 3) * 32 + lane;
-        const uint32_t my_group = NH == 2 ? 0u : (uint32_t)((warp - 4) >> 2);
+        const uint32_t my_group = (uint32_t)((warp - 4) >> 2);
         const uint32_t afull0 = mapa(bar_afull, 0);
-        const uint32_t lane_tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + TC_A_BASE;
-        Ring wring, dring;
+        const uint32_t lane_tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + L::a_base;
+        Ring wring, dring, aring;
         TcPiece pc;
         TcWalk wk;
         wk.start(cluster);
@@ -632,15 +645,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
             if (ex.has_zeros && ex.group == 0 && active) z = __bfloat162float(ex.zeros_pc[nt * 128 + row]);
             const uint32_t zpc = neg_z(z);
             for (int kb = pc.kb0; ok && kb < pc.kb1; ++kb, ++kcount) {
-                const uint32_t ab = kcount & 1u;
-                const bool mine = NH == 2 || ab == my_group;
-                // the buffer is free once the k-block before the last is done
-                const uint32_t free_bar = kcount >= 2 ? bar_done + 8 * dring.stage : 0u;
-                const uint32_t scfull = bar_scfull + 8 * (kcount & (TC_NSC - 1));
+                const bool mine = L::dq_warps == 4 || (kcount & 1u) == my_group;
+                // the buffer is free once the k-block NA ago is done
+                const uint32_t free_bar = kcount >= NA ? bar_done + 8 * dring.stage : 0u;
+                const uint32_t scfull = bar_scfull + 8 * (kcount & (NSC - 1));
                 if (mine && active) {
                     const unsigned char* tile = smem + L::w_off + wring.stage * p.wstage;
-                    __half* scales = s_sc + (kcount & (TC_NSC - 1)) * 512;
-                    const uint32_t wf = bar_wfull + 8 * wring.stage, we = bar_wempty + 8 * wring.stage, at = lane_tmem + ab * TC_A_COLS;
+                    __half* scales = s_sc + (kcount & (NSC - 1)) * 512;
+                    const uint32_t wf = bar_wfull + 8 * wring.stage, we = bar_wempty + 8 * wring.stage, at = lane_tmem + aring.stage * TC_A_COLS;
                     switch (ex.bits) {
                         case 4: ok = dequant_kblock<4>(ex, tile, row, zpc, tile_zeros, scales, scfull, wf, wring.phase, we, free_bar, dring.phase, at, s_abort, p.status); break;
                         case 8: ok = dequant_kblock<8>(ex, tile, row, zpc, tile_zeros, scales, scfull, wf, wring.phase, we, free_bar, dring.phase, at, s_abort, p.status); break;
@@ -655,47 +667,53 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
                 if (mine) {
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) remote_arrive(afull0 + 8 * ab);
+                    if (lane == 0) remote_arrive(afull0 + 8 * aring.stage);
                 }
                 if (active) wring.advance(p.nw);
-                if (kcount >= 2) dring.advance(NX);
+                if (kcount >= NA) dring.advance(NX);
+                aring.advance(NA);
             }
         }
     } else {
-        if constexpr (NH == 2) asm volatile("setmaxnreg.inc.sync.aligned.u32 184;");
+        if constexpr (TN == 256) asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
         else asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
         // ---------------- epilogue warps: scale-and-accumulate, then store ----------------
-        const int ew = warp - L::epi_warp0, quarter = warp & 3, colhalf = ew >> 2;
+        // (Each half tile has its own accfull barriers: a wait tells only two phases of a barrier apart, so a barrier is waited
+        // on by the warps that its buffer's reuse waits for, and by nobody who could fall two uses behind.)
+        // Two groups of four warps.  Of a tile with two half tiles each group drains one (an accumulator buffer then costs a
+        // warp one wait for 128 columns); of a tile with one, each group drains half the columns.
+        const int ew = warp - L::epi_warp0, quarter = warp & 3, eg = ew >> 2;
         const int row = quarter * 32 + lane;               // channel inside the 128-channel tile = TMEM lane
-        const int col0 = colhalf * 64;                     // this warp's columns of every half tile
         const uint32_t accempty0 = mapa(bar_accempty, 0);
-        const uint32_t lane_tmem = tmem_base + ((uint32_t)(quarter * 32) << 16) + col0;
-        int* my_perm = s_perm + ew * 64 * NH;              // private to this warp: no cross-warp barrier
+        const uint32_t lane_tmem = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        int* my_perm = s_perm + ew * L::EC;                // private to this warp: no cross-warp barrier
         TcPiece pc;
         TcWalk wk;
         wk.start(cluster);
         bool ok = true;
         int buf = 0;
-        uint32_t full_phase = 0;                           // bit b: parity of the next arrival on accfull[b]
+        uint32_t full_phase = 0;                           // bit i: parity of the next arrival on accfull[i]
         uint32_t kcount = 0;
         Ring dring;                                        // the k-block whose last accumulator is drained next
         while (ok && wk.next(sc, p, nclusters, pc)) {
             const ExpertDev& ex = p.ex[pc.e];
             const int nt = 2 * pc.ntp + (int)rank, n = nt * 128 + row;
             const bool active = nt < p.NT1;
-            const int nh = NH == 1 ? 1 : (pc.rows > 128 ? 2 : 1);
+            const int nh = NH == 1 ? 1 : (pc.rows > L::HC ? 2 : 1);
+            const int mine_h = nh == 2 ? eg : 0;
+            const int col0 = nh == 2 ? 0 : eg * (L::HC / 2);              // this warp's columns of half tile mine_h
+            const int ncol = min(nh == 2 ? L::HC : L::HC / 2, pc.rows - mine_h * L::HC - col0);   // those with a token (may be <= 0)
+            const int tok0 = mine_h * L::HC + col0;
             __syncwarp();
 #pragma unroll
-            for (int i = 0; i < 2 * NH; ++i) {
-                const int col = (i >> 1) * 128 + col0 + (i & 1) * 32 + lane;
-                my_perm[i * 32 + lane] = col < pc.rows ? __ldcg(p.perm + pc.m0 + col) : -1;
+            for (int i = 0; i < L::EC / 32; ++i) {
+                const int col = i * 32 + lane;
+                my_perm[col] = col < ncol ? __ldcg(p.perm + pc.m0 + tok0 + col) : -1;
             }
             __syncwarp();
-            float acc[NH][64];
+            float acc[L::EC];
 #pragma unroll
-            for (int h = 0; h < NH; ++h)
-#pragma unroll
-                for (int i = 0; i < 64; ++i) acc[h][i] = 0.f;
+            for (int i = 0; i < L::EC; ++i) acc[i] = 0.f;
             // One round per k-block (grouped: every group's buffer is drained, the last one of the k-block being announced by
             // the k-block's own barrier) or one for the whole piece (per channel).  The loops are kept rolled: unrolled over
             // the groups and the barriers' outcomes the kernel was 235 KB of code and spent a quarter of its warps' time
@@ -703,40 +721,41 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
             const bool keep = ex.group == 0;
             const int per = keep ? 1 : moqe_groups_per_tile(ex.group), rounds = keep ? 1 : pc.kb1 - pc.kb0;
             const float s_pc = keep && active ? __half2float(ex.scales_pc[n]) * W8_PRESCALE : 0.f;   // (weights are unpacked as (c - z) * 2^-13)
+            const uint32_t freed = nh == 2 ? 2u : 1u;
 #pragma unroll 1
             for (int it = 0; ok && it < rounds; ++it) {
-                const uint32_t slot = kcount & (TC_NSC - 1);
-                // (slot reuse: the dequant warps write k-block k after k - 2 is done, and three buffers bound how far the
-                // drains may be behind)
-                if (!keep) ok = __all_sync(0xffffffffu, mbar_wait_short(bar_scfull + 8 * slot, (kcount / TC_NSC) & 1u, s_abort, p.status));
-#pragma unroll
-                for (int h = 0; h < NH; ++h) {
-                    if (h < nh) {
-                        const int cols = half_cols(pc.rows, h);
+                const uint32_t slot = kcount & (NSC - 1);
 #pragma unroll 1
-                        for (int j = 0; j < per; ++j) {
-                            const bool by_done = !keep && h + 1 == nh && j + 1 == per;
-                            const uint32_t bar = by_done ? bar_done + 8 * dring.stage : bar_accfull + 8 * buf;
-                            const uint32_t phase = by_done ? dring.phase : (full_phase >> buf) & 1u;
-                            const float s = keep ? s_pc : __half2float(s_sc[slot * 512 + j * 128 + row]) * W8_PRESCALE;
-                            ok &= __all_sync(0xffffffffu, mbar_wait_short(bar, phase, s_abort, p.status));
-                            if (!by_done) full_phase ^= 1u << buf;
-                            tc_fence_after();
+                for (int t = 0; t < nh * per; ++t) {
+                    const int h = t >= per ? 1 : 0, j = t - h * per;
+                    const bool by_done = !keep && t + 1 == nh * per;
+                    if (h == mine_h) {
+                        const uint32_t bar = by_done ? bar_done + 8 * dring.stage : bar_accfull + 8 * (h * TC_NACC + buf);
+                        const uint32_t phase = by_done ? dring.phase : (full_phase >> (h * TC_NACC + buf)) & 1u;
+                        ok &= __all_sync(0xffffffffu, mbar_wait_short(bar, phase, s_abort, p.status));
+                        tc_fence_after();
+                        const uint32_t src = lane_tmem + buf * L::HC + col0;
+                        float s = s_pc;
 #pragma unroll
-                            for (int c = 0; c < 2; ++c) {
-                                if (col0 + 32 * c < cols) {
-                                    uint32_t v[32];
-                                    tmem_ld32(lane_tmem + buf * TC_ACC_COLS + 32 * c, v);
-                                    tmem_ld_wait();
-                                    fma_cols32(acc[h] + 32 * c, v, s);
+                        for (int c = 0; c < L::EC / 32; ++c) {
+                            if (32 * c < ncol) {
+                                uint32_t v[32];
+                                tmem_ld32(src + 32 * c, v);
+                                if (c == 0 && !keep) {
+                                    // the group's scale, fetched while the load is under way
+                                    if (j == 0) ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_scfull + 8 * slot, (kcount / NSC) & 1u, s_abort, p.status));
+                                    s = __half2float(s_sc[slot * 512 + j * 128 + row]) * W8_PRESCALE;
                                 }
+                                tmem_ld_wait();
+                                fma_cols32(acc + 32 * c, v, s);
                             }
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) remote_arrive(accempty0 + 8 * buf);
-                            if (++buf == TC_NACC) buf = 0;
                         }
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) remote_arrive(accempty0 + 8 * buf, freed);
                     }
+                    if (!by_done) full_phase ^= 1u << (h * TC_NACC + buf);
+                    if (++buf == TC_NACC) buf = 0;
                 }
                 if (!keep) { dring.advance(NX); ++kcount; }
             }
@@ -754,17 +773,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
                 const int Gs = sc.misc[0];
                 const int c_a = (int)(first * Gs / C), c_b = (int)((first + (long long)(p.KB - 1) * sc.w[pc.e]) * Gs / C);
                 const size_t slot = (size_t)p.cols * 128;
-                auto slot_of = [&](int c, int which) { return p.partials + ((size_t)(c * 2 + which) * 2 + rank) * slot + (size_t)col0 * 128 + row; };
+                auto slot_of = [&](int c, int which) { return p.partials + ((size_t)(c * 2 + which) * 2 + rank) * slot + (size_t)tok0 * 128 + row; };
                 {
                     float* dst = slot_of(cluster, pc.kb0 == 0 ? 1 : 0);
 #pragma unroll
-                    for (int h = 0; h < NH; ++h)
+                    for (int i0 = 0; i0 < L::EC; i0 += 8)
+                        if (i0 < ncol) {
 #pragma unroll
-                        for (int i0 = 0; i0 < 64; i0 += 8)
-                            if (h * 128 + col0 + i0 < pc.rows) {
-#pragma unroll
-                                for (int i = i0; i < i0 + 8; ++i) __stcg(dst + (size_t)(h * 128 + i) * 128, acc[h][i]);
-                            }
+                            for (int i = i0; i < i0 + 8; ++i) __stcg(dst + (size_t)i * 128, acc[i]);
+                        }
                 }
                 __syncwarp();
                 unsigned* counter = p.counters + (c_a * 2 + (int)rank) * TC_EPI + ew;
@@ -776,23 +793,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
                 if (arrived != (unsigned)(c_b - c_a)) continue;
                 __syncwarp();
 #pragma unroll
-                for (int h = 0; h < NH; ++h)
-#pragma unroll
-                    for (int i = 0; i < 64; ++i) acc[h][i] = 0.f;
+                for (int i = 0; i < L::EC; ++i) acc[i] = 0.f;
 #pragma unroll 1
                 for (int c = c_a; c <= c_b; ++c) {
                     const float* src = slot_of(c, c == c_a ? 1 : 0);
 #pragma unroll
-                    for (int h = 0; h < NH; ++h)
+                    for (int i0 = 0; i0 < L::EC; i0 += 8)
+                        if (i0 < ncol) {
+                            float v[8];
 #pragma unroll
-                        for (int i0 = 0; i0 < 64; i0 += 8)
-                            if (h * 128 + col0 + i0 < pc.rows) {
-                                float v[8];
+                            for (int i = 0; i < 8; ++i) v[i] = __ldcg(src + (size_t)(i0 + i) * 128);
 #pragma unroll
-                                for (int i = 0; i < 8; ++i) v[i] = __ldcg(src + (size_t)(h * 128 + i0 + i) * 128);
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) acc[h][i0 + i] += v[i];
-                            }
+                            for (int i = 0; i < 8; ++i) acc[i0 + i] += v[i];
+                        }
                 }
                 if (lane == 0) *counter = 0u;
             }
@@ -801,19 +814,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<NH>::threads, 
             const int odd = lane & 1;
             uint16_t* y = p.Y + (n & ~1);
 #pragma unroll
-            for (int h = 0; h < NH; ++h)
+            for (int i0 = 0; i0 < L::EC; i0 += 8)
+                if (i0 < ncol) {
 #pragma unroll
-                for (int i0 = 0; i0 < 64; i0 += 8)
-                    if (h * 128 + col0 + i0 < pc.rows) {
-#pragma unroll
-                        for (int i = i0; i < i0 + 8; i += 2) {
-                            const uint32_t mine = pack_bf16x2(acc[h][i], acc[h][i + 1]);
-                            const uint32_t other = __shfl_xor_sync(0xffffffffu, mine, 1);
-                            const uint32_t pair = __byte_perm(mine, other, odd ? 0x3276u : 0x5410u);
-                            const int to = my_perm[h * 64 + i + odd];
-                            if (to >= 0 && n < p.N) *reinterpret_cast<uint32_t*>(y + (size_t)to * p.N) = pair;
-                        }
+                    for (int i = i0; i < i0 + 8; i += 2) {
+                        const uint32_t mine = pack_bf16x2(acc[i], acc[i + 1]);
+                        const uint32_t other = __shfl_xor_sync(0xffffffffu, mine, 1);
+                        const uint32_t pair = __byte_perm(mine, other, odd ? 0x3276u : 0x5410u);
+                        const int to = my_perm[i + odd];
+                        if (to >= 0 && n < p.N) *reinterpret_cast<uint32_t*>(y + (size_t)to * p.N) = pair;
                     }
+                }
         }
     }
 
@@ -865,11 +876,12 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
     if (!ws || ws_bytes < tc_workspace_bytes(M, K, E, ex[0]->Np)) return MOQE_ERR_WORKSPACE;
     EncodeTiledFn enc = encode_fn();
     if (!enc) return MOQE_ERR_CUDA;
-    // tensor map over X[M][K] bf16: boxes of 64 k x 64 rows, 128-byte swizzle, zero fill outside
+    const int tile = tile_tokens ? tile_tokens : (M > 256 ? 256 : (M > 128 ? 128 : 64));
+    // tensor map over X[M][K] bf16: boxes of 64 k x XR rows, 128-byte swizzle, zero fill outside
     CUtensorMap tmap;
     cuuint64_t gdim[2] = {(cuuint64_t)K, (cuuint64_t)M};
     cuuint64_t gstride[1] = {(cuuint64_t)K * 2};
-    cuuint32_t box[2] = {64, 64}, estr[2] = {1, 1};
+    cuuint32_t box[2] = {64, tile == 64 ? 32u : 64u}, estr[2] = {1, 1};
     if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(X), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return MOQE_ERR_CUDA;
@@ -889,7 +901,6 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int clusters = sms / 2 < TC_MAX_CLUSTERS ? sms / 2 : TC_MAX_CLUSTERS;
-    const int nh = tile_tokens ? tile_tokens / 128 : (M > 256 ? 2 : 1);
     auto launch = [&](auto kernel, int threads, int smem, int w_bytes) -> bool {
         p.wstage = (stride + 127) / 128 * 128;
         p.nw = w_bytes / p.wstage < TC_NW_MAX ? w_bytes / p.wstage : TC_NW_MAX;
@@ -903,8 +914,12 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
         cfg.attrs = at; cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kernel, p, tmap) == cudaSuccess;
     };
-    const bool launched = nh == 2 ? launch(qgemm_tc_kernel<2>, TcCfg<2>::threads, TcCfg<2>::dyn_bytes, TcCfg<2>::w_bytes)
-                                  : launch(qgemm_tc_kernel<1>, TcCfg<1>::threads, TcCfg<1>::dyn_bytes, TcCfg<1>::w_bytes);
+    auto run = [&](auto tag) {
+        using L = TcCfg<decltype(tag)::value>;
+        return launch(qgemm_tc_kernel<decltype(tag)::value>, L::threads, L::dyn_bytes, L::w_bytes);
+    };
+    const bool launched = tile == 256 ? run(std::integral_constant<int, 256>{})
+                                      : (tile == 128 ? run(std::integral_constant<int, 128>{}) : run(std::integral_constant<int, 64>{}));
     if (!launched) { cudaGetLastError(); return MOQE_ERR_CUDA; }
     count_launch();
     return cuda_ok(cudaGetLastError());
