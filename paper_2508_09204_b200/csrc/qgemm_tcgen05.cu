@@ -68,23 +68,14 @@ struct TcCfg {
     static constexpr int nsc = NA == 2 ? 8 : 16;
     static_assert(nsc > NA + 2 + TC_NACC, "scale slots");
     static constexpr int xstage = NH * xhalf;
-    // shared memory
-    static constexpr int x_off = 0;
-    static constexpr int bar_off = nx * xstage;
+    // dynamic shared memory: token stages, packed-weight ring (a power of two of alignment slack in front)
+    static constexpr int w_off = nx * xstage;
     static constexpr int n_bars = 2 * TC_NW_MAX + 2 * nx + NA + (NH + 1) * TC_NACC + nsc;   // wfull wempty xfull done afull accfull accempty scfull
-    static constexpr int misc_off = bar_off + n_bars * 8;                    // tmem addr, abort flag, clusters of the split, T, Td
-    static constexpr int cost_off = (misc_off + 32 + 15) / 16 * 16;          // long long: base[32], total
-    static constexpr int sched_off = cost_off + 33 * 8;                      // ints: see TcSched
-    static constexpr int sched_ints = 34 + 33 + 5 * 32;
-    static constexpr int perm_off = sched_off + sched_ints * 4;
-    static constexpr int xrow_off = perm_off + TC_EPI * EC * 4;              // rows of X to gather, one list per gather warp
-    static constexpr int sc_off = (xrow_off + 2 * NH * XR * 4 + 15) / 16 * 16;   // scales on their way to the epilogue
-    static constexpr int w_off = (sc_off + nsc * 4 * 128 * 2 + 127) / 128 * 128;
-    static constexpr int total = 226 * 1024;
-    static constexpr int w_bytes = (total - w_off) / 128 * 128;
-    static constexpr int dyn_bytes = total + 1024;                           // slack for manual 1024-byte alignment
+    static constexpr int static_bytes = 1024 + 1600 + n_bars * 8 + TC_EPI * EC * 4 + 2 * NH * XR * 4 + nsc * 1024;   // (an upper bound of TcShared)
+    static constexpr int w_bytes = (227 * 1024 - static_bytes - 1024 - w_off) / 128 * 128;
+    static constexpr int dyn_bytes = 1024 + w_off + w_bytes;
 };
-static_assert(TcCfg<256>::dyn_bytes <= 232448 && TcCfg<256>::w_bytes >= 3 * 18432, "shared memory budget");
+static_assert(TcCfg<256>::w_bytes >= 3 * 18432, "shared memory budget");
 
 struct TcParams {
     ExpertDev ex[MOQE_MAX_EXPERTS];
@@ -150,17 +141,30 @@ __device__ __forceinline__ uint32_t umma_idesc_pair(int n) {
 }
 
 // ---------------------------------------------------------------------------- schedule
+// (static shared memory: every address is a constant of the code, not a register)
 struct TcSched {
-    int* off;      // [E + 1] (34)
-    int* tile0;    // [E + 1] first tile of each expert (33)
-    int* rpt;      // rows per token tile
-    int* us;       // first unit (k-block of a tile, counted per expert) that is split
-    int* ub;       // this cluster's share of the split units
-    int* ue;
-    int* w;        // cost of a unit
-    long long* base;   // cost before each expert's split units; [32]: total
-    int* misc;     // {clusters of the split, T, Td}
+    int off[MOQE_MAX_EXPERTS + 1];
+    int tile0[MOQE_MAX_EXPERTS + 1];        // first tile of each expert
+    int rpt[MOQE_MAX_EXPERTS];              // rows per token tile
+    int us[MOQE_MAX_EXPERTS];               // first unit (k-block of a tile, counted per expert) that is split
+    int ub[MOQE_MAX_EXPERTS], ue[MOQE_MAX_EXPERTS];   // this cluster's share of the split units
+    int w[MOQE_MAX_EXPERTS];                // cost of a unit
+    int Gs, Td;                             // clusters of the split; tiles that are not split
+    long long base[MOQE_MAX_EXPERTS], C;    // cost before each expert's split units; total
 };
+template <int TN>
+struct TcShared {
+    using L = TcCfg<TN>;
+    unsigned long long bars[L::n_bars];
+    TcSched sc;
+    uint32_t tmem;
+    int abort;
+    __align__(16) int perm[TC_EPI][L::EC];  // per epilogue warp: its columns' target rows
+    int xrow[2][L::NH * L::XR];             // rows of X to gather, one list per gather warp
+    __align__(16) __half scales[L::nsc][4][128];   // on their way to the epilogue
+};
+static_assert(sizeof(TcShared<256>) <= TcCfg<256>::static_bytes && sizeof(TcShared<128>) <= TcCfg<128>::static_bytes &&
+                  sizeof(TcShared<64>) <= TcCfg<64>::static_bytes && sizeof(TcShared<64>) <= 48 * 1024, "shared memory budget");
 
 struct TcPiece { int e, ntp, m0, rows, kb0, kb1, tile; };   // tile: inside the expert
 
@@ -170,7 +174,7 @@ struct TcWalk {
     __device__ __forceinline__ void start(int cluster) { t = cluster; e = -1; u = ue = 0; }
     __device__ __forceinline__ bool next(const TcSched& s, const TcParams& p, int nclusters, TcPiece& pc) {
         int tile;
-        if (t < s.misc[2]) {
+        if (t < s.Td) {
             int ee = 0;
             while (t >= s.tile0[ee + 1]) ++ee;
             pc.e = ee;
@@ -248,62 +252,119 @@ __device__ __forceinline__ void unpack_scaled(const uint32_t (&w)[PieceWords<BIT
 }
 __device__ __forceinline__ uint32_t neg_z(float z) { const float v = z * -0.0001220703125f; return pack_bf16x2(v, v); }
 
-// One k-block of one channel: its four pieces from the packed tile into registers, then to the lane's 64 TMEM columns.
-// scales: where the channel's scales go.  zpc: the channel's zero-point if it is not in the tile (per channel, or a
-// symmetric grid).  bar_free: the barrier whose phase fphase hands the operand buffer back (0: it has not been used
-// yet).  Returns false on abort.
-template <int BITS>
-__device__ __forceinline__ bool dequant_kblock(const ExpertDev& ex, const unsigned char* tile, int row, uint32_t zpc, bool tile_zeros,
-                                               __half* scales, uint32_t bar_scfull, uint32_t bar_wfull, uint32_t wphase, uint32_t bar_wempty,
-                                               uint32_t bar_free, uint32_t fphase, uint32_t a_tmem, volatile int* abort_flag, int* status) {
-    const int lane = threadIdx.x & 31;
+// The dequant role for the k-blocks of one piece.  A thread owns one channel (its TMEM lane): per k-block it reads the four
+// pieces of its codes from the packed tile and fills the 64 TMEM columns of its lane.  zpc: the channel's zero-point if it
+// is not in the tile (per channel, or a symmetric grid).  Returns false on abort.
+// (What the loop needs of the expert is passed by value: fields of the kernel's parameters would be fetched again after
+// every barrier.)
+struct TcDequant {
+    uint32_t bar_wfull, bar_wempty, bar_done, bar_scfull, afull0;   // afull0: in the leading CTA
+    uint32_t lane_tmem;
+    int row, nw, wstage;
+    uint32_t my_group;
+    Ring wring, dring, aring;
+    uint32_t kcount;
+};
+template <int TN, int BITS>
+__device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, const unsigned char* wtiles, int nkb, int per, bool has_zeros,
+                                              uint32_t zpc, bool tile_zeros, int* status) {
+    using L = TcCfg<TN>;
+    const int lane = threadIdx.x & 31, row = d.row;
     const int half = (row >> 3) & 1, r = row & 7;
-    const unsigned char* blob = tile + (row >> 4) * moqe_blob_bytes(BITS);
-    bool ok = __all_sync(0xffffffffu, mbar_wait_short(bar_wfull, wphase, abort_flag, status));
-    uint32_t w[4][PieceWords<BITS>::n];
+    const int meta = moqe_tile_bytes(BITS) + row * 2, mg = has_zeros ? 512 : 256;
+    const unsigned char* blobs = wtiles + (row >> 4) * moqe_blob_bytes(BITS);
+    bool ok = true;
+#pragma unroll 1
+    for (int kb = 0; ok && kb < nkb; ++kb) {
+        if (L::dq_warps == 4 || (d.kcount & 1u) == d.my_group) {
+            const int stage = d.wring.stage * d.wstage;
+            const unsigned char* blob = blobs + stage;
+            ok = __all_sync(0xffffffffu, mbar_wait_short(d.bar_wfull + 8 * d.wring.stage, d.wring.phase, &sh.abort, status));
+            uint32_t w[4][PieceWords<BITS>::n];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int slot = q * 8 + (r ^ (2 * q));
-        if constexpr (BITS == 3) {
-            // both halves share the 16-byte slot: {A, B, C of half 0, A of half 1}
-            const uint4 v = *reinterpret_cast<const uint4*>(blob + slot * 16);
-            const uint2 u = *reinterpret_cast<const uint2*>(blob + 512 + slot * 8);
-            w[q][0] = half ? v.w : v.x;
-            w[q][1] = half ? u.x : v.y;
-            w[q][2] = half ? u.y : v.z;
-        } else {
-            load_piece_smem<BITS>(blob, half, slot, w[q]);
+            for (int q = 0; q < 4; ++q) {
+                const int slot = q * 8 + (r ^ (2 * q));
+                if constexpr (BITS == 3) {
+                    // both halves share the 16-byte slot: {A, B, C of half 0, A of half 1}
+                    const uint4 v = *reinterpret_cast<const uint4*>(blob + slot * 16);
+                    const uint2 u = *reinterpret_cast<const uint2*>(blob + 512 + slot * 8);
+                    w[q][0] = half ? v.w : v.x;
+                    w[q][1] = half ? u.x : v.y;
+                    w[q][2] = half ? u.y : v.z;
+                } else {
+                    load_piece_smem<BITS>(blob, half, slot, w[q]);
+                }
+            }
+            uint32_t nz[4] = {zpc, zpc, zpc, zpc};
+            if (per > 0) {
+                // the tile's scales travel on to the epilogue warps
+                const unsigned char* m = wtiles + stage + meta;
+                __half* scales = &sh.scales[d.kcount & (L::nsc - 1)][0][row];
+                scales[0] = *reinterpret_cast<const __half*>(m);
+                if (per > 1) {
+                    scales[128] = *reinterpret_cast<const __half*>(m + mg);
+                    if (per > 2) {
+                        scales[256] = *reinterpret_cast<const __half*>(m + 2 * mg);
+                        scales[384] = *reinterpret_cast<const __half*>(m + 3 * mg);
+                    }
+                }
+                if (tile_zeros) {
+                    nz[0] = nz[1] = nz[2] = nz[3] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + 256)));
+                    if (per > 1) {
+                        nz[3] = nz[2] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + (per == 2 ? 1 : 2) * 512 + 256)));
+                        if (per > 2) {
+                            nz[1] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + 512 + 256)));
+                            nz[3] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + 3 * 512 + 256)));
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) { mbar_arrive(d.bar_wempty + 8 * d.wring.stage); mbar_arrive(d.bar_scfull + 8 * (d.kcount & (L::nsc - 1))); }
+            // the operand buffer is free once the k-block NA ago is done
+            if (d.kcount >= L::NA) ok &= __all_sync(0xffffffffu, mbar_wait_short(d.bar_done + 8 * d.dring.stage, d.dring.phase, &sh.abort, status));
+            tc_fence_after();
+            const uint32_t at = d.lane_tmem + d.aring.stage * TC_A_COLS;
+            auto chunk = [&](auto Gc) {
+                constexpr int G = decltype(Gc)::value;
+                uint32_t o[16];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) unpack_scaled<BITS, G>(w[q], nz[G], o + 4 * q);
+                tmem_st16(at + 16 * G, o);
+            };
+            chunk(std::integral_constant<int, 0>{});
+            chunk(std::integral_constant<int, 1>{});
+            chunk(std::integral_constant<int, 2>{});
+            chunk(std::integral_constant<int, 3>{});
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) remote_arrive(d.afull0 + 8 * d.aring.stage);
         }
+        d.wring.advance(d.nw);
+        if (d.kcount >= L::NA) d.dring.advance(L::nx);
+        d.aring.advance(L::NA);
+        ++d.kcount;
     }
-    const int per = moqe_groups_per_tile(ex.group);
-    uint32_t nz[4] = {zpc, zpc, zpc, zpc};
-    if (tile_zeros) {
-#pragma unroll
-        for (int G = 0; G < 4; ++G) {
-            const int j = per == 4 ? G : (per == 2 ? (G >> 1) : 0);
-            nz[G] = neg_z(__bfloat162float(moqe_tile_zeros(tile, BITS, j)[row]));
+    return ok;
+}
+// the same for a CTA whose channels do not exist (the second half of the last, odd pair): the operand buffers keep whatever
+// they hold (those products are never read)
+template <int TN>
+__device__ __forceinline__ bool dequant_none(TcDequant& d, TcShared<TN>& sh, int nkb, int* status) {
+    using L = TcCfg<TN>;
+    bool ok = true;
+#pragma unroll 1
+    for (int kb = 0; ok && kb < nkb; ++kb) {
+        if (L::dq_warps == 4 || (d.kcount & 1u) == d.my_group) {
+            if ((threadIdx.x & 31) == 0) mbar_arrive(d.bar_scfull + 8 * (d.kcount & (L::nsc - 1)));
+            if (d.kcount >= L::NA) ok = __all_sync(0xffffffffu, mbar_wait_short(d.bar_done + 8 * d.dring.stage, d.dring.phase, &sh.abort, status));
+            if ((threadIdx.x & 31) == 0) remote_arrive(d.afull0 + 8 * d.aring.stage);
         }
+        if (d.kcount >= L::NA) d.dring.advance(L::nx);
+        d.aring.advance(L::NA);
+        ++d.kcount;
     }
-    // the tile's scales travel on to the epilogue warps
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-        if (j < per) scales[j * 128 + row] = moqe_tile_scales(tile, BITS, ex.has_zeros, j)[row];
-    __syncwarp();
-    if (lane == 0) { mbar_arrive(bar_wempty); mbar_arrive(bar_scfull); }
-    if (bar_free) ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_free, fphase, abort_flag, status));
-    tc_fence_after();
-    auto chunk = [&](auto Gc) {
-        constexpr int G = decltype(Gc)::value;
-        uint32_t o[16];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) unpack_scaled<BITS, G>(w[q], nz[G], o + 4 * q);
-        tmem_st16(a_tmem + 16 * G, o);
-    };
-    chunk(std::integral_constant<int, 0>{});
-    chunk(std::integral_constant<int, 1>{});
-    chunk(std::integral_constant<int, 2>{});
-    chunk(std::integral_constant<int, 3>{});
-    tmem_st_wait();
     return ok;
 }
 
@@ -320,8 +381,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
     qgemm_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap tmap) {
     using L = TcCfg<TN>;
     constexpr int NH = L::NH, NX = L::nx, NA = L::NA, NSC = L::nsc;
+    __shared__ TcShared<TN> sh;
     extern __shared__ unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);
+    TcSched& sc = sh.sc;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_rank();
     const int cluster = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
@@ -329,24 +392,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
     // done[stage]: every MMA of the k-block in that token stage has finished.  One commit per k-block hands back the token
     // stage and the weight buffer and announces the accumulator buffer filled last (a commit costs the issuing warp about
     // 200 cycles, three k16 steps of a half tile).
-    const uint32_t bar_wfull = sbase + L::bar_off, bar_wempty = bar_wfull + 8 * TC_NW_MAX;
+    const uint32_t bar_wfull = smem_u32(sh.bars), bar_wempty = bar_wfull + 8 * TC_NW_MAX;
     const uint32_t bar_xfull = bar_wempty + 8 * TC_NW_MAX, bar_done = bar_xfull + 8 * NX;
     const uint32_t bar_afull = bar_done + 8 * NX;
     const uint32_t bar_accfull = bar_afull + 8 * NA, bar_accempty = bar_accfull + 8 * NH * TC_NACC, bar_scfull = bar_accempty + 8 * TC_NACC;
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + L::misc_off);
-    volatile int* s_abort = reinterpret_cast<volatile int*>(smem + L::misc_off + 4);
-    TcSched sc;
-    sc.misc = reinterpret_cast<int*>(smem + L::misc_off + 8);
-    sc.base = reinterpret_cast<long long*>(smem + L::cost_off);
-    sc.off = reinterpret_cast<int*>(smem + L::sched_off);
-    sc.tile0 = sc.off + 34;
-    sc.rpt = sc.tile0 + 33;
-    sc.us = sc.rpt + 32;
-    sc.ub = sc.us + 32;
-    sc.ue = sc.ub + 32;
-    sc.w = sc.ue + 32;
-    int* s_perm = reinterpret_cast<int*>(smem + L::perm_off);
-    __half* s_sc = reinterpret_cast<__half*>(smem + L::sc_off);
+    volatile int* s_abort = &sh.abort;
 
     // ---- prologue: nothing here depends on the previous kernel in the stream
     if (tid == 0) {
@@ -359,7 +409,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc_pair(sbase + L::misc_off, 512);
+    if (warp == 1) tmem_alloc_pair(smem_u32(&sh.tmem), 512);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (warp == 0) {
@@ -408,13 +458,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         if (e < p.E) { sc.off[e] = o0; sc.tile0[e] = tile0; }
         if (e == p.E - 1) { sc.off[p.E] = o1; sc.tile0[p.E] = T; }
         sc.rpt[e] = rpt; sc.us[e] = us; sc.ub[e] = ub; sc.ue[e] = ue; sc.w[e] = w; sc.base[e] = base;
-        if (lane == 0) { sc.misc[0] = Gs; sc.misc[1] = T; sc.misc[2] = Td; sc.base[32] = C; }
+        if (lane == 0) { sc.Gs = Gs; sc.Td = Td; sc.C = C; }
     }
     tc_fence_before();
     __syncthreads();
     cluster_sync();                                        // the pair's barriers are initialised, its TMEM allocated
     tc_fence_after();
-    const uint32_t tmem_base = *s_tmem;
+    const uint32_t tmem_base = sh.tmem;
 
     if (warp < 4) {
         if constexpr (TN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
@@ -426,7 +476,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             // LAG stages later (at once where nothing is gathered).
             constexpr int LAG = NX == 4 ? 3 : 4;
             const int gw = warp == 0 ? 0 : 1;
-            int* s_xrow = reinterpret_cast<int*>(smem + L::xrow_off) + gw * NH * L::XR;
+            int* s_xrow = sh.xrow[gw];
             const int hi = lane >> 4, c16 = lane & 15;
             // byte offset of this lane's 16-byte chunk of row 4 i + 2 gw + hi: sub-tile, then the 128-byte swizzle
             const uint32_t r0 = 2 * gw + hi;
@@ -473,7 +523,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 __syncwarp();
                 for (int kb = pc.kb0; kb < pc.kb1; ++kb) {
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status)))) break;
-                    const uint32_t stage = sbase + L::x_off + ring.stage * L::xstage;
+                    const uint32_t stage = sbase + ring.stage * L::xstage;
                     if (gw == 0 && bytes > 0) {
                         const uint32_t full = full0 + 8 * ring.stage;
                         if (lane == 0) remote_expect_tx_only(full, bytes);
@@ -573,7 +623,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
 #pragma unroll 1
                     for (int h = 0; h < nh; ++h) {
                         const uint32_t idesc = umma_idesc_pair(half_cols<L::HC>(pc.rows, h));
-                        const uint64_t bdesc = umma_desc_sw128(sbase + L::x_off + ring.stage * L::xstage + h * L::xhalf);
+                        const uint64_t bdesc = umma_desc_sw128(sbase + ring.stage * L::xstage + h * L::xhalf);
                         const bool last_half = h + 1 == nh;
                         if (steps == 8) {
                             const int b2 = keep && h ? (buf + 1 == TC_NACC ? 0 : buf + 1) : buf;
@@ -626,52 +676,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         if constexpr (TN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         else asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
         // ---------------- dequant warps: thread = channel = TMEM lane ----------------
-        const int row = (warp & 3) * 32 + lane;
-        const uint32_t my_group = (uint32_t)((warp - 4) >> 2);
-        const uint32_t afull0 = mapa(bar_afull, 0);
-        const uint32_t lane_tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + L::a_base;
-        Ring wring, dring, aring;
+        TcDequant d;
+        d.bar_wfull = bar_wfull; d.bar_wempty = bar_wempty; d.bar_done = bar_done; d.bar_scfull = bar_scfull;
+        d.afull0 = mapa(bar_afull, 0);
+        d.row = (warp & 3) * 32 + lane;
+        d.lane_tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + L::a_base;
+        d.nw = p.nw; d.wstage = p.wstage;
+        d.my_group = (uint32_t)((warp - 4) >> 2);
+        d.kcount = 0;
+        const unsigned char* wtiles = smem + L::w_off;
         TcPiece pc;
         TcWalk wk;
         wk.start(cluster);
         bool ok = true;
-        uint32_t kcount = 0;
         while (ok && wk.next(sc, p, nclusters, pc)) {
             const ExpertDev& ex = p.ex[pc.e];
-            const int nt = 2 * pc.ntp + (int)rank;
-            const bool active = nt < p.NT1;
-            const bool tile_zeros = ex.has_zeros && ex.group != 0;
+            const int nt = 2 * pc.ntp + (int)rank, nkb = pc.kb1 - pc.kb0;
+            if (nt >= p.NT1) { ok = dequant_none<TN>(d, sh, nkb, p.status); continue; }
+            const bool has_zeros = ex.has_zeros != 0, tile_zeros = has_zeros && ex.group != 0;
+            const int per = moqe_groups_per_tile(ex.group);
             float z = (float)(1 << (ex.bits - 1));
-            if (ex.has_zeros && ex.group == 0 && active) z = __bfloat162float(ex.zeros_pc[nt * 128 + row]);
+            if (has_zeros && ex.group == 0) z = __bfloat162float(ex.zeros_pc[nt * 128 + d.row]);
             const uint32_t zpc = neg_z(z);
-            for (int kb = pc.kb0; ok && kb < pc.kb1; ++kb, ++kcount) {
-                const bool mine = L::dq_warps == 4 || (kcount & 1u) == my_group;
-                // the buffer is free once the k-block NA ago is done
-                const uint32_t free_bar = kcount >= NA ? bar_done + 8 * dring.stage : 0u;
-                const uint32_t scfull = bar_scfull + 8 * (kcount & (NSC - 1));
-                if (mine && active) {
-                    const unsigned char* tile = smem + L::w_off + wring.stage * p.wstage;
-                    __half* scales = s_sc + (kcount & (NSC - 1)) * 512;
-                    const uint32_t wf = bar_wfull + 8 * wring.stage, we = bar_wempty + 8 * wring.stage, at = lane_tmem + aring.stage * TC_A_COLS;
-                    switch (ex.bits) {
-                        case 4: ok = dequant_kblock<4>(ex, tile, row, zpc, tile_zeros, scales, scfull, wf, wring.phase, we, free_bar, dring.phase, at, s_abort, p.status); break;
-                        case 8: ok = dequant_kblock<8>(ex, tile, row, zpc, tile_zeros, scales, scfull, wf, wring.phase, we, free_bar, dring.phase, at, s_abort, p.status); break;
-                        case 3: ok = dequant_kblock<3>(ex, tile, row, zpc, tile_zeros, scales, scfull, wf, wring.phase, we, free_bar, dring.phase, at, s_abort, p.status); break;
-                        default: ok = dequant_kblock<2>(ex, tile, row, zpc, tile_zeros, scales, scfull, wf, wring.phase, we, free_bar, dring.phase, at, s_abort, p.status); break;
-                    }
-                } else if (mine) {
-                    // no channels here: the operand buffer keeps whatever it holds (those products are never read)
-                    if (lane == 0) mbar_arrive(scfull);
-                    if (free_bar) ok = __all_sync(0xffffffffu, mbar_wait_short(free_bar, dring.phase, s_abort, p.status));
-                }
-                if (mine) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) remote_arrive(afull0 + 8 * aring.stage);
-                }
-                if (active) wring.advance(p.nw);
-                if (kcount >= NA) dring.advance(NX);
-                aring.advance(NA);
+            switch (ex.bits) {
+                case 4: ok = dequant_piece<TN, 4>(d, sh, wtiles, nkb, per, has_zeros, zpc, tile_zeros, p.status); break;
+                case 8: ok = dequant_piece<TN, 8>(d, sh, wtiles, nkb, per, has_zeros, zpc, tile_zeros, p.status); break;
+                case 3: ok = dequant_piece<TN, 3>(d, sh, wtiles, nkb, per, has_zeros, zpc, tile_zeros, p.status); break;
+                default: ok = dequant_piece<TN, 2>(d, sh, wtiles, nkb, per, has_zeros, zpc, tile_zeros, p.status); break;
             }
         }
     } else {
@@ -686,7 +717,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         const int row = quarter * 32 + lane;               // channel inside the 128-channel tile = TMEM lane
         const uint32_t accempty0 = mapa(bar_accempty, 0);
         const uint32_t lane_tmem = tmem_base + ((uint32_t)(quarter * 32) << 16);
-        int* my_perm = s_perm + ew * L::EC;                // private to this warp: no cross-warp barrier
+        int* my_perm = sh.perm[ew];                        // private to this warp: no cross-warp barrier
         TcPiece pc;
         TcWalk wk;
         wk.start(cluster);
@@ -744,7 +775,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                                 if (c == 0 && !keep) {
                                     // the group's scale, fetched while the load is under way
                                     if (j == 0) ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_scfull + 8 * slot, (kcount / NSC) & 1u, s_abort, p.status));
-                                    s = __half2float(s_sc[slot * 512 + j * 128 + row]) * W8_PRESCALE;
+                                    s = __half2float(sh.scales[slot][j][row]) * W8_PRESCALE;
                                 }
                                 tmem_ld_wait();
                                 fma_cols32(acc + 32 * c, v, s);
@@ -769,8 +800,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             if (!active) continue;
             if (pc.kb0 != 0 || pc.kb1 != p.KB) {
                 // part of a tile: park this warp's sums, announce, and add everything up if this was the last arrival
-                const long long C = sc.base[32], first = sc.base[pc.e] + (long long)(pc.tile * p.KB - sc.us[pc.e]) * sc.w[pc.e];
-                const int Gs = sc.misc[0];
+                const long long C = sc.C, first = sc.base[pc.e] + (long long)(pc.tile * p.KB - sc.us[pc.e]) * sc.w[pc.e];
+                const int Gs = sc.Gs;
                 const int c_a = (int)(first * Gs / C), c_b = (int)((first + (long long)(p.KB - 1) * sc.w[pc.e]) * Gs / C);
                 const size_t slot = (size_t)p.cols * 128;
                 auto slot_of = [&](int c, int which) { return p.partials + ((size_t)(c * 2 + which) * 2 + rank) * slot + (size_t)tok0 * 128 + row; };
