@@ -44,36 +44,44 @@ constexpr int TC_MAX_CLUSTERS = 80;
 constexpr int TC_EPI = 8;                          // epilogue warps
 constexpr int TC_NW_MAX = 12;                      // packed-weight stages
 constexpr int TC_A_COLS = 64;                      // TMEM columns of one k-block of unpacked weights
-constexpr int TC_NACC = 3;
 
 // TN: tokens of a tile.  256: the tensor core's 1024 cycles a k-block hide one dequant warpgroup's work; 128 and 64: small
-// batches, where unpacking is the critical role and gets two warpgroups that take turns (and, with 64, five weight buffers
-// instead of two, so that they do not wait for the round trip through the tensor core).
+// batches, where unpacking is the critical role and gets two warpgroups.  With 64 tokens every hand-over between the roles
+// costs more than the work handed over, so a step takes KS = 2 k-blocks: the two dequant groups unpack one each, the two
+// epilogue groups drain one each.
 template <int TN>
 struct TcCfg {
     static constexpr int NH = TN == 256 ? 2 : 1;                             // half tiles
+    static constexpr int KS = TN == 64 ? 2 : 1;                              // k-blocks of a step
     static constexpr int HC = TN / NH;                                       // columns of a half tile = of an accumulator buffer
     static constexpr int XR = HC / 2;                                        // token rows a CTA fetches for a half tile
     static constexpr int xhalf = 2 * XR * 128;                               // XR rows x 128 k bf16: two 64-k swizzled sub-tiles
-    static constexpr int a_base = TC_NACC * HC;                              // the weight buffers sit behind the accumulators
-    static constexpr int NA = (512 - a_base) / TC_A_COLS;
-    static constexpr int EC = TN / 2;                                        // columns of an epilogue warp
+    static constexpr int NACC = TN == 64 ? 4 : 3;                            // accumulator buffers
+    static constexpr int a_base = NACC * HC;                                 // the weight buffers sit behind them
+    static constexpr int NA = 2;                                             // weight buffers (of KS k-blocks)
+    static_assert(a_base + NA * KS * TC_A_COLS <= 512, "tensor memory");
+    static constexpr int EC = TN / 2;                                        // columns an epilogue warp stores
+    static constexpr int DC = TN == 64 ? 64 : EC;                            // columns it drains
     static constexpr int dq_warps = TN == 256 ? 4 : 8;
+    static constexpr int dq_arrive = KS == 2 ? 8 : 4;                        // dequant warps that fill one weight buffer
     static constexpr int epi_warp0 = 4 + dq_warps;
     static constexpr int threads = (epi_warp0 + TC_EPI) * 32;
-    static constexpr int nx = TN == 256 ? 4 : 6;                             // token stages: one k-block of the tile
-    static_assert(NA <= nx, "the dequant warps wait for the k-block NA ago on its token stage's barrier");
-    // k-blocks of scales between the dequant warps and the epilogue.  When the scales of k-block k are written, the k-block
-    // NA + 2 before it is done and at most three buffers are still to be drained: slot k - nsc must be older than that.
-    static constexpr int nsc = NA == 2 ? 8 : 16;
-    static_assert(nsc > NA + 2 + TC_NACC, "scale slots");
-    static constexpr int xstage = NH * xhalf;
+    static constexpr int nx = 4;                                             // token stages: one step of the tile
+    // (nx, NA and nsc are powers of two: stage and parity follow from the step's number)
+    static_assert(NA <= nx, "the dequant warps wait for the step NA ago on its token stage's barrier");
+    // Steps of scales between the dequant warps and the epilogue.  When the scales of step k are written, step k - NA - 2
+    // is done and at most NACC buffers are still to be drained: slot k - nsc must be older than that.
+    static constexpr int nsc = 8;
+    static_assert(nsc >= NA + 2 + NACC, "scale slots");
+    static constexpr int xstage = KS * NH * xhalf;
     // dynamic shared memory: token stages, packed-weight ring (a power of two of alignment slack in front)
     static constexpr int w_off = nx * xstage;
-    static constexpr int n_bars = 2 * TC_NW_MAX + 2 * nx + NA + (NH + 1) * TC_NACC + nsc;   // wfull wempty xfull done afull accfull accempty scfull
-    static constexpr int static_bytes = 1024 + 1600 + n_bars * 8 + TC_EPI * EC * 4 + 2 * NH * XR * 4 + nsc * 1024;   // (an upper bound of TcShared)
-    static constexpr int w_bytes = (227 * 1024 - static_bytes - 1024 - w_off) / 128 * 128;
-    static constexpr int dyn_bytes = 1024 + w_off + w_bytes;
+    static constexpr int n_bars = 2 * TC_NW_MAX + 2 * nx + NA + 3 * NACC + nsc + 2 * TC_EPI;   // wfull wempty xfull done afull accfull[2] accempty scfull xchg[2]
+    static constexpr int xchg_bytes = TN == 64 ? TC_EPI * 32 * 32 * 4 : 16;
+    static constexpr int static_bytes = 1024 + 1600 + n_bars * 8 + TC_EPI * EC * 4 + 2 * NH * XR * 4 + nsc * KS * 1024 + 64;   // (an upper bound of TcShared)
+    static constexpr int xchg_off = (227 * 1024 - static_bytes - 1024 - xchg_bytes) / 128 * 128;
+    static constexpr int w_bytes = (xchg_off - w_off) / 128 * 128;
+    static constexpr int dyn_bytes = 1024 + xchg_off + xchg_bytes;
 };
 static_assert(TcCfg<256>::w_bytes >= 3 * 18432, "shared memory budget");
 
@@ -91,6 +99,15 @@ struct TcParams {
     int nw, wstage;           // packed-weight ring
     int split;                // 0: whole tiles only
 };
+
+// A whole warp's bounded wait.  The outcome is per lane (false: the CTA is aborting); the loops vote on it once a step, not
+// after every wait (a vote each time made a wait that does not wait cost 85 cycles instead of 48).
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
+    bool ok = mbar_try_short(bar, parity);
+    if (!ok) ok = mbar_wait_short(bar, parity, abort_flag, status);
+    __syncwarp();
+    return ok;
+}
 
 // ---------------------------------------------------------------------------- PTX of the two-CTA forms
 __device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
@@ -161,7 +178,7 @@ struct TcShared {
     int abort;
     __align__(16) int perm[TC_EPI][L::EC];  // per epilogue warp: its columns' target rows
     int xrow[2][L::NH * L::XR];             // rows of X to gather, one list per gather warp
-    __align__(16) __half scales[L::nsc][4][128];   // on their way to the epilogue
+    __align__(16) __half scales[L::nsc][L::KS][4][128];   // on their way to the epilogue
 };
 static_assert(sizeof(TcShared<256>) <= TcCfg<256>::static_bytes && sizeof(TcShared<128>) <= TcCfg<128>::static_bytes &&
                   sizeof(TcShared<64>) <= TcCfg<64>::static_bytes && sizeof(TcShared<64>) <= 48 * 1024, "shared memory budget");
@@ -262,8 +279,8 @@ struct TcDequant {
     uint32_t lane_tmem;
     int row, nw, wstage;
     uint32_t my_group;
-    Ring wring, dring, aring;
-    uint32_t kcount;
+    Ring wring;
+    uint32_t step;
 };
 template <int TN, int BITS>
 __device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, const unsigned char* wtiles, int nkb, int per, bool has_zeros,
@@ -275,11 +292,15 @@ __device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, co
     const unsigned char* blobs = wtiles + (row >> 4) * moqe_blob_bytes(BITS);
     bool ok = true;
 #pragma unroll 1
-    for (int kb = 0; ok && kb < nkb; ++kb) {
-        if (L::dq_warps == 4 || (d.kcount & 1u) == d.my_group) {
+    for (int kb = 0; ok && kb < nkb; kb += L::KS) {
+        const int nk = min(L::KS, nkb - kb);
+        const int kk = L::KS == 2 ? (int)d.my_group : 0;              // this group's k-block of the step
+        const bool mine = L::KS == 2 ? kk < nk : (L::dq_warps == 4 || (d.step & 1u) == d.my_group);
+        if (mine) {
+            if (L::KS == 2 && kk) d.wring.advance(d.nw);
             const int stage = d.wring.stage * d.wstage;
             const unsigned char* blob = blobs + stage;
-            ok = __all_sync(0xffffffffu, mbar_wait_short(d.bar_wfull + 8 * d.wring.stage, d.wring.phase, &sh.abort, status));
+            ok = warp_wait(d.bar_wfull + 8 * d.wring.stage, d.wring.phase, &sh.abort, status);
             uint32_t w[4][PieceWords<BITS>::n];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -299,7 +320,7 @@ __device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, co
             if (per > 0) {
                 // the tile's scales travel on to the epilogue warps
                 const unsigned char* m = wtiles + stage + meta;
-                __half* scales = &sh.scales[d.kcount & (L::nsc - 1)][0][row];
+                __half* scales = &sh.scales[d.step % L::nsc][kk][0][row];
                 scales[0] = *reinterpret_cast<const __half*>(m);
                 if (per > 1) {
                     scales[128] = *reinterpret_cast<const __half*>(m + mg);
@@ -320,11 +341,11 @@ __device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, co
                 }
             }
             __syncwarp();
-            if (lane == 0) { mbar_arrive(d.bar_wempty + 8 * d.wring.stage); mbar_arrive(d.bar_scfull + 8 * (d.kcount & (L::nsc - 1))); }
-            // the operand buffer is free once the k-block NA ago is done
-            if (d.kcount >= L::NA) ok &= __all_sync(0xffffffffu, mbar_wait_short(d.bar_done + 8 * d.dring.stage, d.dring.phase, &sh.abort, status));
+            if (lane == 0) { mbar_arrive(d.bar_wempty + 8 * d.wring.stage); mbar_arrive(d.bar_scfull + 8 * (d.step % L::nsc)); }
+            // the operand buffer is free once the step NA ago is done
+            if (d.step >= L::NA) ok &= warp_wait(d.bar_done + 8 * ((d.step - L::NA) % L::nx), (d.step - L::NA) / L::nx & 1u, &sh.abort, status);
             tc_fence_after();
-            const uint32_t at = d.lane_tmem + d.aring.stage * TC_A_COLS;
+            const uint32_t at = d.lane_tmem + (d.step % L::NA * L::KS + kk) * TC_A_COLS;
             auto chunk = [&](auto Gc) {
                 constexpr int G = decltype(Gc)::value;
                 uint32_t o[16];
@@ -339,12 +360,18 @@ __device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, co
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) remote_arrive(d.afull0 + 8 * d.aring.stage);
+            if (lane == 0) remote_arrive(d.afull0 + 8 * (d.step % L::NA));
+            d.wring.advance(d.nw);
+            if (L::KS == 2 && nk == 2 && !kk) d.wring.advance(d.nw);
+            ok = __all_sync(0xffffffffu, ok);
+        } else if (L::KS == 2) {
+            // (the step has no k-block for this group)
+            if (lane == 0) { mbar_arrive(d.bar_scfull + 8 * (d.step % L::nsc)); remote_arrive(d.afull0 + 8 * (d.step % L::NA)); }
+            d.wring.advance(d.nw);
+        } else {
+            d.wring.advance(d.nw);
         }
-        d.wring.advance(d.nw);
-        if (d.kcount >= L::NA) d.dring.advance(L::nx);
-        d.aring.advance(L::NA);
-        ++d.kcount;
+        ++d.step;
     }
     return ok;
 }
@@ -355,24 +382,24 @@ __device__ __forceinline__ bool dequant_none(TcDequant& d, TcShared<TN>& sh, int
     using L = TcCfg<TN>;
     bool ok = true;
 #pragma unroll 1
-    for (int kb = 0; ok && kb < nkb; ++kb) {
-        if (L::dq_warps == 4 || (d.kcount & 1u) == d.my_group) {
-            if ((threadIdx.x & 31) == 0) mbar_arrive(d.bar_scfull + 8 * (d.kcount & (L::nsc - 1)));
-            if (d.kcount >= L::NA) ok = __all_sync(0xffffffffu, mbar_wait_short(d.bar_done + 8 * d.dring.stage, d.dring.phase, &sh.abort, status));
-            if ((threadIdx.x & 31) == 0) remote_arrive(d.afull0 + 8 * d.aring.stage);
+    for (int kb = 0; ok && kb < nkb; kb += L::KS) {
+        if (L::KS == 2 || L::dq_warps == 4 || (d.step & 1u) == d.my_group) {
+            if ((threadIdx.x & 31) == 0) mbar_arrive(d.bar_scfull + 8 * (d.step % L::nsc));
+            if (d.step >= L::NA) ok = __all_sync(0xffffffffu, warp_wait(d.bar_done + 8 * ((d.step - L::NA) % L::nx), (d.step - L::NA) / L::nx & 1u, &sh.abort, status));
+            if ((threadIdx.x & 31) == 0) remote_arrive(d.afull0 + 8 * (d.step % L::NA));
         }
-        if (d.kcount >= L::NA) d.dring.advance(L::nx);
-        d.aring.advance(L::NA);
-        ++d.kcount;
+        ++d.step;
     }
     return ok;
 }
 
-// acc[0..31] += s * v
-// (Scalar: the packed two-column form needs aligned register pairs, and the moves that make them cost more than it saves.)
+// acc[0..31] += s * v, two columns per instruction (each half rounds as a scalar fma does)
 __device__ __forceinline__ void fma_cols32(float* acc, const uint32_t (&v)[32], float s) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) acc[i] = fmaf(s, __uint_as_float(v[i]), acc[i]);
+    for (int i = 0; i < 32; i += 2)
+        asm("{\n\t.reg .b64 a, x, s2;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 x, {%3, %4};\n\tmov.b64 s2, {%2, %2};\n\t"
+            "fma.rn.f32x2 a, s2, x, a;\n\tmov.b64 {%0, %1}, a;\n\t}"
+            : "+f"(acc[i]), "+f"(acc[i + 1]) : "f"(s), "r"(v[i]), "r"(v[i + 1]));
 }
 
 // ---------------------------------------------------------------------------- the kernel
@@ -380,7 +407,7 @@ template <int TN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 1)
     qgemm_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap tmap) {
     using L = TcCfg<TN>;
-    constexpr int NH = L::NH, NX = L::nx, NA = L::NA, NSC = L::nsc;
+    constexpr int NH = L::NH, KS = L::KS, NX = L::nx, NA = L::NA, NSC = L::nsc, NACC = L::NACC;
     __shared__ TcShared<TN> sh;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);
@@ -389,23 +416,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
     const uint32_t rank = cluster_rank();
     const int cluster = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
     const uint32_t sbase = smem_u32(smem);
-    // done[stage]: every MMA of the k-block in that token stage has finished.  One commit per k-block hands back the token
+    // done[stage]: every MMA of the step in that token stage has finished.  One commit per step hands back the token
     // stage and the weight buffer and announces the accumulator buffer filled last (a commit costs the issuing warp about
     // 200 cycles, three k16 steps of a half tile).
     const uint32_t bar_wfull = smem_u32(sh.bars), bar_wempty = bar_wfull + 8 * TC_NW_MAX;
     const uint32_t bar_xfull = bar_wempty + 8 * TC_NW_MAX, bar_done = bar_xfull + 8 * NX;
     const uint32_t bar_afull = bar_done + 8 * NX;
-    const uint32_t bar_accfull = bar_afull + 8 * NA, bar_accempty = bar_accfull + 8 * NH * TC_NACC, bar_scfull = bar_accempty + 8 * TC_NACC;
+    const uint32_t bar_accfull = bar_afull + 8 * NA, bar_accempty = bar_accfull + 16 * NACC, bar_scfull = bar_accempty + 8 * NACC, bar_xchg = bar_scfull + 8 * NSC;
     volatile int* s_abort = &sh.abort;
 
     // ---- prologue: nothing here depends on the previous kernel in the stream
     if (tid == 0) {
         for (int i = 0; i < TC_NW_MAX; ++i) { mbar_init(bar_wfull + 8 * i, 1); mbar_init(bar_wempty + 8 * i, 4); }
         for (int i = 0; i < NX; ++i) { mbar_init(bar_xfull + 8 * i, 4); mbar_init(bar_done + 8 * i, 1); }
-        for (int i = 0; i < NA; ++i) mbar_init(bar_afull + 8 * i, 8);
-        for (int i = 0; i < NH * TC_NACC; ++i) mbar_init(bar_accfull + 8 * i, 1);
-        for (int i = 0; i < TC_NACC; ++i) mbar_init(bar_accempty + 8 * i, 2 * TC_EPI);
-        for (int i = 0; i < NSC; ++i) mbar_init(bar_scfull + 8 * i, 4);
+        for (int i = 0; i < NA; ++i) mbar_init(bar_afull + 8 * i, 2 * L::dq_arrive);
+        for (int i = 0; i < 2 * NACC; ++i) mbar_init(bar_accfull + 8 * i, 1);
+        for (int i = 0; i < NACC; ++i) mbar_init(bar_accempty + 8 * i, 2 * TC_EPI);
+        for (int i = 0; i < NSC; ++i) mbar_init(bar_scfull + 8 * i, L::dq_arrive);
+        if (KS == 2)
+            for (int i = 0; i < 2 * TC_EPI; ++i) mbar_init(bar_xchg + 8 * i, 1);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -468,20 +497,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
 
     if (warp < 4) {
         if constexpr (TN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
-        else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
         if (warp == 0 || warp == 3) {
-            // ---------------- X producers: this CTA's XR token rows of every half tile, 128 k per stage ----------------
+            // ---------------- X producers: this CTA's XR token rows of every half tile, KS x 128 k per stage ----------------
             // Both warps walk the stages and arrive on the pair's xfull barrier; warp 0 also adds the byte count of the TMA
             // boxes.  A warp gathers every other pair of rows; its arrival for a stage follows once its copies have landed,
             // LAG stages later (at once where nothing is gathered).
-            constexpr int LAG = NX == 4 ? 3 : 4;
+            constexpr int LAG = 3;
             const int gw = warp == 0 ? 0 : 1;
             int* s_xrow = sh.xrow[gw];
             const int hi = lane >> 4, c16 = lane & 15;
             // byte offset of this lane's 16-byte chunk of row 4 i + 2 gw + hi: sub-tile, then the 128-byte swizzle
             const uint32_t r0 = 2 * gw + hi;
             const uint32_t sw0 = (c16 >> 3) * (L::XR * 128) + r0 * 128 + (((c16 & 7) ^ r0) << 4), sw1 = (c16 >> 3) * (L::XR * 128) + (r0 + 4) * 128 + (((c16 & 7) ^ (r0 + 4)) << 4);
-            Ring ring, aring;                              // aring: the stage whose arrival is due next
+            uint32_t step = 0, due = 0;                    // due: the step whose arrival comes next
             TcPiece pc;
             TcWalk wk;
             wk.start(cluster);
@@ -491,8 +520,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             auto arrive = [&]() {
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) remote_arrive(full0 + 8 * aring.stage);
-                aring.advance(NX);
+                if (lane == 0) remote_arrive(full0 + 8 * (due % NX));
+                ++due;
             };
             while (ok && wk.next(sc, p, nclusters, pc)) {
                 const int nh = NH == 1 ? 1 : (pc.rows > L::HC ? 2 : 1);
@@ -521,36 +550,44 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                     }
                 }
                 __syncwarp();
-                for (int kb = pc.kb0; kb < pc.kb1; ++kb) {
-                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status)))) break;
-                    const uint32_t stage = sbase + ring.stage * L::xstage;
+                for (int kb0 = pc.kb0; kb0 < pc.kb1; kb0 += KS) {
+                    const int nk = min(KS, pc.kb1 - kb0);
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * (step % NX), (step / NX & 1u) ^ 1u, s_abort, p.status)))) break;
+                    const uint32_t full = full0 + 8 * (step % NX);
                     if (gw == 0 && bytes > 0) {
-                        const uint32_t full = full0 + 8 * ring.stage;
-                        if (lane == 0) remote_expect_tx_only(full, bytes);
-                        __syncwarp();
-#pragma unroll
-                        for (int h = 0; h < NH; ++h)
-                            if (src[h] >= 0 && lane < 2) tma_box_pair(stage + h * L::xhalf + lane * (L::XR * 128), &tmap, kb * 128 + lane * 64, src[h], full);
+                        if (lane == 0) remote_expect_tx_only(full, bytes * nk);
                         __syncwarp();
                     }
-                    const int k = kb * 128 + c16 * 8;
-                    const int real = k < p.K ? 16 : 0;
-                    const char* xk = reinterpret_cast<const char*>(p.X) + (real ? (size_t)k * 2 : 0);
 #pragma unroll
-                    for (int h = 0; h < NH; ++h) {
-                        if (src[h] < 0) {
-                            const uint32_t dst = stage + h * L::xhalf;
+                    for (int kk = 0; kk < KS; ++kk) {
+                        if (kk >= nk) break;
+                        const int kb = kb0 + kk;
+                        const uint32_t stage = sbase + (step % NX) * L::xstage + kk * (NH * L::xhalf);
+                        if (gw == 0 && bytes > 0) {
+#pragma unroll
+                            for (int h = 0; h < NH; ++h)
+                                if (src[h] >= 0 && lane < 2) tma_box_pair(stage + h * L::xhalf + lane * (L::XR * 128), &tmap, kb * 128 + lane * 64, src[h], full);
+                            __syncwarp();
+                        }
+                        const int k = kb * 128 + c16 * 8;
+                        const int real = k < p.K ? 16 : 0;
+                        const char* xk = reinterpret_cast<const char*>(p.X) + (real ? (size_t)k * 2 : 0);
+#pragma unroll
+                        for (int h = 0; h < NH; ++h) {
+                            if (src[h] < 0) {
+                                const uint32_t dst = stage + h * L::xhalf;
 #pragma unroll 4
-                            for (int i = 0; i < L::XR / 4; ++i) {
-                                const int r = 4 * i + (int)r0;
-                                if (4 * i + 2 * gw >= cnt[h]) break;
-                                if (r < cnt[h])
-                                    cp_async16(dst + ((i & 1) ? sw1 : sw0) + (i >> 1) * 1024, xk + (size_t)s_xrow[h * L::XR + r] * (size_t)(p.K * 2), real);
+                                for (int i = 0; i < L::XR / 4; ++i) {
+                                    const int r = 4 * i + (int)r0;
+                                    if (4 * i + 2 * gw >= cnt[h]) break;
+                                    if (r < cnt[h])
+                                        cp_async16(dst + ((i & 1) ? sw1 : sw0) + (i >> 1) * 1024, xk + (size_t)s_xrow[h * L::XR + r] * (size_t)(p.K * 2), real);
+                                }
                             }
                         }
                     }
                     asm volatile("cp.async.commit_group;" ::: "memory");
-                    ring.advance(NX);
+                    ++step;
                     ++pending;
                     if (!gathers) {
                         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -566,8 +603,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             for (; ok && pending > 0; --pending) arrive();
             // every stage handed back (the commits come from the leading CTA) before this CTA may exit
             for (int i = 0; ok && i < NX; ++i) {
-                ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status));
-                ring.advance(NX);
+                ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * (step % NX), (step / NX & 1u) ^ 1u, s_abort, p.status));
+                ++step;
             }
         } else if (warp == 2) {
             // ---------------- W producer: one packed 128x128-code tile per k-block ----------------
@@ -599,48 +636,55 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             // The WHOLE warp walks the pieces, so that control flow stays warp-uniform, and one elected lane issues
             // straight-line MMAs whose operands were all computed beforehand: issued from a loop that only lane 0
             // runs, every MMA costs ~250 cycles.
-            Ring ring;
             TcPiece pc;
             TcWalk wk;
             wk.start(cluster);
             bool ok = true;
-            Ring aring;                                    // weight buffers
+            uint32_t step = 0;
             int buf = 0;
             uint32_t buf_phase = 1;                        // parity of "empty" for the buffers of this round
-            auto next_buf = [&]() { if (++buf == TC_NACC) { buf = 0; buf_phase ^= 1u; } };
+            auto next_buf = [&]() { if (++buf == NACC) { buf = 0; buf_phase ^= 1u; } };
             while (ok && wk.next(sc, p, nclusters, pc)) {
                 const int nh = NH == 1 ? 1 : (pc.rows > L::HC ? 2 : 1);
                 const int group = p.ex[pc.e].group;
                 // A per-channel expert's half tile h stays in buffer (buf + h) of the rotation for the whole piece.
                 const bool keep = group == 0;
                 const int steps = keep || group >= 128 ? 8 : group >> 4;         // MMAs into one accumulator buffer
-                for (int kb = pc.kb0; ok && kb < pc.kb1; ++kb) {
-                    ok = __all_sync(0xffffffffu, mbar_wait_short(bar_xfull + 8 * ring.stage, ring.phase, s_abort, p.status));
-                    ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_afull + 8 * aring.stage, aring.phase, s_abort, p.status));
+                for (int kb0 = pc.kb0; ok && kb0 < pc.kb1; kb0 += KS) {
+                    const int nk = min(KS, pc.kb1 - kb0);
+                    ok = warp_wait(bar_xfull + 8 * (step % NX), step / NX & 1u, s_abort, p.status);
+                    ok &= warp_wait(bar_afull + 8 * (step % NA), step / NA & 1u, s_abort, p.status);
                     tc_fence_after();
-                    const uint32_t a_tmem = tmem_base + L::a_base + aring.stage * TC_A_COLS;
-                    const uint32_t done = bar_done + 8 * ring.stage;
+                    const uint32_t done = bar_done + 8 * (step % NX);
+                    const uint64_t xdesc = umma_desc_sw128(sbase + (step % NX) * L::xstage);
+                    // sub-steps: the half tiles of the k-block, or the k-blocks of the step.  Sub-step u is drained by epilogue
+                    // group u (see there).
+                    const int nu = KS == 2 ? nk : nh;
 #pragma unroll 1
-                    for (int h = 0; h < nh; ++h) {
+                    for (int u = 0; u < nu; ++u) {
+                        const int h = KS == 2 ? 0 : u, kk = KS == 2 ? u : 0;
+                        const uint32_t a_tmem = tmem_base + L::a_base + ((step % NA) * KS + kk) * TC_A_COLS;
                         const uint32_t idesc = umma_idesc_pair(half_cols<L::HC>(pc.rows, h));
-                        const uint64_t bdesc = umma_desc_sw128(sbase + ring.stage * L::xstage + h * L::xhalf);
-                        const bool last_half = h + 1 == nh;
+                        const uint64_t bdesc = xdesc + u * (L::xhalf / 16);
+                        const bool last = u + 1 == nu;
                         if (steps == 8) {
-                            const int b2 = keep && h ? (buf + 1 == TC_NACC ? 0 : buf + 1) : buf;
-                            const uint32_t ph = keep && h && buf + 1 == TC_NACC ? buf_phase ^ 1u : buf_phase;
-                            const uint32_t add = keep && kb > pc.kb0 ? 1u : 0u;
-                            if (!add) ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_accempty + 8 * b2, ph, s_abort, p.status));
-                            tc_fence_after();
+                            const int b2 = keep && h ? (buf + 1 == NACC ? 0 : buf + 1) : buf;
+                            const uint32_t ph = keep && h && buf + 1 == NACC ? buf_phase ^ 1u : buf_phase;
+                            const uint32_t add = keep && kb0 + kk > pc.kb0 ? 1u : 0u;
+                            if (!add) {
+                                ok &= warp_wait(bar_accempty + 8 * b2, ph, s_abort, p.status);
+                                tc_fence_after();
+                            }
                             const uint32_t d = tmem_base + b2 * L::HC;
                             if (elect_one()) {
 #pragma unroll
                                 for (int i = 0; i < 8; ++i)
                                     umma_pair_ts(d, a_tmem + 8 * i, bdesc + (i >> 2) * (L::XR * 8) + (i & 3) * 2, idesc, i > 0 ? 1u : add);
                                 if (keep) {
-                                    if (last_half) umma_commit_pair(done);
-                                    if (kb + 1 == pc.kb1) umma_commit_pair(bar_accfull + 8 * (h * TC_NACC + b2));
+                                    if (last) umma_commit_pair(done);
+                                    if (kb0 + kk + 1 == pc.kb1) umma_commit_pair(bar_accfull + 8 * (h * NACC + b2));
                                 } else {
-                                    umma_commit_pair(last_half ? done : bar_accfull + 8 * (h * TC_NACC + b2));
+                                    umma_commit_pair(last ? done : bar_accfull + 8 * (u * NACC + b2));
                                 }
                             }
                             __syncwarp();
@@ -648,7 +692,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                         } else {
 #pragma unroll 1
                             for (int i0 = 0; i0 < 8; i0 += steps) {
-                                ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_accempty + 8 * buf, buf_phase, s_abort, p.status));
+                                ok &= warp_wait(bar_accempty + 8 * buf, buf_phase, s_abort, p.status);
                                 tc_fence_after();
                                 const uint32_t d = tmem_base + buf * L::HC;
                                 const uint64_t bd = bdesc + (i0 >> 2) * (L::XR * 8) + (i0 & 3) * 2;
@@ -659,15 +703,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                                         umma_pair_ts(d, a_tmem + 8 * i0 + 16, bd + 4, idesc, 1u);
                                         umma_pair_ts(d, a_tmem + 8 * i0 + 24, bd + 6, idesc, 1u);
                                     }
-                                    umma_commit_pair(last_half && i0 + steps == 8 ? done : bar_accfull + 8 * (h * TC_NACC + buf));
+                                    umma_commit_pair(last && i0 + steps == 8 ? done : bar_accfull + 8 * (u * NACC + buf));
                                 }
                                 __syncwarp();
                                 next_buf();
                             }
                         }
                     }
-                    ring.advance(NX);
-                    aring.advance(NA);
+                    ok = __all_sync(0xffffffffu, ok);
+                    ++step;
                 }
                 if (keep) for (int h = 0; h < nh; ++h) next_buf();
             }
@@ -683,7 +727,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         d.lane_tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + L::a_base;
         d.nw = p.nw; d.wstage = p.wstage;
         d.my_group = (uint32_t)((warp - 4) >> 2);
-        d.kcount = 0;
+        d.step = 0;
         const unsigned char* wtiles = smem + L::w_off;
         TcPiece pc;
         TcWalk wk;
@@ -709,10 +753,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         if constexpr (TN == 256) asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
         else asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
         // ---------------- epilogue warps: scale-and-accumulate, then store ----------------
-        // (Each half tile has its own accfull barriers: a wait tells only two phases of a barrier apart, so a barrier is waited
-        // on by the warps that its buffer's reuse waits for, and by nobody who could fall two uses behind.)
-        // Two groups of four warps.  Of a tile with two half tiles each group drains one (an accumulator buffer then costs a
-        // warp one wait for 128 columns); of a tile with one, each group drains half the columns.
+        // Two groups of four warps.  Of a tile with two half tiles each group drains one, of a step with two k-blocks each
+        // drains one (an accumulator buffer then costs a warp one wait for all its columns); otherwise both drain every
+        // buffer, half the columns each.
+        // (Each of the two sub-steps has its own accfull barriers: a wait tells only two phases of a barrier apart, so a barrier
+        // is waited on by the warps that its buffer's reuse waits for, and by nobody who could fall two uses behind.)
         const int ew = warp - L::epi_warp0, quarter = warp & 3, eg = ew >> 2;
         const int row = quarter * 32 + lane;               // channel inside the 128-channel tile = TMEM lane
         const uint32_t accempty0 = mapa(bar_accempty, 0);
@@ -724,17 +769,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         bool ok = true;
         int buf = 0;
         uint32_t full_phase = 0;                           // bit i: parity of the next arrival on accfull[i]
-        uint32_t kcount = 0;
-        Ring dring;                                        // the k-block whose last accumulator is drained next
+        uint32_t step = 0, xphase = 0;                     // steps so far; parity of the exchange
         while (ok && wk.next(sc, p, nclusters, pc)) {
             const ExpertDev& ex = p.ex[pc.e];
             const int nt = 2 * pc.ntp + (int)rank, n = nt * 128 + row;
             const bool active = nt < p.NT1;
             const int nh = NH == 1 ? 1 : (pc.rows > L::HC ? 2 : 1);
-            const int mine_h = nh == 2 ? eg : 0;
-            const int col0 = nh == 2 ? 0 : eg * (L::HC / 2);              // this warp's columns of half tile mine_h
-            const int ncol = min(nh == 2 ? L::HC : L::HC / 2, pc.rows - mine_h * L::HC - col0);   // those with a token (may be <= 0)
-            const int tok0 = mine_h * L::HC + col0;
+            // the columns this warp stores: ncol (may be <= 0) from token tok0 of the tile on
+            const int tok0 = nh == 2 ? eg * L::HC : eg * (L::HC / 2);
+            const int ncol = min(nh == 2 ? L::HC : L::HC / 2, pc.rows - tok0);
             __syncwarp();
 #pragma unroll
             for (int i = 0; i < L::EC / 32; ++i) {
@@ -742,59 +785,101 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 my_perm[col] = col < ncol ? __ldcg(p.perm + pc.m0 + tok0 + col) : -1;
             }
             __syncwarp();
-            float acc[L::EC];
+            float acc[L::DC];
 #pragma unroll
-            for (int i = 0; i < L::EC; ++i) acc[i] = 0.f;
-            // One round per k-block (grouped: every group's buffer is drained, the last one of the k-block being announced by
-            // the k-block's own barrier) or one for the whole piece (per channel).  The loops are kept rolled: unrolled over
-            // the groups and the barriers' outcomes the kernel was 235 KB of code and spent a quarter of its warps' time
-            // fetching instructions.
+            for (int i = 0; i < L::DC; ++i) acc[i] = 0.f;
             const bool keep = ex.group == 0;
-            const int per = keep ? 1 : moqe_groups_per_tile(ex.group), rounds = keep ? 1 : pc.kb1 - pc.kb0;
+            const int per = keep ? 1 : moqe_groups_per_tile(ex.group), nkb = pc.kb1 - pc.kb0;
             const float s_pc = keep && active ? __half2float(ex.scales_pc[n]) * W8_PRESCALE : 0.f;   // (weights are unpacked as (c - z) * 2^-13)
-            const uint32_t freed = nh == 2 ? 2u : 1u;
-#pragma unroll 1
-            for (int it = 0; ok && it < rounds; ++it) {
-                const uint32_t slot = kcount & (NSC - 1);
-#pragma unroll 1
-                for (int t = 0; t < nh * per; ++t) {
-                    const int h = t >= per ? 1 : 0, j = t - h * per;
-                    const bool by_done = !keep && t + 1 == nh * per;
-                    if (h == mine_h) {
-                        const uint32_t bar = by_done ? bar_done + 8 * dring.stage : bar_accfull + 8 * (h * TC_NACC + buf);
-                        const uint32_t phase = by_done ? dring.phase : (full_phase >> (h * TC_NACC + buf)) & 1u;
-                        ok &= __all_sync(0xffffffffu, mbar_wait_short(bar, phase, s_abort, p.status));
-                        tc_fence_after();
-                        const uint32_t src = lane_tmem + buf * L::HC + col0;
-                        float s = s_pc;
+            const bool alone = KS == 2 || nh == 2;             // a buffer is drained by one group
+            const uint32_t freed = alone ? 2u : 1u;
+            const int col0 = alone ? 0 : tok0;                 // first column drained, and how many hold a token
+            const int dcol = KS == 2 ? pc.rows : ncol;
+            // waits for an accumulator buffer, adds it to the sums and hands it back; scl: the group's scale in shared memory
+            // (or nullptr: s_pc), complete once the step's scfull barrier is
+            auto drain = [&](uint32_t bar, uint32_t phase, int b, const __half* scl, bool wait_scales) {
+                ok &= warp_wait(bar, phase, s_abort, p.status);
+                tc_fence_after();
+                const uint32_t src = lane_tmem + b * L::HC + col0;
+                float sv = s_pc;
 #pragma unroll
-                        for (int c = 0; c < L::EC / 32; ++c) {
-                            if (32 * c < ncol) {
-                                uint32_t v[32];
-                                tmem_ld32(src + 32 * c, v);
-                                if (c == 0 && !keep) {
-                                    // the group's scale, fetched while the load is under way
-                                    if (j == 0) ok &= __all_sync(0xffffffffu, mbar_wait_short(bar_scfull + 8 * slot, (kcount / NSC) & 1u, s_abort, p.status));
-                                    s = __half2float(sh.scales[slot][j][row]) * W8_PRESCALE;
-                                }
-                                tmem_ld_wait();
-                                fma_cols32(acc + 32 * c, v, s);
-                            }
+                for (int c = 0; c < L::DC / 32; ++c) {
+                    if (32 * c < dcol) {
+                        uint32_t v[32];
+                        tmem_ld32(src + 32 * c, v);
+                        if (c == 0 && scl) {
+                            // (fetched while the load is under way)
+                            if (wait_scales) ok &= warp_wait(bar_scfull + 8 * (step % NSC), step / NSC & 1u, s_abort, p.status);
+                            sv = __half2float(*scl) * W8_PRESCALE;
                         }
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) remote_arrive(accempty0 + 8 * buf, freed);
+                        tmem_ld_wait();
+                        fma_cols32(acc + 32 * c, v, sv);
                     }
-                    if (!by_done) full_phase ^= 1u << (h * TC_NACC + buf);
-                    if (++buf == TC_NACC) buf = 0;
                 }
-                if (!keep) { dring.advance(NX); ++kcount; }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) remote_arrive(accempty0 + 8 * b, freed);
+            };
+            int left = nkb;
+            if (!keep && per == 1) {
+                // one buffer a step for this warp (the common formats): the loop is kept short, since a warp gets an
+                // instruction through every nine cycles or so and nothing else of the epilogue runs in parallel
+                const bool by_done = !alone || eg == 1;
+                const int mine = alone ? eg : 0, uses = alone ? 2 : 1;
+#pragma unroll 1
+                for (; ok && left >= KS; left -= KS) {
+                    int ob = buf + mine;
+                    if (ob >= NACC) ob -= NACC;
+                    drain(by_done ? bar_done + 8 * (step % NX) : bar_accfull + 8 * ob, by_done ? step / NX & 1u : (full_phase >> ob) & 1u, ob,
+                          &sh.scales[step % NSC][KS == 2 ? eg : 0][0][row], true);
+                    if (alone) full_phase ^= 1u << buf;
+                    buf += uses;
+                    if (buf >= NACC) buf -= NACC;
+                    ++step;
+                    ok = __all_sync(0xffffffffu, ok);
+                }
             }
-            if (keep) {
-                const int k = dring.stage + (pc.kb1 - pc.kb0);
-                dring.phase ^= (uint32_t)(k / NX) & 1u;
-                dring.stage = k % NX;
-                kcount += pc.kb1 - pc.kb0;
+            // The rest: one round per step (every group's buffer is drained, the last one of the step being announced by the
+            // step's own barrier), or one for the whole piece (per channel).  The loops are kept rolled: unrolled over the
+            // groups and the barriers' outcomes the kernel was 235 KB of code and spent a quarter of its warps' time fetching
+            // instructions.
+#pragma unroll 1
+            while (ok && left > 0) {
+                const int nu = KS == 2 ? (keep ? 1 : min(KS, left)) : nh;
+#pragma unroll 1
+                for (int t = 0; t < nu * per; ++t) {
+                    const int u = t >= per ? 1 : 0, j = t - u * per;
+                    const bool by_done = !keep && t + 1 == nu * per;
+                    const int fb = u * NACC + buf;
+                    if (!alone || u == eg)
+                        drain(by_done ? bar_done + 8 * (step % NX) : bar_accfull + 8 * fb, by_done ? step / NX & 1u : (full_phase >> fb) & 1u, buf,
+                              keep ? nullptr : &sh.scales[step % NSC][KS == 2 ? u : 0][j][row], j == 0);
+                    if (!by_done) full_phase ^= 1u << fb;
+                    if (++buf == NACC) buf = 0;
+                }
+                step += keep ? (nkb + KS - 1) / KS : 1;
+                left = keep ? 0 : left - KS;
+                ok = __all_sync(0xffffffffu, ok);
+            }
+            if constexpr (KS == 2) {
+                // the two groups hold sums over different k-blocks: each takes half of the columns and hands over the others
+                float* x = reinterpret_cast<float*>(smem + L::xchg_off) + lane;
+                float* out = x + ew * 1024;
+                const float* in = x + (ew ^ 4) * 1024;
+                // (on mbarriers: every wait of this kernel is bounded)
+                const uint32_t xfull = bar_xchg, xempty = bar_xchg + 8 * TC_EPI;
+                ok &= warp_wait(xempty + 8 * ew, xphase ^ 1u, s_abort, p.status);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) out[i * 32] = eg ? acc[i] : acc[i + 32];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(xfull + 8 * ew);
+                ok &= warp_wait(xfull + 8 * (ew ^ 4), xphase, s_abort, p.status);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) acc[i] = (eg ? acc[i + 32] : acc[i]) + in[i * 32];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(xempty + 8 * (ew ^ 4));
+                xphase ^= 1u;
+                ok = __all_sync(0xffffffffu, ok);
             }
             if (!ok) break;
             if (!active) continue;
