@@ -144,8 +144,8 @@ __device__ __forceinline__ void umma_pair_ts(uint32_t d_tmem, uint32_t a_tmem, u
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5, %5, %5, %5, %5}, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(0u) : "memory");
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
 // arrives at the same barrier of both CTAs when every MMA issued so far is done
 __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
@@ -650,7 +650,56 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 // A per-channel expert's half tile h stays in buffer (buf + h) of the rotation for the whole piece.
                 const bool keep = group == 0;
                 const int steps = keep || group >= 128 ? 8 : group >> 4;         // MMAs into one accumulator buffer
-                for (int kb0 = pc.kb0; ok && kb0 < pc.kb1; kb0 += KS) {
+                int kb0 = pc.kb0;
+                const uint32_t idesc0 = umma_idesc_pair(half_cols<L::HC>(pc.rows, 0)), idesc1 = KS == 2 ? idesc0 : umma_idesc_pair(half_cols<L::HC>(pc.rows, nh - 1));
+                // eight MMAs: one k-block (xd: its token rows, at: its weights) into the accumulator at d
+                auto mma_kblock = [&](uint32_t d, uint32_t at, uint64_t xd, uint32_t idesc) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) umma_pair_ts(d, at + 8 * i, xd + (i >> 2) * (L::XR * 8) + (i & 3) * 2, idesc, i > 0 ? 1u : 0u);
+                };
+                if (!keep && steps == 8 && (KS == 2 || nh == 2)) {
+                    // two buffers a step (the common grouped formats): this warp's instructions are on the critical path of
+                    // every step, so there are as few of them as can be
+                    const uint32_t xd0 = sbase, at0 = tmem_base + L::a_base;
+#pragma unroll 1
+                    for (; ok && kb0 + KS <= pc.kb1; kb0 += KS, ++step) {
+                        const uint32_t st = step % NX;
+                        const int b1 = buf + 1 == NACC ? 0 : buf + 1;
+                        const uint32_t ph1 = b1 == 0 ? buf_phase ^ 1u : buf_phase;
+                        ok = warp_wait(bar_xfull + 8 * st, step / NX & 1u, s_abort, p.status);
+                        ok &= warp_wait(bar_afull + 8 * (step % NA), step / NA & 1u, s_abort, p.status);
+                        ok &= warp_wait(bar_accempty + 8 * buf, buf_phase, s_abort, p.status);
+                        if (KS == 2) ok &= warp_wait(bar_accempty + 8 * b1, ph1, s_abort, p.status);
+                        tc_fence_after();
+                        const uint64_t xd = umma_desc_sw128(xd0 + st * L::xstage);
+                        const uint32_t at = at0 + (step % NA) * (KS * TC_A_COLS);
+                        if (KS == 2) {
+                            if (elect_one()) {
+                                mma_kblock(tmem_base + buf * L::HC, at, xd, idesc0);
+                                umma_commit_pair(bar_accfull + 8 * buf);
+                                mma_kblock(tmem_base + b1 * L::HC, at + TC_A_COLS, xd + L::xhalf / 16, idesc0);
+                                umma_commit_pair(bar_done + 8 * st);
+                            }
+                        } else {
+                            if (elect_one()) {
+                                mma_kblock(tmem_base + buf * L::HC, at, xd, idesc0);
+                                umma_commit_pair(bar_accfull + 8 * buf);
+                            }
+                            __syncwarp();
+                            ok &= warp_wait(bar_accempty + 8 * b1, ph1, s_abort, p.status);
+                            tc_fence_after();
+                            if (elect_one()) {
+                                mma_kblock(tmem_base + b1 * L::HC, at, xd + L::xhalf / 16, idesc1);
+                                umma_commit_pair(bar_done + 8 * st);
+                            }
+                        }
+                        buf_phase = ph1;
+                        buf = b1;
+                        next_buf();
+                        ok = __all_sync(0xffffffffu, ok);
+                    }
+                }
+                for (; ok && kb0 < pc.kb1; kb0 += KS) {
                     const int nk = min(KS, pc.kb1 - kb0);
                     ok = warp_wait(bar_xfull + 8 * (step % NX), step / NX & 1u, s_abort, p.status);
                     ok &= warp_wait(bar_afull + 8 * (step % NA), step / NA & 1u, s_abort, p.status);
