@@ -91,7 +91,7 @@ struct TcParams {
     const int32_t* offsets;
     const uint16_t* X;
     uint16_t* Y;
-    float* partials;          // [cluster][2][rank][cols][128]
+    float* partials;          // [cluster][2][rank][cols / 4][128][4]
     uint32_t* counters;       // [cluster][rank][warp]; zero on entry, left zero
     int* status;
     int M, N, K, KB, E, NT1, NTP;    // NT1: 128-channel tiles, NTP: pairs of them
@@ -116,9 +116,8 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
     return d;
 }
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // (Arrivals on the other CTA's barriers order tensor-memory work and async copies only, so they need no cluster-scope
 // release; with one, 16384 rows of a per-channel expert took 9.1 ms a LLaMA block instead of 4.9.)
 __device__ __forceinline__ void remote_arrive(uint32_t cluster_addr, uint32_t count = 1) {
@@ -167,7 +166,7 @@ struct TcSched {
     int ub[MOQE_MAX_EXPERTS], ue[MOQE_MAX_EXPERTS];   // this cluster's share of the split units
     int w[MOQE_MAX_EXPERTS];                // cost of a unit
     int Gs, Td;                             // clusters of the split; tiles that are not split
-    long long base[MOQE_MAX_EXPERTS], C;    // cost before each expert's split units; total
+    int base[MOQE_MAX_EXPERTS], C;          // cost before each expert's split units; total
 };
 template <int TN>
 struct TcShared {
@@ -438,6 +437,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // (the pair's barriers are initialised when both CTAs have arrived here; every role waits for that before it first touches
+    // the other CTA, so the round trip hides behind the schedule)
+    __syncwarp();
+    cluster_arrive();
     if (warp == 1) tmem_alloc_pair(smem_u32(&sh.tmem), 512);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -456,33 +459,38 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             if (lane >= d) incl += o;
         }
         const int T = __shfl_sync(0xffffffffu, incl, 31), tile0 = incl - T_e;
+        // cost of a k-block, in units of 64 cycles: the tensor core's for its token columns, or what streaming and unpacking takes
+        const int bits = e < p.E ? p.ex[e].bits : 4;
+        const int w = max(min(rpt, TN) >> 4, bits == 8 ? 11 : 7);
+        // Whole rounds of tiles stay whole; what is left over is split by k-blocks if a whole tile less on the clusters that
+        // would have got one is worth the parking and adding up (some 8000 cycles).
         int Td = T;
-        if (p.split && T % nclusters != 0) Td = T >= 2 * nclusters ? (T / nclusters - 1) * nclusters : 0;
+        if (p.split) {
+            const int left = T % nclusters;
+            int wmean = mt > 0 ? w : 0;
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) wmean = max(wmean, __shfl_xor_sync(0xffffffffu, wmean, d));
+            if (left != 0 && (nclusters - left) * p.KB * wmean > 125 * nclusters) Td = T - left;
+        }
         const int us = min(max(Td - tile0, 0), T_e) * p.KB;
         const int cnt = T_e * p.KB - us;
-        // cost of a k-block: tensor cycles of its token columns, or what streaming and unpacking it takes
-        const int bits = e < p.E ? p.ex[e].bits : 4;
-        const int floor_cost = bits == 8 ? 700 : 450;
-        const int w = max(4 * min(rpt, TN), floor_cost);
-        const long long cost = (long long)cnt * w;
-        long long cincl = cost;
+        const int cost = cnt * w;                          // (at most 80 tiles are split: the host keeps this within 32 bits)
+        int cincl = cost;
         int wmax = cnt > 0 ? w : 1;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const long long o = __shfl_up_sync(0xffffffffu, cincl, d);
+            const int o = __shfl_up_sync(0xffffffffu, cincl, d);
             if (lane >= d) cincl += o;
             wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, d));
         }
-        const long long C = __shfl_sync(0xffffffffu, cincl, 31), base = cincl - cost;
-        // every cluster's share holds at least one unit's start
-        const int Gs = (int)min((long long)nclusters, C / wmax);
-        int ub = 0, ue = 0;
+        const int C = __shfl_sync(0xffffffffu, cincl, 31), base = cincl - cost;
+        // every cluster's share holds at least the start of two units
+        const int Gs = min(nclusters, C / (2 * wmax));
+        int ub = us, ue = us;
         if (cnt > 0 && cluster < Gs) {
-            const long long den = (long long)w * Gs;
-            const long long n0 = (long long)cluster * C - base * Gs, n1 = (long long)(cluster + 1) * C - base * Gs;
-            const long long t0 = n0 <= 0 ? 0 : (n0 + den - 1) / den, t1 = n1 <= 0 ? 0 : (n1 + den - 1) / den;
-            ub = us + (int)min(t0, (long long)cnt);
-            ue = us + (int)min(t1, (long long)cnt);
+            const int den = w * Gs, n0 = cluster * C - base * Gs, n1 = n0 + C;
+            ub = us + min(n0 <= 0 ? 0 : (n0 + den - 1) / den, cnt);
+            ue = us + min(n1 <= 0 ? 0 : (n1 + den - 1) / den, cnt);
         }
         if (e < p.E) { sc.off[e] = o0; sc.tile0[e] = tile0; }
         if (e == p.E - 1) { sc.off[p.E] = o1; sc.tile0[p.E] = T; }
@@ -491,7 +499,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
     }
     tc_fence_before();
     __syncthreads();
-    cluster_sync();                                        // the pair's barriers are initialised, its TMEM allocated
+    if (warp != 2) cluster_wait();                         // (the weight producer touches its own CTA only)
     tc_fence_after();
     const uint32_t tmem_base = sh.tmem;
 
@@ -629,6 +637,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                     }
                 }
             }
+            __syncwarp();
+            cluster_wait();
         } else if (warp == 1 && rank == 0) {
             // ---------------- MMA issuer (the leading CTA's, for the pair) ----------------
             // (Its waits spin on the plain try_wait: they sit on the critical path and coming round a short spin is
@@ -934,19 +944,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             if (!active) continue;
             if (pc.kb0 != 0 || pc.kb1 != p.KB) {
                 // part of a tile: park this warp's sums, announce, and add everything up if this was the last arrival
-                const long long C = sc.C, first = sc.base[pc.e] + (long long)(pc.tile * p.KB - sc.us[pc.e]) * sc.w[pc.e];
-                const int Gs = sc.Gs;
-                const int c_a = (int)(first * Gs / C), c_b = (int)((first + (long long)(p.KB - 1) * sc.w[pc.e]) * Gs / C);
+                const int C = sc.C, Gs = sc.Gs, first = sc.base[pc.e] + (pc.tile * p.KB - sc.us[pc.e]) * sc.w[pc.e];
+                const int c_a = first * Gs / C, c_b = (first + (p.KB - 1) * sc.w[pc.e]) * Gs / C;
                 const size_t slot = (size_t)p.cols * 128;
-                auto slot_of = [&](int c, int which) { return p.partials + ((size_t)(c * 2 + which) * 2 + rank) * slot + (size_t)tok0 * 128 + row; };
+                auto slot_of = [&](int c, int which) { return p.partials + ((size_t)(c * 2 + which) * 2 + rank) * slot + (size_t)tok0 * 128 + row * 4; };
                 {
                     float* dst = slot_of(cluster, pc.kb0 == 0 ? 1 : 0);
 #pragma unroll
-                    for (int i0 = 0; i0 < L::EC; i0 += 8)
-                        if (i0 < ncol) {
-#pragma unroll
-                            for (int i = i0; i < i0 + 8; ++i) __stcg(dst + (size_t)i * 128, acc[i]);
-                        }
+                    for (int i = 0; i < L::EC; i += 4)
+                        if (i < ncol) __stcg(reinterpret_cast<float4*>(dst + i * 128), make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]));
                 }
                 __syncwarp();
                 unsigned* counter = p.counters + (c_a * 2 + (int)rank) * TC_EPI + ew;
@@ -959,35 +965,56 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 __syncwarp();
 #pragma unroll
                 for (int i = 0; i < L::EC; ++i) acc[i] = 0.f;
+                // several clusters' sums are fetched in one round trip (as many as there are registers for), then added in
+                // cluster order
+                constexpr int CB = TN == 64 ? 2 : 1, CC = TN == 64 ? 32 : 32;
 #pragma unroll 1
-                for (int c = c_a; c <= c_b; ++c) {
-                    const float* src = slot_of(c, c == c_a ? 1 : 0);
+                for (int c = c_a; c <= c_b; c += CB) {
 #pragma unroll
-                    for (int i0 = 0; i0 < L::EC; i0 += 8)
+                    for (int i0 = 0; i0 < L::EC; i0 += CC)
                         if (i0 < ncol) {
-                            float v[8];
+                            float4 v[CB][CC / 4];
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) v[i] = __ldcg(src + (size_t)(i0 + i) * 128);
+                            for (int b = 0; b < CB; ++b) {
+                                const float* src = slot_of(min(c + b, c_b), c + b == c_a ? 1 : 0) + i0 * 128;
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) acc[i0 + i] += v[i];
+                                for (int i = 0; i < CC / 4; ++i)
+                                    v[b][i] = i0 + 4 * i < ncol && c + b <= c_b ? __ldcg(reinterpret_cast<const float4*>(src + i * 512)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            }
+#pragma unroll
+                            for (int b = 0; b < CB; ++b)
+#pragma unroll
+                                for (int i = 0; i < CC / 4; ++i) {
+                                    acc[i0 + 4 * i] += v[b][i].x;
+                                    acc[i0 + 4 * i + 1] += v[b][i].y;
+                                    acc[i0 + 4 * i + 2] += v[b][i].z;
+                                    acc[i0 + 4 * i + 3] += v[b][i].w;
+                                }
                         }
                 }
                 if (lane == 0) *counter = 0u;
             }
-            // Store: lanes hold neighbouring channels, registers tokens.  Neighbouring lanes swap one of every two tokens, so
-            // that a lane writes two channels of one token.
-            const int odd = lane & 1;
-            uint16_t* y = p.Y + (n & ~1);
+            // Store: lanes hold neighbouring channels, registers tokens.  Four neighbouring lanes transpose four tokens between
+            // them (two exchanges), so that a lane writes four channels of one token.  The store is predicated, not branched
+            // around: with a branch each, 64 stores took a warp 9500 cycles.
+            const int sub = lane & 3;
+            uint16_t* y = p.Y + (n & ~3);
+            const int* to_list = my_perm + sub;
+            const bool in_n = n < p.N;
 #pragma unroll
-            for (int i0 = 0; i0 < L::EC; i0 += 8)
+            for (int i0 = 0; i0 < L::EC; i0 += 16)
                 if (i0 < ncol) {
 #pragma unroll
-                    for (int i = i0; i < i0 + 8; i += 2) {
-                        const uint32_t mine = pack_bf16x2(acc[i], acc[i + 1]);
-                        const uint32_t other = __shfl_xor_sync(0xffffffffu, mine, 1);
-                        const uint32_t pair = __byte_perm(mine, other, odd ? 0x3276u : 0x5410u);
-                        const int to = my_perm[i + odd];
-                        if (to >= 0 && n < p.N) *reinterpret_cast<uint32_t*>(y + (size_t)to * p.N) = pair;
+                    for (int i = i0; i < i0 + 16; i += 4) {
+                        const uint32_t p01 = pack_bf16x2(acc[i], acc[i + 1]), p23 = pack_bf16x2(acc[i + 2], acc[i + 3]);
+                        const uint32_t q01 = __shfl_xor_sync(0xffffffffu, p01, 1), q23 = __shfl_xor_sync(0xffffffffu, p23, 1);
+                        const uint32_t a = __byte_perm(p01, q01, sub & 1 ? 0x3276u : 0x5410u);       // two channels of token i + (sub & 1)
+                        const uint32_t b = __byte_perm(p23, q23, sub & 1 ? 0x3276u : 0x5410u);       // ... of token i + 2 + (sub & 1)
+                        const uint32_t other = __shfl_xor_sync(0xffffffffu, sub & 2 ? a : b, 2);
+                        const int to = to_list[i];
+                        uint16_t* at = y + (size_t)(uint32_t)max(to, 0) * (uint32_t)p.N;
+                        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %3, 0;\n\t@q st.global.v2.b32 [%0], {%1, %2};\n\t}"
+                                     ::"l"(at), "r"(sub & 2 ? other : a), "r"(sub & 2 ? b : other), "r"((int)(in_n && to >= 0)) : "memory");
                     }
                 }
         }
@@ -1001,7 +1028,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         unsigned long long t0 = global_ns();
         while (global_ns() - t0 < 200000ull) __nanosleep(1000);
     }
-    cluster_sync();                                        // the peer no longer touches this CTA's barriers or TMEM
+    cluster_arrive();
+    cluster_wait();                                        // the peer no longer touches this CTA's barriers or TMEM
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc_pair(tmem_base, 512);
@@ -1061,7 +1089,7 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
     p.partials = (float*)((char*)ws + (tc_zero_bytes() + 255) / 256 * 256);
     p.M = M; p.N = N; p.K = K; p.KB = ex[0]->Kp / 128; p.E = E; p.NT1 = ex[0]->Np / 128; p.NTP = (p.NT1 + 1) / 2;
     p.cols = tc_cols(M);
-    p.split = tile_tokens == 0 ? 1 : 0;
+    p.split = tile_tokens == 0 && p.KB <= 4096 ? 1 : 0;
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
