@@ -176,7 +176,7 @@ struct TcShared {
     uint32_t tmem;
     int abort;
     __align__(16) int perm[TC_EPI][L::EC];  // per epilogue warp: its columns' target rows
-    int xrow[2][L::NH * L::XR];             // rows of X to gather, one list per gather warp
+    __align__(16) int xrow[2][L::NH * L::XR];   // rows of X to gather, one list per gather warp: row 4 i + j at [j][i]
     __align__(16) __half scales[L::nsc][L::KS][4][128];   // on their way to the epilogue
 };
 static_assert(sizeof(TcShared<256>) <= TcCfg<256>::static_bytes && sizeof(TcShared<128>) <= TcCfg<128>::static_bytes &&
@@ -524,7 +524,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             wk.start(cluster);
             bool ok = true;
             int pending = 0;
-            const uint32_t full0 = mapa(bar_xfull, 0);
+            const uint32_t full0 = mapa(bar_xfull, 0), pitch = (uint32_t)p.K * 2;
             auto arrive = [&]() {
                 fence_proxy_async();
                 __syncwarp();
@@ -547,8 +547,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                         const int b = lane + 32 < c ? __ldcg(p.perm + pc.m0 + first_row + lane + 32) : 0;
                         const int first = __shfl_sync(0xffffffffu, a, 0);
                         const bool run = __all_sync(0xffffffffu, (lane >= c || a == first + lane) && (lane + 32 >= c || b == first + lane + 32));
-                        s_xrow[h * L::XR + lane] = a;
-                        if (L::XR > 32) s_xrow[h * L::XR + lane + 32] = b;
+                        s_xrow[h * L::XR + (lane & 3) * (L::XR / 4) + (lane >> 2)] = a;
+                        if (L::XR > 32) s_xrow[h * L::XR + (lane & 3) * (L::XR / 4) + 8 + (lane >> 2)] = b;
                         // (a box fetches XR rows whatever it needs; operand rows beyond the real ones yield columns that are
                         // never stored, so they may hold anything)
                         src[h] = run && 2 * c >= L::XR ? first : -1;
@@ -584,12 +584,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                         for (int h = 0; h < NH; ++h) {
                             if (src[h] < 0) {
                                 const uint32_t dst = stage + h * L::xhalf;
-#pragma unroll 4
-                                for (int i = 0; i < L::XR / 4; ++i) {
-                                    const int r = 4 * i + (int)r0;
-                                    if (4 * i + 2 * gw >= cnt[h]) break;
-                                    if (r < cnt[h])
-                                        cp_async16(dst + ((i & 1) ? sw1 : sw0) + (i >> 1) * 1024, xk + (size_t)s_xrow[h * L::XR + r] * (size_t)(p.K * 2), real);
+                                const int4* list = reinterpret_cast<const int4*>(s_xrow + h * L::XR + r0 * (L::XR / 4));
+                                // (no branch per row: a list entry beyond the real rows is row 0, copied in vain)
+#pragma unroll 1
+                                for (int i = 0; 4 * i < cnt[h]; i += 4) {
+                                    const int4 r4 = list[i >> 2];
+                                    const uint32_t d = dst + (i >> 1) * 1024;
+                                    cp_async16(d + sw0, xk + (size_t)(uint32_t)r4.x * pitch, real);
+                                    cp_async16(d + sw1, xk + (size_t)(uint32_t)r4.y * pitch, real);
+                                    cp_async16(d + sw0 + 1024, xk + (size_t)(uint32_t)r4.z * pitch, real);
+                                    cp_async16(d + sw1 + 1024, xk + (size_t)(uint32_t)r4.w * pitch, real);
                                 }
                             }
                         }
