@@ -54,7 +54,11 @@ WsLayout ws_layout(int M, int Np, int K, int E) {
     return w;
 }
 
-constexpr int AUTO_STREAM_MAX_ROWS = 128;
+// Batches the decode kernel does not take: up to this many rows the streaming kernel, if it is the formats that keep the
+// decode kernel away (groups narrower than 128 k: four Qwen experts, layer by layer, streaming / grouped GEMM: 24 rows
+// 25 / 28, 73 / 71, 76 / 107 us; 64 rows 32 / 28, 106 / 72, 110 / 108); everything else is the grouped GEMM's (4096 x 4096,
+// three LLaMA experts, 48 rows: 30 / 22 us).
+constexpr int AUTO_STREAM_MAX_ROWS = 48;
 constexpr int LAST_PATH = 6;
 
 bool g_auto_decode = true;   // whether the automatic choice takes a decode kernel where it applies
@@ -67,7 +71,7 @@ int pick_kernel(int path, int M, const moqe_expert* const* ex, int E) {
     if (path == 1) return 1;
     if (path == 0) {
         if (g_auto_decode && decode_supported_multi(M, ex, 1, E)) return 2;
-        if (M <= AUTO_STREAM_MAX_ROWS) return 1;
+        if (M <= AUTO_STREAM_MAX_ROWS && !(g_auto_decode && decode_supported_multi(1, ex, 1, E))) return 1;
         return (g_auto_dense && dense_supported(M, ex[0]->N, ex[0]->K, ex, E)) ? 3 : 0;
     }
     return 0;

@@ -218,6 +218,15 @@ struct TcWalk {
         return true;
     }
 };
+// What a k-block of a tile costs, in units of 64 cycles (measured, every cluster busy): by tile size, rows of the tile and
+// quantization groups per k-block.
+template <int TN>
+__device__ __forceinline__ int kblock_cost(int rows, int bits, int per) {
+    const int wide = bits == 8 || bits == 3 ? 2 : 0;
+    if (TN == 64) return (per <= 1 ? 13 : (per == 2 ? 22 : 36)) + wide;
+    if (TN == 128) return (per == 0 ? 16 : (per == 1 ? 20 : (per == 2 ? 30 : 50))) + wide;
+    return (rows <= 128 ? (per == 0 ? 18 : (per == 1 ? 23 : (per == 2 ? 39 : 68))) : (per == 0 ? 24 : (per == 1 ? 30 : (per == 2 ? 54 : 108)))) + wide;
+}
 // MMA columns of half tile h of a tile with `rows` tokens
 template <int HC>
 __device__ __forceinline__ int half_cols(int rows, int h) { return (min(HC, rows - HC * h) + 31) & ~31; }
@@ -459,18 +468,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             if (lane >= d) incl += o;
         }
         const int T = __shfl_sync(0xffffffffu, incl, 31), tile0 = incl - T_e;
-        // cost of a k-block, in units of 64 cycles: the tensor core's for its token columns, or what streaming and unpacking takes
-        const int bits = e < p.E ? p.ex[e].bits : 4;
-        const int w = max(min(rpt, TN) >> 4, bits == 8 ? 11 : 7);
+        const int w = e < p.E ? kblock_cost<TN>(rpt, p.ex[e].bits, moqe_groups_per_tile(p.ex[e].group)) : 1;
         // Whole rounds of tiles stay whole; what is left over is split by k-blocks if a whole tile less on the clusters that
-        // would have got one is worth the parking and adding up (some 8000 cycles).
+        // would have got one is worth the parking and adding up (10 us: 16 tiles of 16 k-blocks, split, 19.9 us, whole 13.4).
         int Td = T;
         if (p.split) {
             const int left = T % nclusters;
             int wmean = mt > 0 ? w : 0;
 #pragma unroll
             for (int d = 16; d > 0; d >>= 1) wmean = max(wmean, __shfl_xor_sync(0xffffffffu, wmean, d));
-            if (left != 0 && (nclusters - left) * p.KB * wmean > 125 * nclusters) Td = T - left;
+            if (left != 0 && (nclusters - left) * p.KB * wmean > 300 * nclusters) Td = T - left;
         }
         const int us = min(max(Td - tile0, 0), T_e) * p.KB;
         const int cnt = T_e * p.KB - us;
@@ -1073,7 +1080,9 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
     if (!ws || ws_bytes < tc_workspace_bytes(M, K, E, ex[0]->Np)) return MOQE_ERR_WORKSPACE;
     EncodeTiledFn enc = encode_fn();
     if (!enc) return MOQE_ERR_CUDA;
-    const int tile = tile_tokens ? tile_tokens : (M > 256 ? 256 : (M > 128 ? 128 : 64));
+    // Tile by batch size (the routing is not known here): LLaMA blocks, three experts, rows dealt evenly, 64 / 128 / 256
+    // tokens: 192 rows 235 / 275 / 302 us, 256 rows 367 / 299 / 318, 384 rows 383 / 323 / 346, 512 rows 474 / 489 / 414.
+    const int tile = tile_tokens ? tile_tokens : (M > 448 ? 256 : (M > 192 ? 128 : 64));
     // tensor map over X[M][K] bf16: boxes of 64 k x XR rows, 128-byte swizzle, zero fill outside
     CUtensorMap tmap;
     cuuint64_t gdim[2] = {(cuuint64_t)K, (cuuint64_t)M};
