@@ -316,7 +316,9 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
                 cs_e = ti.e;
             }
             const bool live = row < ti.rows;
-            const uint32_t out_row = out_base + row * out_pitch;
+            // This thread's half of the staged row.  The halves lie where those of a full chunk do, whatever the chunk's width:
+            // in a narrower last chunk the second half would otherwise be written over the first warp's copy still under way.
+            const uint32_t out_row = out_base + row * out_pitch + colhalf * nc_rows;
             for (int nc = 0; ok && nc < nchunks; ++nc) {
                 const int wrows = min(DN_NC, p.Nw - nc * DN_NC);
                 const int half_cols = wrows >> 1, c_lo = colhalf * half_cols;          // this warp's channels of the chunk
@@ -341,7 +343,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
                                                                      __uint_as_float(v[8 * j + 2 * i + 1]) * sc[2 * i + 1]);
                             o[i] = *reinterpret_cast<uint32_t*>(&h);
                         }
-                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(out_row + (c + 8 * j) * 2), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
+                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(out_row + (c - c_lo + 8 * j) * 2), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
                     }
                 }
                 tc_fence_before();
@@ -353,7 +355,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
                 if (live && nbytes > 0) {
                     fence_proxy_async();
                     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                                 ::"l"(p.Y + yrow * p.N + n0), "r"(out_row + c_lo * 2), "r"(nbytes) : "memory");
+                                 ::"l"(p.Y + yrow * p.N + n0), "r"(out_row), "r"(nbytes) : "memory");
                 }
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
