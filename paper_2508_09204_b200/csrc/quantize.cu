@@ -8,6 +8,7 @@
 // math), so codes, scales and zero-points are reproducible bit for bit.
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "dequant.cuh"
@@ -174,6 +175,19 @@ __device__ __forceinline__ MetaSlot meta_slot(uint8_t* tiles, __half* scales_pc,
     return m;
 }
 
+// scale and zero-point of a group from its extremes, exactly as moqe.h states them
+struct GroupGrid { __half sh; float s; int z; };
+__device__ __forceinline__ GroupGrid group_grid(float lo, float hi, float a, int bits, int sym) {
+    GroupGrid g;
+    const int L = (1 << bits) - 1, qmax = (1 << (bits - 1)) - 1;
+    const float s32 = sym ? __fdiv_rn(a, (float)qmax) : __fdiv_rn(__fsub_rn(hi, lo), (float)L);
+    g.sh = __float2half_rn(s32);
+    g.s = __half2float(g.sh);
+    if (!(g.s > 0.f) || isinf(g.s)) { g.sh = __float2half_rn(1.0f); g.s = 1.0f; }
+    g.z = sym ? 1 << (bits - 1) : max(0, min(L, (int)rintf(__fdiv_rn(-lo, g.s))));
+    return g;
+}
+
 __global__ void rtn_scales_kernel(const float* __restrict__ W, int N, int K, int bits, int group, int G, int sym, int KB,
                                   uint8_t* __restrict__ tiles, __half* __restrict__ scales_pc,
                                   __nv_bfloat16* __restrict__ zeros_pc) {
@@ -197,21 +211,11 @@ __global__ void rtn_scales_kernel(const float* __restrict__ W, int N, int K, int
         a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
     }
     if (lane != 0) return;
-    const int L = (1 << bits) - 1;
-    const int qmax = (1 << (bits - 1)) - 1;
-    float s32 = sym ? __fdiv_rn(a, (float)qmax) : __fdiv_rn(__fsub_rn(hi, lo), (float)L);
-    __half sh = __float2half_rn(s32);
-    float s = __half2float(sh);
-    if (!(s > 0.f) || isinf(s)) { sh = __float2half_rn(1.0f); s = 1.0f; }
-    int z = 0;
-    if (!sym) {
-        z = (int)rintf(__fdiv_rn(-lo, s));
-        z = max(0, min(L, z));
-    }
+    const GroupGrid g2 = group_grid(lo, hi, a, bits, sym);
     for (int c = 0; c < meta_copies(group); ++c) {
         MetaSlot m = meta_slot(tiles, scales_pc, zeros_pc, bits, group, !sym, KB, n, gi, c);
-        *m.s = sh;
-        if (!sym) *m.z = __float2bfloat16_rn((float)z);            // exact: z <= 255
+        *m.s = g2.sh;
+        if (!sym) *m.z = __float2bfloat16_rn((float)g2.z);         // exact: z <= 255
     }
 }
 
@@ -267,6 +271,168 @@ __global__ void encode_pack_kernel(const float* __restrict__ W, const uint8_t* _
                       pc.slot, w);
 }
 
+// ---------------------------------------------------------------------------
+// K1: scales, zero-points, codes and packing in one kernel, for per-channel experts and groups within a k-block
+// (wider groups take K1a and K1b above).  Bound by the fp32 weights' bytes, which are read from HBM once: a warp holds
+// the 16 channels x 128 k of a blob in registers between finding the groups' extremes and rounding.  A per-channel
+// expert's block goes over its 16 rows twice, the second time out of L2 (16 rows are 256 KB at K = 4096).  Every byte of
+// the tiles is written here, padding included.  11008 x 4096, 4-bit g128: 63 us (the two kernels: 92 + 60); three blocks
+// to an SM (two: 68 us, four: 65).
+// ---------------------------------------------------------------------------
+// rint(w / s) as IEEE division and rounding give it, from a multiplication by 1 / s.  The product is off by at most
+// 2^-22 of its size; only where it comes that close to the middle between two integers does the division decide.
+// Adding 1.5 * 2^23 rounds to the nearest even integer and leaves it in the low bits: no conversion instructions, which
+// run at a quarter of the rate.
+template <int BITS>
+__device__ __forceinline__ void round_chunk(const float (&w)[8], float s, float inv, int (&q)[8]) {
+    constexpr float SIZE = (float)(1 << (BITS + 1)), MAGIC = 12582912.f;
+    bool slow = false;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const float x = __fmul_rn(w[t], inv), y = __fadd_rn(x, MAGIC), d = __fsub_rn(x, __fsub_rn(y, MAGIC));
+        slow |= !(fabsf(d) < 0.5f - SIZE * 0x1p-21f) || !(fabsf(x) < SIZE);
+        q[t] = __float_as_int(y) - 0x4B400000;
+    }
+    if (slow) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) q[t] = (int)rintf(__fdiv_rn(w[t], s));
+    }
+}
+
+template <int BITS>
+__global__ void __launch_bounds__(256, 3) quantize_pack_kernel(const float* __restrict__ W, int N, int K, int group /* 0, 32, 64 or 128 */, int sym, int KB,
+                                                            uint8_t* __restrict__ tiles, __half* __restrict__ scales_pc,
+                                                            __nv_bfloat16* __restrict__ zeros_pc) {
+    constexpr int L = (1 << BITS) - 1, half_code = 1 << (BITS - 1), qmax = half_code - 1;
+    __shared__ float s_ext[8][3][16];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nt = blockIdx.x >> 3, nb = blockIdx.x & 7;
+    const int q = lane >> 3, r = (lane & 7) ^ (2 * q);                  // this lane's slot: piece (q, r) of both halves
+    const int row0 = nt * 128 + nb * 16 + r;
+    const int stride = moqe_tile_stride(BITS, group, !sym);
+    // the lane that holds (q ^ d, r)
+    auto partner = [&](int d) { const int p = q ^ d; return p * 8 + (r ^ (2 * p)); };
+    auto load = [&](int n, int kb, float (&v)[32]) {
+#pragma unroll
+        for (int G = 0; G < 4; ++G) {
+            const int k0 = kb * 128 + 32 * G + 8 * q;
+            const bool live = n < N && k0 < K;                          // K % 8 == 0: a chunk is wholly inside or outside
+            const float4* src = reinterpret_cast<const float4*>(W + (live ? (size_t)n * K + k0 : 0));
+            const float4 a = live ? src[0] : make_float4(0.f, 0.f, 0.f, 0.f), b = live ? src[1] : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[8 * G] = a.x; v[8 * G + 1] = a.y; v[8 * G + 2] = a.z; v[8 * G + 3] = a.w;
+            v[8 * G + 4] = b.x; v[8 * G + 5] = b.y; v[8 * G + 6] = b.z; v[8 * G + 7] = b.w;
+        }
+    };
+    // (a symmetric grid needs max |w| only, an asymmetric one min and max; max |w| is the larger of -min and max)
+    GroupGrid pc[2];
+    if (group == 0) {
+        float lo[2] = {0.f, 0.f}, hi[2] = {0.f, 0.f};
+        for (int kb = warp; kb < KB; kb += 8) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float v[32];
+                load(row0 + 8 * h, kb, v);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) { lo[h] = fminf(lo[h], v[i]); hi[h] = fmaxf(hi[h], v[i]); }
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int d = 1; d < 4; d <<= 1) {
+                lo[h] = fminf(lo[h], __shfl_sync(0xffffffffu, lo[h], partner(d)));
+                hi[h] = fmaxf(hi[h], __shfl_sync(0xffffffffu, hi[h], partner(d)));
+            }
+            if (q == 0) { s_ext[warp][0][8 * h + r] = lo[h]; s_ext[warp][1][8 * h + r] = hi[h]; }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            for (int w = 0; w < 8; ++w) { lo[h] = fminf(lo[h], s_ext[w][0][8 * h + r]); hi[h] = fmaxf(hi[h], s_ext[w][1][8 * h + r]); }
+            pc[h] = group_grid(lo[h], hi[h], fmaxf(-lo[h], hi[h]), BITS, sym);
+            const int n = row0 + 8 * h;
+            if (warp == 0 && q == 0 && blockIdx.y == 0) {
+                scales_pc[n] = n < N ? pc[h].sh : __float2half_rn(0.f);
+                if (!sym) zeros_pc[n] = __float2bfloat16_rn(n < N ? (float)pc[h].z : 0.f);
+            }
+        }
+    }
+    const int per = moqe_groups_per_tile(group), meta_g = moqe_meta_group_bytes(!sym);
+    for (int kb = blockIdx.y * 8 + warp; kb < KB; kb += gridDim.y * 8) {
+        uint8_t* tile = tiles + ((size_t)nt * KB + kb) * (size_t)stride;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int n = row0 + 8 * h;
+            float v[32];
+            load(n, kb, v);
+            float s[4], inv[4];
+            int z[4];
+            if (group == 0) {
+                const float iv = __frcp_rn(pc[h].s);
+#pragma unroll
+                for (int G = 0; G < 4; ++G) { s[G] = pc[h].s; inv[G] = iv; z[G] = pc[h].z; }
+            } else {
+                float lo[4], hi[4];
+#pragma unroll
+                for (int G = 0; G < 4; ++G) {
+                    lo[G] = hi[G] = 0.f;
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) { lo[G] = fminf(lo[G], v[8 * G + t]); hi[G] = fmaxf(hi[G], v[8 * G + t]); }
+                }
+                if (per < 4) {
+                    lo[0] = lo[1] = fminf(lo[0], lo[1]); hi[0] = hi[1] = fmaxf(hi[0], hi[1]);
+                    lo[2] = lo[3] = fminf(lo[2], lo[3]); hi[2] = hi[3] = fmaxf(hi[2], hi[3]);
+                }
+                if (per == 1) { lo[0] = fminf(lo[0], lo[2]); hi[0] = fmaxf(hi[0], hi[2]); }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (j < per) {
+                        const int G = per == 4 ? j : (per == 2 ? 2 * j : 0);
+                        float l = lo[0], u = hi[0];
+                        if (G == 1) { l = lo[1]; u = hi[1]; }
+                        if (G == 2) { l = lo[2]; u = hi[2]; }
+                        if (G == 3) { l = lo[3]; u = hi[3]; }
+#pragma unroll
+                        for (int d = 1; d < 4; d <<= 1) {
+                            l = fminf(l, __shfl_sync(0xffffffffu, l, partner(d)));
+                            u = fmaxf(u, __shfl_sync(0xffffffffu, u, partner(d)));
+                        }
+                        const GroupGrid g = group_grid(l, u, fmaxf(-l, u), BITS, sym);
+                        const float iv = __frcp_rn(g.s);
+#pragma unroll
+                        for (int G2 = 0; G2 < 4; ++G2)
+                            if (per == 1 || (per == 2 ? (G2 >> 1) == j : G2 == j)) { s[G2] = g.s; inv[G2] = iv; z[G2] = g.z; }
+                        if (q == 0) {
+                            const bool live = n < N && kb * 128 + j * (128 / per) < K;
+                            uint8_t* m = tile + moqe_tile_bytes(BITS) + j * meta_g + (nb * 16 + 8 * h + r) * 2;
+                            *reinterpret_cast<__half*>(m) = live ? g.sh : __float2half_rn(0.f);
+                            if (!sym) *reinterpret_cast<__nv_bfloat16*>(m + 256) = __float2bfloat16_rn(live ? (float)g.z : 0.f);
+                        }
+                    }
+                }
+            }
+            uint32_t c[32];
+#pragma unroll
+            for (int G = 0; G < 4; ++G) {
+                const bool live = n < N && kb * 128 + 32 * G + 8 * q < K;
+                float w8[8];
+                int qi[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) w8[t] = v[8 * G + t];
+                round_chunk<BITS>(w8, s[G], inv[G], qi);
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    const int code = sym ? max(-qmax, min(qmax, qi[t])) + half_code : max(0, min(L, qi[t] + z[G]));
+                    c[8 * G + t] = live ? (uint32_t)code : 0u;
+                }
+            }
+            uint32_t w[PieceWords<BITS>::n];
+            encode_piece<BITS>(c, w);
+            store_piece<BITS>(tile + nb * moqe_blob_bytes(BITS), h, lane, w);
+        }
+    }
+}
+
 template <int BITS>
 __global__ void unpack_kernel(const uint8_t* __restrict__ tiles, int N, int K, int KB, int tile_stride,
                               uint8_t* __restrict__ canon, long long npieces) {
@@ -318,6 +484,50 @@ __global__ void meta_import_kernel(const uint16_t* __restrict__ scales_in, const
     }
 }
 
+// Experts' device memory comes from a memory pool of the library's own, one per device: building an 11008 x 4096 expert
+// spent 520 of its 830 us in cudaMalloc and cudaFree.  The pool keeps at most POOL_KEEP bytes of freed memory for the next
+// expert (what is above goes back to the device at the next synchronisation) and is safe for any threads and streams.
+constexpr uint64_t POOL_KEEP = 128ull << 20;
+std::mutex g_pool_mutex;
+cudaMemPool_t g_pools[64] = {nullptr};
+
+cudaMemPool_t expert_pool(int device) {
+    if (device < 0 || device >= 64) return nullptr;
+    std::lock_guard<std::mutex> lock(g_pool_mutex);
+    if (!g_pools[device]) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        cudaMemPool_t pool = nullptr;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+        uint64_t keep = POOL_KEEP;
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        g_pools[device] = pool;
+    }
+    return g_pools[device];
+}
+
+// Memory for an expert that is filled on `st`.  nullptr: none to be had, or `st` is being captured (the memory would
+// belong to the graph).
+void* expert_malloc(size_t bytes, int device, cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) { cudaGetLastError(); return nullptr; }
+    cudaMemPool_t pool = expert_pool(device);
+    void* p = nullptr;
+    if (!pool || cudaMallocFromPoolAsync(&p, bytes, pool, st) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return p;
+}
+// Gives it back once nothing on the device can be using it any more.
+bool expert_free(void* p, int device) {
+    int now = 0;
+    if (cudaGetDevice(&now) != cudaSuccess) return false;
+    bool ok = now == device || cudaSetDevice(device) == cudaSuccess;
+    ok = ok && cudaDeviceSynchronize() == cudaSuccess && cudaFreeAsync(p, nullptr) == cudaSuccess;
+    if (now != device) ok = cudaSetDevice(now) == cudaSuccess && ok;
+    return ok;
+}
+
 moqe_status check_format(int N, int K, int bits, int group) {
     if (N <= 0 || K <= 0) return MOQE_ERR_SHAPE;
     if (bits != 2 && bits != 3 && bits != 4 && bits != 8) return MOQE_ERR_UNSUPPORTED;
@@ -330,7 +540,9 @@ moqe_status check_format(int N, int K, int bits, int group) {
     return MOQE_OK;
 }
 
-moqe_status alloc_expert(int N, int K, int bits, int group, int sym, cudaStream_t st, moqe_expert** out) {
+// clear: zero the buffers on `st` (padded channels / padded k: codes 0, scale 0, zero-point 0); a caller that writes every
+// byte itself does without
+moqe_status alloc_expert(int N, int K, int bits, int group, int sym, bool clear, cudaStream_t st, moqe_expert** out) {
     moqe_expert* e = new (std::nothrow) moqe_expert();
     if (!e) return MOQE_ERR_ALLOC;
     e->N = N; e->K = K; e->bits = bits; e->group = group; e->sym = sym ? 1 : 0;
@@ -341,23 +553,33 @@ moqe_status alloc_expert(int N, int K, int bits, int group, int sym, cudaStream_
     if (cudaGetDevice(&e->device) != cudaSuccess) { delete e; return MOQE_ERR_CUDA; }
     e->tiles_alloc = (size_t)(e->Np / 128) * (e->Kp / 128) * moqe_tile_stride(bits, group, !e->sym);
     e->pc_alloc = group == 0 ? (size_t)e->Np * 2 : 0;
-    bool ok = cudaMalloc(&e->tiles, e->tiles_alloc) == cudaSuccess;
-    if (ok && group == 0) {
-        ok = cudaMalloc(&e->scales_pc, e->pc_alloc) == cudaSuccess &&
-             (e->sym || cudaMalloc(&e->zeros_pc, e->pc_alloc) == cudaSuccess);
+    // one block: the tiles, then (per channel) scales and zero-points
+    const size_t pc_total = e->pc_alloc * (e->sym ? 1 : 2);
+    e->tiles = (uint8_t*)expert_malloc(e->tiles_alloc + pc_total, e->device, st);
+    if (!e->tiles) { delete e; return MOQE_ERR_ALLOC; }
+    if (group == 0) {
+        e->scales_pc = (__half*)(e->tiles + e->tiles_alloc);
+        if (!e->sym) e->zeros_pc = (__nv_bfloat16*)(e->tiles + e->tiles_alloc + e->pc_alloc);
     }
-    if (!ok) {
-        cudaGetLastError();
-        cudaFree(e->tiles); cudaFree(e->scales_pc); cudaFree(e->zeros_pc);
-        delete e;
-        return MOQE_ERR_ALLOC;
-    }
-    // padded channels / padded k: codes 0, scale 0, zero-point 0
-    cudaMemsetAsync(e->tiles, 0, e->tiles_alloc, st);
-    if (e->scales_pc) cudaMemsetAsync(e->scales_pc, 0, e->pc_alloc, st);
-    if (e->zeros_pc) cudaMemsetAsync(e->zeros_pc, 0, e->pc_alloc, st);
+    if (clear && cudaMemsetAsync(e->tiles, 0, e->tiles_alloc + pc_total, st) != cudaSuccess) { moqe_expert_destroy(e); return MOQE_ERR_CUDA; }
     *out = e;
     return MOQE_OK;
+}
+
+moqe_status launch_quantize(const moqe_expert* e, const float* W, cudaStream_t st) {
+    const int KB = e->Kp / 128, strips = e->Np / 16;
+    // a per-channel strip belongs to one block; grouped strips are cut along K until there are four blocks or so to an SM
+    int cuts = e->group == 0 ? 1 : 600 / strips + 1;
+    if (cuts > (KB + 7) / 8) cuts = (KB + 7) / 8;
+    const dim3 grid(strips, cuts);
+#define MOQE_QP(B) quantize_pack_kernel<B><<<grid, 256, 0, st>>>(W, e->N, e->K, e->group, e->sym, KB, e->tiles, e->scales_pc, e->zeros_pc)
+    if (e->bits == 4) MOQE_QP(4);
+    else if (e->bits == 8) MOQE_QP(8);
+    else if (e->bits == 2) MOQE_QP(2);
+    else MOQE_QP(3);
+#undef MOQE_QP
+    count_launch();
+    return cuda_ok(cudaGetLastError());
 }
 
 template <bool FROM_CODES>
@@ -390,8 +612,15 @@ extern "C" moqe_status moqe_quantize_rtn(const float* W, int N, int K, int bits,
     if (reinterpret_cast<uintptr_t>(W) % 16 != 0) return MOQE_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)stream;
     moqe_expert* e = nullptr;
-    s = alloc_expert(N, K, bits, group, sym, st, &e);
+    const bool one_pass = group <= 128;
+    s = alloc_expert(N, K, bits, group, sym, !one_pass, st, &e);
     if (s != MOQE_OK) return s;
+    if (one_pass) {
+        s = launch_quantize(e, W, st);
+        if (s != MOQE_OK) { moqe_expert_destroy(e); return s; }
+        *out = e;
+        return MOQE_OK;
+    }
     long long warps = (long long)N * e->G;
     unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
     rtn_scales_kernel<<<blocks, 256, 0, st>>>(W, N, K, bits, group, e->G, e->sym, e->Kp / 128, e->tiles, e->scales_pc,
@@ -414,7 +643,7 @@ extern "C" moqe_status moqe_expert_import(int N, int K, int bits, int group, int
     if (reinterpret_cast<uintptr_t>(codes) % 8 != 0) return MOQE_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)stream;
     moqe_expert* e = nullptr;
-    s = alloc_expert(N, K, bits, group, sym, st, &e);
+    s = alloc_expert(N, K, bits, group, sym, true, st, &e);
     if (s != MOQE_OK) return s;
     long long n = (long long)N * e->G;
     meta_import_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(scales_f16, zeros_f16, N, e->G, e->Kp / 128, bits, group,
@@ -469,9 +698,9 @@ extern "C" moqe_status moqe_expert_info(const moqe_expert* e, int* N, int* K, in
 
 extern "C" moqe_status moqe_expert_destroy(moqe_expert* e) {
     if (!e) return MOQE_ERR_NULL;
-    cudaError_t a = cudaFree(e->tiles), b = cudaFree(e->scales_pc), c = cudaFree(e->zeros_pc);
+    const bool ok = expert_free(e->tiles, e->device);
     delete e;
-    return (a == cudaSuccess && b == cudaSuccess && c == cudaSuccess) ? MOQE_OK : MOQE_ERR_CUDA;
+    return ok ? MOQE_OK : MOQE_ERR_CUDA;
 }
 
 // ---------------------------------------------------------------------------- dense copy of a small expert
@@ -629,7 +858,7 @@ extern "C" moqe_status moqe_expert_prefetch(const moqe_expert_host* hx, void* st
     if (s != MOQE_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     moqe_expert* e = nullptr;
-    s = alloc_expert(hx->h.N, hx->h.K, hx->h.bits, hx->h.group, hx->h.sym, st, &e);
+    s = alloc_expert(hx->h.N, hx->h.K, hx->h.bits, hx->h.group, hx->h.sym, false, st, &e);
     if (s != MOQE_OK) return s;
     cudaError_t err = cudaMemcpyAsync(e->tiles, hx->image, e->tiles_alloc, cudaMemcpyHostToDevice, st);
     if (err == cudaSuccess && e->scales_pc) err = cudaMemcpyAsync(e->scales_pc, hx->image + e->tiles_alloc, e->pc_alloc, cudaMemcpyHostToDevice, st);

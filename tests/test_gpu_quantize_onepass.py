@@ -1,0 +1,38 @@
+"""Expert construction in one kernel: bit-exact codes, scales and zero-points where its rounding shortcut has to fall back
+to the division (weights exactly halfway between two codes), at padded sizes, and in memory that an earlier, destroyed
+expert has used (nothing of it may be left in the padding, which the products read)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import moqe_workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("bits,group,sym", [(8, 0, True), (4, 0, False), (3, 32, True), (2, 64, False), (4, 128, False), (8, 64, False)])
+@pytest.mark.parametrize("N,K", [(8, 64), (136, 192), (264, 1088), (16, 8192)])
+def test_halfway_weights_and_reused_memory(N, K, bits, group, sym):
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_close, assert_expert_matches, bf16_to_torch, dev, torch_to_bits
+    if group and K % group:
+        pytest.skip("the group does not divide K")
+    g = np.random.default_rng(bits * 1000 + group + N)
+    # multiples of half a step of a power-of-two grid; the extremes pin the grid's scale
+    top = 2 ** (bits - 1) - 1
+    W = (g.integers(-2 * top, 2 * top + 1, size=(N, K)) * 0.5).astype(np.float32)
+    per = group or K
+    W[:, ::per], W[:, 1::per] = top, (-top if sym else -(2 ** bits - 1 - top))
+    W *= np.float32(2.0 ** -7)
+    big = moqe.moqe_quantize_rtn(torch.full((2 * N + 128, 2 * K), 3.0, device=dev()), 8, 0, False)
+    big.close()
+    e = moqe.moqe_quantize_rtn(torch.from_numpy(W).to(dev()), bits, group, sym)
+    c, s, z = oracle.quantize_rtn(W, bits, group, sym)
+    assert_expert_matches(e, (c, s, z))
+    M = 136
+    X = wl.activations_bf16(f"onepass/{K}", M, K)
+    ids = np.zeros(M, np.int32)
+    Y = moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), [e], path=moqe.PATH_TCGEN05)
+    assert moqe.moqe_async_status() == moqe.OK
+    assert_close(torch_to_bits(Y), oracle.routed_gemm(X, ids, [oracle.dequantize(c, s, z, group)]), "product")
