@@ -12,8 +12,11 @@
 //               through `perm` by the producer warp's 16-byte cp.async copies into the same swizzled layout -- the
 //               fused permutation, no gathered copy of X exists
 //   epilogue  : one thread per token row reads its accumulator row from TMEM, multiplies by the per-channel scale,
-//               rounds to bf16 and writes up to 512 contiguous bytes of Y at the row's ORIGINAL position (fused
-//               un-permutation).  X is read once per channel chunk and Y written once.
+//               rounds to bf16 and stages it in shared memory, 32 rows x 64 channels at a time.  Such a box goes out as ONE
+//               TMA store where its rows are consecutive in Y, else in 16-byte stores, to the rows' ORIGINAL positions
+//               (fused un-permutation).  X is read once per channel chunk and Y written once.
+//               (A bulk copy per row half, as before, is bound by the copy engine's 23 cycles a request: 131 / 125 us on the
+//               56 x 56 layers at 256 images, whatever their width.)
 //
 // Per-channel experts reach the tensor core as the exact integers c - z (scale applied to the fp32 sums).  Grouped
 // experts as TWO bf16 numbers per weight, hi + lo = s * (c - z) to 2^-17, and the k loop runs over both halves (the
@@ -37,6 +40,7 @@ namespace {
 constexpr int DN_THREADS = 416;                 // warp 0: producer (TMA + gather), warp 1: MMA issuer, warps 2..9: epilogue,
                                                 // warps 10..12: gather helpers
 constexpr int DN_GATHER_WARPS = 4;              // warp 0 and the helpers
+constexpr int DN_OUT_BOX = 32 * 128;            // staged output: 32 rows x 64 channels bf16, 128-byte swizzle
 constexpr int DN_EPI_THREADS = 256;
 constexpr int DN_MAX_STAGES = 8;
 constexpr int DN_XSTAGE = 128 * 128;            // 128 token rows x 64 k bf16
@@ -75,6 +79,10 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar) : "memory");
 }
 
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int c0, int c1, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(map), "r"(c0), "r"(c1), "r"(src) : "memory");
+}
+
 struct DnTile { int e, m0, rows, box0; };
 // token tile t of the call: expert, first sorted row, rows, index of its first 64-row box
 __device__ __forceinline__ bool dn_tile(const int* s_off, int E, int t, DnTile& ti) {
@@ -97,7 +105,8 @@ __device__ __forceinline__ bool dn_tile(const int* s_off, int E, int t, DnTile& 
 
 __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid_constant__ DnParams p,
                                                                     const __grid_constant__ CUtensorMap tmap_x,
-                                                                    const __grid_constant__ CUtensorMap tmap_w) {
+                                                                    const __grid_constant__ CUtensorMap tmap_w,
+                                                                    const __grid_constant__ CUtensorMap tmap_y) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     using L = DnSmem;
@@ -106,12 +115,12 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
     const uint32_t bar_full = sbase + L::bar_off, bar_empty = bar_full + 8 * DN_MAX_STAGES;
     const uint32_t bar_accfull = bar_empty + 8 * DN_MAX_STAGES, bar_accempty = bar_accfull + 16;
     const uint32_t bar_wres_full = bar_accempty + 16, bar_wres_empty = bar_wres_full + 8;
-    // Shared-memory plan.  Output rows are staged with a padded pitch; an expert's dense weights stay resident when all
+    // Shared-memory plan.  Output boxes of the epilogue warps; an expert's dense weights stay resident when all
     // their 64-k steps fit DN_WRES_MAX (the token rows are then the only stream); the rest is cut into operand stages of
     // 128 token rows (+ the channel rows of one accumulator when the weights are streamed too).
     const int nc_rows = min(DN_NC, p.Nw);
-    const int out_pitch = nc_rows * 2 + 16;
-    const int out_bytes = (128 * out_pitch + 1023) & ~1023;
+    const int out_boxes = (nc_rows / 64 + 1) / 2;            // 64-channel boxes an epilogue warp has in a chunk
+    const int out_bytes = 8 * out_boxes * DN_OUT_BOX;
     const int wres_bytes = p.resident ? p.max_steps * p.Nw * 128 : 0;
     const int stage_bytes = DN_XSTAGE + (p.resident ? 0 : nc_rows * 128);
     const int nstg = min(DN_MAX_STAGES, (DN_POOL_BYTES - out_bytes - wres_bytes) / stage_bytes);
@@ -201,7 +210,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
             for (int nc = 0; ok && nc < nchunks; ++nc) {
                 const int wrows = min(DN_NC, p.Nw - nc * DN_NC);
                 for (int ks = 0; ks < steps; ++ks) {
-                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(bar_empty + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status)))) break;
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait_short(bar_empty + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status)))) break;
                     const uint32_t full = bar_full + 8 * ring.stage;
                     const uint32_t xd = ring_base + ring.stage * stage_bytes;
                     const int xcol = (ks < kstages ? ks : ks - kstages) * 64;             // the second half re-reads the tokens
@@ -233,7 +242,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
                         }
                         asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(full) : "memory");
                     } else {
-                        mbar_arrive(full);
+                        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], 32;" ::"r"(full) : "memory");   // the warp's 32 at once
                     }
                     ring.advance(nstg);
                 }
@@ -315,49 +324,70 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
                 asm volatile("bar.sync 1, %0;" ::"n"(DN_EPI_THREADS) : "memory");
                 cs_e = ti.e;
             }
-            const bool live = row < ti.rows;
-            // This thread's half of the staged row.  The halves lie where those of a full chunk do, whatever the chunk's width:
-            // in a narrower last chunk the second half would otherwise be written over the first warp's copy still under way.
-            const uint32_t out_row = out_base + row * out_pitch + colhalf * nc_rows;
+            // this warp's 32 rows: one TMA store a box if they are all there and consecutive in Y
+            const int first = __shfl_sync(0xffffffffu, (int)yrow, 0), live_rows = ti.rows - quarter * 32;
+            const bool run = __all_sync(0xffffffffu, live_rows >= 32 && (int)yrow == first + lane);
             for (int nc = 0; ok && nc < nchunks; ++nc) {
-                const int wrows = min(DN_NC, p.Nw - nc * DN_NC);
-                const int half_cols = wrows >> 1, c_lo = colhalf * half_cols;          // this warp's channels of the chunk
-                if (!(ok = mbar_wait(bar_accfull + 8 * buf, acc_use[buf] & 1u, s_abort, p.status))) break;
+                const int wrows = min(DN_NC, p.Nw - nc * DN_NC), boxes = wrows >> 6, split = (boxes + 1) >> 1;
+                const int b_lo = colhalf ? split : 0, b_hi = colhalf ? boxes : split;          // this warp's boxes of the chunk
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait_short(bar_accfull + 8 * buf, acc_use[buf] & 1u, s_abort, p.status)))) break;
                 tc_fence_after();
-                // the previous chunk's row has left shared memory (this thread's own bulk store) before it is overwritten
-                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                for (int c = c_lo; c < c_lo + half_cols; c += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * DN_NC + c, v);
-                    tmem_ld_wait();
-                    const uint32_t cs = cs_base + (nc * DN_NC + c) * 4;
+                // the previous boxes have left shared memory (lane 0's own stores) before they are overwritten
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                __syncwarp();
+                for (int b = b_lo; b < b_hi; ++b) {
+                    const uint32_t box = out_base + ((warp - 2) * out_boxes + (b - b_lo)) * DN_OUT_BOX;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        float sc[8];
-                        asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(sc[0]), "=f"(sc[1]), "=f"(sc[2]), "=f"(sc[3]) : "r"(cs + j * 32));
-                        asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(sc[4]), "=f"(sc[5]), "=f"(sc[6]), "=f"(sc[7]) : "r"(cs + j * 32 + 16));
-                        uint32_t o[4];
+                    for (int half = 0; half < 2; ++half) {
+                        const int c = b * 64 + half * 32;
+                        uint32_t v[32];
+                        tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * DN_NC + c, v);
+                        tmem_ld_wait();
+                        const uint32_t cs = cs_base + (nc * DN_NC + c) * 4;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v[8 * j + 2 * i]) * sc[2 * i],
-                                                                     __uint_as_float(v[8 * j + 2 * i + 1]) * sc[2 * i + 1]);
-                            o[i] = *reinterpret_cast<uint32_t*>(&h);
+                        for (int j = 0; j < 4; ++j) {
+                            float sc[8];
+                            asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(sc[0]), "=f"(sc[1]), "=f"(sc[2]), "=f"(sc[3]) : "r"(cs + j * 32));
+                            asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(sc[4]), "=f"(sc[5]), "=f"(sc[6]), "=f"(sc[7]) : "r"(cs + j * 32 + 16));
+                            uint32_t o[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v[8 * j + 2 * i]) * sc[2 * i],
+                                                                         __uint_as_float(v[8 * j + 2 * i + 1]) * sc[2 * i + 1]);
+                                o[i] = *reinterpret_cast<uint32_t*>(&h);
+                            }
+                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(box + lane * 128 + (((half * 4 + j) ^ (lane & 7)) << 4)), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
                         }
-                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(out_row + (c - c_lo + 8 * j) * 2), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
                     }
                 }
                 tc_fence_before();
-                mbar_arrive(bar_accempty + 8 * buf);
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], 32;" ::"r"(bar_accempty + 8 * buf) : "memory");
                 acc_use[buf]++;
                 buf ^= 1;
-                // this warp's channels of the row go out as ONE contiguous copy to the row's original position
-                const int n0 = nc * DN_NC + c_lo, nbytes = min(half_cols, p.N - n0) * 2;
-                if (live && nbytes > 0) {
+                if (run) {
                     fence_proxy_async();
-                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                                 ::"l"(p.Y + yrow * p.N + n0), "r"(out_row), "r"(nbytes) : "memory");
+                    __syncwarp();
+                    if (lane == 0)
+                        for (int b = b_lo; b < b_hi; ++b)
+                            tma_store_2d(&tmap_y, nc * DN_NC + b * 64, first, out_base + ((warp - 2) * out_boxes + (b - b_lo)) * DN_OUT_BOX);
+                } else {
+                    // rows scattered in Y, or the ragged end of a tile: 16 bytes a lane, eight lanes to a row's 128 bytes
+                    for (int b = b_lo; b < b_hi; ++b) {
+                        const uint32_t box = out_base + ((warp - 2) * out_boxes + (b - b_lo)) * DN_OUT_BOX;
+                        const int n0 = nc * DN_NC + b * 64 + (lane & 7) * 8;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int r = 4 * i + (lane >> 3);
+                            const int to = __shfl_sync(0xffffffffu, (int)yrow, r);
+                            uint32_t o[4];
+                            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3]) : "r"(box + r * 128 + (((lane & 7) ^ (r & 7)) << 4)));
+                            if (r < live_rows && n0 < p.N) *reinterpret_cast<uint4*>(p.Y + (size_t)to * p.N + n0) = make_uint4(o[0], o[1], o[2], o[3]);
+                        }
+                    }
+                    __syncwarp();
                 }
-                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                if (lane == 0) asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
         }
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
@@ -388,10 +418,10 @@ EncodeTiledFn dn_encode_fn() {
         return (EncodeTiledFn)f;
     return nullptr;
 }
-bool dn_map(EncodeTiledFn enc, CUtensorMap* m, const void* base, size_t rows, size_t cols) {
+bool dn_map(EncodeTiledFn enc, CUtensorMap* m, const void* base, size_t rows, size_t cols, unsigned box_rows = 64) {
     cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t gstride[1] = {(cuuint64_t)cols * 2};
-    cuuint32_t box[2] = {64, 64};
+    cuuint32_t box[2] = {64, box_rows};
     cuuint32_t estr[2] = {1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -426,8 +456,8 @@ moqe_status launch_qgemm_dense(const void* X, int M, int N, int K, const moqe_ex
     float* cs = (float*)(base + al256((size_t)E * Np * Kp * 4));
     moqe_status s = launch_dense_unpack(ex, E, Wd, cs, st);
     if (s != MOQE_OK) return s;
-    CUtensorMap tmap_x, tmap_w;
-    if (!dn_map(enc, &tmap_x, X, M, K) || !dn_map(enc, &tmap_w, Wd, (size_t)E * Np, 2 * (size_t)Kp))
+    CUtensorMap tmap_x, tmap_w, tmap_y;
+    if (!dn_map(enc, &tmap_x, X, M, K) || !dn_map(enc, &tmap_w, Wd, (size_t)E * Np, 2 * (size_t)Kp) || !dn_map(enc, &tmap_y, Y, M, N, 32))
         return MOQE_ERR_CUDA;
     DnParams p;
     p.perm = perm; p.offsets = offsets; p.X = (const uint16_t*)X; p.col_scale = cs; p.Y = (uint16_t*)Y;
@@ -446,7 +476,7 @@ moqe_status launch_qgemm_dense(const void* X, int M, int N, int K, const moqe_ex
     const int grid = (int)(tiles < sms ? tiles : sms);
     if (cudaFuncSetAttribute(qgemm_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DnSmem::dyn_bytes) != cudaSuccess)
         return MOQE_ERR_CUDA;
-    qgemm_dense_kernel<<<grid, DN_THREADS, DnSmem::dyn_bytes, st>>>(p, tmap_x, tmap_w);
+    qgemm_dense_kernel<<<grid, DN_THREADS, DnSmem::dyn_bytes, st>>>(p, tmap_x, tmap_w, tmap_y);
     count_launch();
     return cuda_ok(cudaGetLastError());
 }
