@@ -72,7 +72,10 @@ int pick_kernel(int path, int M, const moqe_expert* const* ex, int E) {
     if (path == 0) {
         if (g_auto_decode && decode_supported_multi(M, ex, 1, E)) return 2;
         if (M <= AUTO_STREAM_MAX_ROWS && !(g_auto_decode && decode_supported_multi(1, ex, 1, E))) return 1;
-        return (g_auto_dense && dense_supported(M, ex[0]->N, ex[0]->K, ex, E)) ? 3 : 0;
+        // (the dense-weights GEMM streams or re-reads an expert's whole matrix per 128 rows; three experts, dense / grouped GEMM:
+        // 1024 -> 256 channels, 980 rows 27 / 21 us, 12544 rows 32 / 31; 256 -> 1024, 980 rows 31 / 11, 3920 rows 35 / 16)
+        const bool few = M < 12000 && (long long)ex[0]->N * ex[0]->K > 65536;
+        return (g_auto_dense && !few && dense_supported(M, ex[0]->N, ex[0]->K, ex, E)) ? 3 : 0;
     }
     return 0;
 }

@@ -19,8 +19,8 @@
 //               56 x 56 layers at 256 images, whatever their width.)
 //
 // Per-channel experts reach the tensor core as the exact integers c - z (scale applied to the fp32 sums).  Grouped
-// experts as TWO bf16 numbers per weight, hi + lo = s * (c - z) to 2^-17, and the k loop runs over both halves (the
-// token stage is fetched again from L2 for the second half): twice the tensor work on a path the tensor cores do not
+// experts as TWO bf16 numbers per weight, hi + lo = s * (c - z) to 2^-17: resident weights meet each token stage with both
+// halves, streamed ones run the k loop over both (the token stage is fetched again from L2 for the second half): twice the tensor work on a path the tensor cores do not
 // bound, and no rounding of weights that the tolerance of the routed product would see.
 //
 // Every mbarrier wait is bounded; on expiry the CTA raises its abort flag, latches MOQE_ERR_TIMEOUT, lets copies in
@@ -138,8 +138,9 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = tid; i <= p.E; i += DN_THREADS) s_off[i] = p.offsets[i];
     if (warp == 1) tmem_alloc(sbase + L::misc_off, 512);
+    asm volatile("griddepcontrol.wait;" ::: "memory");            // (nothing above depends on the kernels before)
+    for (int i = tid; i <= p.E; i += DN_THREADS) s_off[i] = p.offsets[i];
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -209,7 +210,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
             }
             for (int nc = 0; ok && nc < nchunks; ++nc) {
                 const int wrows = min(DN_NC, p.Nw - nc * DN_NC);
-                for (int ks = 0; ks < steps; ++ks) {
+                for (int ks = 0; ks < (p.resident ? kstages : steps); ++ks) {
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait_short(bar_empty + 8 * ring.stage, ring.phase ^ 1u, s_abort, p.status)))) break;
                     const uint32_t full = bar_full + 8 * ring.stage;
                     const uint32_t xd = ring_base + ring.stage * stage_bytes;
@@ -275,20 +276,29 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
                 if (!(ok = __all_sync(0xffffffffu, mbar_wait(bar_accempty + 8 * buf, (acc_use[buf] & 1u) ^ 1u, s_abort, p.status)))) break;
                 const uint32_t d = tmem_base + buf * DN_NC;
                 const int steps = ((p.split_mask >> ti.e) & 1u) ? 2 * kstages : kstages;
-                for (int ks = 0; ks < steps; ++ks) {
-                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(bar_full + 8 * ring.stage, ring.phase, s_abort, p.status)))) break;
+                const int xsteps = p.resident ? kstages : steps;
+                const bool both = p.resident && steps > kstages;            // hi and lo halves against one token stage
+                for (int ks = 0; ks < xsteps; ++ks) {
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait_short(bar_full + 8 * ring.stage, ring.phase, s_abort, p.status)))) break;
                     fence_proxy_async();                 // gathered token rows were written by plain (generic-proxy) copies
                     tc_fence_after();
                     const uint32_t stage = ring_base + ring.stage * stage_bytes;
                     const uint64_t adesc = umma_desc_sw128(stage);
                     const uint64_t bdesc = umma_desc_sw128(p.resident ? wres_base + ks * p.Nw * 128 + nc * DN_NC * 128 : stage + DN_XSTAGE);
                     const uint32_t empty_bar = bar_empty + 8 * ring.stage;
-                    const bool last = ks + 1 == steps;
+                    const uint64_t bdesc2 = bdesc + (uint32_t)(kstages * p.Nw * 128) / 16;
+                    const bool last = ks + 1 == xsteps;
                     if (elect_one()) {
                         umma_bf16(d, adesc, bdesc, idesc, ks > 0 ? 1u : 0u);
                         umma_bf16(d, adesc + 2, bdesc + 2, idesc, 1u);
                         umma_bf16(d, adesc + 4, bdesc + 4, idesc, 1u);
                         umma_bf16(d, adesc + 6, bdesc + 6, idesc, 1u);
+                        if (both) {
+                            umma_bf16(d, adesc, bdesc2, idesc, 1u);
+                            umma_bf16(d, adesc + 2, bdesc2 + 2, idesc, 1u);
+                            umma_bf16(d, adesc + 4, bdesc2 + 4, idesc, 1u);
+                            umma_bf16(d, adesc + 6, bdesc2 + 6, idesc, 1u);
+                        }
                         umma_commit(empty_bar);
                         if (last) umma_commit(bar_accfull + 8 * buf);
                     }
@@ -476,7 +486,13 @@ moqe_status launch_qgemm_dense(const void* X, int M, int N, int K, const moqe_ex
     const int grid = (int)(tiles < sms ? tiles : sms);
     if (cudaFuncSetAttribute(qgemm_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DnSmem::dyn_bytes) != cudaSuccess)
         return MOQE_ERR_CUDA;
-    qgemm_dense_kernel<<<grid, DN_THREADS, DnSmem::dyn_bytes, st>>>(p, tmap_x, tmap_w, tmap_y);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(DN_THREADS); cfg.dynamicSmemBytes = DnSmem::dyn_bytes; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, qgemm_dense_kernel, p, tmap_x, tmap_w, tmap_y) != cudaSuccess) { cudaGetLastError(); return MOQE_ERR_CUDA; }
     count_launch();
     return cuda_ok(cudaGetLastError());
 }

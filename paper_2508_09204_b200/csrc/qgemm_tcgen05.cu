@@ -1082,7 +1082,16 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
     if (!enc) return MOQE_ERR_CUDA;
     // Tile by batch size (the routing is not known here): LLaMA blocks, three experts, rows dealt evenly, 64 / 128 / 256
     // tokens: 192 rows 235 / 275 / 302 us, 256 rows 367 / 299 / 318, 384 rows 383 / 323 / 346, 512 rows 474 / 489 / 414.
-    const int tile = tile_tokens ? tile_tokens : (M > 448 ? 256 : (M > 192 ? 128 : 64));
+    // A layer that would leave clusters without a tile takes smaller ones while they still fit one round (980 rows of
+    // 256 x 1024, 128 against 256 tokens: 11 / 16 us).
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int clusters = sms / 2 < TC_MAX_CLUSTERS ? sms / 2 : TC_MAX_CLUSTERS;
+    int tile = tile_tokens ? tile_tokens : (M > 448 ? 256 : (M > 192 ? 128 : 64));
+    const int ntp = (ex[0]->Np / 128 + 1) / 2;
+    if (!tile_tokens)
+        while (tile > 64 && (long long)(2 * M / tile + E) * ntp <= clusters) tile /= 2;
     // tensor map over X[M][K] bf16: boxes of 64 k x XR rows, 128-byte swizzle, zero fill outside
     CUtensorMap tmap;
     cuuint64_t gdim[2] = {(cuuint64_t)K, (cuuint64_t)M};
@@ -1103,10 +1112,6 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
     p.M = M; p.N = N; p.K = K; p.KB = ex[0]->Kp / 128; p.E = E; p.NT1 = ex[0]->Np / 128; p.NTP = (p.NT1 + 1) / 2;
     p.cols = tc_cols(M);
     p.split = tile_tokens == 0 && p.KB <= 4096 ? 1 : 0;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int clusters = sms / 2 < TC_MAX_CLUSTERS ? sms / 2 : TC_MAX_CLUSTERS;
     auto launch = [&](auto kernel, int threads, int smem, int w_bytes) -> bool {
         p.wstage = (stride + 127) / 128 * 128;
         p.nw = w_bytes / p.wstage < TC_NW_MAX ? w_bytes / p.wstage : TC_NW_MAX;

@@ -763,6 +763,7 @@ __device__ __forceinline__ void dense_unpack_piece(const uint8_t* __restrict__ t
 // blockIdx.y = expert
 __global__ void dense_unpack_kernel(const __grid_constant__ DenseSrc src, int N, int K, int Np, int Kp, int KB,
                                     uint16_t* __restrict__ Wd, float* __restrict__ col_scale, long long npieces) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");     // (the GEMM behind may start its prologue)
     const long long pid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (pid >= npieces) return;
     const int e = blockIdx.y;
