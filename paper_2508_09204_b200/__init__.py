@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from array import array
 from typing import List, Optional, Sequence, Tuple
 
 import torch
@@ -70,11 +71,11 @@ def lib() -> C.CDLL:
         L.moqe_routed_qgemm_workspace.argtypes = [i32, i32, i32, i32]
         L.moqe_routed_qgemm_workspace.restype = sz
         L.moqe_routed_qgemm.argtypes = [vp, vp, i32, C.POINTER(vp), i32, vp, vp, sz, vp]
-        L.moqe_routed_qgemm_path.argtypes = [vp, vp, i32, C.POINTER(vp), i32, vp, vp, sz, vp, i32]
-        L.moqe_routed_qgemm_sorted.argtypes = [vp, vp, vp, i32, C.POINTER(vp), i32, vp, vp, sz, vp, i32]
-        L.moqe_routed_qgemm_sorted_multi.argtypes = [C.POINTER(vp), vp, vp, i32, i32, C.POINTER(vp), i32, C.POINTER(vp), vp, sz, vp]
-        L.moqe_routed_qgemm_sorted_gated.argtypes = [vp, vp, vp, i32, C.POINTER(vp), C.POINTER(vp), i32, vp, vp, sz, vp]
-        L.moqe_routed_qgemm_sorted_residual.argtypes = [vp, vp, vp, i32, C.POINTER(vp), i32, vp, vp, vp, sz, vp]
+        L.moqe_routed_qgemm_path.argtypes = [vp, vp, i32, vp, i32, vp, vp, sz, vp, i32]
+        L.moqe_routed_qgemm_sorted.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, sz, vp, i32]
+        L.moqe_routed_qgemm_sorted_multi.argtypes = [vp, vp, vp, i32, i32, vp, i32, vp, vp, sz, vp]
+        L.moqe_routed_qgemm_sorted_gated.argtypes = [vp, vp, vp, i32, vp, vp, i32, vp, vp, sz, vp]
+        L.moqe_routed_qgemm_sorted_residual.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, vp, sz, vp]
         L.moqe_routed_qgemm_workspace_clear.argtypes = [vp, sz, i32, i32, i32, i32, vp]
         L.moqe_async_status.argtypes = [vp]
         L.moqe_status_str.argtypes = [i32]
@@ -106,12 +107,26 @@ def _check(code: int, where: str):
         raise MoqeError(code, where)
 
 
+_raw_stream = None
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    """The current CUDA stream's handle (by the short way where torch has it: a Stream object costs 2 us a call)."""
+    global _raw_stream
+    if _raw_stream is None:
+        torch.cuda.init()
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+            (lambda dev: torch.cuda.current_stream(dev).cuda_stream)
+    return _raw_stream(torch._C._cuda_getDevice())
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+def _handles(experts) -> array:
+    """The experts' handles as a C array; pass ``.buffer_info()[0]`` and keep the array until the call returns."""
+    return array("Q", [e.address for e in experts])
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
@@ -119,7 +134,7 @@ def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
         raise ValueError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise ValueError(f"{name} must be {dtype}")
-    return t.contiguous()
+    return t if t.is_contiguous() else t.contiguous()
 
 
 class Expert:
@@ -132,6 +147,10 @@ class Expert:
         _check(lib().moqe_expert_info(self.handle, N, K, bits, group, sym, cb, mb, ab), "moqe_expert_info")
         self.N, self.K, self.bits, self.group, self.sym = N.value, K.value, bits.value, group.value, bool(sym.value)
         self.code_bytes, self.meta_bytes, self.alloc_bytes = cb.value, mb.value, ab.value
+
+    @property
+    def address(self) -> int:
+        return (self.handle.value or 0) if self.handle is not None else 0
 
     @property
     def groups_per_row(self) -> int:
@@ -308,6 +327,11 @@ def moqe_unpermute(Yp: torch.Tensor, perm: torch.Tensor) -> torch.Tensor:
     return Y
 
 
+def _at(a):
+    """What a C-array argument is passed as: the address of an ``array``, a ctypes array as it is."""
+    return a.buffer_info()[0] if isinstance(a, array) else a
+
+
 def moqe_routed_qgemm_workspace(M: int, N: int, K: int, E: int) -> int:
     return int(lib().moqe_routed_qgemm_workspace(int(M), int(N), int(K), int(E)))
 
@@ -333,8 +357,8 @@ def moqe_routed_qgemm(X: torch.Tensor, row_ids: torch.Tensor, experts: Sequence[
         Y = torch.empty((M, N), dtype=torch.bfloat16, device=X.device)
     if workspace is None:
         workspace = alloc_workspace(moqe_routed_qgemm_workspace(M, N, K, E), X.device)
-    arr = (C.c_void_p * E)(*[e.handle for e in experts])
-    _check(lib().moqe_routed_qgemm_path(_ptr(X), _ptr(row_ids), M, arr, E, _ptr(Y), _ptr(workspace), workspace.numel(),
+    arr = _handles(experts)
+    _check(lib().moqe_routed_qgemm_path(_ptr(X), _ptr(row_ids), M, arr.buffer_info()[0], E, _ptr(Y), _ptr(workspace), workspace.numel(),
                                         _stream(), int(path)), "moqe_routed_qgemm")
     return Y
 
@@ -353,8 +377,8 @@ def moqe_routed_qgemm_sorted(X: torch.Tensor, perm: torch.Tensor, offsets: torch
     """
     M, K = X.shape
     E = len(experts)
-    arr = _arr if _arr is not None else (C.c_void_p * E)(*[e.handle for e in experts])
-    _check(lib().moqe_routed_qgemm_sorted(_ptr(X), _ptr(perm), _ptr(offsets), M, arr, E, _ptr(Y), _ptr(workspace),
+    arr = _arr if _arr is not None else _handles(experts)
+    _check(lib().moqe_routed_qgemm_sorted(_ptr(X), _ptr(perm), _ptr(offsets), M, _at(arr), E, _ptr(Y), _ptr(workspace),
                                           workspace.numel(), _stream(), int(path)), "moqe_routed_qgemm_sorted")
     return Y
 
@@ -364,8 +388,8 @@ def moqe_routed_qgemm_sorted_gated(X: torch.Tensor, perm: torch.Tensor, offsets:
     """``Y = silu(X . Wgate_e^T) * (X . Wup_e^T)`` for a sorted decode batch, one launch."""
     M = X.shape[0]
     E = len(gate)
-    ag, au = _arrs if _arrs is not None else ((C.c_void_p * E)(*[e.handle for e in gate]), (C.c_void_p * E)(*[e.handle for e in up]))
-    _check(lib().moqe_routed_qgemm_sorted_gated(_ptr(X), _ptr(perm), _ptr(offsets), M, ag, au, E, _ptr(Y), _ptr(workspace),
+    ag, au = _arrs if _arrs is not None else (_handles(gate), _handles(up))
+    _check(lib().moqe_routed_qgemm_sorted_gated(_ptr(X), _ptr(perm), _ptr(offsets), M, _at(ag), _at(au), E, _ptr(Y), _ptr(workspace),
                                                 workspace.numel(), _stream()), "moqe_routed_qgemm_sorted_gated")
     return Y
 
@@ -375,8 +399,8 @@ def moqe_routed_qgemm_sorted_residual(X: torch.Tensor, perm: torch.Tensor, offse
     """``Y = X . W_e^T + R`` for a sorted decode batch (``R`` bf16 ``[M][N]``, may be ``Y``)."""
     M = X.shape[0]
     E = len(experts)
-    arr = _arr if _arr is not None else (C.c_void_p * E)(*[e.handle for e in experts])
-    _check(lib().moqe_routed_qgemm_sorted_residual(_ptr(X), _ptr(perm), _ptr(offsets), M, arr, E, _ptr(R), _ptr(Y),
+    arr = _arr if _arr is not None else _handles(experts)
+    _check(lib().moqe_routed_qgemm_sorted_residual(_ptr(X), _ptr(perm), _ptr(offsets), M, _at(arr), E, _ptr(R), _ptr(Y),
                                                    _ptr(workspace), workspace.numel(), _stream()), "moqe_routed_qgemm_sorted_residual")
     return Y
 
@@ -391,12 +415,12 @@ def moqe_routed_qgemm_sorted_multi(Xs: Sequence[torch.Tensor], perm: torch.Tenso
     E = len(experts[0])
     M = Xs[0].shape[0]
     if _arrs is None:
-        xa = (C.c_void_p * nl)(*[_ptr(x) for x in Xs])
-        ya = (C.c_void_p * nl)(*[_ptr(y) for y in Ys])
-        ea = (C.c_void_p * (nl * E))(*[e.handle for layer in experts for e in layer])
+        xa = array("Q", [x.data_ptr() for x in Xs])
+        ya = array("Q", [y.data_ptr() for y in Ys])
+        ea = array("Q", [e.address for layer in experts for e in layer])
     else:
         xa, ya, ea = _arrs
-    _check(lib().moqe_routed_qgemm_sorted_multi(xa, _ptr(perm), _ptr(offsets), M, nl, ea, E, ya, _ptr(workspace),
+    _check(lib().moqe_routed_qgemm_sorted_multi(_at(xa), _ptr(perm), _ptr(offsets), M, nl, _at(ea), E, _at(ya), _ptr(workspace),
                                                 workspace.numel(), _stream()), "moqe_routed_qgemm_sorted_multi")
     return Ys
 

@@ -12,7 +12,8 @@ namespace moqe {
 namespace {
 std::atomic<unsigned long long> g_launches{0};
 std::mutex g_status_mutex;
-int* g_status_words[64] = {nullptr};
+std::atomic<int*> g_status_words[64] = {};
+std::atomic<int> g_sm_counts[64] = {};
 }  // namespace
 
 void count_launch(unsigned n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
@@ -20,14 +21,36 @@ void count_launch(unsigned n) { g_launches.fetch_add(n, std::memory_order_relaxe
 int* device_status_word() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    if (int* p = g_status_words[dev].load(std::memory_order_acquire)) return p;
     std::lock_guard<std::mutex> lock(g_status_mutex);
-    if (!g_status_words[dev]) {
+    if (!g_status_words[dev].load(std::memory_order_relaxed)) {
         int* p = nullptr;
         if (cudaMalloc(&p, sizeof(int)) != cudaSuccess) { cudaGetLastError(); return nullptr; }
         if (cudaMemset(p, 0, sizeof(int)) != cudaSuccess) { cudaFree(p); return nullptr; }
-        g_status_words[dev] = p;
+        g_status_words[dev].store(p, std::memory_order_release);
     }
-    return g_status_words[dev];
+    return g_status_words[dev].load(std::memory_order_relaxed);
+}
+
+int device_sm_count() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+    n = g_sm_counts[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
+        g_sm_counts[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+
+bool ensure_dynamic_smem(const void* kernel, int bytes, std::atomic<unsigned long long>& done) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+    if (bit && (done.load(std::memory_order_relaxed) & bit)) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    done.fetch_or(bit, std::memory_order_relaxed);
+    return true;
 }
 
 namespace {

@@ -44,6 +44,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/moqe.h"
 
 static __host__ __device__ inline int moqe_blob_bytes(int bits) { return 16 * 128 * bits / 8; }
@@ -94,6 +96,9 @@ namespace moqe {
 
 // first device-detected error of this device (0 = none); kernels latch with atomicCAS
 int* device_status_word();                 // allocates on first use for the current device
+int device_sm_count();                     // of the current device (148 if it cannot be asked)
+// cudaFuncAttributeMaxDynamicSharedMemorySize of a kernel, set once per device: `done` is the kernel's own word of flags
+bool ensure_dynamic_smem(const void* kernel, int bytes, std::atomic<unsigned long long>& done);
 void count_launch(unsigned n = 1);
 
 inline moqe_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? MOQE_OK : MOQE_ERR_CUDA; }

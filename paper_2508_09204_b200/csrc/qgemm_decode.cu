@@ -938,13 +938,6 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
     }
 }
 
-int dec_sm_count() {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    return n > 0 ? n : 148;
-}
-
 // relative cost of one super-tile in the work split, by code width (measured: a 3-bit super-tile takes the consumers
 // about a tenth longer than a 4-bit one, an 8-bit one lies between -- its copies are twice as large)
 int g_dec_cost[9] = {0, 0, 20, 22, 20, 0, 0, 0, 21};
@@ -1022,14 +1015,15 @@ moqe_status launch_qgemm_decode_ext(const void* const* X, int M, int nl, const m
     p.R = E;
     p.P = nl * E;
     p.status = device_status_word();
-    int grid = dec_sm_count();
+    int grid = device_sm_count();
     if (grid > GV_MAX_GRID) grid = GV_MAX_GRID;
     p.small = total_cost * (grid + 1) < (1ll << 31) ? 1 : 0;
     const bool fused = ex2 != nullptr || R != nullptr;
     if (fused && M > 16) return MOQE_ERR_UNSUPPORTED;     // gated pairs and residual adds: batches of at most 16 rows
     const int smem = fused ? GvSmem<true>::dyn_bytes : GvSmem<false>::dyn_bytes;
     auto kernel = fused ? qgemm_decode_kernel<true, 2> : (M > 16 ? qgemm_decode_kernel<false, 4> : qgemm_decode_kernel<false, 2>);
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static std::atomic<unsigned long long> attr[3] = {};
+    cudaError_t err = ensure_dynamic_smem((const void*)kernel, smem, attr[fused ? 0 : (M > 16 ? 1 : 2)]) ? cudaSuccess : cudaErrorInvalidValue;
     if (err == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(grid); cfg.blockDim = dim3(GV_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;

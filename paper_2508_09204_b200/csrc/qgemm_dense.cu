@@ -422,11 +422,14 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn dn_encode_fn() {
-    void* f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
-        return (EncodeTiledFn)f;
-    return nullptr;
+    static const EncodeTiledFn fn = []() -> EncodeTiledFn {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+            return (EncodeTiledFn)f;
+        return nullptr;
+    }();
+    return fn;
 }
 bool dn_map(EncodeTiledFn enc, CUtensorMap* m, const void* base, size_t rows, size_t cols, unsigned box_rows = 64) {
     cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
@@ -479,13 +482,11 @@ moqe_status launch_qgemm_dense(const void* X, int M, int N, int K, const moqe_ex
         if (ex[e]->group != 0) p.split_mask |= 1u << e;
     p.max_steps = p.Ksteps * (p.split_mask ? 2 : 1);
     p.resident = (size_t)p.max_steps * p.Nw * 128 <= (size_t)DN_WRES_MAX ? 1 : 0;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = device_sm_count();
     const long long tiles = (long long)(M + 127) / 128 + E;
     const int grid = (int)(tiles < sms ? tiles : sms);
-    if (cudaFuncSetAttribute(qgemm_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DnSmem::dyn_bytes) != cudaSuccess)
-        return MOQE_ERR_CUDA;
+    static std::atomic<unsigned long long> attr{0};
+    if (!ensure_dynamic_smem((const void*)qgemm_dense_kernel, DnSmem::dyn_bytes, attr)) return MOQE_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(DN_THREADS); cfg.dynamicSmemBytes = DnSmem::dyn_bytes; cfg.stream = st;
     cudaLaunchAttribute at[1];

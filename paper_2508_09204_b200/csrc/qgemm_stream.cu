@@ -618,12 +618,6 @@ int pick_ntmax(int M) { return M <= 8 ? 1 : (M <= 16 ? 2 : 4); }
 
 constexpr int MAX_GRID = 512;                 // bound on resident CTAs the partial slots are sized for
 
-int sm_count() {                              // of the current device (asked every time: a process may drive several)
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    return n > 0 ? n : 148;
-}
 
 // relative cost of one packed tile in the work split.  Measured: a tile costs about the same time whatever its
 // width (the per-tile latency of a consumer warp, not its bytes, sets the pace), hence equal costs.
@@ -664,7 +658,7 @@ moqe_status launch_qgemm_stream(const void* X, int M, int N, int K, const moqe_e
         s.C += (long long)s.TT * s.w[e];
     }
     s.split = M <= SPLIT_MAX_ROWS ? 1 : 0;
-    int ctas = 2 * sm_count();
+    int ctas = 2 * device_sm_count();
     if (ctas > MAX_GRID) ctas = MAX_GRID;
     // split mode: every CTA's cost share must be at least one tile of the dearest kind, so that every CTA
     // between the owners of a segment's first and last tile really owns a tile of it (the reduction counts them)
@@ -698,7 +692,8 @@ moqe_status launch_qgemm_stream(const void* X, int M, int N, int K, const moqe_e
 #define MOQE_LAUNCH(NT)                                                                                           \
     do {                                                                                                          \
         const int smem = StreamSmem<NT>::dyn_bytes;                                                               \
-        err = cudaFuncSetAttribute(qgemm_stream_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);   \
+        static std::atomic<unsigned long long> attr{0};                                                           \
+        err = ensure_dynamic_smem((const void*)qgemm_stream_kernel<NT>, smem, attr) ? cudaSuccess : cudaErrorInvalidValue; \
         if (err == cudaSuccess) {                                                                                 \
             cudaLaunchConfig_t cfg = {};                                                                          \
             cfg.gridDim = dim3(grid); cfg.blockDim = dim3(STREAM_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st; \

@@ -1084,9 +1084,7 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
     // tokens: 192 rows 235 / 275 / 302 us, 256 rows 367 / 299 / 318, 384 rows 383 / 323 / 346, 512 rows 474 / 489 / 414.
     // A layer that would leave clusters without a tile takes smaller ones while they still fit one round (980 rows of
     // 256 x 1024, 128 against 256 tokens: 11 / 16 us).
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = device_sm_count();
     const int clusters = sms / 2 < TC_MAX_CLUSTERS ? sms / 2 : TC_MAX_CLUSTERS;
     int tile = tile_tokens ? tile_tokens : (M > 448 ? 256 : (M > 192 ? 128 : 64));
     const int ntp = (ex[0]->Np / 128 + 1) / 2;
@@ -1112,11 +1110,10 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
     p.M = M; p.N = N; p.K = K; p.KB = ex[0]->Kp / 128; p.E = E; p.NT1 = ex[0]->Np / 128; p.NTP = (p.NT1 + 1) / 2;
     p.cols = tc_cols(M);
     p.split = tile_tokens == 0 && p.KB <= 4096 ? 1 : 0;
-    auto launch = [&](auto kernel, int threads, int smem, int w_bytes) -> bool {
+    auto launch = [&](auto kernel, int threads, int smem, int w_bytes, std::atomic<unsigned long long>& attr) -> bool {
         p.wstage = (stride + 127) / 128 * 128;
         p.nw = w_bytes / p.wstage < TC_NW_MAX ? w_bytes / p.wstage : TC_NW_MAX;
-        // (the attribute is set at every launch: it belongs to the current device, and the call is cheap)
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return false;
+        if (!ensure_dynamic_smem((const void*)kernel, smem, attr)) return false;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(2 * clusters); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
         cudaLaunchAttribute at[1];
@@ -1127,7 +1124,8 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
     };
     auto run = [&](auto tag) {
         using L = TcCfg<decltype(tag)::value>;
-        return launch(qgemm_tc_kernel<decltype(tag)::value>, L::threads, L::dyn_bytes, L::w_bytes);
+        static std::atomic<unsigned long long> attr{0};
+        return launch(qgemm_tc_kernel<decltype(tag)::value>, L::threads, L::dyn_bytes, L::w_bytes, attr);
     };
     const bool launched = tile == 256 ? run(std::integral_constant<int, 256>{})
                                       : (tile == 128 ? run(std::integral_constant<int, 128>{}) : run(std::integral_constant<int, 64>{}));
