@@ -1,0 +1,51 @@
+"""The routing chain where its kernels change shape: the two-kernel sort up to 2048 blocks of 1024 rows and the three-kernel
+one beyond (33 buckets, invalid ids among them), rows expanded four at a time, samples of the router's hidden layer taken
+eight to a warp.  All of it is integer work or fp32 sums, compared as the other tests of these calls do."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import moqe_workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,E", [(1025, 32), (2048, 1), (2 * 1024 * 1024, 4), (2 * 1024 * 1024 + 1, 4), (2 * 1024 * 1024 + 1, 32)])
+def test_sort_with_invalid_ids(M, E):
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import dev
+    ids = np.random.default_rng(M + E).integers(-1, E + 1, size=M).astype(np.int32)
+    bucket = np.where((ids < 0) | (ids >= E), E, ids)
+    _, perm, offsets = moqe.moqe_permute(None, torch.from_numpy(ids).to(dev()), E)
+    counts = np.bincount(bucket, minlength=E + 1)
+    assert np.array_equal(offsets.cpu().numpy(), np.concatenate([[0], np.cumsum(counts[:E])]))
+    assert np.array_equal(perm.cpu().numpy(), np.argsort(bucket, kind="stable"))
+    assert moqe.moqe_async_status() == moqe.ERR_EXPERT_ID
+
+
+@pytest.mark.parametrize("rows", [(1,), (3, 0, 0, 2), (5, 1020, 0, 1), (1, 1, 1, 1, 1, 1, 4093)])
+def test_expand_rows(rows):
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import dev
+    off = np.concatenate([[0], np.cumsum(rows)]).astype(np.int32)
+    ids = np.arange(len(rows), dtype=np.int32)[::-1].copy()
+    got = moqe.moqe_expand_ids(torch.from_numpy(ids).to(dev()), torch.from_numpy(off).to(dev()), int(off[-1]))
+    assert np.array_equal(got.cpu().numpy(), np.repeat(ids, rows))
+
+
+@pytest.mark.parametrize("S,H,D", [(1, 8, 1), (7, 264, 9), (8, 128, 8), (9, 136, 17), (17, 512, 7)])
+def test_router_sample_groups(S, H, D):
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import dev, bf16_to_torch
+    n = 1 + (np.arange(S) * 37) % 70
+    off = np.concatenate([[0], np.cumsum(n)]).astype(np.int32)
+    X = wl.activations_bf16(f"route/groups/{S}", int(off[-1]), H)
+    W1 = wl.normal_f32(f"route/groups/w1/{S}", (D, H), 1.0 / np.sqrt(H))
+    W2 = wl.normal_f32(f"route/groups/w2/{S}", (3, D), 1.0 / np.sqrt(D))
+    ref, _ = oracle.router_mlp(X, off, W1, W2)
+    lg, ids = moqe.moqe_router_mlp(bf16_to_torch(X), torch.from_numpy(off).to(dev()), torch.from_numpy(W1).to(dev()),
+                                   torch.from_numpy(W2).to(dev()))
+    # fp32 sums of at most 70 + 512 terms of size ~1: 1e-6 relative, a hundredth of the bound
+    assert np.all(np.abs(lg.cpu().numpy().astype(np.float64) - ref) <= 1e-4 * (1.0 + np.abs(ref)))
+    assert np.array_equal(ids.cpu().numpy(), oracle.route(lg.cpu().numpy()))
