@@ -77,10 +77,10 @@ WsLayout ws_layout(int M, int Np, int K, int E) {
     return w;
 }
 
-// Batches the decode kernel does not take: up to this many rows the streaming kernel, if it is the formats that keep the
-// decode kernel away (groups narrower than 128 k: four Qwen experts, layer by layer, streaming / grouped GEMM: 24 rows
-// 25 / 28, 73 / 71, 76 / 107 us; 64 rows 32 / 28, 106 / 72, 110 / 108); everything else is the grouped GEMM's (4096 x 4096,
-// three LLaMA experts, 48 rows: 30 / 22 us).
+// Batches beyond the decode kernel's 32 rows: up to this many the streaming kernel, if an expert has groups narrower than
+// 128 k (four Qwen experts, layer by layer, streaming / grouped GEMM: 24 rows 25 / 28, 73 / 71, 76 / 107 us; 64 rows
+// 32 / 28, 106 / 72, 110 / 108); everything else is the grouped GEMM's (4096 x 4096, three LLaMA experts, 48 rows:
+// 30 / 22 us).
 constexpr int AUTO_STREAM_MAX_ROWS = 48;
 constexpr int LAST_PATH = 6;
 
@@ -93,7 +93,7 @@ int pick_kernel(int path, int M, const moqe_expert* const* ex, int E) {
     if (path == 6) return 3;
     if (path == 1) return 1;
     if (path == 0) {
-        if (g_auto_decode && decode_supported_multi(M, ex, 1, E)) return 2;
+        if (g_auto_decode && decode_supported(M, ex, E)) return 2;
         if (M <= AUTO_STREAM_MAX_ROWS && !(g_auto_decode && decode_supported_multi(1, ex, 1, E))) return 1;
         // (the dense-weights GEMM streams or re-reads an expert's whole matrix per 128 rows; three experts, dense / grouped GEMM:
         // 1024 -> 256 channels, 980 rows 27 / 21 us, 12544 rows 32 / 31; 256 -> 1024, 980 rows 31 / 11, 3920 rows 35 / 16)
@@ -142,7 +142,7 @@ moqe_status single_layer_args(const void* X, const void* ids_or_perm, const void
     w = ws_layout(M, ex[0]->Np, K, E);
     if (!workspace || workspace_bytes < w.total || (uintptr_t)workspace % 256) return MOQE_ERR_WORKSPACE;
     kernel = pick_kernel(path, M, ex, E);
-    if (kernel == 2 && !decode_supported_multi(M, ex, 1, E)) return MOQE_ERR_UNSUPPORTED;
+    if (kernel == 2 && !(path == 5 ? decode_supported_multi(M, ex, 1, E) : decode_supported(M, ex, E))) return MOQE_ERR_UNSUPPORTED;
     return MOQE_OK;
 }
 

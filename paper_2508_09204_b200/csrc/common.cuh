@@ -119,10 +119,12 @@ moqe_status launch_qgemm_stream(const void* X, int M, int N, int K, const moqe_e
 size_t stream_zero_bytes(int M, int Np);
 void stream_set_tile_cost(int bits, int cost);   // relative cost of one packed tile in the work split (measurement knob)
 
-// qgemm_decode.cu: decode shapes -- at most DECODE_MAX_ROWS rows, experts per-channel or with groups of >= 128 k;
+// qgemm_decode.cu: decode shapes -- at most DECODE_MAX_ROWS rows, experts per-channel or with groups of >= 128 k (narrower
+// ones in single-layer calls);
 // nl layers that share the routing go down as one launch (ex[l * E + e] = expert e of layer l)
 constexpr int DECODE_MAX_ROWS = 32;
 bool decode_supported_multi(int M, const moqe_expert* const* ex, int nl, int E);
+bool decode_supported(int M, const moqe_expert* const* ex, int E);   // one layer, plain: groups of 32 and 64 k too
 size_t decode_workspace_bytes(int M);
 size_t decode_zero_bytes(int M);
 moqe_status launch_qgemm_decode_multi(const void* const* X, int M, int nl, const moqe_expert* const* ex, int E,

@@ -15,6 +15,11 @@
 //                           with their sums.  Chunk descriptors travel with the buffers, so the consumers follow the
 //                           work split without walking it themselves.
 //
+//   Groups of 32 and 64 k (an instantiation of its own): the service warps sum the token values per group, and a consumer
+//   restarts its accumulators from them and scales once per group instead of once per k-block.  Against the streaming kernel,
+//   which took these formats before (W8, two W4-g128 and a W3-g64 expert; 8 / 24 rows): 3584 x 18944 67 / 75 -> 40 / 41 us,
+//   512 x 3584 12 / 16 -> 11 / 11 us.
+//
 //   Unpacking costs 5 integer instructions per 8 four-bit codes (1 per 2 eight-bit codes, 23 per 32 three-bit
 //   codes, 10 per 16 two-bit codes): a masked code dropped into the mantissa of the fp16 number 1024 becomes 1024 + c, or 1024 + 16c
 //   for a code that sits four bits higher -- no shift, no subtraction.  The tensor core multiplies by token
@@ -54,20 +59,23 @@ constexpr int GV_MAX_STAGES = 12;
 constexpr int GV_XCHG_BYTES = 8 * 8 * 32 * 4;                  // gated pairs: [8 blobs][8 values][32 lanes] floats
 constexpr int GV_XBUF = 32 * 1024;                             // one chunk of staged token rows
 constexpr int GV_CHUNK_KB = 16;                                // k-blocks per chunk for one token block (8 for two)
-constexpr int GV_SBUF = GV_CHUNK_KB * 8 * 2 * 4;               // the chunk's sums: [k-block][token block][t][4] floats
+constexpr int GV_SBUF = GV_CHUNK_KB * 8 * 2 * 4;               // the chunk's sums: [k-block][token block][group][t][4] floats
+constexpr int GV_FINE = 4;                                     // groups of a k-block in the variant for groups of 32 and 64 k
 // a parked partial sum: 256 channels x 8 * NTMAX tokens
 __host__ __device__ constexpr int gv_slot_floats(int ntmax) { return GV_CONS * ntmax * 4 * 32; }
 constexpr int GV_MAX_GRID = 256;
 constexpr int GV_PREFETCH_TILES = 4;                           // super-tiles asked of L2 before the dependency wait
 
-// FUSED: the variant with gated pairs and residual adds (it gives 8 KB of the ring to the exchange buffer)
-template <bool FUSED>
+// FUSED: the variant with gated pairs and residual adds (it gives 8 KB of the ring to the exchange buffer); FINE: the one
+// that also takes groups of 32 and 64 k (6 KB of the ring go to the sums of four groups to a k-block)
+template <bool FUSED, bool FINE>
 struct GvSmem {
-    static constexpr int ring_bytes = (FUSED ? 150 : 158) * 1024;
+    static constexpr int sbuf = GV_SBUF * (FINE ? GV_FINE : 1);
+    static constexpr int ring_bytes = (FUSED ? 150 : (FINE ? 152 : 158)) * 1024;
     static constexpr int ring_off = 0;
     static constexpr int x_off = ring_bytes;
     static constexpr int s_off = x_off + 2 * GV_XBUF;
-    static constexpr int xchg_off = s_off + 2 * GV_SBUF;
+    static constexpr int xchg_off = s_off + 2 * sbuf;
     static constexpr int desc_off = xchg_off + (FUSED ? GV_XCHG_BYTES : 0);   // 2 chunk descriptors of 32 bytes
     static constexpr int bar_off = desc_off + 2 * 32;                     // wfull[12] wempty[12] xfull[2] xempty[2]
     static constexpr int off_off = bar_off + (2 * GV_MAX_STAGES + 4) * 8;
@@ -79,7 +87,8 @@ struct GvSmem {
     static constexpr int total = ps_off + MOQE_MAX_EXPERTS * 48;
     static constexpr int dyn_bytes = total;
 };
-static_assert(GvSmem<false>::dyn_bytes <= 227 * 1024 && GvSmem<true>::dyn_bytes <= 227 * 1024, "shared memory budget");
+static_assert(GvSmem<false, false>::dyn_bytes <= 227 * 1024 && GvSmem<true, false>::dyn_bytes <= 227 * 1024 &&
+              GvSmem<false, true>::dyn_bytes <= 227 * 1024, "shared memory budget");
 
 // what the kernel needs to know about a (layer, expert) pair besides pointers; copied to shared memory on entry
 struct PairS {
@@ -88,7 +97,7 @@ struct PairS {
     int rexp;                               // the routing expert whose rows the pair takes
     int w;                                  // cost of one super-tile
     int gated;                              // a gated pair (see tiles2)
-    int pad;
+    int ng;                                 // scale groups of a k-block (1, 2 or 4)
 };
 static_assert(sizeof(PairS) == 48, "PairS is copied word by word");
 
@@ -109,6 +118,7 @@ struct GvParams {
     uint32_t* counters;                     // [CTA][warp]: arrivals for the segment whose head that CTA holds; zero on entry, left zero
     int* status;
     int M, R, P;                            // rows of the batch, routing experts, pairs
+    int slot_nt;                            // token blocks a parked partial sum has room for
     int small;                              // (total cost) x (grid) fits 31 bits: the work split runs in 32-bit arithmetic
 };
 
@@ -251,27 +261,16 @@ __device__ __forceinline__ int sigma_shift(int bits, int p) {
     return p == 15 ? 6 : 3 * ((p % 5) % 3);
 }
 
-template <int BITS, int NT, bool GROUPED, bool ASYM>
+template <int BITS, int NT, bool GROUPED, bool ASYM, int NG = 1>
 struct GvTag {
-    static constexpr int bits = BITS, nt = NT;
+    static constexpr int bits = BITS, nt = NT, ng = NG;
     static constexpr bool grouped = GROUPED, asym = ASYM;
 };
 
-// The MMAs of one tile for one lane: `blob` is the shared-memory address of the warp's blob, `xb` that of the
-// lane's token fragments of this k-block.
-// The same for more than two token blocks: the token fragments are fetched where they are used (holding them all
-// would take 16 registers per block).
-template <int BITS, int NT>
-__device__ __forceinline__ void tile_mma_wide(const GvConst& kc, uint32_t blob, int slot16, uint32_t xb, float (&acc)[NT][4]) {
-    auto step = [&](int G, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
-        // one 32-k group of both channel rows against every token block: a* = row g pairs 0..3, c* = row g + 8
-#pragma unroll
-        for (int tb = 0; tb < NT; ++tb) {
-            const uint4 b = lds128(xb + ((tb * 4 + G) << 9));
-            mma_f16(acc[tb], a0, c0, a1, c1, b.x, b.y);
-            mma_f16(acc[tb], a2, c2, a3, c3, b.z, b.w);
-        }
-    };
+// One tile's codes of one lane, unpacked 32 k at a time: step(G, row g pairs 0..3, row g + 8 pairs 0..3) for the 32-k groups
+// G = 0..3 in order.  `blob` is the shared-memory address of the warp's blob.
+template <int BITS, class Step>
+__device__ __forceinline__ void tile_steps(const GvConst& kc, uint32_t blob, int slot16, const Step& step) {
     if constexpr (BITS == 4) {
         const uint4 w0 = lds128(blob + slot16), w1 = lds128(blob + 512 + slot16);
         const uint32_t a0[4] = {w0.x, w0.y, w0.z, w0.w}, a1[4] = {w1.x, w1.y, w1.z, w1.w};
@@ -318,6 +317,74 @@ __device__ __forceinline__ void tile_mma_wide(const GvConst& kc, uint32_t blob, 
             step(G, ar[4 * G], ar[4 * G + 1], ar[4 * G + 2], ar[4 * G + 3], a8[4 * G], a8[4 * G + 1], a8[4 * G + 2], a8[4 * G + 3]);
     }
 }
+
+// The MMAs of one tile for more than two token blocks: the token fragments (`xb`: the lane's, of this k-block) are fetched
+// where they are used (holding them all would take 16 registers per block).
+template <int BITS, int NT>
+__device__ __forceinline__ void tile_mma_wide(const GvConst& kc, uint32_t blob, int slot16, uint32_t xb, float (&acc)[NT][4]) {
+    tile_steps<BITS>(kc, blob, slot16, [&](int G, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
+#pragma unroll
+        for (int tb = 0; tb < NT; ++tb) {
+            const uint4 b = lds128(xb + ((tb * 4 + G) << 9));
+            mma_f16(acc[tb], a0, c0, a1, c1, b.x, b.y);
+            mma_f16(acc[tb], a2, c2, a3, c3, b.z, b.w);
+        }
+    });
+}
+
+// One tile whose k-block holds NG = 2 or 4 scale groups: every group starts from its own sums (`sS`: [token block][group][t])
+// and is scaled into the running sums when its 128 / NG values of k are done.  meta: the lane's first scale in the tile.
+template <int BITS, int NT, int NG>
+__device__ __forceinline__ void tile_mma_fine(const GvConst& kc, uint32_t blob, int slot16, uint32_t xb, const float4* sS, uint32_t meta,
+                                              bool zeros, float* fin) {
+    constexpr int GS = 4 / NG;
+    uint4 bh[NT > 2 ? 1 : NT][4];
+    if constexpr (NT <= 2) {
+#pragma unroll
+        for (int G = 0; G < 4; ++G)
+#pragma unroll
+            for (int tb = 0; tb < NT; ++tb) bh[tb][G] = lds128(xb + ((tb * 4 + G) << 9));
+    }
+    float acc[NT][4], S0[NT][2], s0, s8, z0, z8;
+    tile_steps<BITS>(kc, blob, slot16, [&](int G, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
+        if (G % GS == 0) {
+            const uint32_t m = meta + (G / GS) * (zeros ? 512 : 256);
+            s0 = __half2float(__ushort_as_half((unsigned short)lds16(m)));
+            s8 = __half2float(__ushort_as_half((unsigned short)lds16(m + 16)));
+            // (without zero-points these read what follows in the stage and drop it: a branch costs more)
+            const uint32_t y0 = lds16(m + 256) << 16, y8 = lds16(m + 256 + 16) << 16;
+            z0 = zeros ? __uint_as_float(y0) : 0.f;
+            z8 = zeros ? __uint_as_float(y8) : 0.f;
+#pragma unroll
+            for (int tb = 0; tb < NT; ++tb) {
+                const float4 sv = sS[(tb * NG + G / GS) * 4];
+                acc[tb][0] = acc[tb][2] = sv.x;
+                acc[tb][1] = acc[tb][3] = sv.y;
+                S0[tb][0] = sv.z;
+                S0[tb][1] = sv.w;
+            }
+        }
+#pragma unroll
+        for (int tb = 0; tb < NT; ++tb) {
+            uint4 b;
+            if constexpr (NT <= 2) b = bh[tb][G];
+            else b = lds128(xb + ((tb * 4 + G) << 9));
+            mma_f16(acc[tb], a0, c0, a1, c1, b.x, b.y);
+            mma_f16(acc[tb], a2, c2, a3, c3, b.z, b.w);
+        }
+        if (G % GS == GS - 1) {
+#pragma unroll
+            for (int tb = 0; tb < NT; ++tb) {
+                fin[4 * tb + 0] = fmaf(s0, fmaf(-z0, S0[tb][0], acc[tb][0]), fin[4 * tb + 0]);
+                fin[4 * tb + 1] = fmaf(s0, fmaf(-z0, S0[tb][1], acc[tb][1]), fin[4 * tb + 1]);
+                fin[4 * tb + 2] = fmaf(s8, fmaf(-z8, S0[tb][0], acc[tb][2]), fin[4 * tb + 2]);
+                fin[4 * tb + 3] = fmaf(s8, fmaf(-z8, S0[tb][1], acc[tb][3]), fin[4 * tb + 3]);
+            }
+        }
+    });
+}
+
+// The MMAs of one tile for one lane.
 
 template <int BITS, int NT>
 __device__ __forceinline__ void tile_mma(const GvConst& kc, uint32_t blob, int slot16, uint32_t xb, float (&acc)[NT][4]) {
@@ -399,12 +466,15 @@ __device__ __forceinline__ void tile_mma(const GvConst& kc, uint32_t blob, int s
 
 // ---------------------------------------------------------------------------- the kernel
 // NTMAX: token blocks of 8 rows an expert may get: 2 (batches of at most 16 rows), or 4 (at most 32 rows; its own
-// instantiation, so that the common one keeps its registers)
-template <bool FUSED, int NTMAX>
+// instantiation, so that the common one keeps its registers).  FINE: groups of 32 and 64 k are taken too (an instantiation of
+// its own, for the registers, the ring and the size of the code)
+template <bool FUSED, int NTMAX, bool FINE>
 __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __grid_constant__ GvParams p) {
-    using L = GvSmem<FUSED>;
+    using L = GvSmem<FUSED, FINE>;
     static_assert(NTMAX == 2 || (NTMAX == 4 && !FUSED), "gated pairs and residuals exist for batches of at most 16 rows");
-    constexpr int SLOT_FLOATS = gv_slot_floats(NTMAX);
+    static_assert(!FINE || NTMAX == 4, "groups of 32 and 64 k: one instantiation for every batch size");
+    const int slot_nt = FINE ? p.slot_nt : NTMAX;             // (a batch of at most 16 rows has the smaller workspace)
+    const int SLOT_FLOATS = gv_slot_floats(slot_nt);
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = smem_u32(smem);
@@ -553,7 +623,8 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
         const int bits = s_ps[v].bits, K = s_ps[v].K;
         const float fold = s_ps[v].has_zeros ? 0.f : (float)(1 << (bits - 1));   // a constant zero-point goes into the sums
         const uint32_t xbuf = sbase + L::x_off + buf * GV_XBUF;
-        float* sbuf = reinterpret_cast<float*>(smem + L::s_off + buf * GV_SBUF);
+        float* sbuf = reinterpret_cast<float*>(smem + L::s_off + buf * L::sbuf);
+        const int ng = FINE ? s_ps[v].ng : 1;
         // (the format's scale exponents are compile-time constants: one instantiation of the loop per code width)
         auto stage_units = [&](auto bits_tag) {
             // one 16-byte fetch (chunk a = 4G + q of the k-block: k = 32G + 8q ..) -> four fp16 pairs in MMA fragment order at
@@ -604,10 +675,22 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
 #pragma unroll
                         for (int i = 0; i < 4; ++i) convert(data[i], 4 * part + i, xdst, S0, S1);
                     }
-                    S0 += __shfl_xor_sync(0xffffffffu, S0, 1);
-                    S1 += __shfl_xor_sync(0xffffffffu, S1, 1);
-                    S0 += __shfl_xor_sync(0xffffffffu, S0, 2);
-                    S1 += __shfl_xor_sync(0xffffffffu, S1, 2);
+                    if (!FINE || ng < 4) {
+                        S0 += __shfl_xor_sync(0xffffffffu, S0, 1);
+                        S1 += __shfl_xor_sync(0xffffffffu, S1, 1);
+                    }
+                    if (!FINE || ng < 2) {
+                        S0 += __shfl_xor_sync(0xffffffffu, S0, 2);
+                        S1 += __shfl_xor_sync(0xffffffffu, S1, 2);
+                    }
+                    if constexpr (FINE) {
+                        // sums at [slab][group][t = mm / 2][4]
+                        if (live && part % (4 / ng) == 0) {
+                            float* S = sbuf + (slab * ng + part / (4 / ng)) * 16 + (mm >> 1) * 4 + (mm & 1);
+                            S[0] = fmaf(-1024.f, S1, -fold * S0);
+                            S[2] = S0;
+                        }
+                    }
                 } else {
                     float g0[4] = {0.f, 0.f, 0.f, 0.f}, g1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -626,9 +709,22 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                     }
                     S0 = (g0[0] + g0[1]) + (g0[2] + g0[3]);
                     S1 = (g1[0] + g1[1]) + (g1[2] + g1[3]);
+                    if constexpr (FINE) {
+                        if (live) {
+                            float* S = sbuf + slab * ng * 16 + (mm >> 1) * 4 + (mm & 1);
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                if (i >= ng) break;
+                                const float a0 = ng == 1 ? S0 : (ng == 2 ? g0[(2 * i) & 3] + g0[(2 * i + 1) & 3] : g0[i]);
+                                const float a1 = ng == 1 ? S1 : (ng == 2 ? g1[(2 * i) & 3] + g1[(2 * i + 1) & 3] : g1[i]);
+                                S[16 * i] = fmaf(-1024.f, a1, -fold * a0);
+                                S[16 * i + 2] = a0;
+                            }
+                        }
+                    }
                 }
                 // sums at [slab][t = mm / 2][4]
-                if (live && part == 0) {
+                if (!FINE && live && part == 0) {
                     float* S = sbuf + slab * 16 + (mm >> 1) * 4 + (mm & 1);
                     S[0] = fmaf(-1024.f, S1, -fold * S0);              // what the accumulator starts from
                     S[2] = S0;
@@ -709,26 +805,29 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
         const int slot16 = (t * 8 + (g ^ (2 * t))) * 16;          // this lane's 16-byte slot inside a 512-byte half blob
         const uint32_t tile_base = sbase + L::ring_off + half * (stage_bytes >> 1);
         Ring ring;
-        float fin[4 * NTMAX];                             // the running sums of the current piece: [token block][4]
-#pragma unroll
-        for (int i = 0; i < 4 * NTMAX; ++i) fin[i] = 0.f;
-        float sc_r = 0.f, sc_r8 = 0.f, z_r = 0.f, z_r8 = 0.f;     // per-channel experts: scale / zero-point of rows g, g + 8
         bool ok = true;
 
         // One chunk of k-blocks of one piece, for a format fixed at compile time.
-        auto run_chunk = [&](auto tag, int nkb, int buf, bool active) {
+        // fin: the piece's running sums [token block][4]; sc / z: per-channel experts' scales / zero-points of rows g, g + 8
+        auto run_chunk = [&](auto tag, int nkb, int buf, bool active, bool zeros, auto& fin, const float (&sc)[2], const float (&z)[2]) {
             constexpr int BITS = decltype(tag)::bits, NT = decltype(tag)::nt;
             constexpr bool GROUPED = decltype(tag)::grouped, ASYM = decltype(tag)::asym;
+            constexpr int NG = decltype(tag)::ng;
             GvConst kc;
             kc.template init<BITS>();
             const uint32_t xb0 = sbase + L::x_off + buf * GV_XBUF + lane * 16;
-            const float4* sS = reinterpret_cast<const float4*>(smem + L::s_off + buf * GV_SBUF) + t;
+            const float4* sS = reinterpret_cast<const float4*>(smem + L::s_off + buf * L::sbuf) + t;
             const uint32_t blob_off = blob * (BITS * 256);
             const uint32_t meta_off = moqe_tile_bytes(BITS) + (blob * 16 + g) * 2;
 #pragma unroll 1
             for (int kbl = 0; kbl < nkb; ++kbl) {
                 if (!__all_sync(0xffffffffu, mbar_wait_short(bar_wfull + 8 * ring.stage, ring.phase, s_abort, p.status))) { ok = false; return; }
-                if (active) {
+                if (NG > 1) {
+                    if constexpr (NG > 1) {
+                        const uint32_t tile = tile_base + ring.stage * stage_bytes;
+                        if (active) tile_mma_fine<BITS, NT, NG>(kc, tile + blob_off, slot16, xb0 + ((kbl * NT * 4) << 9), sS + kbl * NT * NG * 4, tile + meta_off, zeros, fin);
+                    }
+                } else if (active) {
                     const uint32_t tile = tile_base + ring.stage * stage_bytes;
                     float acc[NT][4], S0[NT][2];
 #pragma unroll
@@ -739,7 +838,7 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                         S0[tb][0] = sv.z;
                         S0[tb][1] = sv.w;
                     }
-                    float s0 = sc_r, s8 = sc_r8, z0 = z_r, z8 = z_r8;
+                    float s0 = sc[0], s8 = sc[1], z0 = z[0], z8 = z[1];
                     if constexpr (GROUPED) {
                         const uint32_t meta = tile + meta_off;
                         s0 = __half2float(__ushort_as_half((unsigned short)lds16(meta)));
@@ -772,160 +871,175 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
             }
         };
 
-        for (int n = 0; ok; ++n) {
-            const int buf = n & 1;
-            if (n > 0 && !__all_sync(0xffffffffu, mbar_wait(bar_xfull + 8 * buf, (uint32_t)((n - 1) >> 1) & 1u, s_abort, p.status))) break;
-            const ChunkDesc* d = s_desc + buf;
-            if (!d->valid) break;
-            const int v = d->v, nt2 = d->nt2, kbc = d->kbc, nkb = d->nkb, kb0 = d->kb0, kb1 = d->kb1;
+        // One piece, for a number of token blocks fixed at compile time: all its chunks, then the result.  The sums live in
+        // here, so that one token block does not carry the registers of four (24 rows over four experts, 18944 x 3584:
+        // 45 -> 41 us; the values that had been spilled were loaded in every k-block).  `n` is the CTA's chunk count; the piece's first chunk is there already.
+        int n = 0;
+        auto run_piece = [&](auto nt_tag) {
+            constexpr int NT = decltype(nt_tag)::value;
+            const ChunkDesc* d = s_desc + (n & 1);
+            const int v = d->v, nt2 = d->nt2, kb0 = d->kb0, kb1 = d->kb1;
             const int row0 = s_off[s_ps[v].rexp], rows = s_off[s_ps[v].rexp + 1] - row0;
             const int bits = s_ps[v].bits, group = s_ps[v].group, has_zeros = s_ps[v].has_zeros;
+            const int ng = FINE ? s_ps[v].ng : 1;
             const bool gated = FUSED && s_ps[v].gated;
             const int nt = gated ? nt2 : 2 * nt2 + half;
             const bool active = nt < s_ps[v].NT1;
             const int n_r = nt * 128 + blob * 16 + g;
-            if (kbc == kb0) {
+            float fin[4 * NT], sc[2] = {0.f, 0.f}, z[2] = {0.f, 0.f};
 #pragma unroll
-                for (int i = 0; i < 4 * NTMAX; ++i) fin[i] = 0.f;
-                if (group == 0 && active) {
-                    const __half* sp = gated && half ? p.scales_pc2[v] : p.ex[v].scales_pc;
-                    sc_r = __half2float(sp[n_r]);
-                    sc_r8 = __half2float(sp[n_r + 8]);
-                    if (has_zeros) {
-                        const __nv_bfloat16* zp = gated && half ? p.zeros_pc2[v] : p.ex[v].zeros_pc;
-                        z_r = __bfloat162float(zp[n_r]);
-                        z_r8 = __bfloat162float(zp[n_r + 8]);
-                    }
+            for (int i = 0; i < 4 * NT; ++i) fin[i] = 0.f;
+            if (group == 0 && active) {
+                const __half* sp = gated && half ? p.scales_pc2[v] : p.ex[v].scales_pc;
+                sc[0] = __half2float(sp[n_r]);
+                sc[1] = __half2float(sp[n_r + 8]);
+                if (has_zeros) {
+                    const __nv_bfloat16* zp = gated && half ? p.zeros_pc2[v] : p.ex[v].zeros_pc;
+                    z[0] = __bfloat162float(zp[n_r]);
+                    z[1] = __bfloat162float(zp[n_r + 8]);
                 }
             }
-            // dispatch on the format (uniform over the CTA)
-            const int nti = (NTMAX > 2 && rows > 16) ? 2 : (rows > 8 ? 1 : 0);                  // 1, 2 or 4 token blocks
-            const int fmt = (bits == 4 ? 0 : (bits == 8 ? 1 : (bits == 3 ? 2 : 3))) * 12 + nti * 4 + (group != 0 ? 2 : 0) + (has_zeros ? 1 : 0);
-            switch (fmt) {
-#define GV_CASE(B, BI, NTI, GR, AS) \
-                case BI * 12 + NTI * 4 + GR * 2 + AS: \
-                    if constexpr ((1 << NTI) <= NTMAX) run_chunk(GvTag<B, (1 << NTI), GR != 0, AS != 0>{}, nkb, buf, active); \
-                    break;
-#define GV_CASES(B, BI) GV_CASE(B, BI, 0, 0, 0) GV_CASE(B, BI, 0, 0, 1) GV_CASE(B, BI, 0, 1, 0) GV_CASE(B, BI, 0, 1, 1) \
-                        GV_CASE(B, BI, 1, 0, 0) GV_CASE(B, BI, 1, 0, 1) GV_CASE(B, BI, 1, 1, 0) GV_CASE(B, BI, 1, 1, 1) \
-                        GV_CASE(B, BI, 2, 0, 0) GV_CASE(B, BI, 2, 0, 1) GV_CASE(B, BI, 2, 1, 0) GV_CASE(B, BI, 2, 1, 1)
-                GV_CASES(4, 0)
-                GV_CASES(8, 1)
-                GV_CASES(3, 2)
-                GV_CASES(2, 3)
+            const int b4 = bits == 4 ? 0 : (bits == 8 ? 1 : (bits == 3 ? 2 : 3));
+            const int fmt = b4 * 6 + (ng > 1 ? 4 + (ng >> 2) : (group != 0 ? 2 : 0) + (has_zeros ? 1 : 0));
+            for (int kbc = kb0; kbc < kb1;) {
+                const int buf = n & 1;
+                if (kbc > kb0 && !__all_sync(0xffffffffu, mbar_wait(bar_xfull + 8 * buf, (uint32_t)((n - 1) >> 1) & 1u, s_abort, p.status))) { ok = false; return; }
+                const int nkb = s_desc[buf].nkb;
+                // dispatch on the format (uniform over the CTA)
+                switch (fmt) {
+#define GV_CASE(B, BI, GR, AS) case BI * 6 + GR * 2 + AS: run_chunk(GvTag<B, NT, GR != 0, AS != 0>{}, nkb, buf, active, false, fin, sc, z); break;
+#define GV_FINE_CASE(B, BI, G4) \
+                    case BI * 6 + 4 + G4: if constexpr (FINE) run_chunk(GvTag<B, NT, true, true, G4 ? 4 : 2>{}, nkb, buf, active, has_zeros != 0, fin, sc, z); break;
+#define GV_CASES(B, BI) GV_CASE(B, BI, 0, 0) GV_CASE(B, BI, 0, 1) GV_CASE(B, BI, 1, 0) GV_CASE(B, BI, 1, 1) GV_FINE_CASE(B, BI, 0) GV_FINE_CASE(B, BI, 1)
+                    GV_CASES(4, 0)
+                    GV_CASES(8, 1)
+                    GV_CASES(3, 2)
+                    GV_CASES(2, 3)
 #undef GV_CASES
+#undef GV_FINE_CASE
 #undef GV_CASE
-                default: break;
+                    default: break;
+                }
+                if (!ok) return;
+                kbc += nkb;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_xempty + 8 * buf);       // the token rows are used up: the next chunk may be staged
+                ++n;
             }
-            if (!ok) break;
+            if (!active) return;
 
-            if (kbc + nkb == kb1 && active) {
-                // ---- the piece is complete
-                const int NT = 1 << nti;
-                const int KB = s_ps[v].KB, N = s_ps[v].N;
-                uint16_t* Y = p.Y[v];
-                const uint16_t* R = FUSED ? p.Res[v] : nullptr;
-                auto store_rows = [&]() {
+            // ---- the piece is complete
+            const int KB = s_ps[v].KB, N = s_ps[v].N;
+            uint16_t* Y = p.Y[v];
+            const uint16_t* R = FUSED ? p.Res[v] : nullptr;
+            auto store_rows = [&]() {
 #pragma unroll
-                    for (int tb = 0; tb < NTMAX; ++tb) {
+                for (int tb = 0; tb < NT; ++tb) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int m = 8 * tb + 2 * t + (j & 1), nn = n_r + (j >> 1) * 8;
-                            if (tb < NT && m < rows && nn < N) {
-                                const size_t at = (size_t)s_perm[row0 + m] * N + nn;
-                                float y = fin[4 * tb + j];
-                                if (R) y += __uint_as_float((uint32_t)R[at] << 16);
-                                Y[at] = __bfloat16_as_ushort(__float2bfloat16_rn(y));
-                            }
+                    for (int j = 0; j < 4; ++j) {
+                        const int m = 8 * tb + 2 * t + (j & 1), nn = n_r + (j >> 1) * 8;
+                        if (m < rows && nn < N) {
+                            const size_t at = (size_t)s_perm[row0 + m] * N + nn;
+                            float y = fin[4 * tb + j];
+                            if (R) y += __uint_as_float((uint32_t)R[at] << 16);
+                            Y[at] = __bfloat16_as_ushort(__float2bfloat16_rn(y));
                         }
-                    }
-                };
-                // gated pair: fin <- silu(fin) * other, the second expert's product of the same channels and rows
-                auto gate_with = [&](const float (&other)[4 * NTMAX]) {
-#pragma unroll
-                    for (int i = 0; i < 4 * NTMAX; ++i) fin[i] = fin[i] / (1.f + expf(-fin[i])) * other[i];
-                };
-                float* xchg = reinterpret_cast<float*>(smem + L::xchg_off) + blob * 256 + lane;
-                if (kb0 == 0 && kb1 == KB) {
-                    if (FUSED && gated) {
-                        // warps w and w + 8 hold the two products of the same channels: hand the second to the first
-                        if (half == 1) {
-#pragma unroll
-                            for (int i = 0; i < 4 * NTMAX; ++i) xchg[i * 32] = fin[i];
-                        }
-                        asm volatile("bar.sync %0, 64;" ::"r"(2 + blob) : "memory");
-                        if (half == 0) {
-                            float other[4 * NTMAX];
-#pragma unroll
-                            for (int i = 0; i < 4 * NTMAX; ++i) other[i] = xchg[i * 32];
-                            gate_with(other);
-                            store_rows();
-                        }
-                        asm volatile("bar.sync %0, 64;" ::"r"(2 + blob) : "memory");     // the buffer may be written again
-                    } else {
-                        store_rows();
-                    }
-                } else {
-                    // part of a segment: park this warp's sums, announce, and add everything up if this was the last arrival
-                    // (for a gated pair the two warps of a blob share one counter and whoever is last finishes both products)
-                    const long long C = *s_C, base = s_base[v];
-                    const int G = *s_G, wv = s_ps[v].w;
-                    const int c_a = (int)(((base + (long long)(nt2 * KB) * wv) * G) / C);
-                    const int c_b = (int)(((base + (long long)(nt2 * KB + KB - 1) * wv) * G) / C);
-                    float* slot = p.partials + (size_t)(2 * blockIdx.x + (kb0 == 0 ? 1 : 0)) * SLOT_FLOATS;
-#pragma unroll
-                    for (int tb = 0; tb < NTMAX; ++tb)
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (tb < NT) __stcg(slot + ((warp * NTMAX + tb) * 4 + j) * 32 + lane, fin[4 * tb + j]);
-                    __syncwarp();
-                    unsigned* counter = p.counters + c_a * GV_CONS + (gated ? blob : warp);
-                    const unsigned last = (unsigned)(gated ? 2 * (c_b - c_a) + 1 : c_b - c_a);
-                    unsigned arrived = 0;
-                    // one acquire-release increment: the release side publishes the warp's parked sums (ordered before it
-                    // by the warp barrier above), the acquire side lets the last arriver read everybody else's
-                    if (lane == 0) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(counter) : "memory");
-                    arrived = __shfl_sync(0xffffffffu, arrived, 0);
-                    if (arrived == last) {
-                        __syncwarp();
-                        auto gather = [&](int wsrc, float (&dst)[4 * NTMAX]) {
-#pragma unroll
-                            for (int i = 0; i < 4 * NTMAX; ++i) dst[i] = 0.f;
-                            // several CTAs' sums are fetched together (one round trip), then added in CTA order
-                            constexpr int GB = NTMAX == 2 ? 4 : 2;
-                            for (int c0 = c_a; c0 <= c_b; c0 += GB) {
-                                float part[GB][4 * NTMAX];
-#pragma unroll
-                                for (int u = 0; u < GB; ++u) {
-                                    const int c = c0 + u;
-                                    const float* src = p.partials + (size_t)(2 * c + (c == c_a ? 1 : 0)) * SLOT_FLOATS;
-#pragma unroll
-                                    for (int tb = 0; tb < NTMAX; ++tb)
-#pragma unroll
-                                        for (int j = 0; j < 4; ++j)
-                                            part[u][4 * tb + j] = (c <= c_b && tb < NT) ? __ldcg(src + ((wsrc * NTMAX + tb) * 4 + j) * 32 + lane) : 0.f;
-                                }
-#pragma unroll
-                                for (int u = 0; u < GB; ++u)
-#pragma unroll
-                                    for (int i = 0; i < 4 * NTMAX; ++i) dst[i] += part[u][i];
-                            }
-                        };
-                        if (FUSED && gated) {
-                            float other[4 * NTMAX];
-                            gather(blob, fin);
-                            gather(blob + 8, other);
-                            gate_with(other);
-                        } else {
-                            gather(warp, fin);
-                        }
-                        store_rows();
-                        if (lane == 0) *counter = 0u;
                     }
                 }
+            };
+            // gated pair: fin <- silu(fin) * other, the second expert's product of the same channels and rows
+            auto gate_with = [&](const float (&other)[4 * NT]) {
+#pragma unroll
+                for (int i = 0; i < 4 * NT; ++i) fin[i] = fin[i] / (1.f + expf(-fin[i])) * other[i];
+            };
+            float* xchg = reinterpret_cast<float*>(smem + L::xchg_off) + blob * 256 + lane;
+            if (kb0 == 0 && kb1 == KB) {
+                if (FUSED && gated) {
+                    // warps w and w + 8 hold the two products of the same channels: hand the second to the first
+                    if (half == 1) {
+#pragma unroll
+                        for (int i = 0; i < 4 * NT; ++i) xchg[i * 32] = fin[i];
+                    }
+                    asm volatile("bar.sync %0, 64;" ::"r"(2 + blob) : "memory");
+                    if (half == 0) {
+                        float other[4 * NT];
+#pragma unroll
+                        for (int i = 0; i < 4 * NT; ++i) other[i] = xchg[i * 32];
+                        gate_with(other);
+                        store_rows();
+                    }
+                    asm volatile("bar.sync %0, 64;" ::"r"(2 + blob) : "memory");     // the buffer may be written again
+                } else {
+                    store_rows();
+                }
+            } else {
+                // part of a segment: park this warp's sums, announce, and add everything up if this was the last arrival
+                // (for a gated pair the two warps of a blob share one counter and whoever is last finishes both products)
+                const long long C = *s_C, base = s_base[v];
+                const int G = *s_G, wv = s_ps[v].w;
+                const int c_a = (int)(((base + (long long)(nt2 * KB) * wv) * G) / C);
+                const int c_b = (int)(((base + (long long)(nt2 * KB + KB - 1) * wv) * G) / C);
+                float* slot = p.partials + (size_t)(2 * blockIdx.x + (kb0 == 0 ? 1 : 0)) * SLOT_FLOATS;
+#pragma unroll
+                for (int tb = 0; tb < NT; ++tb)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        __stcg(slot + ((warp * slot_nt + tb) * 4 + j) * 32 + lane, fin[4 * tb + j]);
+                __syncwarp();
+                unsigned* counter = p.counters + c_a * GV_CONS + (gated ? blob : warp);
+                const unsigned last = (unsigned)(gated ? 2 * (c_b - c_a) + 1 : c_b - c_a);
+                unsigned arrived = 0;
+                // one acquire-release increment: the release side publishes the warp's parked sums (ordered before it
+                // by the warp barrier above), the acquire side lets the last arriver read everybody else's
+                if (lane == 0) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(counter) : "memory");
+                arrived = __shfl_sync(0xffffffffu, arrived, 0);
+                if (arrived == last) {
+                    __syncwarp();
+                    // several CTAs' sums are fetched together (one round trip to L2, 32 registers whatever the number of
+                    // token blocks), then added in CTA order
+                    auto gather = [&](int wsrc, float (&dst)[4 * NT]) {
+                        constexpr int GB = 8 / NT;
+#pragma unroll
+                        for (int i = 0; i < 4 * NT; ++i) dst[i] = 0.f;
+                        const float* src0 = p.partials + (size_t)(wsrc * slot_nt * 4) * 32 + lane;
+                        for (int c0 = c_a; c0 <= c_b; c0 += GB) {
+                            float part[GB][4 * NT];
+#pragma unroll
+                            for (int u = 0; u < GB; ++u) {
+                                const int c = c0 + u;
+                                const float* src = src0 + (size_t)(2 * c + (c == c_a ? 1 : 0)) * SLOT_FLOATS;
+#pragma unroll
+                                for (int i = 0; i < 4 * NT; ++i) part[u][i] = c <= c_b ? __ldcg(src + i * 32) : 0.f;
+                            }
+#pragma unroll
+                            for (int u = 0; u < GB; ++u)
+#pragma unroll
+                                for (int i = 0; i < 4 * NT; ++i) dst[i] += part[u][i];
+                        }
+                    };
+                    if (FUSED && gated) {
+                        float other[4 * NT];
+                        gather(blob, fin);
+                        gather(blob + 8, other);
+                        gate_with(other);
+                    } else {
+                        gather(warp, fin);
+                    }
+                    store_rows();
+                    if (lane == 0) *counter = 0u;
+                }
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_xempty + 8 * buf);
+        };
+        for (;;) {
+            const int buf = n & 1;
+            if (n > 0 && !__all_sync(0xffffffffu, mbar_wait(bar_xfull + 8 * buf, (uint32_t)((n - 1) >> 1) & 1u, s_abort, p.status))) break;
+            const ChunkDesc* d = s_desc + buf;
+            if (!d->valid) break;
+            const int rexp = s_ps[d->v].rexp, rows = s_off[rexp + 1] - s_off[rexp];
+            if (rows <= 8) run_piece(std::integral_constant<int, 1>{});
+            else if (NTMAX == 2 || rows <= 16) run_piece(std::integral_constant<int, 2>{});
+            else run_piece(std::integral_constant<int, NTMAX>{});
+            if (!ok) break;
         }
     }
 
@@ -942,9 +1056,14 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
 // about a tenth longer than a 4-bit one, an 8-bit one lies between -- its copies are twice as large)
 int g_dec_cost[9] = {0, 0, 20, 22, 20, 0, 0, 0, 21};
 
-bool dec_formats_ok(const moqe_expert* const* ex, int n) {
+// ... a quarter more with two scale groups to a k-block, three eighths with four (3584 x 18944, W8 / two W4 / one W3 expert, 24
+// rows, the W3 one with groups of 64: 41 us with this, 45 when all cost alike and 43 at a half more)
+int dec_cost(int bits, int group) { return g_dec_cost[bits] * (group == 32 ? 22 : (group == 64 ? 20 : 16)) / 16; }
+
+bool dec_formats_ok(const moqe_expert* const* ex, int n, bool fine) {
     for (int v = 0; v < n; ++v) {
         if (ex[v]->bits != 2 && ex[v]->bits != 3 && ex[v]->bits != 4 && ex[v]->bits != 8) return false;
+        if (fine && (ex[v]->group == 32 || ex[v]->group == 64)) continue;
         if (ex[v]->group != 0 && (ex[v]->group < 128 || ex[v]->group % 128 != 0)) return false;
     }
     return true;
@@ -955,7 +1074,10 @@ bool dec_formats_ok(const moqe_expert* const* ex, int n) {
 void decode_set_tile_cost(int bits, int cost) { if (bits >= 0 && bits <= 8 && cost > 0) g_dec_cost[bits] = cost; }
 
 bool decode_supported_multi(int M, const moqe_expert* const* ex, int nl, int E) {
-    return M <= DECODE_MAX_ROWS && nl >= 1 && nl * E <= MOQE_MAX_EXPERTS && dec_formats_ok(ex, nl * E);
+    return M <= DECODE_MAX_ROWS && nl >= 1 && nl * E <= MOQE_MAX_EXPERTS && dec_formats_ok(ex, nl * E, false);
+}
+bool decode_supported(int M, const moqe_expert* const* ex, int E) {
+    return M <= DECODE_MAX_ROWS && E <= MOQE_MAX_EXPERTS && dec_formats_ok(ex, E, true);
 }
 
 size_t decode_zero_bytes(int M) { return M > DECODE_MAX_ROWS ? 0 : (size_t)GV_MAX_GRID * GV_CONS * sizeof(uint32_t); }
@@ -978,7 +1100,8 @@ moqe_status launch_qgemm_decode_ext(const void* const* X, int M, int nl, const m
                                   const moqe_expert* const* ex2, int E, void* const* Y, const void* const* R,
                                   const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes, cudaStream_t st) {
     if (M == 0) return MOQE_OK;
-    if (!decode_supported_multi(M, ex, nl, E)) return MOQE_ERR_UNSUPPORTED;
+    const bool fine = !decode_supported_multi(M, ex, nl, E);
+    if (fine && (nl != 1 || ex2 || R || !decode_supported(M, ex, E))) return MOQE_ERR_UNSUPPORTED;
     if (ex2)
         for (int v = 0; v < nl * E; ++v)
             if (ex2[v] && (ex2[v]->N != ex[v]->N || ex2[v]->K != ex[v]->K || ex2[v]->bits != ex[v]->bits ||
@@ -998,9 +1121,9 @@ moqe_status launch_qgemm_decode_ext(const void* const* X, int M, int nl, const m
             q.bits = p.ex[v].bits; q.group = p.ex[v].group; q.has_zeros = p.ex[v].has_zeros; q.stride = p.ex[v].tile_stride;
             q.N = ex[v]->N; q.K = ex[v]->K; q.KB = ex[v]->Kp / 128; q.NT1 = ex[v]->Np / 128;
             q.rexp = e;
-            q.w = g_dec_cost[ex[v]->bits];
+            q.w = dec_cost(ex[v]->bits, ex[v]->group);
             q.gated = second ? 1 : 0;
-            q.pad = 0;
+            q.ng = q.group == 32 ? 4 : (q.group == 64 ? 2 : 1);
             total_cost += (long long)(second ? q.NT1 : (q.NT1 + 1) / 2) * q.KB * q.w;
             p.tiles2[v] = second ? second->tiles : nullptr;
             p.scales_pc2[v] = second ? second->scales_pc : nullptr;
@@ -1014,16 +1137,19 @@ moqe_status launch_qgemm_decode_ext(const void* const* X, int M, int nl, const m
     p.M = M;
     p.R = E;
     p.P = nl * E;
+    p.slot_nt = M > 16 ? 4 : 2;
     p.status = device_status_word();
     int grid = device_sm_count();
     if (grid > GV_MAX_GRID) grid = GV_MAX_GRID;
     p.small = total_cost * (grid + 1) < (1ll << 31) ? 1 : 0;
     const bool fused = ex2 != nullptr || R != nullptr;
     if (fused && M > 16) return MOQE_ERR_UNSUPPORTED;     // gated pairs and residual adds: batches of at most 16 rows
-    const int smem = fused ? GvSmem<true>::dyn_bytes : GvSmem<false>::dyn_bytes;
-    auto kernel = fused ? qgemm_decode_kernel<true, 2> : (M > 16 ? qgemm_decode_kernel<false, 4> : qgemm_decode_kernel<false, 2>);
-    static std::atomic<unsigned long long> attr[3] = {};
-    cudaError_t err = ensure_dynamic_smem((const void*)kernel, smem, attr[fused ? 0 : (M > 16 ? 1 : 2)]) ? cudaSuccess : cudaErrorInvalidValue;
+    const int smem = fused ? GvSmem<true, false>::dyn_bytes : (fine ? GvSmem<false, true>::dyn_bytes : GvSmem<false, false>::dyn_bytes);
+    auto kernel = fused ? qgemm_decode_kernel<true, 2, false> : (fine ? qgemm_decode_kernel<false, 4, true> :
+                          (M > 16 ? qgemm_decode_kernel<false, 4, false> : qgemm_decode_kernel<false, 2, false>));
+    static std::atomic<unsigned long long> attr[4] = {};
+    std::atomic<unsigned long long>& done = attr[fused ? 0 : (fine ? 3 : (M > 16 ? 1 : 2))];
+    cudaError_t err = ensure_dynamic_smem((const void*)kernel, smem, done) ? cudaSuccess : cudaErrorInvalidValue;
     if (err == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(grid); cfg.blockDim = dim3(GV_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;

@@ -1,0 +1,30 @@
+"""Batches of at most 32 rows on experts with groups of 32 and 64 k, beside wider formats: the edges of a token block (8, 16
+rows of one expert), a last k-block that is only partly there, a ragged last channel tile, pieces split over many CTAs."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import moqe_workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("one", [False, True])
+@pytest.mark.parametrize("M,N,K", [(1, 128, 64), (8, 200, 320), (9, 1000, 192), (16, 264, 1088), (17, 384, 640), (32, 128, 4096)])
+def test_fine_groups(M, N, K, one):
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_close, bf16_to_torch, build_experts, dev, torch_to_bits
+    specs = [(b, g, sym) for b in (8, 4, 3, 2) for g, sym in ((32, True), (32, False), (64, True), (64, False))] + [(8, 0, True), (3, 0, False)]
+    if K % 128 == 0:
+        specs.append((4, 128, False))
+    W = wl.weights_f32(f"fine/{N}/{K}", N, K)
+    X = wl.activations_bf16(f"fine/{M}/{K}", M, K)
+    gpu, What, _ = build_experts(W, specs)
+    turns = range(len(specs)) if one else range(2)               # every expert alone with all rows / spread over the experts
+    for i in turns:
+        ids = np.full(M, i, np.int32) if one else ((np.arange(M) * 5 + i) % len(specs)).astype(np.int32)
+        before = moqe.moqe_launch_count()
+        Y = moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), gpu)
+        assert moqe.moqe_launch_count() > before and moqe.moqe_async_status() == moqe.OK
+        assert_close(torch_to_bits(Y), oracle.routed_gemm(X, ids, What), f"fine M{M} N{N} K{K} {i}")
