@@ -67,18 +67,14 @@ struct TcCfg {
     static constexpr int epi_warp0 = 4 + dq_warps;
     static constexpr int threads = (epi_warp0 + TC_EPI) * 32;
     static constexpr int nx = 4;                                             // token stages: one step of the tile
-    // (nx, NA and nsc are powers of two: stage and parity follow from the step's number)
+    // (nx and NA are powers of two: stage and parity follow from the step's number)
     static_assert(NA <= nx, "the dequant warps wait for the step NA ago on its token stage's barrier");
-    // Steps of scales between the dequant warps and the epilogue.  When the scales of step k are written, step k - NA - 2
-    // is done and at most NACC buffers are still to be drained: slot k - nsc must be older than that.
-    static constexpr int nsc = 8;
-    static_assert(nsc >= NA + 2 + NACC, "scale slots");
     static constexpr int xstage = KS * NH * xhalf;
     // dynamic shared memory: token stages, packed-weight ring (a power of two of alignment slack in front)
     static constexpr int w_off = nx * xstage;
-    static constexpr int n_bars = 2 * TC_NW_MAX + 2 * nx + NA + 3 * NACC + nsc + 2 * TC_EPI;   // wfull wempty xfull done afull accfull[2] accempty scfull xchg[2]
+    static constexpr int n_bars = 2 * TC_NW_MAX + 2 * nx + NA + 3 * NACC + 2 * TC_EPI;   // wfull wempty xfull done afull accfull[2] accempty xchg[2]
     static constexpr int xchg_bytes = TN == 64 ? TC_EPI * 32 * 32 * 4 : 16;
-    static constexpr int static_bytes = 1024 + 1600 + n_bars * 8 + TC_EPI * EC * 4 + 2 * NH * XR * 4 + nsc * KS * 1024 + 64;   // (an upper bound of TcShared)
+    static constexpr int static_bytes = 1024 + 1600 + n_bars * 8 + TC_EPI * EC * 4 + 2 * NH * XR * 4 + 64;   // (an upper bound of TcShared)
     static constexpr int xchg_off = (227 * 1024 - static_bytes - 1024 - xchg_bytes) / 128 * 128;
     static constexpr int w_bytes = (xchg_off - w_off) / 128 * 128;
     static constexpr int dyn_bytes = 1024 + xchg_off + xchg_bytes;
@@ -122,6 +118,15 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // release; with one, 16384 rows of a per-channel expert took 9.1 ms a LLaMA block instead of 4.9.)
 __device__ __forceinline__ void remote_arrive(uint32_t cluster_addr, uint32_t count = 1) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_addr), "r"(count) : "memory");
+}
+// One lane of a warp arrives.  Predicated: as a branch of one lane each of these cost the warp 100 cycles and more, several
+// times a k-block (see dequant_piece).
+__device__ __forceinline__ void mbar_arrive_if(bool yes, uint32_t bar) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"((uint32_t)yes) : "memory");
+}
+__device__ __forceinline__ void remote_arrive_if(bool yes, uint32_t cluster_addr, uint32_t count = 1) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p mbarrier.arrive.shared::cluster.b64 _, [%0], %1;\n\t}"
+                 ::"r"(cluster_addr), "r"(count), "r"((uint32_t)yes) : "memory");
 }
 __device__ __forceinline__ void remote_expect_tx_only(uint32_t cluster_addr, uint32_t bytes) {
     asm volatile("mbarrier.expect_tx.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(cluster_addr), "r"(bytes) : "memory");
@@ -177,7 +182,6 @@ struct TcShared {
     int abort;
     __align__(16) int perm[TC_EPI][L::EC];  // per epilogue warp: its columns' target rows
     __align__(16) int xrow[2][L::NH * L::XR];   // rows of X to gather, one list per gather warp: row 4 i + j at [j][i]
-    __align__(16) __half scales[L::nsc][L::KS][4][128];   // on their way to the epilogue
 };
 static_assert(sizeof(TcShared<256>) <= TcCfg<256>::static_bytes && sizeof(TcShared<128>) <= TcCfg<128>::static_bytes &&
                   sizeof(TcShared<64>) <= TcCfg<64>::static_bytes && sizeof(TcShared<64>) <= 48 * 1024, "shared memory budget");
@@ -222,10 +226,10 @@ struct TcWalk {
 // quantization groups per k-block.
 template <int TN>
 __device__ __forceinline__ int kblock_cost(int rows, int bits, int per) {
-    const int wide = bits == 8 || bits == 3 ? 2 : 0;
+    const int wide = bits == 8 || bits == 3 ? 2 : 0;       // (the 8-bit tiles are larger, the 3-bit ones take longer to unpack)
     if (TN == 64) return (per <= 1 ? 13 : (per == 2 ? 22 : 36)) + wide;
-    if (TN == 128) return (per == 0 ? 16 : (per == 1 ? 20 : (per == 2 ? 30 : 50))) + wide;
-    return (rows <= 128 ? (per == 0 ? 18 : (per == 1 ? 23 : (per == 2 ? 39 : 68))) : (per == 0 ? 24 : (per == 1 ? 30 : (per == 2 ? 54 : 108)))) + wide;
+    if (TN == 128) return (per == 0 ? 16 : (per == 1 ? 18 : (per == 2 ? 32 : 57))) + wide / 2;
+    return (rows <= 128 ? (per == 0 ? 18 : (per == 1 ? 23 : (per == 2 ? 39 : 68))) : (per == 0 ? 22 : (per == 1 ? 23 : (per == 2 ? 50 : 106)))) + wide / 2;
 }
 // MMA columns of half tile h of a tile with `rows` tokens
 template <int HC>
@@ -283,7 +287,7 @@ __device__ __forceinline__ uint32_t neg_z(float z) { const float v = z * -0.0001
 // (What the loop needs of the expert is passed by value: fields of the kernel's parameters would be fetched again after
 // every barrier.)
 struct TcDequant {
-    uint32_t bar_wfull, bar_wempty, bar_done, bar_scfull, afull0;   // afull0: in the leading CTA
+    uint32_t bar_wfull, bar_wempty, bar_done, afull0;   // afull0: in the leading CTA
     uint32_t lane_tmem;
     int row, nw, wstage;
     uint32_t my_group;
@@ -291,12 +295,12 @@ struct TcDequant {
     uint32_t step;
 };
 template <int TN, int BITS>
-__device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, const unsigned char* wtiles, int nkb, int per, bool has_zeros,
+__device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, const unsigned char* wtiles, int nkb, int per,
                                               uint32_t zpc, bool tile_zeros, int* status) {
     using L = TcCfg<TN>;
     const int lane = threadIdx.x & 31, row = d.row;
     const int half = (row >> 3) & 1, r = row & 7;
-    const int meta = moqe_tile_bytes(BITS) + row * 2, mg = has_zeros ? 512 : 256;
+    const int meta = moqe_tile_bytes(BITS) + row * 2 + 256;               // its zero-points in the tile
     const unsigned char* blobs = wtiles + (row >> 4) * moqe_blob_bytes(BITS);
     bool ok = true;
 #pragma unroll 1
@@ -325,31 +329,19 @@ __device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, co
                 }
             }
             uint32_t nz[4] = {zpc, zpc, zpc, zpc};
-            if (per > 0) {
-                // the tile's scales travel on to the epilogue warps
+            if (tile_zeros) {
                 const unsigned char* m = wtiles + stage + meta;
-                __half* scales = &sh.scales[d.step % L::nsc][kk][0][row];
-                scales[0] = *reinterpret_cast<const __half*>(m);
+                nz[0] = nz[1] = nz[2] = nz[3] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m)));
                 if (per > 1) {
-                    scales[128] = *reinterpret_cast<const __half*>(m + mg);
+                    nz[3] = nz[2] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + (per == 2 ? 1 : 2) * 512)));
                     if (per > 2) {
-                        scales[256] = *reinterpret_cast<const __half*>(m + 2 * mg);
-                        scales[384] = *reinterpret_cast<const __half*>(m + 3 * mg);
-                    }
-                }
-                if (tile_zeros) {
-                    nz[0] = nz[1] = nz[2] = nz[3] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + 256)));
-                    if (per > 1) {
-                        nz[3] = nz[2] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + (per == 2 ? 1 : 2) * 512 + 256)));
-                        if (per > 2) {
-                            nz[1] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + 512 + 256)));
-                            nz[3] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + 3 * 512 + 256)));
-                        }
+                        nz[1] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + 512)));
+                        nz[3] = neg_z(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(m + 3 * 512)));
                     }
                 }
             }
             __syncwarp();
-            if (lane == 0) { mbar_arrive(d.bar_wempty + 8 * d.wring.stage); mbar_arrive(d.bar_scfull + 8 * (d.step % L::nsc)); }
+            mbar_arrive_if(lane == 0, d.bar_wempty + 8 * d.wring.stage);
             // the operand buffer is free once the step NA ago is done
             if (d.step >= L::NA) ok &= warp_wait(d.bar_done + 8 * ((d.step - L::NA) % L::nx), (d.step - L::NA) / L::nx & 1u, &sh.abort, status);
             tc_fence_after();
@@ -368,13 +360,13 @@ __device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, co
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) remote_arrive(d.afull0 + 8 * (d.step % L::NA));
+            remote_arrive_if(lane == 0, d.afull0 + 8 * (d.step % L::NA));
             d.wring.advance(d.nw);
             if (L::KS == 2 && nk == 2 && !kk) d.wring.advance(d.nw);
             ok = __all_sync(0xffffffffu, ok);
         } else if (L::KS == 2) {
             // (the step has no k-block for this group)
-            if (lane == 0) { mbar_arrive(d.bar_scfull + 8 * (d.step % L::nsc)); remote_arrive(d.afull0 + 8 * (d.step % L::NA)); }
+            remote_arrive_if(lane == 0, d.afull0 + 8 * (d.step % L::NA));
             d.wring.advance(d.nw);
         } else {
             d.wring.advance(d.nw);
@@ -392,7 +384,6 @@ __device__ __forceinline__ bool dequant_none(TcDequant& d, TcShared<TN>& sh, int
 #pragma unroll 1
     for (int kb = 0; ok && kb < nkb; kb += L::KS) {
         if (L::KS == 2 || L::dq_warps == 4 || (d.step & 1u) == d.my_group) {
-            if ((threadIdx.x & 31) == 0) mbar_arrive(d.bar_scfull + 8 * (d.step % L::nsc));
             if (d.step >= L::NA) ok = __all_sync(0xffffffffu, warp_wait(d.bar_done + 8 * ((d.step - L::NA) % L::nx), (d.step - L::NA) / L::nx & 1u, &sh.abort, status));
             if ((threadIdx.x & 31) == 0) remote_arrive(d.afull0 + 8 * (d.step % L::NA));
         }
@@ -415,7 +406,7 @@ template <int TN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 1)
     qgemm_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap tmap) {
     using L = TcCfg<TN>;
-    constexpr int NH = L::NH, KS = L::KS, NX = L::nx, NA = L::NA, NSC = L::nsc, NACC = L::NACC;
+    constexpr int NH = L::NH, KS = L::KS, NX = L::nx, NA = L::NA, NACC = L::NACC;
     __shared__ TcShared<TN> sh;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);
@@ -430,7 +421,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
     const uint32_t bar_wfull = smem_u32(sh.bars), bar_wempty = bar_wfull + 8 * TC_NW_MAX;
     const uint32_t bar_xfull = bar_wempty + 8 * TC_NW_MAX, bar_done = bar_xfull + 8 * NX;
     const uint32_t bar_afull = bar_done + 8 * NX;
-    const uint32_t bar_accfull = bar_afull + 8 * NA, bar_accempty = bar_accfull + 16 * NACC, bar_scfull = bar_accempty + 8 * NACC, bar_xchg = bar_scfull + 8 * NSC;
+    const uint32_t bar_accfull = bar_afull + 8 * NA, bar_accempty = bar_accfull + 16 * NACC, bar_xchg = bar_accempty + 8 * NACC;
     volatile int* s_abort = &sh.abort;
 
     // ---- prologue: nothing here depends on the previous kernel in the stream
@@ -440,7 +431,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         for (int i = 0; i < NA; ++i) mbar_init(bar_afull + 8 * i, 2 * L::dq_arrive);
         for (int i = 0; i < 2 * NACC; ++i) mbar_init(bar_accfull + 8 * i, 1);
         for (int i = 0; i < NACC; ++i) mbar_init(bar_accempty + 8 * i, 2 * TC_EPI);
-        for (int i = 0; i < NSC; ++i) mbar_init(bar_scfull + 8 * i, L::dq_arrive);
         if (KS == 2)
             for (int i = 0; i < 2 * TC_EPI; ++i) mbar_init(bar_xchg + 8 * i, 1);
         *s_abort = 0;
@@ -512,7 +502,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
 
     if (warp < 4) {
         if constexpr (TN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
-        else asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
         if (warp == 0 || warp == 3) {
             // ---------------- X producers: this CTA's XR token rows of every half tile, KS x 128 k per stage ----------------
             // Both warps walk the stages and arrive on the pair's xfull barrier; warp 0 also adds the byte count of the TMA
@@ -535,7 +525,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             auto arrive = [&]() {
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) remote_arrive(full0 + 8 * (due % NX));
+                remote_arrive_if(lane == 0, full0 + 8 * (due % NX));
                 ++due;
             };
             while (ok && wk.next(sc, p, nclusters, pc)) {
@@ -674,14 +664,52 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 int kb0 = pc.kb0;
                 const uint32_t idesc0 = umma_idesc_pair(half_cols<L::HC>(pc.rows, 0)), idesc1 = KS == 2 ? idesc0 : umma_idesc_pair(half_cols<L::HC>(pc.rows, nh - 1));
                 // eight MMAs: one k-block (xd: its token rows, at: its weights) into the accumulator at d
-                auto mma_kblock = [&](uint32_t d, uint32_t at, uint64_t xd, uint32_t idesc) {
+                auto mma_kblock = [&](uint32_t d, uint32_t at, uint64_t xd, uint32_t idesc, uint32_t add = 0u) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) umma_pair_ts(d, at + 8 * i, xd + (i >> 2) * (L::XR * 8) + (i & 3) * 2, idesc, i > 0 ? 1u : 0u);
+                    for (int i = 0; i < 8; ++i) umma_pair_ts(d, at + 8 * i, xd + (i >> 2) * (L::XR * 8) + (i & 3) * 2, idesc, i > 0 ? 1u : add);
                 };
-                if (!keep && steps == 8 && (KS == 2 || nh == 2)) {
-                    // two buffers a step (the common grouped formats): this warp's instructions are on the critical path of
-                    // every step, so there are as few of them as can be
-                    const uint32_t xd0 = sbase, at0 = tmem_base + L::a_base;
+                // This warp's instructions are on the critical path of every step (the tensor core runs dry while it waits, votes
+                // and commits), so the loops of the common formats hold as few of them as can be (8192 rows x 4096 x 4096, per
+                // channel: 211 -> 194 us against one loop for every format).
+                const uint32_t xd0 = sbase, at0 = tmem_base + L::a_base;
+                if (keep) {
+                    const int b1 = buf + 1 == NACC ? 0 : buf + 1;
+                    const uint32_t ph1 = b1 == 0 ? buf_phase ^ 1u : buf_phase;
+                    const uint32_t d0 = tmem_base + buf * L::HC, d1 = tmem_base + b1 * L::HC;
+                    ok = warp_wait(bar_accempty + 8 * buf, buf_phase, s_abort, p.status);
+                    if (nh == 2) ok &= warp_wait(bar_accempty + 8 * b1, ph1, s_abort, p.status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    uint32_t add = 0u;
+#pragma unroll 1
+                    for (; ok && kb0 < pc.kb1; kb0 += KS, ++step) {
+                        const uint32_t st = step % NX;
+                        ok = warp_wait(bar_xfull + 8 * st, step / NX & 1u, s_abort, p.status);
+                        ok &= warp_wait(bar_afull + 8 * (step % NA), step / NA & 1u, s_abort, p.status);
+                        tc_fence_after();
+                        const uint64_t xd = umma_desc_sw128(xd0 + st * L::xstage);
+                        const uint32_t at = at0 + (step % NA) * (KS * TC_A_COLS);
+                        const bool two = KS == 2 ? kb0 + 1 < pc.kb1 : nh == 2;
+                        if (elect_one()) {
+                            mma_kblock(d0, at, xd, idesc0, add);
+                            if (two) {
+                                if (KS == 2) mma_kblock(d0, at + TC_A_COLS, xd + L::xhalf / 16, idesc0, 1u);
+                                else mma_kblock(d1, at, xd + L::xhalf / 16, idesc1, add);
+                            }
+                            umma_commit_pair(bar_done + 8 * st);
+                        }
+                        add = 1u;
+                        ok = __all_sync(0xffffffffu, ok);
+                    }
+                    if (ok && elect_one()) {
+                        umma_commit_pair(bar_accfull + 8 * buf);
+                        if (nh == 2) umma_commit_pair(bar_accfull + 8 * (NACC + b1));
+                    }
+                    __syncwarp();
+                    for (int h = 0; h < nh; ++h) next_buf();
+                    continue;
+                }
+                if (steps == 8 && (KS == 2 || nh == 2)) {
+                    // two buffers a step
 #pragma unroll 1
                     for (; ok && kb0 + KS <= pc.kb1; kb0 += KS, ++step) {
                         const uint32_t st = step % NX;
@@ -720,6 +748,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                         ok = __all_sync(0xffffffffu, ok);
                     }
                 }
+                if (KS == 1 && steps == 8 && nh == 1) {
+                    // one buffer a step
+#pragma unroll 1
+                    for (; ok && kb0 < pc.kb1; ++kb0, ++step) {
+                        const uint32_t st = step % NX;
+                        ok = warp_wait(bar_xfull + 8 * st, step / NX & 1u, s_abort, p.status);
+                        ok &= warp_wait(bar_afull + 8 * (step % NA), step / NA & 1u, s_abort, p.status);
+                        ok &= warp_wait(bar_accempty + 8 * buf, buf_phase, s_abort, p.status);
+                        tc_fence_after();
+                        const uint64_t xd = umma_desc_sw128(xd0 + st * L::xstage);
+                        if (elect_one()) {
+                            mma_kblock(tmem_base + buf * L::HC, at0 + (step % NA) * (KS * TC_A_COLS), xd, idesc0);
+                            umma_commit_pair(bar_done + 8 * st);
+                        }
+                        next_buf();
+                        ok = __all_sync(0xffffffffu, ok);
+                    }
+                }
+                // groups narrower than 128 k, and the odd k-block of a step of two
                 for (; ok && kb0 < pc.kb1; kb0 += KS) {
                     const int nk = min(KS, pc.kb1 - kb0);
                     ok = warp_wait(bar_xfull + 8 * (step % NX), step / NX & 1u, s_abort, p.status);
@@ -738,27 +785,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                         const uint64_t bdesc = xdesc + u * (L::xhalf / 16);
                         const bool last = u + 1 == nu;
                         if (steps == 8) {
-                            const int b2 = keep && h ? (buf + 1 == NACC ? 0 : buf + 1) : buf;
-                            const uint32_t ph = keep && h && buf + 1 == NACC ? buf_phase ^ 1u : buf_phase;
-                            const uint32_t add = keep && kb0 + kk > pc.kb0 ? 1u : 0u;
-                            if (!add) {
-                                ok &= warp_wait(bar_accempty + 8 * b2, ph, s_abort, p.status);
-                                tc_fence_after();
-                            }
-                            const uint32_t d = tmem_base + b2 * L::HC;
+                            ok &= warp_wait(bar_accempty + 8 * buf, buf_phase, s_abort, p.status);
+                            tc_fence_after();
                             if (elect_one()) {
-#pragma unroll
-                                for (int i = 0; i < 8; ++i)
-                                    umma_pair_ts(d, a_tmem + 8 * i, bdesc + (i >> 2) * (L::XR * 8) + (i & 3) * 2, idesc, i > 0 ? 1u : add);
-                                if (keep) {
-                                    if (last) umma_commit_pair(done);
-                                    if (kb0 + kk + 1 == pc.kb1) umma_commit_pair(bar_accfull + 8 * (h * NACC + b2));
-                                } else {
-                                    umma_commit_pair(last ? done : bar_accfull + 8 * (u * NACC + b2));
-                                }
+                                mma_kblock(tmem_base + buf * L::HC, a_tmem, bdesc, idesc);
+                                umma_commit_pair(last ? done : bar_accfull + 8 * (u * NACC + buf));
                             }
                             __syncwarp();
-                            if (!keep) next_buf();
+                            next_buf();
                         } else {
 #pragma unroll 1
                             for (int i0 = 0; i0 < 8; i0 += steps) {
@@ -783,15 +817,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                     ok = __all_sync(0xffffffffu, ok);
                     ++step;
                 }
-                if (keep) for (int h = 0; h < nh; ++h) next_buf();
             }
         }
     } else if (warp < L::epi_warp0) {
         if constexpr (TN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
-        else asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         // ---------------- dequant warps: thread = channel = TMEM lane ----------------
         TcDequant d;
-        d.bar_wfull = bar_wfull; d.bar_wempty = bar_wempty; d.bar_done = bar_done; d.bar_scfull = bar_scfull;
+        d.bar_wfull = bar_wfull; d.bar_wempty = bar_wempty; d.bar_done = bar_done;
         d.afull0 = mapa(bar_afull, 0);
         d.row = (warp & 3) * 32 + lane;
         d.lane_tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + L::a_base;
@@ -813,15 +846,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             if (has_zeros && ex.group == 0) z = __bfloat162float(ex.zeros_pc[nt * 128 + d.row]);
             const uint32_t zpc = neg_z(z);
             switch (ex.bits) {
-                case 4: ok = dequant_piece<TN, 4>(d, sh, wtiles, nkb, per, has_zeros, zpc, tile_zeros, p.status); break;
-                case 8: ok = dequant_piece<TN, 8>(d, sh, wtiles, nkb, per, has_zeros, zpc, tile_zeros, p.status); break;
-                case 3: ok = dequant_piece<TN, 3>(d, sh, wtiles, nkb, per, has_zeros, zpc, tile_zeros, p.status); break;
-                default: ok = dequant_piece<TN, 2>(d, sh, wtiles, nkb, per, has_zeros, zpc, tile_zeros, p.status); break;
+                case 4: ok = dequant_piece<TN, 4>(d, sh, wtiles, nkb, per, zpc, tile_zeros, p.status); break;
+                case 8: ok = dequant_piece<TN, 8>(d, sh, wtiles, nkb, per, zpc, tile_zeros, p.status); break;
+                case 3: ok = dequant_piece<TN, 3>(d, sh, wtiles, nkb, per, zpc, tile_zeros, p.status); break;
+                default: ok = dequant_piece<TN, 2>(d, sh, wtiles, nkb, per, zpc, tile_zeros, p.status); break;
             }
         }
     } else {
         if constexpr (TN == 256) asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
-        else asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
+        // (what the producers and the dequant warps can do without: with 120 the sums were spilled in every step; 96 rows x 4096 x
+        // 11008: 42 -> 38 us)
+        else asm volatile("setmaxnreg.inc.sync.aligned.u32 136;");
         // ---------------- epilogue warps: scale-and-accumulate, then store ----------------
         // Two groups of four warps.  Of a tile with two half tiles each group drains one, of a step with two k-blocks each
         // drains one (an accumulator buffer then costs a warp one wait for all its columns); otherwise both drain every
@@ -865,22 +900,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             const uint32_t freed = alone ? 2u : 1u;
             const int col0 = alone ? 0 : tok0;                 // first column drained, and how many hold a token
             const int dcol = KS == 2 ? pc.rows : ncol;
-            // waits for an accumulator buffer, adds it to the sums and hands it back; scl: the group's scale in shared memory
-            // (or nullptr: s_pc), complete once the step's scfull barrier is
-            auto drain = [&](uint32_t bar, uint32_t phase, int b, const __half* scl, bool wait_scales) {
+            // Scales come straight from the tiles in global memory (the packed tile has just been fetched, so they are in L2),
+            // two drains ahead of their use.  Handed on by the dequant warps through shared memory and a barrier of their own,
+            // they cost both roles some 200 cycles a k-block.
+            const int mg = ex.has_zeros ? 512 : 256, round = KS * ex.tile_stride;
+            const unsigned char* meta = ex.tiles + ((size_t)(active ? nt : 0) * p.KB + pc.kb0) * ex.tile_stride + moqe_tile_bytes(ex.bits) + row * 2;
+            const int off_end = (nkb - 1) * ex.tile_stride + (per - 1) * mg;
+            int off = min(KS == 2 ? eg * ex.tile_stride : 0, (nkb - 1) * ex.tile_stride), oj = 0;
+            auto fetch_scale = [&]() { return keep ? (unsigned short)0 : __ldg(reinterpret_cast<const unsigned short*>(meta + off)); };
+            auto next_scale = [&](bool one) {                      // one: a group to a k-block
+                if (one) off = min(off + round, off_end);
+                else {
+                    const bool wrap = ++oj == per;
+                    off = min(off + (wrap ? round - (per - 1) * mg : mg), off_end);
+                    oj = wrap ? 0 : oj;
+                }
+            };
+            unsigned short s_now = fetch_scale();                  // (as loaded: converting waits for the load)
+            next_scale(per == 1);
+            unsigned short s_next = fetch_scale();
+            // waits for an accumulator buffer, adds it to the sums and hands it back
+            auto drain = [&](auto chunks, bool one, uint32_t bar, uint32_t phase, int b) {
                 ok &= warp_wait(bar, phase, s_abort, p.status);
                 tc_fence_after();
                 const uint32_t src = lane_tmem + b * L::HC + col0;
                 float sv = s_pc;
 #pragma unroll
                 for (int c = 0; c < L::DC / 32; ++c) {
-                    if (32 * c < dcol) {
+                    if (decltype(chunks)::value > 0 ? c < decltype(chunks)::value : 32 * c < dcol) {
                         uint32_t v[32];
                         tmem_ld32(src + 32 * c, v);
-                        if (c == 0 && scl) {
-                            // (fetched while the load is under way)
-                            if (wait_scales) ok &= warp_wait(bar_scfull + 8 * (step % NSC), step / NSC & 1u, s_abort, p.status);
-                            sv = __half2float(*scl) * W8_PRESCALE;
+                        if (c == 0) {
+                            // (while the load is under way)
+                            if (one || !keep) sv = __half2float(__ushort_as_half(s_now)) * W8_PRESCALE;
+                            s_now = s_next;
+                            next_scale(one);
+                            s_next = fetch_scale();
                         }
                         tmem_ld_wait();
                         fma_cols32(acc + 32 * c, v, sv);
@@ -888,7 +943,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) remote_arrive(accempty0 + 8 * b, freed);
+                remote_arrive_if(lane == 0, accempty0 + 8 * b, freed);
             };
             int left = nkb;
             if (!keep && per == 1) {
@@ -896,17 +951,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 // instruction through every nine cycles or so and nothing else of the epilogue runs in parallel
                 const bool by_done = !alone || eg == 1;
                 const int mine = alone ? eg : 0, uses = alone ? 2 : 1;
+                auto steps = [&](auto chunks) {
 #pragma unroll 1
-                for (; ok && left >= KS; left -= KS) {
-                    int ob = buf + mine;
-                    if (ob >= NACC) ob -= NACC;
-                    drain(by_done ? bar_done + 8 * (step % NX) : bar_accfull + 8 * ob, by_done ? step / NX & 1u : (full_phase >> ob) & 1u, ob,
-                          &sh.scales[step % NSC][KS == 2 ? eg : 0][0][row], true);
-                    if (alone) full_phase ^= 1u << buf;
-                    buf += uses;
-                    if (buf >= NACC) buf -= NACC;
-                    ++step;
-                    ok = __all_sync(0xffffffffu, ok);
+                    for (; ok && left >= KS; left -= KS) {
+                        int ob = buf + mine;
+                        if (ob >= NACC) ob -= NACC;
+                        drain(chunks, true, by_done ? bar_done + 8 * (step % NX) : bar_accfull + 8 * ob, by_done ? step / NX & 1u : (full_phase >> ob) & 1u, ob);
+                        if (alone) full_phase ^= 1u << buf;
+                        buf += uses;
+                        if (buf >= NACC) buf -= NACC;
+                        ++step;
+                        ok = __all_sync(0xffffffffu, ok);
+                    }
+                };
+                if constexpr (TN == 256) {
+                    // The number of 32-column chunks is fixed at compile time: no branch between them, and the loads of a chunk
+                    // start before the sums of the last are done (16384 x 11008 x 4096, three LLaMA experts: 1430 -> 1395
+                    // us).  The smaller tiles, with one or two chunks, are faster with the branches (38.3 against 39.0).
+                    const int nch = (dcol + 31) >> 5;
+                    if (nch <= 1) steps(std::integral_constant<int, 1>{});
+                    else if (nch == 2) steps(std::integral_constant<int, 2>{});
+                    else if (nch == 3) steps(std::integral_constant<int, 3>{});
+                    else steps(std::integral_constant<int, 4>{});
+                } else {
+                    steps(std::integral_constant<int, 0>{});
                 }
             }
             // The rest: one round per step (every group's buffer is drained, the last one of the step being announced by the
@@ -918,12 +986,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 const int nu = KS == 2 ? (keep ? 1 : min(KS, left)) : nh;
 #pragma unroll 1
                 for (int t = 0; t < nu * per; ++t) {
-                    const int u = t >= per ? 1 : 0, j = t - u * per;
+                    const int u = t >= per ? 1 : 0;
                     const bool by_done = !keep && t + 1 == nu * per;
                     const int fb = u * NACC + buf;
                     if (!alone || u == eg)
-                        drain(by_done ? bar_done + 8 * (step % NX) : bar_accfull + 8 * fb, by_done ? step / NX & 1u : (full_phase >> fb) & 1u, buf,
-                              keep ? nullptr : &sh.scales[step % NSC][KS == 2 ? u : 0][j][row], j == 0);
+                        drain(std::integral_constant<int, 0>{}, false, by_done ? bar_done + 8 * (step % NX) : bar_accfull + 8 * fb, by_done ? step / NX & 1u : (full_phase >> fb) & 1u, buf);
                     if (!by_done) full_phase ^= 1u << fb;
                     if (++buf == NACC) buf = 0;
                 }
@@ -942,12 +1009,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
 #pragma unroll
                 for (int i = 0; i < 32; ++i) out[i * 32] = eg ? acc[i] : acc[i + 32];
                 __syncwarp();
-                if (lane == 0) mbar_arrive(xfull + 8 * ew);
+                mbar_arrive_if(lane == 0, xfull + 8 * ew);
                 ok &= warp_wait(xfull + 8 * (ew ^ 4), xphase, s_abort, p.status);
 #pragma unroll
                 for (int i = 0; i < 32; ++i) acc[i] = (eg ? acc[i + 32] : acc[i]) + in[i * 32];
                 __syncwarp();
-                if (lane == 0) mbar_arrive(xempty + 8 * (ew ^ 4));
+                mbar_arrive_if(lane == 0, xempty + 8 * (ew ^ 4));
                 xphase ^= 1u;
                 ok = __all_sync(0xffffffffu, ok);
             }
