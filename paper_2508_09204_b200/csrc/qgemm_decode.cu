@@ -815,13 +815,16 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
             constexpr int NG = decltype(tag)::ng;
             GvConst kc;
             kc.template init<BITS>();
+            bool good = true;
             const uint32_t xb0 = sbase + L::x_off + buf * GV_XBUF + lane * 16;
             const float4* sS = reinterpret_cast<const float4*>(smem + L::s_off + buf * L::sbuf) + t;
             const uint32_t blob_off = blob * (BITS * 256);
             const uint32_t meta_off = moqe_tile_bytes(BITS) + (blob * 16 + g) * 2;
 #pragma unroll 1
             for (int kbl = 0; kbl < nkb; ++kbl) {
-                if (!__all_sync(0xffffffffu, mbar_wait_short(bar_wfull + 8 * ring.stage, ring.phase, s_abort, p.status))) { ok = false; return; }
+                // (the outcome is voted on once a chunk: a vote after every wait costs as much again as the wait)
+                good &= mbar_wait_short(bar_wfull + 8 * ring.stage, ring.phase, s_abort, p.status);
+                __syncwarp();
                 if (NG > 1) {
                     if constexpr (NG > 1) {
                         const uint32_t tile = tile_base + ring.stage * stage_bytes;
@@ -832,11 +835,14 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                     float acc[NT][4], S0[NT][2];
 #pragma unroll
                     for (int tb = 0; tb < NT; ++tb) {
-                        const float4 sv = sS[(kbl * NT + tb) * 4];
-                        acc[tb][0] = acc[tb][2] = sv.x;
-                        acc[tb][1] = acc[tb][3] = sv.y;
-                        S0[tb][0] = sv.z;
-                        S0[tb][1] = sv.w;
+                        const float2 start = *reinterpret_cast<const float2*>(sS + (kbl * NT + tb) * 4);
+                        acc[tb][0] = acc[tb][2] = start.x;
+                        acc[tb][1] = acc[tb][3] = start.y;
+                        if constexpr (ASYM) {
+                            const float2 s = *(reinterpret_cast<const float2*>(sS + (kbl * NT + tb) * 4) + 1);
+                            S0[tb][0] = s.x;
+                            S0[tb][1] = s.y;
+                        }
                     }
                     float s0 = sc[0], s8 = sc[1], z0 = z[0], z8 = z[1];
                     if constexpr (GROUPED) {
@@ -866,9 +872,10 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                     }
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar_wempty + 8 * ring.stage);
+                mbar_arrive_if(lane == 0, bar_wempty + 8 * ring.stage);
                 ring.advance(nstg);
             }
+            ok = __all_sync(0xffffffffu, good);
         };
 
         // One piece, for a number of token blocks fixed at compile time: all its chunks, then the result.  The sums live in

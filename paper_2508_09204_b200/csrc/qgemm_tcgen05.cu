@@ -121,9 +121,6 @@ __device__ __forceinline__ void remote_arrive(uint32_t cluster_addr, uint32_t co
 }
 // One lane of a warp arrives.  Predicated: as a branch of one lane each of these cost the warp 100 cycles and more, several
 // times a k-block (see dequant_piece).
-__device__ __forceinline__ void mbar_arrive_if(bool yes, uint32_t bar) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"((uint32_t)yes) : "memory");
-}
 __device__ __forceinline__ void remote_arrive_if(bool yes, uint32_t cluster_addr, uint32_t count = 1) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p mbarrier.arrive.shared::cluster.b64 _, [%0], %1;\n\t}"
                  ::"r"(cluster_addr), "r"(count), "r"((uint32_t)yes) : "memory");
