@@ -276,8 +276,8 @@ __global__ void encode_pack_kernel(const float* __restrict__ W, const uint8_t* _
 // (wider groups take K1a and K1b above).  Bound by the fp32 weights' bytes, which are read from HBM once: a warp holds
 // the 16 channels x 128 k of a blob in registers between finding the groups' extremes and rounding.  A per-channel
 // expert's block goes over its 16 rows twice, the second time out of L2 (16 rows are 256 KB at K = 4096).  Every byte of
-// the tiles is written here, padding included.  11008 x 4096, 4-bit g128: 63 us (the two kernels: 92 + 60); three blocks
-// to an SM (two: 68 us, four: 65).
+// the tiles is written here, padding included.  11008 x 4096, 4-bit g128: 57 us (the two kernels: 92 + 60); three blocks
+// to an SM (four: 54 us, but 3-bit g64 68 instead of 65; the loads through shared memory, a half piece ahead: 69).
 // ---------------------------------------------------------------------------
 // rint(w / s) as IEEE division and rounding give it, from a multiplication by 1 / s.  The product is off by at most
 // 2^-22 of its size; only where it comes that close to the middle between two integers does the division decide.
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(256, 3) quantize_pack_kernel(const float* __re
                                                             uint8_t* __restrict__ tiles, __half* __restrict__ scales_pc,
                                                             __nv_bfloat16* __restrict__ zeros_pc) {
     constexpr int L = (1 << BITS) - 1, half_code = 1 << (BITS - 1), qmax = half_code - 1;
-    __shared__ float s_ext[8][3][16];
+    __shared__ float s_ext[8][2][16];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nt = blockIdx.x >> 3, nb = blockIdx.x & 7;
     const int q = lane >> 3, r = (lane & 7) ^ (2 * q);                  // this lane's slot: piece (q, r) of both halves
@@ -433,9 +433,34 @@ __global__ void __launch_bounds__(256, 3) quantize_pack_kernel(const float* __re
     }
 }
 
+// canonical [N][G] fp16 scales / zero-points out of the per-tile (or per-channel) device copies, by one thread each
+struct MetaExport {
+    const __half* scales_pc;
+    const __nv_bfloat16* zeros_pc;
+    uint16_t *scales_out, *zeros_out;       // either may be nullptr
+    int G, group, sym;
+};
+__device__ __forceinline__ void meta_export(const uint8_t* tiles, const MetaExport& x, int N, int KB, int bits, long long i) {
+    if (i >= (long long)N * x.G) return;
+    const int n = (int)(i / x.G), gi = (int)(i % x.G);
+    MetaSlot m = meta_slot(const_cast<uint8_t*>(tiles), const_cast<__half*>(x.scales_pc), const_cast<__nv_bfloat16*>(x.zeros_pc), bits,
+                           x.group, !x.sym, KB, n, gi, 0);
+    if (x.scales_out) x.scales_out[i] = __half_as_ushort(*m.s);
+    if (x.zeros_out) {
+        const float z = x.sym ? (float)(1 << (bits - 1)) : __bfloat162float(*m.z);
+        x.zeros_out[i] = __half_as_ushort(__float2half_rn(z));
+    }
+}
+
+// The codes' blocks first, then those of the scales and zero-points (11008 x 4096, 4-bit g128: 14.7 us for the codes, and 5.7
+// and a launch for a kernel of 1400 blocks that waits on scattered loads; together 17.7).
 template <int BITS>
 __global__ void unpack_kernel(const uint8_t* __restrict__ tiles, int N, int K, int KB, int tile_stride,
-                              uint8_t* __restrict__ canon, long long npieces) {
+                              uint8_t* __restrict__ canon, long long npieces, unsigned code_blocks, const MetaExport x) {
+    if (blockIdx.x >= code_blocks) {
+        meta_export(tiles, x, N, KB, BITS, (long long)(blockIdx.x - code_blocks) * blockDim.x + threadIdx.x);
+        return;
+    }
     long long pid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (pid >= npieces) return;
     PieceCoord pc = piece_coord(pid, KB);
@@ -455,22 +480,7 @@ __global__ void unpack_kernel(const uint8_t* __restrict__ tiles, int N, int K, i
     }
 }
 
-// canonical [N][G] fp16 scales / zero-points  <->  the per-tile (or per-channel) device copies
-__global__ void meta_export_kernel(const uint8_t* __restrict__ tiles, const __half* __restrict__ scales_pc,
-                                   const __nv_bfloat16* __restrict__ zeros_pc, int N, int G, int KB, int bits, int group, int sym,
-                                   uint16_t* __restrict__ scales_out, uint16_t* __restrict__ zeros_out) {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)N * G) return;
-    int n = (int)(i / G), gi = (int)(i % G);
-    MetaSlot m = meta_slot(const_cast<uint8_t*>(tiles), const_cast<__half*>(scales_pc), const_cast<__nv_bfloat16*>(zeros_pc), bits,
-                           group, !sym, KB, n, gi, 0);
-    if (scales_out) scales_out[i] = __half_as_ushort(*m.s);
-    if (zeros_out) {
-        float z = sym ? (float)(1 << (bits - 1)) : __bfloat162float(*m.z);
-        zeros_out[i] = __half_as_ushort(__float2half_rn(z));
-    }
-}
-
+// canonical [N][G] fp16 scales / zero-points -> the per-tile (or per-channel) device copies
 __global__ void meta_import_kernel(const uint16_t* __restrict__ scales_in, const uint16_t* __restrict__ zeros_in, int N, int G,
                                    int KB, int bits, int group, int sym, uint8_t* __restrict__ tiles,
                                    __half* __restrict__ scales_pc, __nv_bfloat16* __restrict__ zeros_pc) {
@@ -568,9 +578,9 @@ moqe_status alloc_expert(int N, int K, int bits, int group, int sym, bool clear,
 
 moqe_status launch_quantize(const moqe_expert* e, const float* W, cudaStream_t st) {
     const int KB = e->Kp / 128, strips = e->Np / 16;
-    // a per-channel strip belongs to one block; grouped strips are cut along K until there are four blocks or so to an SM
-    int cuts = e->group == 0 ? 1 : 600 / strips + 1;
-    if (cuts > (KB + 7) / 8) cuts = (KB + 7) / 8;
+    // a per-channel strip belongs to one block; grouped strips are cut along K as far as they go, a k-block to a warp (so many
+    // small blocks leave no wave half empty: 63 -> 57 us for 688 strips)
+    const int cuts = e->group == 0 ? 1 : (KB + 7) / 8;
     const dim3 grid(strips, cuts);
 #define MOQE_QP(B) quantize_pack_kernel<B><<<grid, 256, 0, st>>>(W, e->N, e->K, e->group, e->sym, KB, e->tiles, e->scales_pc, e->zeros_pc)
     if (e->bits == 4) MOQE_QP(4);
@@ -660,23 +670,18 @@ extern "C" moqe_status moqe_expert_export(const moqe_expert* e, uint8_t* codes, 
                                           uint16_t* zeros_f16, void* stream) {
     if (!e) return MOQE_ERR_NULL;
     cudaStream_t st = (cudaStream_t)stream;
-    if (codes) {
-        if (reinterpret_cast<uintptr_t>(codes) % 8 != 0) return MOQE_ERR_UNSUPPORTED;
-        int KB = e->Kp / 128;
-        long long npieces = (long long)(e->Np / 128) * KB * 512;
-        unsigned blocks = (unsigned)((npieces + 127) / 128);
-        const int stride = moqe_tile_stride(e->bits, e->group, !e->sym);
-        if (e->bits == 4) unpack_kernel<4><<<blocks, 128, 0, st>>>(e->tiles, e->N, e->K, KB, stride, codes, npieces);
-        else if (e->bits == 8) unpack_kernel<8><<<blocks, 128, 0, st>>>(e->tiles, e->N, e->K, KB, stride, codes, npieces);
-        else if (e->bits == 2) unpack_kernel<2><<<blocks, 128, 0, st>>>(e->tiles, e->N, e->K, KB, stride, codes, npieces);
-        else unpack_kernel<3><<<blocks, 128, 0, st>>>(e->tiles, e->N, e->K, KB, stride, codes, npieces);
-        count_launch();
-    }
-    if (scales_f16 || zeros_f16) {
-        long long n = (long long)e->N * e->G;
-        meta_export_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(e->tiles, e->scales_pc, e->zeros_pc, e->N, e->G,
-                                                                        e->Kp / 128, e->bits, e->group, e->sym, scales_f16,
-                                                                        zeros_f16);
+    if (codes && reinterpret_cast<uintptr_t>(codes) % 8 != 0) return MOQE_ERR_UNSUPPORTED;
+    const int KB = e->Kp / 128, stride = moqe_tile_stride(e->bits, e->group, !e->sym);
+    const long long npieces = codes ? (long long)(e->Np / 128) * KB * 512 : 0;
+    const unsigned code_blocks = (unsigned)((npieces + 127) / 128);
+    const bool meta = scales_f16 || zeros_f16;
+    const unsigned blocks = code_blocks + (meta ? (unsigned)(((long long)e->N * e->G + 127) / 128) : 0u);
+    const MetaExport x = {e->scales_pc, e->zeros_pc, scales_f16, zeros_f16, e->G, e->group, e->sym};
+    if (blocks > 0) {
+        if (e->bits == 4) unpack_kernel<4><<<blocks, 128, 0, st>>>(e->tiles, e->N, e->K, KB, stride, codes, npieces, code_blocks, x);
+        else if (e->bits == 8) unpack_kernel<8><<<blocks, 128, 0, st>>>(e->tiles, e->N, e->K, KB, stride, codes, npieces, code_blocks, x);
+        else if (e->bits == 2) unpack_kernel<2><<<blocks, 128, 0, st>>>(e->tiles, e->N, e->K, KB, stride, codes, npieces, code_blocks, x);
+        else unpack_kernel<3><<<blocks, 128, 0, st>>>(e->tiles, e->N, e->K, KB, stride, codes, npieces, code_blocks, x);
         count_launch();
     }
     return cuda_ok(cudaGetLastError());
