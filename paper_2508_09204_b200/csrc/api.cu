@@ -95,9 +95,14 @@ int pick_kernel(int path, int M, const moqe_expert* const* ex, int E) {
     if (path == 0) {
         if (g_auto_decode && decode_supported(M, ex, E)) return 2;
         if (M <= AUTO_STREAM_MAX_ROWS && !(g_auto_decode && decode_supported_multi(1, ex, 1, E))) return 1;
-        // (the dense-weights GEMM streams or re-reads an expert's whole matrix per 128 rows; three experts, dense / grouped GEMM:
-        // 1024 -> 256 channels, 980 rows 27 / 21 us, 12544 rows 32 / 31; 256 -> 1024, 980 rows 31 / 11, 3920 rows 35 / 16)
-        const bool few = M < 12000 && (long long)ex[0]->N * ex[0]->K > 65536;
+        // The dense-weights GEMM streams or re-reads an expert's whole matrix per 128 rows, the grouped GEMM drains every group
+        // of 32 k by itself.  Dense / grouped, three experts of which one has groups of 32: 1024 -> 256 channels, 3920 rows
+        // 35 / 19 us, 12544 rows 37 / 41; 256 -> 1024, 12544 rows 39 / 31, 25088 rows 57 / 52, 50176 rows 75 / 92.  Two experts
+        // without such groups: 1024 -> 256, 12544 rows 35 / 26, 25088 rows 50 / 39; 256 -> 1024, 39 / 29, 55 / 46, 50176 rows
+        // 84 / 81.  (64 x 256 weights stay resident: dense from 3920 rows 14 / 11 to 12544 rows 14 / 19 on the better one.)
+        bool fine = false;
+        for (int e = 0; e < E; ++e) fine |= ex[e]->group == 32;
+        const bool few = M < (fine && ex[0]->K > ex[0]->N ? 12000 : 30000) && (long long)ex[0]->N * ex[0]->K > 65536;
         return (g_auto_dense && !few && dense_supported(M, ex[0]->N, ex[0]->K, ex, E)) ? 3 : 0;
     }
     return 0;
