@@ -219,6 +219,16 @@ struct TcWalk {
         return true;
     }
 };
+// Tokens of the first half tile, a multiple of 32: half of them, not as many as fit, so that the two epilogue groups have the
+// same work (512 rows over three experts, 171 to a tile: 96 + 75 instead of 128 + 43).
+template <int HC>
+__device__ __forceinline__ int half_split(int rows) { return rows <= HC ? HC : ((rows + 1) / 2 + 31) & ~31; }
+// MMA columns of half tile h of a tile with `rows` tokens
+template <int HC>
+__device__ __forceinline__ int half_cols(int rows, int h) {
+    const int hs = half_split<HC>(rows);
+    return (min(hs, rows - hs * h) + 31) & ~31;
+}
 // What a k-block of a tile costs, in units of 64 cycles (measured, every cluster busy): by tile size, rows of the tile and
 // quantization groups per k-block.
 template <int TN>
@@ -228,9 +238,6 @@ __device__ __forceinline__ int kblock_cost(int rows, int bits, int per) {
     if (TN == 128) return (per == 0 ? 16 : (per == 1 ? 18 : (per == 2 ? 32 : 57))) + wide / 2;
     return (rows <= 128 ? (per == 0 ? 18 : (per == 1 ? 23 : (per == 2 ? 39 : 68))) : (per == 0 ? 22 : (per == 1 ? 23 : (per == 2 ? 50 : 106)))) + wide / 2;
 }
-// MMA columns of half tile h of a tile with `rows` tokens
-template <int HC>
-__device__ __forceinline__ int half_cols(int rows, int h) { return (min(HC, rows - HC * h) + 31) & ~31; }
 
 // ---------------------------------------------------------------------------- unpacking
 __device__ __forceinline__ uint32_t fma_bf16x2(uint32_t a, uint32_t b, uint32_t c) {
@@ -535,7 +542,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                     src[h] = -1; cnt[h] = 0;
                     if (h < nh) {
                         const int per_cta = half_cols<L::HC>(pc.rows, h) >> 1;
-                        const int first_row = h * L::HC + (int)rank * per_cta;
+                        const int first_row = h * half_split<L::HC>(pc.rows) + (int)rank * per_cta;
                         const int c = max(min(per_cta, pc.rows - first_row), 0);         // real rows of this CTA
                         const int a = lane < c ? __ldcg(p.perm + pc.m0 + first_row + lane) : 0;
                         const int b = lane + 32 < c ? __ldcg(p.perm + pc.m0 + first_row + lane + 32) : 0;
@@ -878,8 +885,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             const bool active = nt < p.NT1;
             const int nh = NH == 1 ? 1 : (pc.rows > L::HC ? 2 : 1);
             // the columns this warp stores: ncol (may be <= 0) from token tok0 of the tile on
-            const int tok0 = nh == 2 ? eg * L::HC : eg * (L::HC / 2);
-            const int ncol = min(nh == 2 ? L::HC : L::HC / 2, pc.rows - tok0);
+            const int hs = nh == 2 ? half_split<L::HC>(pc.rows) : L::HC / 2;
+            const int tok0 = eg * hs, ncol = min(hs, pc.rows - tok0);
             __syncwarp();
 #pragma unroll
             for (int i = 0; i < L::EC / 32; ++i) {
