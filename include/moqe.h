@@ -79,8 +79,8 @@ typedef struct moqe_expert moqe_expert;
  *               z = clamp(rint(-lo/s), 0, 2^b-1), c = clamp(rint(w/s)+z, 0, 2^b-1)
  *   s == 0 or non-finite after the fp16 rounding -> s = 1;   dequant = s*(c-z).
  * W: device fp32 [N][K], finite.  bits in {2,3,4,8}; group 0, 32, 64 or a multiple
- * of 128, dividing K.  On success *out owns new device buffers (cudaMalloc'ed by
- * this call; it is therefore not capturable in a CUDA graph) and must be
+ * of 128, dividing K.  On success *out owns new device buffers (from a memory
+ * pool of the library, ordered on `stream`; the call is therefore not capturable in a CUDA graph) and must be
  * released with moqe_expert_destroy.  The kernels run on `stream`.
  * ------------------------------------------------------------------------- */
 MOQE_API moqe_status moqe_quantize_rtn(const float* W, int N, int K, int bits, int group, int sym,
@@ -107,7 +107,8 @@ MOQE_API moqe_status moqe_expert_import(int N, int K, int bits, int group, int s
 MOQE_API moqe_status moqe_expert_info(const moqe_expert* e, int* N, int* K, int* bits, int* group, int* sym,
                              size_t* code_bytes, size_t* meta_bytes, size_t* alloc_bytes);
 
-/* Frees the expert's device buffers (cudaFree: synchronises the device). */
+/* Gives the expert's device buffers back (synchronises the device).  The library's pool keeps up to 1 GB of freed
+ * expert memory per device for experts built later; the rest goes back to the device. */
 MOQE_API moqe_status moqe_expert_destroy(moqe_expert* e);
 
 /* ---------------------------------------------------------------------------
@@ -241,12 +242,12 @@ MOQE_API moqe_status moqe_router_load_report(const float* logits, const int32_t*
  * invalid id are written as zeros).  M == 0 is valid.  workspace:
  * moqe_routed_qgemm_workspace(M, N, K, E) bytes, contents irrelevant on entry;
  * calls that share a workspace must not overlap on the device.
- * Decode batches (at most 32 rows, experts per-channel or with groups of 128 k or more) stream each touched
- * expert's packed weights once through the decode kernel (bulk-copy ring, warp-level MMAs on fp16 operands,
+ * Decode batches (at most 32 rows) stream each touched expert's packed weights once through the decode kernel (bulk-copy ring, warp-level MMAs on fp16 operands,
  * stream-K split that follows the routing: experts without rows cost nothing).  That kernel converts the bf16
- * activations to fp16: values with |x| > 65504 are outside its domain (they become infinities); every other
- * kernel takes the whole bf16 range.  Other small batches take the split-K mma.sync streaming kernel; large
- * batches run the persistent tcgen05 grouped GEMM.
+ * activations to fp16: values with |x| > 65504 are outside its domain (they become infinities), unless one of the
+ * call's experts has groups narrower than 128 k (then rows are scaled block by block); every other kernel takes the
+ * whole bf16 range.  33 to 48 rows with such an expert take the split-K mma.sync streaming kernel; all other
+ * batches run the persistent tcgen05 grouped GEMM, or the dense-weights one on small layers.
  * ------------------------------------------------------------------------- */
 MOQE_API size_t moqe_routed_qgemm_workspace(int M, int N, int K, int E);
 MOQE_API moqe_status moqe_routed_qgemm(const void* X_bf16, const int32_t* row_ids, int M,
@@ -255,7 +256,7 @@ MOQE_API moqe_status moqe_routed_qgemm(const void* X_bf16, const int32_t* row_id
 
 /* Same, with the kernel chosen by the caller (testing / measurement):
  * path 0 = automatic, 1 = split-K dequant-MMA streaming kernel, 2 = tcgen05 grouped GEMM (automatic
- * token tile), 3 / 4 = tcgen05 grouped GEMM with 128- / 256-token tiles, 5 = decode kernel
+ * token tile), 3 / 4 = tcgen05 grouped GEMM with 128- / 256-token tiles, never split along K, 5 = decode kernel
  * (MOQE_ERR_UNSUPPORTED if the batch has more than 32 rows or an expert has groups narrower than 128 k),
  * 6 = dense-weights tcgen05 GEMM for large batches on small layers (more than 128 rows, K <= 1024, at most 1024
  * output channels; the automatic choice there: the layer is bound by its activations, so each expert's weights

@@ -17,8 +17,9 @@
 //
 //   Groups of 32 and 64 k (an instantiation of its own): the service warps sum the token values per group, and a consumer
 //   restarts its accumulators from them and scales once per group instead of once per k-block.  Against the streaming kernel,
-//   which took these formats before (W8, two W4-g128 and a W3-g64 expert; 8 / 24 rows): 3584 x 18944 67 / 75 -> 40 / 41 us,
-//   512 x 3584 12 / 16 -> 11 / 11 us.
+//   which took these formats before (W8, two W4-g128 and a W3-g64 expert; 8 / 24 rows): 3584 x 18944 67 / 75 -> 45 / 45 us,
+//   512 x 3584 12 / 16 -> 13 / 13 us.  That instantiation also takes the whole bf16 range: a row tile (128 values) is divided by
+//   a power of two that fits it into fp16, and the k-block's contribution multiplied by it (without that 41 / 42 us).
 //
 //   Unpacking costs 5 integer instructions per 8 four-bit codes (1 per 2 eight-bit codes, 23 per 32 three-bit
 //   codes, 10 per 16 two-bit codes): a masked code dropped into the mantissa of the fp16 number 1024 becomes 1024 + c, or 1024 + 16c
@@ -53,8 +54,8 @@ namespace moqe {
 namespace {
 
 constexpr int GV_CONS = 16;                                    // consumer warps
-constexpr int GV_SERV = 2;                                     // service warps
-constexpr int GV_THREADS = (GV_CONS + GV_SERV + 1) * 32;       // + the producer's warp
+__host__ __device__ constexpr int gv_serv(bool fine) { return fine ? 3 : 2; }                       // service warps
+__host__ __device__ constexpr int gv_threads(bool fine) { return (GV_CONS + gv_serv(fine) + 1) * 32; }   // + the producer's warp
 constexpr int GV_MAX_STAGES = 12;
 constexpr int GV_XCHG_BYTES = 8 * 8 * 32 * 4;                  // gated pairs: [8 blobs][8 values][32 lanes] floats
 constexpr int GV_XBUF = 32 * 1024;                             // one chunk of staged token rows
@@ -68,11 +69,11 @@ constexpr int GV_ALIGN = 5;                                    // super-tiles a 
 constexpr int GV_PREFETCH_TILES = 4;                           // super-tiles asked of L2 before the dependency wait
 
 // FUSED: the variant with gated pairs and residual adds (it gives 8 KB of the ring to the exchange buffer); FINE: the one
-// that also takes groups of 32 and 64 k (6 KB of the ring go to the sums of four groups to a k-block)
+// that also takes groups of 32 and 64 k (7 KB of the ring go to the sums of four groups to a k-block and the row scales)
 template <bool FUSED, bool FINE>
 struct GvSmem {
-    static constexpr int sbuf = GV_SBUF * (FINE ? GV_FINE : 1);
-    static constexpr int ring_bytes = (FUSED ? 150 : (FINE ? 152 : 158)) * 1024;
+    static constexpr int sbuf = FINE ? GV_SBUF * GV_FINE + GV_SBUF / 2 : GV_SBUF;     // (FINE: + the row tiles' scales [slab][8])
+    static constexpr int ring_bytes = (FUSED ? 150 : (FINE ? 151 : 158)) * 1024;
     static constexpr int ring_off = 0;
     static constexpr int x_off = ring_bytes;
     static constexpr int s_off = x_off + 2 * GV_XBUF;
@@ -338,7 +339,7 @@ __device__ __forceinline__ void tile_mma_wide(const GvConst& kc, uint32_t blob, 
 // and is scaled into the running sums when its 128 / NG values of k are done.  meta: the lane's first scale in the tile.
 template <int BITS, int NT, int NG>
 __device__ __forceinline__ void tile_mma_fine(const GvConst& kc, uint32_t blob, int slot16, uint32_t xb, const float4* sS, uint32_t meta,
-                                              bool zeros, float* fin) {
+                                              bool zeros, const float (&rs)[NT][2], float* fin) {
     constexpr int GS = 4 / NG;
     uint4 bh[NT > 2 ? 1 : NT][4];
     if constexpr (NT <= 2) {
@@ -377,10 +378,10 @@ __device__ __forceinline__ void tile_mma_fine(const GvConst& kc, uint32_t blob, 
         if (G % GS == GS - 1) {
 #pragma unroll
             for (int tb = 0; tb < NT; ++tb) {
-                fin[4 * tb + 0] = fmaf(s0, fmaf(-z0, S0[tb][0], acc[tb][0]), fin[4 * tb + 0]);
-                fin[4 * tb + 1] = fmaf(s0, fmaf(-z0, S0[tb][1], acc[tb][1]), fin[4 * tb + 1]);
-                fin[4 * tb + 2] = fmaf(s8, fmaf(-z8, S0[tb][0], acc[tb][2]), fin[4 * tb + 2]);
-                fin[4 * tb + 3] = fmaf(s8, fmaf(-z8, S0[tb][1], acc[tb][3]), fin[4 * tb + 3]);
+                fin[4 * tb + 0] = fmaf(rs[tb][0], s0 * fmaf(-z0, S0[tb][0], acc[tb][0]), fin[4 * tb + 0]);
+                fin[4 * tb + 1] = fmaf(rs[tb][1], s0 * fmaf(-z0, S0[tb][1], acc[tb][1]), fin[4 * tb + 1]);
+                fin[4 * tb + 2] = fmaf(rs[tb][0], s8 * fmaf(-z8, S0[tb][0], acc[tb][2]), fin[4 * tb + 2]);
+                fin[4 * tb + 3] = fmaf(rs[tb][1], s8 * fmaf(-z8, S0[tb][1], acc[tb][3]), fin[4 * tb + 3]);
             }
         }
     });
@@ -471,8 +472,9 @@ __device__ __forceinline__ void tile_mma(const GvConst& kc, uint32_t blob, int s
 // instantiation, so that the common one keeps its registers).  FINE: groups of 32 and 64 k are taken too (an instantiation of
 // its own, for the registers, the ring and the size of the code)
 template <bool FUSED, int NTMAX, bool FINE>
-__global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __grid_constant__ GvParams p) {
+__global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const __grid_constant__ GvParams p) {
     using L = GvSmem<FUSED, FINE>;
+    constexpr int GV_SERV = gv_serv(FINE);
     static_assert(NTMAX == 2 || (NTMAX == 4 && !FUSED), "gated pairs and residuals exist for batches of at most 16 rows");
     static_assert(!FINE || NTMAX == 4, "groups of 32 and 64 k: one instantiation for every batch size");
     const int slot_nt = FINE ? p.slot_nt : NTMAX;             // (a batch of at most 16 rows has the smaller workspace)
@@ -655,7 +657,7 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
         auto stage_units = [&](auto bits_tag) {
             // one 16-byte fetch (chunk a = 4G + q of the k-block: k = 32G + 8q ..) -> four fp16 pairs in MMA fragment order at
             // [slab][G][lane = 4 mm + q]; the pair sums go into the group's partial sums
-            auto convert = [&](const uint4& dat, int a, uint32_t xdst, float& S0, float& S1) {
+            auto convert = [&](const uint4& dat, int a, uint32_t xdst, float inv, float& S0, float& S1) {
                 const int G = a >> 2, q = a & 3;
                 const uint32_t w[4] = {dat.x, dat.y, dat.z, dat.w};
                 uint32_t o[4];
@@ -664,7 +666,8 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                     // pair p = 4G + j of the piece: scaled by sigma = 2^-e, e fixed by the format
                     constexpr int BITS = decltype(bits_tag)::value;
                     const int e = sigma_shift(BITS, 4 * G + j);
-                    const float lo = __uint_as_float(w[j] << 16), hi = __uint_as_float(w[j] & 0xFFFF0000u);
+                    float lo = __uint_as_float(w[j] << 16), hi = __uint_as_float(w[j] & 0xFFFF0000u);
+                    if constexpr (FINE) { lo *= inv; hi *= inv; }
                     const float sum = lo + hi;
                     S0 += sum;
                     S1 = fmaf(__int_as_float((127 - e) << 23), sum, S1);
@@ -688,6 +691,14 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                 const uint16_t* src = live && m < rows ? p.X[v] + (size_t)s_perm[row0 + m] * K + k0 : nullptr;
                 const uint32_t xdst = xbuf + (slab << 11) + (mm << 6);
                 float S0, S1;
+                // FINE: a row tile is divided by a power of two that brings its largest value to 2^14 .. 2^15, so that any bf16
+                // value fits (exactly, unless it is 2^-22 of the largest and below).  top: the largest magnitude's bits.
+                auto top_of = [&](uint32_t top, const uint4& d) {
+                    return __vmaxu2(__vmaxu2(top, __vmaxu2(d.x & 0x7FFF7FFFu, d.y & 0x7FFF7FFFu)), __vmaxu2(d.z & 0x7FFF7FFFu, d.w & 0x7FFF7FFFu));
+                };
+                auto exponent = [&](uint32_t top) { return min(268 - (int)(max(top & 0xFFFFu, top >> 16) >> 7), 253); };   // of 1 / the divisor
+                auto put_scale = [&](int ex) { sbuf[GV_SBUF * GV_FINE / 4 + slab * 8 + mm] = __int_as_float((254 - ex) << 23); };
+                float inv = 1.f;
                 if constexpr (PARTS == 4) {
                     uint4 data[4];
 #pragma unroll
@@ -696,10 +707,20 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                         data[i] = make_uint4(0, 0, 0, 0);
                         if (src != nullptr && k0 + a * 8 < K) data[i] = __ldg(reinterpret_cast<const uint4*>(src + a * 8));
                     }
+                    if constexpr (FINE) {
+                        uint32_t top = 0;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) top = top_of(top, data[i]);
+                        top = __vmaxu2(top, __shfl_xor_sync(0xffffffffu, top, 1));
+                        top = __vmaxu2(top, __shfl_xor_sync(0xffffffffu, top, 2));
+                        const int ex = exponent(top);
+                        inv = __int_as_float(ex << 23);
+                        if (live && part == 0) put_scale(ex);
+                    }
                     S0 = 0.f; S1 = 0.f;
                     if (live) {
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) convert(data[i], 4 * part + i, xdst, S0, S1);
+                        for (int i = 0; i < 4; ++i) convert(data[i], 4 * part + i, xdst, inv, S0, S1);
                     }
                     if (!FINE || ng < 4) {
                         S0 += __shfl_xor_sync(0xffffffffu, S0, 1);
@@ -719,6 +740,15 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                     }
                 } else {
                     float g0[4] = {0.f, 0.f, 0.f, 0.f}, g1[4] = {0.f, 0.f, 0.f, 0.f};
+                    if constexpr (FINE) {
+                        uint32_t top = 0;                          // (the loads below find their lines in L1)
+#pragma unroll
+                        for (int a = 0; a < 16; ++a)
+                            if (src != nullptr && k0 + a * 8 < K) top = top_of(top, __ldg(reinterpret_cast<const uint4*>(src + a * 8)));
+                        const int ex = exponent(top);
+                        inv = __int_as_float(ex << 23);
+                        if (live) put_scale(ex);
+                    }
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         uint4 data[8];
@@ -730,7 +760,7 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                         }
                         if (live) {
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) convert(data[i], 8 * h + i, xdst, g0[2 * h + (i >> 2)], g1[2 * h + (i >> 2)]);
+                            for (int i = 0; i < 8; ++i) convert(data[i], 8 * h + i, xdst, inv, g0[2 * h + (i >> 2)], g1[2 * h + (i >> 2)]);
                         }
                     }
                     S0 = (g0[0] + g0[1]) + (g0[2] + g0[3]);
@@ -851,10 +881,16 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                 // (the outcome is voted on once a chunk: a vote after every wait costs as much again as the wait)
                 good &= mbar_wait_short(bar_wfull + 8 * ring.stage, ring.phase, s_abort, p.status);
                 __syncwarp();
+                float rs[NT][2];                                  // FINE: what the row tiles were divided by
+                if constexpr (FINE) {
+                    const float2* T = reinterpret_cast<const float2*>(smem + L::s_off + buf * L::sbuf + GV_SBUF * GV_FINE) + kbl * NT * 4 + t;
+#pragma unroll
+                    for (int tb = 0; tb < NT; ++tb) { const float2 v2 = T[tb * 4]; rs[tb][0] = v2.x; rs[tb][1] = v2.y; }
+                }
                 if (NG > 1) {
                     if constexpr (NG > 1) {
                         const uint32_t tile = tile_base + ring.stage * stage_bytes;
-                        if (active) tile_mma_fine<BITS, NT, NG>(kc, tile + blob_off, slot16, xb0 + ((kbl * NT * 4) << 9), sS + kbl * NT * NG * 4, tile + meta_off, zeros, fin);
+                        if (active) tile_mma_fine<BITS, NT, NG>(kc, tile + blob_off, slot16, xb0 + ((kbl * NT * 4) << 9), sS + kbl * NT * NG * 4, tile + meta_off, zeros, rs, fin);
                     }
                 } else if (active) {
                     const uint32_t tile = tile_base + ring.stage * stage_bytes;
@@ -884,7 +920,13 @@ __global__ void __launch_bounds__(GV_THREADS, 1) qgemm_decode_kernel(const __gri
                     // the k-block is complete: scale and add
 #pragma unroll
                     for (int tb = 0; tb < NT; ++tb) {
-                        if constexpr (ASYM) {
+                        if constexpr (FINE) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const float u = ASYM ? fmaf(j < 2 ? -z0 : -z8, S0[tb][j & 1], acc[tb][j]) : acc[tb][j];
+                                fin[4 * tb + j] = fmaf(rs[tb][j & 1], (j < 2 ? s0 : s8) * u, fin[4 * tb + j]);
+                            }
+                        } else if constexpr (ASYM) {
                             fin[4 * tb + 0] = fmaf(s0, fmaf(-z0, S0[tb][0], acc[tb][0]), fin[4 * tb + 0]);
                             fin[4 * tb + 1] = fmaf(s0, fmaf(-z0, S0[tb][1], acc[tb][1]), fin[4 * tb + 1]);
                             fin[4 * tb + 2] = fmaf(s8, fmaf(-z8, S0[tb][0], acc[tb][2]), fin[4 * tb + 2]);
@@ -1185,7 +1227,7 @@ moqe_status launch_qgemm_decode_ext(const void* const* X, int M, int nl, const m
     cudaError_t err = ensure_dynamic_smem((const void*)kernel, smem, done) ? cudaSuccess : cudaErrorInvalidValue;
     if (err == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(grid); cfg.blockDim = dim3(GV_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+        cfg.gridDim = dim3(grid); cfg.blockDim = dim3(gv_threads(fine)); cfg.dynamicSmemBytes = smem; cfg.stream = st;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[0].val.programmaticStreamSerializationAllowed = 1;

@@ -28,3 +28,22 @@ def test_fine_groups(M, N, K, one):
         Y = moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), gpu)
         assert moqe.moqe_launch_count() > before and moqe.moqe_async_status() == moqe.OK
         assert_close(torch_to_bits(Y), oracle.routed_gemm(X, ids, What), f"fine M{M} N{N} K{K} {i}")
+
+
+def test_fine_groups_take_the_whole_bf16_range():
+    """Rows of 2^100, 2^-100 and ordinary size: the kernel multiplies fp16 tokens, so a row tile is divided by a power of two
+    first (batches with such experts took any bf16 value before this kernel did them)."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_close, bf16_to_torch, build_experts, dev, torch_to_bits
+    M, N, K = 24, 256, 2432
+    W = wl.weights_f32("fine/range", N, K)
+    gpu, What, _ = build_experts(W, [(3, 64, False), (4, 128, False), (8, 0, True)])
+    for e in (100, -100, 0):
+        X = torch.from_numpy(wl.activations_bf16("fine/range/X", M, K).view(np.int16)).view(torch.bfloat16)
+        X = torch_to_bits(X * 2.0 ** e)
+        ids = (np.arange(M) % 3).astype(np.int32)
+        Y = moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), gpu)
+        # (both sides are scaled back by the exact power of two before they are compared)
+        back = lambda bits: torch_to_bits(torch.from_numpy(np.ascontiguousarray(bits).view(np.int16)).view(torch.bfloat16) * 2.0 ** -e)
+        assert_close(back(torch_to_bits(Y)), back(oracle.routed_gemm(X, ids, What)), f"rows of 2^{e}")
+    assert moqe.moqe_async_status() == moqe.OK
