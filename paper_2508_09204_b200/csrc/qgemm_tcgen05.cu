@@ -369,7 +369,9 @@ __device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, co
             if (L::KS == 2 && nk == 2 && !kk) d.wring.advance(d.nw);
             ok = __all_sync(0xffffffffu, ok);
         } else if (L::KS == 2) {
-            // (the step has no k-block for this group)
+            // The step has no k-block for this group.  Its arrivals wait for the step NA ago like everyone's: earlier ones would
+            // complete that step's phase in the place of a warp of the other group that has yet to store its weights.
+            if (d.step >= L::NA) ok = __all_sync(0xffffffffu, warp_wait(d.bar_done + 8 * ((d.step - L::NA) % L::nx), (d.step - L::NA) / L::nx & 1u, &sh.abort, status));
             remote_arrive_if(lane == 0, d.afull0 + 8 * (d.step % L::NA));
             d.wring.advance(d.nw);
         } else {

@@ -61,3 +61,18 @@ def test_pair_kernel_split_is_deterministic_and_clears_its_counters():
     assert_close(first, oracle.routed_gemm(X, ids, What), "split")
     for _ in range(3):
         assert np.array_equal(_run(X, ids, gpu, 2), first)
+
+
+@pytest.mark.parametrize("M,N,K", [(192, 19200, 64), (192, 19200, 128), (96, 9600, 640), (48, 6000, 1152)])
+def test_steps_of_one_k_block(M, N, K):
+    """64-token tiles take two k-blocks a step; here every step, or the last of every piece, has one, and a cluster has several
+    tiles or pieces in a row: the dequant group without a k-block must not run ahead of the other.  Same bits every time."""
+    from gpu_helpers import build_experts, assert_close
+    W = wl.weights_f32(f"pair/{N}/{K}", N, K)
+    X = wl.activations_bf16(f"pair/{M}/{K}", M, K)
+    gpu, What, _ = build_experts(W, [(4, 64, False), (8, 0, True), (3, 0, False)])
+    ids = (np.arange(M) % 3).astype(np.int32)
+    first = _run(X, ids, gpu, 2)
+    assert_close(first, oracle.routed_gemm(X, ids, What), f"odd steps M{M} N{N} K{K}")
+    for _ in range(30):
+        assert np.array_equal(_run(X, ids, gpu, 2), first)
