@@ -17,9 +17,14 @@
 //
 //   Groups of 32 and 64 k (an instantiation of its own): the service warps sum the token values per group, and a consumer
 //   restarts its accumulators from them and scales once per group instead of once per k-block.  Against the streaming kernel,
-//   which took these formats before (W8, two W4-g128 and a W3-g64 expert; 8 / 24 rows): 3584 x 18944 67 / 75 -> 45 / 45 us,
-//   512 x 3584 12 / 16 -> 13 / 13 us.  That instantiation also takes the whole bf16 range: a row tile (128 values) is divided by
-//   a power of two that fits it into fp16, and the k-block's contribution multiplied by it (without that 41 / 42 us).
+//   which took these formats before (W8, two W4-g128 and a W3-g64 expert; 8 / 24 rows): 3584 x 18944 69 / 77 -> 47 / 48 us,
+//   512 x 3584 12.6 / 16.0 -> 13.0 / 13.0 us.  That instantiation also takes the whole bf16 range: a row tile (128 values) is
+//   divided by a power of two that fits it into fp16, and the k-block's contribution multiplied by it (without that 4 to 6 us
+//   less).  And it is at least as exact as the streaming kernel, whose 2- to 4-bit codes carry an offset of 128 (see below) and
+//   whose 8-bit codes none: its codes sit higher in the mantissa (see HIGH), for an offset of at most 64 or, with 3 bits, 128,
+//   and 8-bit codes lose theirs before the MMA.  2048 x 4096, 24 rows, outputs that are not the bf16 number nearest to the exact
+//   sum, streaming / here / with the offsets of the other instantiations: W8-pc 0.02 / 0.01 / 0.43 %, W4-g64 0.20 / 0.05 / 1.04,
+//   W3-g64 0.37 / 0.11 / 1.39, W2-g64 0.92 / 0.12 / 4.8.  (3584 x 18944 with those offsets: 45 / 46 us.)
 //
 //   Unpacking costs 5 integer instructions per 8 four-bit codes (1 per 2 eight-bit codes, 23 per 32 three-bit
 //   codes, 10 per 16 two-bit codes): a masked code dropped into the mantissa of the fp16 number 1024 becomes 1024 + c, or 1024 + 16c
@@ -28,7 +33,7 @@
 //   contribute is removed in fp32 with per-(token, k-block) sums of the token values:
 //     Y[m][n] = sum_G s[n][G] * ( sum_{k in G} A[n][k] * B[m][k]  -  1024 * S1[m][G]  -  z[n][G] * S0[m][G] )
 //   A = 1024 + c / sigma_k,  B = sigma_k * x,  S1 = sum sigma_k x,  S0 = sum x.  All products are exact
-//   (11-bit x 8-bit significands).  bf16 token values beyond the fp16 range (|x| > 65504) are outside the
+//   (11-bit x 8-bit significands); the sums are rounded at the size of 1024 * sigma_k in units of a code.  bf16 token values beyond the fp16 range (|x| > 65504) are outside the
 //   kernel's domain: they turn into infinities.
 //
 // Work split ("stream-K" over super-tiles, cut at the ends of segments where that costs little): the super-tiles of every (layer, expert) pair whose expert received
@@ -178,25 +183,31 @@ __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, ui
 // Constants of the unpacking, held in registers the compiler cannot see through: (v & mask) | 0x64006400 is ONE
 // three-input logic instruction when mask and constant are registers, two when they are immediates.
 struct GvConst {
-    uint32_t base, m4lo, m4hi, m3a, m3b, m3c, m3s0, m3s1, m3s2, m2a, m2b, m2c;
+    uint32_t base, m4lo, m4hi, m3a, m3b, m3c, m3s0, m3s1, m3s2, m2a, m2b, m2c, m8;
     // only the constants of one code width are set (and live) at a time
-    template <int BITS>
+    template <int BITS, bool HIGH>
     __device__ __forceinline__ void init() {
         asm volatile("mov.u32 %0, 0x64006400;" : "=r"(base));
         if constexpr (BITS == 4) {
-            asm volatile("mov.u32 %0, 0x000F000F;" : "=r"(m4lo));
+            if constexpr (!HIGH) asm volatile("mov.u32 %0, 0x000F000F;" : "=r"(m4lo));
             asm volatile("mov.u32 %0, 0x00F000F0;" : "=r"(m4hi));
         } else if constexpr (BITS == 3) {
-            asm volatile("mov.u32 %0, 0x00070007;" : "=r"(m3a));
+            if constexpr (!HIGH) asm volatile("mov.u32 %0, 0x00070007;" : "=r"(m3a));
             asm volatile("mov.u32 %0, 0x00380038;" : "=r"(m3b));
             asm volatile("mov.u32 %0, 0x01C001C0;" : "=r"(m3c));
             asm volatile("mov.u32 %0, 0x00400040;" : "=r"(m3s0));
             asm volatile("mov.u32 %0, 0x00800080;" : "=r"(m3s1));
             asm volatile("mov.u32 %0, 0x01000100;" : "=r"(m3s2));
+        } else if constexpr (BITS == 2 && HIGH) {
+            asm volatile("mov.u32 %0, 0x00300030;" : "=r"(m2a));
+            asm volatile("mov.u32 %0, 0x00C000C0;" : "=r"(m2b));
+            asm volatile("mov.u32 %0, 0x03000300;" : "=r"(m2c));
         } else if constexpr (BITS == 2) {
             asm volatile("mov.u32 %0, 0x00030003;" : "=r"(m2a));
             asm volatile("mov.u32 %0, 0x000C000C;" : "=r"(m2b));
             asm volatile("mov.u32 %0, 0x00300030;" : "=r"(m2c));
+        } else if constexpr (HIGH) {
+            asm volatile("mov.u32 %0, 0xE480E480;" : "=r"(m8));       // -1152
         }
     }
 };
@@ -207,8 +218,20 @@ __device__ __forceinline__ uint32_t and_or(uint32_t v, uint32_t mask, uint32_t c
     return d;
 }
 
-// pairs 0..3 of one 4-bit word (8 consecutive k): {1024 + c, 1024 + 16c, 1024 + c, 1024 + 16c}
+// HIGH: the variant with less to be cancelled (see the head of this file): no code sits lower than needed for an offset of at
+// most 64 (4- and 2-bit) or 128 (3-bit codes) in units of a code, and 8-bit codes lose theirs before the MMA.  Two more shifts
+// per 8 four-bit codes, four more per 32 three-bit codes, none for two-bit codes, one addition per pair of 8-bit codes.
+
+// pairs 0..3 of one 4-bit word (8 consecutive k): {1024 + c, 1024 + 16c, 1024 + c, 1024 + 16c}; HIGH: 1024 + 16c
+template <bool HIGH>
 __device__ __forceinline__ void unpack_w4(const GvConst& k, uint32_t v, uint32_t (&o)[4]) {
+    if constexpr (HIGH) {
+        o[0] = and_or(v << 4, k.m4hi, k.base);
+        o[1] = and_or(v, k.m4hi, k.base);
+        o[2] = and_or(v >> 4, k.m4hi, k.base);
+        o[3] = and_or(v >> 8, k.m4hi, k.base);
+        return;
+    }
     o[0] = and_or(v, k.m4lo, k.base);
     o[1] = and_or(v, k.m4hi, k.base);
     const uint32_t u = v >> 8;
@@ -216,8 +239,22 @@ __device__ __forceinline__ void unpack_w4(const GvConst& k, uint32_t v, uint32_t
     o[3] = and_or(u, k.m4hi, k.base);
 }
 // the 8 pairs of one 2-bit word (two chunks; pair f is field f of both halfwords, at bits 2f): 1024 + {1, 4, 16} * c --
-// fields 0..2 straight from the word, 3..5 after a shift by 6, 6..7 after a shift by 12
+// fields 0..2 straight from the word, 3..5 after a shift by 6, 6..7 after a shift by 12; HIGH: {16, 64, 256} * c, fields 0..1
+// after a shift up by 4, 2..4 straight, 5..7 after a shift by 6
+template <bool HIGH>
 __device__ __forceinline__ void unpack_w2(const GvConst& k, uint32_t v, uint32_t (&o)[8]) {
+    if constexpr (HIGH) {
+        const uint32_t l = v << 4, h = v >> 6;
+        o[0] = and_or(l, k.m2a, k.base);
+        o[1] = and_or(l, k.m2b, k.base);
+        o[2] = and_or(v, k.m2a, k.base);
+        o[3] = and_or(v, k.m2b, k.base);
+        o[4] = and_or(v, k.m2c, k.base);
+        o[5] = and_or(h, k.m2a, k.base);
+        o[6] = and_or(h, k.m2b, k.base);
+        o[7] = and_or(h, k.m2c, k.base);
+        return;
+    }
     o[0] = and_or(v, k.m2a, k.base);
     o[1] = and_or(v, k.m2b, k.base);
     o[2] = and_or(v, k.m2c, k.base);
@@ -229,20 +266,36 @@ __device__ __forceinline__ void unpack_w2(const GvConst& k, uint32_t v, uint32_t
     o[6] = and_or(t, k.m2a, k.base);
     o[7] = and_or(t, k.m2b, k.base);
 }
-// pairs 0..3 of an 8-bit chunk held in two words: 1024 + c
-__device__ __forceinline__ void unpack_w8(uint32_t w0, uint32_t w1, uint32_t (&o)[4]) {
+// pairs 0..3 of an 8-bit chunk held in two words: 1024 + c; HIGH: c - 128
+template <bool HIGH>
+__device__ __forceinline__ void unpack_w8(const GvConst& k, uint32_t w0, uint32_t w1, uint32_t (&o)[4]) {
     o[0] = __byte_perm(w0, 0x64646464u, 0x4140u);
     o[1] = __byte_perm(w0, 0x64646464u, 0x4342u);
     o[2] = __byte_perm(w1, 0x64646464u, 0x4140u);
     o[3] = __byte_perm(w1, 0x64646464u, 0x4342u);
+    if constexpr (HIGH) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) asm("add.f16x2 %0, %0, %1;" : "+r"(o[i]) : "r"(k.m8));      // (exact)
+    }
 }
 // the 16 pairs of a 3-bit piece (words A, B, C): pair p < 15 is field p % 5 of word p / 5 -> 1024 + {1, 8, 64, 1, 8} * c;
-// pair 15 is spread over bit 15 / 31 of the three words -> 1024 + 64c
+// pair 15 is spread over bit 15 / 31 of the three words -> 1024 + 64c; HIGH: fields 0..4 -> 1024 + {8, 64, 64, 8, 64} * c
+template <bool HIGH>
 __device__ __forceinline__ void unpack_w3(const GvConst& k, uint32_t A, uint32_t B, uint32_t C, uint32_t (&o)[16]) {
     const uint32_t w[3] = {A, B, C};
     uint32_t s0 = 0;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
+        if constexpr (HIGH) {
+            const uint32_t l = w[i] << 3, h = w[i] >> 6;
+            if (i == 0) s0 = w[i] >> 9;
+            o[5 * i + 0] = and_or(l, k.m3b, k.base);
+            o[5 * i + 1] = and_or(l, k.m3c, k.base);
+            o[5 * i + 2] = and_or(w[i], k.m3c, k.base);
+            o[5 * i + 3] = and_or(h, k.m3b, k.base);
+            o[5 * i + 4] = and_or(h, k.m3c, k.base);
+            continue;
+        }
         const uint32_t u = w[i] >> 9;
         if (i == 0) s0 = u;
         o[5 * i + 0] = and_or(w[i], k.m3a, k.base);
@@ -257,8 +310,14 @@ __device__ __forceinline__ void unpack_w3(const GvConst& k, uint32_t A, uint32_t
     o[15] = r;
 }
 // log2 of 1 / sigma for pair p (0..15) of a piece: how far the code sits above the mantissa's unit
+template <bool HIGH>
 __device__ __forceinline__ int sigma_shift(int bits, int p) {
     if (bits == 8) return 0;
+    if (HIGH) {
+        if (bits == 4) return 4;
+        if (bits == 2) return (p & 7) < 2 ? 4 + 2 * (p & 7) : 4 + 2 * (((p & 7) - 2) % 3);
+        return p == 15 || (p % 5) % 3 != 0 ? 6 : 3;
+    }
     if (bits == 4) return (p & 1) ? 4 : 0;
     if (bits == 2) return (p & 7) < 6 ? 2 * ((p & 7) % 3) : 2 * ((p & 7) - 6);
     return p == 15 ? 6 : 3 * ((p % 5) % 3);
@@ -272,7 +331,7 @@ struct GvTag {
 
 // One tile's codes of one lane, unpacked 32 k at a time: step(G, row g pairs 0..3, row g + 8 pairs 0..3) for the 32-k groups
 // G = 0..3 in order.  `blob` is the shared-memory address of the warp's blob.
-template <int BITS, class Step>
+template <int BITS, bool HIGH, class Step>
 __device__ __forceinline__ void tile_steps(const GvConst& kc, uint32_t blob, int slot16, const Step& step) {
     if constexpr (BITS == 4) {
         const uint4 w0 = lds128(blob + slot16), w1 = lds128(blob + 512 + slot16);
@@ -280,8 +339,8 @@ __device__ __forceinline__ void tile_steps(const GvConst& kc, uint32_t blob, int
 #pragma unroll
         for (int G = 0; G < 4; ++G) {
             uint32_t ar[4], a8[4];
-            unpack_w4(kc, a0[G], ar);
-            unpack_w4(kc, a1[G], a8);
+            unpack_w4<HIGH>(kc, a0[G], ar);
+            unpack_w4<HIGH>(kc, a1[G], a8);
             step(G, ar[0], ar[1], ar[2], ar[3], a8[0], a8[1], a8[2], a8[3]);
         }
     } else if constexpr (BITS == 2) {
@@ -290,8 +349,8 @@ __device__ __forceinline__ void tile_steps(const GvConst& kc, uint32_t blob, int
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             uint32_t ar[8], a8[8];
-            unpack_w2(kc, a0[h], ar);
-            unpack_w2(kc, a1[h], a8);
+            unpack_w2<HIGH>(kc, a0[h], ar);
+            unpack_w2<HIGH>(kc, a1[h], a8);
 #pragma unroll
             for (int gg = 0; gg < 2; ++gg)
                 step(2 * h + gg, ar[4 * gg], ar[4 * gg + 1], ar[4 * gg + 2], ar[4 * gg + 3], a8[4 * gg], a8[4 * gg + 1], a8[4 * gg + 2], a8[4 * gg + 3]);
@@ -304,8 +363,8 @@ __device__ __forceinline__ void tile_steps(const GvConst& kc, uint32_t blob, int
 #pragma unroll
             for (int gg = 0; gg < 2; ++gg) {
                 uint32_t ar[4], a8[4];
-                unpack_w8(a0[2 * gg], a0[2 * gg + 1], ar);
-                unpack_w8(a1[2 * gg], a1[2 * gg + 1], a8);
+                unpack_w8<HIGH>(kc, a0[2 * gg], a0[2 * gg + 1], ar);
+                unpack_w8<HIGH>(kc, a1[2 * gg], a1[2 * gg + 1], a8);
                 step(2 * u + gg, ar[0], ar[1], ar[2], ar[3], a8[0], a8[1], a8[2], a8[3]);
             }
         }
@@ -313,8 +372,8 @@ __device__ __forceinline__ void tile_steps(const GvConst& kc, uint32_t blob, int
         const uint4 w0 = lds128(blob + slot16);
         const uint2 w1 = lds64(blob + 512 + (slot16 >> 1));
         uint32_t ar[16], a8[16];
-        unpack_w3(kc, w0.x, w0.y, w0.z, ar);
-        unpack_w3(kc, w0.w, w1.x, w1.y, a8);
+        unpack_w3<HIGH>(kc, w0.x, w0.y, w0.z, ar);
+        unpack_w3<HIGH>(kc, w0.w, w1.x, w1.y, a8);
 #pragma unroll
         for (int G = 0; G < 4; ++G)
             step(G, ar[4 * G], ar[4 * G + 1], ar[4 * G + 2], ar[4 * G + 3], a8[4 * G], a8[4 * G + 1], a8[4 * G + 2], a8[4 * G + 3]);
@@ -323,9 +382,9 @@ __device__ __forceinline__ void tile_steps(const GvConst& kc, uint32_t blob, int
 
 // The MMAs of one tile for more than two token blocks: the token fragments (`xb`: the lane's, of this k-block) are fetched
 // where they are used (holding them all would take 16 registers per block).
-template <int BITS, int NT>
+template <int BITS, int NT, bool HIGH>
 __device__ __forceinline__ void tile_mma_wide(const GvConst& kc, uint32_t blob, int slot16, uint32_t xb, float (&acc)[NT][4]) {
-    tile_steps<BITS>(kc, blob, slot16, [&](int G, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
+    tile_steps<BITS, HIGH>(kc, blob, slot16, [&](int G, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
 #pragma unroll
         for (int tb = 0; tb < NT; ++tb) {
             const uint4 b = lds128(xb + ((tb * 4 + G) << 9));
@@ -349,15 +408,15 @@ __device__ __forceinline__ void tile_mma_fine(const GvConst& kc, uint32_t blob, 
             for (int tb = 0; tb < NT; ++tb) bh[tb][G] = lds128(xb + ((tb * 4 + G) << 9));
     }
     float acc[NT][4], S0[NT][2], s0, s8, z0, z8;
-    tile_steps<BITS>(kc, blob, slot16, [&](int G, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
+    tile_steps<BITS, true>(kc, blob, slot16, [&](int G, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
         if (G % GS == 0) {
             const uint32_t m = meta + (G / GS) * (zeros ? 512 : 256);
             s0 = __half2float(__ushort_as_half((unsigned short)lds16(m)));
             s8 = __half2float(__ushort_as_half((unsigned short)lds16(m + 16)));
             // (without zero-points these read what follows in the stage and drop it: a branch costs more)
             const uint32_t y0 = lds16(m + 256) << 16, y8 = lds16(m + 256 + 16) << 16;
-            z0 = zeros ? __uint_as_float(y0) : 0.f;
-            z8 = zeros ? __uint_as_float(y8) : 0.f;
+            z0 = zeros ? __uint_as_float(y0) - (BITS == 8 ? 128.f : 0.f) : 0.f;
+            z8 = zeros ? __uint_as_float(y8) - (BITS == 8 ? 128.f : 0.f) : 0.f;
 #pragma unroll
             for (int tb = 0; tb < NT; ++tb) {
                 const float4 sv = sS[(tb * NG + G / GS) * 4];
@@ -388,11 +447,10 @@ __device__ __forceinline__ void tile_mma_fine(const GvConst& kc, uint32_t blob, 
 }
 
 // The MMAs of one tile for one lane.
-
-template <int BITS, int NT>
+template <int BITS, int NT, bool HIGH>
 __device__ __forceinline__ void tile_mma(const GvConst& kc, uint32_t blob, int slot16, uint32_t xb, float (&acc)[NT][4]) {
     if constexpr (NT > 2) {
-        tile_mma_wide<BITS, NT>(kc, blob, slot16, xb, acc);
+        tile_mma_wide<BITS, NT, HIGH>(kc, blob, slot16, xb, acc);
         return;
     }
     uint4 b[NT][4];
@@ -406,8 +464,8 @@ __device__ __forceinline__ void tile_mma(const GvConst& kc, uint32_t blob, int s
 #pragma unroll
         for (int G = 0; G < 4; ++G) {
             uint32_t ar[4], a8[4];
-            unpack_w4(kc, a0[G], ar);
-            unpack_w4(kc, a1[G], a8);
+            unpack_w4<HIGH>(kc, a0[G], ar);
+            unpack_w4<HIGH>(kc, a1[G], a8);
 #pragma unroll
             for (int tb = 0; tb < NT; ++tb) {
                 mma_f16(acc[tb], ar[0], a8[0], ar[1], a8[1], b[tb][G].x, b[tb][G].y);
@@ -421,8 +479,8 @@ __device__ __forceinline__ void tile_mma(const GvConst& kc, uint32_t blob, int s
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             uint32_t ar[8], a8[8];
-            unpack_w2(kc, a0[h], ar);
-            unpack_w2(kc, a1[h], a8);
+            unpack_w2<HIGH>(kc, a0[h], ar);
+            unpack_w2<HIGH>(kc, a1[h], a8);
 #pragma unroll
             for (int gg = 0; gg < 2; ++gg) {
 #pragma unroll
@@ -441,8 +499,8 @@ __device__ __forceinline__ void tile_mma(const GvConst& kc, uint32_t blob, int s
 #pragma unroll
             for (int gg = 0; gg < 2; ++gg) {
                 uint32_t ar[4], a8[4];
-                unpack_w8(a0[2 * gg], a0[2 * gg + 1], ar);
-                unpack_w8(a1[2 * gg], a1[2 * gg + 1], a8);
+                unpack_w8<HIGH>(kc, a0[2 * gg], a0[2 * gg + 1], ar);
+                unpack_w8<HIGH>(kc, a1[2 * gg], a1[2 * gg + 1], a8);
 #pragma unroll
                 for (int tb = 0; tb < NT; ++tb) {
                     mma_f16(acc[tb], ar[0], a8[0], ar[1], a8[1], b[tb][2 * u + gg].x, b[tb][2 * u + gg].y);
@@ -454,8 +512,8 @@ __device__ __forceinline__ void tile_mma(const GvConst& kc, uint32_t blob, int s
         const uint4 w0 = lds128(blob + slot16);
         const uint2 w1 = lds64(blob + 512 + (slot16 >> 1));
         uint32_t ar[16], a8[16];
-        unpack_w3(kc, w0.x, w0.y, w0.z, ar);
-        unpack_w3(kc, w0.w, w1.x, w1.y, a8);
+        unpack_w3<HIGH>(kc, w0.x, w0.y, w0.z, ar);
+        unpack_w3<HIGH>(kc, w0.w, w1.x, w1.y, a8);
 #pragma unroll
         for (int G = 0; G < 4; ++G) {
 #pragma unroll
@@ -653,6 +711,8 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
         const uint32_t xbuf = sbase + L::x_off + buf * GV_XBUF;
         float* sbuf = reinterpret_cast<float*>(smem + L::s_off + buf * L::sbuf);
         const int ng = FINE ? s_ps[v].ng : 1;
+        // what an accumulator starts from (FINE: 8-bit codes come without an offset, and less a symmetric zero-point)
+        auto start = [&](float S1, float S0) { return FINE && bits == 8 ? 0.f : fmaf(-1024.f, S1, -fold * S0); };
         // (the format's scale exponents are compile-time constants: one instantiation of the loop per code width)
         auto stage_units = [&](auto bits_tag) {
             // one 16-byte fetch (chunk a = 4G + q of the k-block: k = 32G + 8q ..) -> four fp16 pairs in MMA fragment order at
@@ -665,7 +725,7 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
                 for (int j = 0; j < 4; ++j) {
                     // pair p = 4G + j of the piece: scaled by sigma = 2^-e, e fixed by the format
                     constexpr int BITS = decltype(bits_tag)::value;
-                    const int e = sigma_shift(BITS, 4 * G + j);
+                    const int e = sigma_shift<FINE>(BITS, 4 * G + j);
                     float lo = __uint_as_float(w[j] << 16), hi = __uint_as_float(w[j] & 0xFFFF0000u);
                     if constexpr (FINE) { lo *= inv; hi *= inv; }
                     const float sum = lo + hi;
@@ -734,7 +794,7 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
                         // sums at [slab][group][t = mm / 2][4]
                         if (live && part % (4 / ng) == 0) {
                             float* S = sbuf + (slab * ng + part / (4 / ng)) * 16 + (mm >> 1) * 4 + (mm & 1);
-                            S[0] = fmaf(-1024.f, S1, -fold * S0);
+                            S[0] = start(S1, S0);
                             S[2] = S0;
                         }
                     }
@@ -773,7 +833,7 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
                                 if (i >= ng) break;
                                 const float a0 = ng == 1 ? S0 : (ng == 2 ? g0[(2 * i) & 3] + g0[(2 * i + 1) & 3] : g0[i]);
                                 const float a1 = ng == 1 ? S1 : (ng == 2 ? g1[(2 * i) & 3] + g1[(2 * i + 1) & 3] : g1[i]);
-                                S[16 * i] = fmaf(-1024.f, a1, -fold * a0);
+                                S[16 * i] = start(a1, a0);
                                 S[16 * i + 2] = a0;
                             }
                         }
@@ -782,7 +842,7 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
                 // sums at [slab][t = mm / 2][4]
                 if (!FINE && live && part == 0) {
                     float* S = sbuf + slab * 16 + (mm >> 1) * 4 + (mm & 1);
-                    S[0] = fmaf(-1024.f, S1, -fold * S0);              // what the accumulator starts from
+                    S[0] = start(S1, S0);
                     S[2] = S0;
                 }
             }
@@ -870,7 +930,7 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
             constexpr bool GROUPED = decltype(tag)::grouped, ASYM = decltype(tag)::asym;
             constexpr int NG = decltype(tag)::ng;
             GvConst kc;
-            kc.template init<BITS>();
+            kc.template init<BITS, FINE>();
             bool good = true;
             const uint32_t xb0 = sbase + L::x_off + buf * GV_XBUF + lane * 16;
             const float4* sS = reinterpret_cast<const float4*>(smem + L::s_off + buf * L::sbuf) + t;
@@ -916,7 +976,8 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
                             z8 = __uint_as_float(lds16(meta + 256 + 16) << 16);
                         }
                     }
-                    tile_mma<BITS, NT>(kc, tile + blob_off, slot16, xb0 + ((kbl * NT * 4) << 9), acc);
+                    if constexpr (FINE && ASYM && BITS == 8) { z0 -= 128.f; z8 -= 128.f; }
+                    tile_mma<BITS, NT, FINE>(kc, tile + blob_off, slot16, xb0 + ((kbl * NT * 4) << 9), acc);
                     // the k-block is complete: scale and add
 #pragma unroll
                     for (int tb = 0; tb < NT; ++tb) {

@@ -47,3 +47,24 @@ def test_fine_groups_take_the_whole_bf16_range():
         back = lambda bits: torch_to_bits(torch.from_numpy(np.ascontiguousarray(bits).view(np.int16)).view(torch.bfloat16) * 2.0 ** -e)
         assert_close(back(torch_to_bits(Y)), back(oracle.routed_gemm(X, ids, What)), f"rows of 2^{e}")
     assert moqe.moqe_async_status() == moqe.OK
+
+
+@pytest.mark.parametrize("bits,group,sym", [(8, 64, True), (8, 0, False), (4, 32, False), (4, 64, True), (4, 128, False), (3, 64, False), (3, 0, True),
+                                            (2, 32, True), (2, 0, False)])
+def test_sums_are_as_exact_as_the_streaming_kernels(bits, group, sym):
+    """Codes enter the MMA with an offset that is taken out of the fp32 sums again, and the sums' error goes with its size.
+    What shows of it is how many outputs are not the bf16 number nearest to the sum in 64 bits: no more than the streaming
+    kernel has, which takes the same batches (plus three standard deviations of the two counts)."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import bf16_to_torch, dev
+    M, N, K = 32, 2048, 3968
+    W = torch.from_numpy(wl.weights_f32("fine/exact", N, K)).to(dev())
+    X = bf16_to_torch(wl.activations_bf16("fine/exact/X", M, K))
+    experts = [moqe.moqe_quantize_rtn(W, bits, group, sym), moqe.moqe_quantize_rtn(W, 4, 64, False)]
+    ids = torch.zeros(M, dtype=torch.int32, device=dev())
+    c, s, z = (t.double() for t in moqe.moqe_expert_export(experts[0]))
+    What = ((c.view(N, s.shape[1], -1) - z[:, :, None]) * s[:, :, None]).view(N, K)
+    nearest = (X.double() @ What.T).to(torch.bfloat16)
+    off = [int((moqe.moqe_routed_qgemm(X, ids, experts, path=path) != nearest).sum()) for path in (moqe.PATH_AUTO, moqe.PATH_STREAM)]
+    assert moqe.moqe_async_status() == moqe.OK
+    assert off[0] <= off[1] + 3 * (off[0] + off[1]) ** 0.5, off
