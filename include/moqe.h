@@ -269,11 +269,12 @@ MOQE_API moqe_status moqe_routed_qgemm_path(const void* X_bf16, const int32_t* r
  * [E+1] as moqe_permute wrote them (device pointers; rows perm[offsets[E]..M) are
  * left untouched in Y).  One sort then serves every linear layer of a block,
  * since a sample keeps its expert through the whole model (Section 3.1).
- * The split-K arrival counters at the head of the workspace body must be zero on
- * entry -- clear them once with moqe_routed_qgemm_workspace_clear after
- * allocating the workspace (same M, N, K, E) -- and every call leaves them zero,
- * except a call that ended in MOQE_ERR_TIMEOUT (moqe_async_status): clear the
- * workspace again before it is reused after that.
+ * The workspace holds arrival counters, which must be zero on entry -- clear them once with
+ * moqe_routed_qgemm_workspace_clear after allocating the workspace (same M, N, K, E) -- and every call leaves them
+ * zero, whichever kernel it takes, except a call that ended in MOQE_ERR_TIMEOUT (moqe_async_status): clear the
+ * workspace again before it is reused after that.  So one workspace serves any calls of the same M, N, K and E,
+ * whatever their experts' formats and `path`; with more than 64 rows any calls of the same M and E, if it is as
+ * large as the largest of them asks for.
  * `path` as for moqe_routed_qgemm_path. */
 MOQE_API moqe_status moqe_routed_qgemm_sorted(const void* X_bf16, const int32_t* perm, const int32_t* offsets, int M,
                                               const moqe_expert* const* h_experts, int E, void* Y_bf16,

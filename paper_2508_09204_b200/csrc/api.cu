@@ -57,9 +57,16 @@ namespace {
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
+// The arrival counters of the split-K kernels have a region of their own (they share it: each leaves it zero) that no kernel
+// uses as scratch, so that any of them may follow any other on one workspace.  Above 64 rows its place and size depend on M and
+// E alone: one workspace then serves layers of any shape.
 struct WsLayout {
-    size_t perm, offsets, sort, body, total;
+    size_t perm, offsets, sort, counters, body, total;
 };
+size_t counter_bytes(int M, int Np) {
+    const size_t a = stream_zero_bytes(M, Np), b = decode_zero_bytes(M), c = tc_zero_bytes();
+    return align256(a > b ? (a > c ? a : c) : (b > c ? b : c));
+}
 
 WsLayout ws_layout(int M, int Np, int K, int E) {
     WsLayout w;
@@ -67,6 +74,7 @@ WsLayout ws_layout(int M, int Np, int K, int E) {
     w.perm = off;    off += align256((size_t)M * sizeof(int32_t) + 16);
     w.offsets = off; off += align256((MOQE_MAX_EXPERTS + 2) * sizeof(int32_t));
     w.sort = off;    off += align256(sort_workspace_bytes(M, E));
+    w.counters = off; off += counter_bytes(M, Np);
     w.body = off;
     size_t a = stream_workspace_bytes(M, Np, E), b = tc_workspace_bytes(M, K, E, Np), c = decode_workspace_bytes(M);
     const size_t d = dense_workspace_bytes(M, K, E, Np, (K + 127) / 128 * 128);
@@ -108,12 +116,6 @@ int pick_kernel(int path, int M, const moqe_expert* const* ex, int E) {
     return 0;
 }
 
-// the arrival counters at the head of the workspace body (all split-K kernels keep theirs there)
-size_t body_zero_bytes(int M, int Np) {
-    const size_t a = stream_zero_bytes(M, Np), b = decode_zero_bytes(M), c = tc_zero_bytes();
-    return a > b ? (a > c ? a : c) : (b > c ? b : c);
-}
-
 }  // namespace
 }  // namespace moqe
 
@@ -153,12 +155,15 @@ moqe_status single_layer_args(const void* X, const void* ids_or_perm, const void
 
 // the grouped product on sorted rows with the kernel `pick_kernel` chose
 moqe_status run_sorted(int kernel, int path, const void* X, int M, const moqe_expert* const* ex, int E, void* Y,
-                       const int32_t* perm, const int32_t* offsets, void* body, size_t body_bytes, cudaStream_t st) {
+                       const int32_t* perm, const int32_t* offsets, char* base, const WsLayout& w, cudaStream_t st) {
     const int N = ex[0]->N, K = ex[0]->K;
-    if (kernel == 2) return launch_qgemm_decode_multi(&X, M, 1, ex, E, &Y, perm, offsets, body, body_bytes, st);
-    if (kernel == 1) return launch_qgemm_stream(X, M, N, K, ex, E, Y, perm, offsets, body, body_bytes, st);
+    uint32_t* counters = (uint32_t*)(base + w.counters);
+    void* body = base + w.body;
+    const size_t body_bytes = w.total - w.body;
+    if (kernel == 2) return launch_qgemm_decode_multi(&X, M, 1, ex, E, &Y, perm, offsets, counters, body, body_bytes, st);
+    if (kernel == 1) return launch_qgemm_stream(X, M, N, K, ex, E, Y, perm, offsets, counters, body, body_bytes, st);
     if (kernel == 3) return launch_qgemm_dense(X, M, N, K, ex, E, Y, perm, offsets, body, body_bytes, st);
-    return launch_qgemm_tc(X, M, N, K, ex, E, Y, perm, offsets, body, body_bytes, path == 3 ? 128 : (path == 4 ? 256 : 0), st);
+    return launch_qgemm_tc(X, M, N, K, ex, E, Y, perm, offsets, counters, body, body_bytes, path == 3 ? 128 : (path == 4 ? 256 : 0), st);
 }
 }  // namespace
 
@@ -174,11 +179,11 @@ extern "C" moqe_status moqe_routed_qgemm_path(const void* X_bf16, const int32_t*
     char* base = (char*)workspace;
     int32_t* perm = (int32_t*)(base + w.perm);
     int32_t* offsets = (int32_t*)(base + w.offsets);
-    const size_t zero_bytes = kernel != 3 ? body_zero_bytes(M, h_experts[0]->Np) : 0;
-    s = launch_sort(row_ids, M, E, perm, offsets, base + w.sort, w.body - w.sort, base + w.body, zero_bytes, Y_bf16,
+    const size_t zero_bytes = kernel != 3 ? w.body - w.counters : 0;
+    s = launch_sort(row_ids, M, E, perm, offsets, base + w.sort, w.counters - w.sort, base + w.counters, zero_bytes, Y_bf16,
                     h_experts[0]->N, st);
     if (s != MOQE_OK) return s;
-    return run_sorted(kernel, path, X_bf16, M, h_experts, E, Y_bf16, perm, offsets, base + w.body, w.total - w.body, st);
+    return run_sorted(kernel, path, X_bf16, M, h_experts, E, Y_bf16, perm, offsets, base, w, st);
 }
 
 extern "C" moqe_status moqe_routed_qgemm_sorted(const void* X_bf16, const int32_t* perm, const int32_t* offsets, int M,
@@ -189,9 +194,7 @@ extern "C" moqe_status moqe_routed_qgemm_sorted(const void* X_bf16, const int32_
     bool done = false;
     moqe_status s = single_layer_args(X_bf16, perm, offsets, M, h_experts, E, Y_bf16, workspace, workspace_bytes, path, w, kernel, done);
     if (s != MOQE_OK || done) return s;
-    char* base = (char*)workspace;
-    return run_sorted(kernel, path, X_bf16, M, h_experts, E, Y_bf16, perm, offsets, base + w.body, w.total - w.body,
-                      (cudaStream_t)stream);
+    return run_sorted(kernel, path, X_bf16, M, h_experts, E, Y_bf16, perm, offsets, (char*)workspace, w, (cudaStream_t)stream);
 }
 
 extern "C" moqe_status moqe_routed_qgemm_sorted_multi(const void* const* h_X_bf16, const int32_t* perm, const int32_t* offsets,
@@ -216,14 +219,14 @@ extern "C" moqe_status moqe_routed_qgemm_sorted_multi(const void* const* h_X_bf1
     WsLayout w = ws_layout(M, h_experts[0]->Np, h_experts[0]->K, E);
     if (!workspace || workspace_bytes < w.total || (uintptr_t)workspace % 256) return MOQE_ERR_WORKSPACE;
     char* base = (char*)workspace;
-    return launch_qgemm_decode_multi(h_X_bf16, M, n_layers, h_experts, E, h_Y_bf16, perm, offsets, base + w.body,
-                             w.total - w.body, (cudaStream_t)stream);
+    return launch_qgemm_decode_multi(h_X_bf16, M, n_layers, h_experts, E, h_Y_bf16, perm, offsets, (uint32_t*)(base + w.counters),
+                                     base + w.body, w.total - w.body, (cudaStream_t)stream);
 }
 
 namespace {
 // shared argument checks of the decode-only fused entry points
 moqe_status fused_args(const void* X, const int32_t* perm, const int32_t* offsets, int M, const moqe_expert* const* ex, int E,
-                       const void* Y, void* workspace, size_t workspace_bytes, size_t& body, size_t& total) {
+                       const void* Y, void* workspace, size_t workspace_bytes, WsLayout& w) {
     if (!ex) return MOQE_ERR_NULL;
     if (E <= 0 || M < 0) return MOQE_ERR_SHAPE;
     if (E > MOQE_MAX_EXPERTS) return MOQE_ERR_UNSUPPORTED;
@@ -236,10 +239,8 @@ moqe_status fused_args(const void* X, const int32_t* perm, const int32_t* offset
     if (!X || !perm || !offsets || !Y) return MOQE_ERR_NULL;
     if (N % 8 != 0 || K % 8 != 0 || (uintptr_t)X % 16 || (uintptr_t)Y % 16) return MOQE_ERR_UNSUPPORTED;
     if (!decode_supported_multi(M, ex, 1, E)) return MOQE_ERR_UNSUPPORTED;
-    WsLayout w = ws_layout(M, ex[0]->Np, K, E);
+    w = ws_layout(M, ex[0]->Np, K, E);
     if (!workspace || workspace_bytes < w.total || (uintptr_t)workspace % 256) return MOQE_ERR_WORKSPACE;
-    body = w.body;
-    total = w.total;
     return MOQE_OK;
 }
 }  // namespace
@@ -248,24 +249,26 @@ extern "C" moqe_status moqe_routed_qgemm_sorted_gated(const void* X_bf16, const 
                                                       const moqe_expert* const* h_gate, const moqe_expert* const* h_up, int E,
                                                       void* Y_bf16, void* workspace, size_t workspace_bytes, void* stream) {
     if (!h_up) return MOQE_ERR_NULL;
-    size_t body = 0, total = 0;
-    moqe_status s = fused_args(X_bf16, perm, offsets, M, h_gate, E, Y_bf16, workspace, workspace_bytes, body, total);
+    WsLayout w;
+    moqe_status s = fused_args(X_bf16, perm, offsets, M, h_gate, E, Y_bf16, workspace, workspace_bytes, w);
     if (s != MOQE_OK || M == 0) return s;
     for (int e = 0; e < E; ++e)
         if (!h_up[e]) return MOQE_ERR_NULL;
-    return launch_qgemm_decode_ext(&X_bf16, M, 1, h_gate, h_up, E, &Y_bf16, nullptr, perm, offsets, (char*)workspace + body,
-                                   total - body, (cudaStream_t)stream);
+    char* base = (char*)workspace;
+    return launch_qgemm_decode_ext(&X_bf16, M, 1, h_gate, h_up, E, &Y_bf16, nullptr, perm, offsets, (uint32_t*)(base + w.counters),
+                                   base + w.body, w.total - w.body, (cudaStream_t)stream);
 }
 
 extern "C" moqe_status moqe_routed_qgemm_sorted_residual(const void* X_bf16, const int32_t* perm, const int32_t* offsets, int M,
                                                          const moqe_expert* const* h_experts, int E, const void* R_bf16,
                                                          void* Y_bf16, void* workspace, size_t workspace_bytes, void* stream) {
-    size_t body = 0, total = 0;
-    moqe_status s = fused_args(X_bf16, perm, offsets, M, h_experts, E, Y_bf16, workspace, workspace_bytes, body, total);
+    WsLayout w;
+    moqe_status s = fused_args(X_bf16, perm, offsets, M, h_experts, E, Y_bf16, workspace, workspace_bytes, w);
     if (s != MOQE_OK || M == 0) return s;
     if (!R_bf16) return MOQE_ERR_NULL;
+    char* base = (char*)workspace;
     return launch_qgemm_decode_ext(&X_bf16, M, 1, h_experts, nullptr, E, &Y_bf16, &R_bf16, perm, offsets,
-                                   (char*)workspace + body, total - body, (cudaStream_t)stream);
+                                   (uint32_t*)(base + w.counters), base + w.body, w.total - w.body, (cudaStream_t)stream);
 }
 
 extern "C" moqe_status moqe_routed_qgemm_workspace_clear(void* workspace, size_t workspace_bytes, int M, int N, int K,
@@ -274,9 +277,7 @@ extern "C" moqe_status moqe_routed_qgemm_workspace_clear(void* workspace, size_t
     const int Np = (N + 127) / 128 * 128;
     WsLayout w = ws_layout(M, Np, K, E);
     if (!workspace || workspace_bytes < w.total || (uintptr_t)workspace % 256) return MOQE_ERR_WORKSPACE;
-    size_t zb = body_zero_bytes(M, Np);
-    if (zb == 0) return MOQE_OK;
-    return cuda_ok(cudaMemsetAsync((char*)workspace + w.body, 0, zb, (cudaStream_t)stream));
+    return cuda_ok(cudaMemsetAsync((char*)workspace + w.counters, 0, w.body - w.counters, (cudaStream_t)stream));
 }
 
 extern "C" moqe_status moqe_routed_qgemm(const void* X_bf16, const int32_t* row_ids, int M,

@@ -111,10 +111,12 @@ size_t sort_workspace_bytes(int M, int E);
 moqe_status launch_gather(const void* X, const int32_t* perm, const int32_t* offsets_E, int M, int C, void* Xp,
                           cudaStream_t st);
 
+// The split-K kernels count arrivals in `counters` (*_zero_bytes of them; zero on entry, left zero) and park partial sums in `ws`
+// (*_workspace_bytes; contents irrelevant on entry).
 // qgemm_stream.cu
 size_t stream_workspace_bytes(int M, int Np, int E);
 moqe_status launch_qgemm_stream(const void* X, int M, int N, int K, const moqe_expert* const* ex, int E, void* Y,
-                                const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes,
+                                const int32_t* perm, const int32_t* offsets, uint32_t* counters, void* ws, size_t ws_bytes,
                                 cudaStream_t st);
 size_t stream_zero_bytes(int M, int Np);
 void stream_set_tile_cost(int bits, int cost);   // relative cost of one packed tile in the work split (measurement knob)
@@ -128,11 +130,12 @@ bool decode_supported(int M, const moqe_expert* const* ex, int E);   // one laye
 size_t decode_workspace_bytes(int M);
 size_t decode_zero_bytes(int M);
 moqe_status launch_qgemm_decode_multi(const void* const* X, int M, int nl, const moqe_expert* const* ex, int E,
-                                      void* const* Y, const int32_t* perm, const int32_t* offsets, void* ws,
+                                      void* const* Y, const int32_t* perm, const int32_t* offsets, uint32_t* counters, void* ws,
                                       size_t ws_bytes, cudaStream_t st);
 moqe_status launch_qgemm_decode_ext(const void* const* X, int M, int nl, const moqe_expert* const* ex,
                                     const moqe_expert* const* ex2, int E, void* const* Y, const void* const* R,
-                                    const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes, cudaStream_t st);
+                                    const int32_t* perm, const int32_t* offsets, uint32_t* counters, void* ws, size_t ws_bytes,
+                                    cudaStream_t st);
 void decode_set_tile_cost(int bits, int cost);   // relative cost of one super-tile in the work split, by code width
 
 // quantize.cu: a plain bf16 copy Wd[Np][2 Kp] (hi | lo halves) of a (small) expert and its per-channel output scale, for qgemm_dense.cu
@@ -149,7 +152,8 @@ moqe_status launch_qgemm_dense(const void* X, int M, int N, int K, const moqe_ex
 size_t tc_zero_bytes();
 size_t tc_workspace_bytes(int M, int K, int E, int Np);
 moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_expert* const* ex, int E, void* Y,
-                            const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes, int tile_tokens, cudaStream_t st);
+                            const int32_t* perm, const int32_t* offsets, uint32_t* counters, void* ws, size_t ws_bytes, int tile_tokens,
+                            cudaStream_t st);
 
 __device__ __forceinline__ void latch_status(int* status, int code) {
     if (status) atomicCAS(status, 0, code);

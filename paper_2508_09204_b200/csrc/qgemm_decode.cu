@@ -1220,21 +1220,22 @@ size_t decode_zero_bytes(int M) { return M > DECODE_MAX_ROWS ? 0 : (size_t)GV_MA
 
 size_t decode_workspace_bytes(int M) {
     if (M > DECODE_MAX_ROWS) return 0;
-    return (decode_zero_bytes(M) + 255) / 256 * 256 + (size_t)GV_MAX_GRID * 2 * gv_slot_floats(M > 16 ? 4 : 2) * sizeof(float);
+    return (size_t)GV_MAX_GRID * 2 * gv_slot_floats(M > 16 ? 4 : 2) * sizeof(float);
 }
 
 // nl layers that share the routing; ex[l * E + e] = expert e of layer l; X[l] / Y[l] the layer's input / output
 moqe_status launch_qgemm_decode_multi(const void* const* X, int M, int nl, const moqe_expert* const* ex, int E,
-                                    void* const* Y, const int32_t* perm, const int32_t* offsets, void* ws,
+                                    void* const* Y, const int32_t* perm, const int32_t* offsets, uint32_t* counters, void* ws,
                                     size_t ws_bytes, cudaStream_t st) {
-    return launch_qgemm_decode_ext(X, M, nl, ex, nullptr, E, Y, nullptr, perm, offsets, ws, ws_bytes, st);
+    return launch_qgemm_decode_ext(X, M, nl, ex, nullptr, E, Y, nullptr, perm, offsets, counters, ws, ws_bytes, st);
 }
 
 // ex2 (or nullptr): per (layer, expert) the second expert of a gated pair, Y = silu(X.W1^T) * (X.W2^T), or nullptr for a
 // plain layer; R (or nullptr): per layer a residual [M][N] added before the rounding, or nullptr
 moqe_status launch_qgemm_decode_ext(const void* const* X, int M, int nl, const moqe_expert* const* ex,
                                   const moqe_expert* const* ex2, int E, void* const* Y, const void* const* R,
-                                  const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes, cudaStream_t st) {
+                                  const int32_t* perm, const int32_t* offsets, uint32_t* counters, void* ws, size_t ws_bytes,
+                                  cudaStream_t st) {
     if (M == 0) return MOQE_OK;
     const bool fine = !decode_supported_multi(M, ex, nl, E);
     if (fine && (nl != 1 || ex2 || R || !decode_supported(M, ex, E))) return MOQE_ERR_UNSUPPORTED;
@@ -1266,8 +1267,8 @@ moqe_status launch_qgemm_decode_ext(const void* const* X, int M, int nl, const m
             p.zeros_pc2[v] = second ? second->zeros_pc : nullptr;
             p.Res[v] = R ? (const uint16_t*)R[l] : nullptr;
         }
-    p.counters = (uint32_t*)ws;
-    p.partials = (float*)((char*)ws + (decode_zero_bytes(M) + 255) / 256 * 256);
+    p.counters = counters;
+    p.partials = (float*)ws;
     p.perm = perm;
     p.offsets = offsets;
     p.M = M;

@@ -633,15 +633,14 @@ size_t stream_zero_bytes(int M, int Np) {
 }
 
 size_t stream_workspace_bytes(int M, int Np, int E) {
-    (void)E;
+    (void)Np; (void)E;
     if (M > SPLIT_MAX_ROWS) return 0;
-    size_t counters = (stream_zero_bytes(M, Np) + 255) / 256 * 256;
-    size_t partials = (size_t)MAX_GRID * 2 * MAX_CHUNKS_SPLIT * (8 * pick_ntmax(M)) * 128 * sizeof(float);
-    return counters + partials;
+    return (size_t)MAX_GRID * 2 * MAX_CHUNKS_SPLIT * (8 * pick_ntmax(M)) * 128 * sizeof(float);
 }
 
 moqe_status launch_qgemm_stream(const void* X, int M, int N, int K, const moqe_expert* const* ex, int E, void* Y,
-                                const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes, cudaStream_t st) {
+                                const int32_t* perm, const int32_t* offsets, uint32_t* counters, void* ws, size_t ws_bytes,
+                                cudaStream_t st) {
     if (M == 0) return MOQE_OK;
     StreamParams p;
     p.KB = ex[0]->Kp / 128;
@@ -684,8 +683,8 @@ moqe_status launch_qgemm_stream(const void* X, int M, int N, int K, const moqe_e
     p.partials = nullptr;
     if (s.split) {
         if (!ws || ws_bytes < stream_workspace_bytes(M, p.Np, E)) return MOQE_ERR_WORKSPACE;
-        p.counters = (uint32_t*)ws;
-        p.partials = (float*)((char*)ws + (stream_zero_bytes(M, p.Np) + 255) / 256 * 256);
+        p.counters = counters;
+        p.partials = (float*)ws;
     }
     const int nt = pick_ntmax(M);
     cudaError_t err = cudaSuccess;

@@ -1144,11 +1144,12 @@ size_t tc_zero_bytes() { return (size_t)TC_MAX_CLUSTERS * 2 * TC_EPI * sizeof(ui
 
 size_t tc_workspace_bytes(int M, int K, int E, int Np) {
     (void)K; (void)E; (void)Np;
-    return (tc_zero_bytes() + 255) / 256 * 256 + (size_t)TC_MAX_CLUSTERS * 4 * tc_cols(M) * 128 * sizeof(float);
+    return (size_t)TC_MAX_CLUSTERS * 4 * tc_cols(M) * 128 * sizeof(float);
 }
 
 moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_expert* const* ex, int E, void* Y,
-                            const int32_t* perm, const int32_t* offsets, void* ws, size_t ws_bytes, int tile_tokens, cudaStream_t st) {
+                            const int32_t* perm, const int32_t* offsets, uint32_t* counters, void* ws, size_t ws_bytes, int tile_tokens,
+                            cudaStream_t st) {
     if (M == 0) return MOQE_OK;
     if (!ws || ws_bytes < tc_workspace_bytes(M, K, E, ex[0]->Np)) return MOQE_ERR_WORKSPACE;
     EncodeTiledFn enc = encode_fn();
@@ -1178,8 +1179,8 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
         stride = p.ex[e].tile_stride > stride ? p.ex[e].tile_stride : stride;
     }
     p.perm = perm; p.offsets = offsets; p.X = (const uint16_t*)X; p.Y = (uint16_t*)Y; p.status = device_status_word();
-    p.counters = (uint32_t*)ws;
-    p.partials = (float*)((char*)ws + (tc_zero_bytes() + 255) / 256 * 256);
+    p.counters = counters;
+    p.partials = (float*)ws;
     p.M = M; p.N = N; p.K = K; p.KB = ex[0]->Kp / 128; p.E = E; p.NT1 = ex[0]->Np / 128; p.NTP = (p.NT1 + 1) / 2;
     p.cols = tc_cols(M);
     p.split = tile_tokens == 0 && p.KB <= 4096 ? 1 : 0;
