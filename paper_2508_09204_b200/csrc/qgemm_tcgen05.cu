@@ -44,6 +44,11 @@ constexpr int TC_MAX_CLUSTERS = 80;
 constexpr int TC_EPI = 8;                          // epilogue warps
 constexpr int TC_NW_MAX = 12;                      // packed-weight stages
 constexpr int TC_A_COLS = 64;                      // TMEM columns of one k-block of unpacked weights
+constexpr int TC_COST_MAX = 107;                   // of a k-block (kblock_cost)
+// Whether the split by k-blocks may work in 32 bits.  It multiplies costs by clusters, and splits at most one tile less than there
+// are clusters.
+constexpr bool tc_split_fits(int clusters, int KB) { return (long long)clusters * ((long long)(clusters - 1) * KB + 1) * TC_COST_MAX < 1ll << 31; }
+static_assert(tc_split_fits(74, 3715) && !tc_split_fits(74, 3768) && !tc_split_fits(TC_MAX_CLUSTERS, 4096), "74 * 73 * 3768 * 107 > 2^31");
 
 // TN: tokens of a tile.  256: the tensor core's 1024 cycles a k-block hide one dequant warpgroup's work; 128 and 64: small
 // batches, where unpacking is the critical role and gets two warpgroups.  With 64 tokens every hand-over between the roles
@@ -230,7 +235,7 @@ __device__ __forceinline__ int half_cols(int rows, int h) {
     return (min(hs, rows - hs * h) + 31) & ~31;
 }
 // What a k-block of a tile costs, in units of 64 cycles (measured, every cluster busy): by tile size, rows of the tile and
-// quantization groups per k-block.
+// quantization groups per k-block.  At most TC_COST_MAX.
 template <int TN>
 __device__ __forceinline__ int kblock_cost(int rows, int bits, int per) {
     const int wide = bits == 8 || bits == 3 ? 2 : 0;       // (the 8-bit tiles are larger, the 3-bit ones take longer to unpack)
@@ -477,7 +482,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         }
         const int us = min(max(Td - tile0, 0), T_e) * p.KB;
         const int cnt = T_e * p.KB - us;
-        const int cost = cnt * w;                          // (at most 80 tiles are split: the host keeps this within 32 bits)
+        const int cost = cnt * w;                          // (times the clusters within 32 bits: tc_split_fits)
         int cincl = cost;
         int wmax = cnt > 0 ? w : 1;
 #pragma unroll
@@ -1183,7 +1188,7 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
     p.partials = (float*)ws;
     p.M = M; p.N = N; p.K = K; p.KB = ex[0]->Kp / 128; p.E = E; p.NT1 = ex[0]->Np / 128; p.NTP = (p.NT1 + 1) / 2;
     p.cols = tc_cols(M);
-    p.split = tile_tokens == 0 && p.KB <= 4096 ? 1 : 0;
+    p.split = tile_tokens == 0 && tc_split_fits(clusters, p.KB) ? 1 : 0;
     auto launch = [&](auto kernel, int threads, int smem, int w_bytes, std::atomic<unsigned long long>& attr) -> bool {
         p.wstage = (stride + 127) / 128 * 128;
         p.nw = w_bytes / p.wstage < TC_NW_MAX ? w_bytes / p.wstage : TC_NW_MAX;
