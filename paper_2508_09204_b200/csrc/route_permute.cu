@@ -61,12 +61,14 @@ __global__ void expand_ids_kernel(const int32_t* __restrict__ ids, const int32_t
         if (row_offsets[mid] <= m0) lo = mid; else hi = mid;
     }
     int32_t v[4];
-    int next = lo + 1 < S ? row_offsets[lo + 1] : 0x7fffffff, id = ids[lo];
+    constexpr long long NONE = 1ll << 62;               // (no row comes after the last sample; row 2^31 - 1 is one of the last thread's)
+    long long next = lo + 1 < S ? row_offsets[lo + 1] : NONE;
+    int id = ids[lo];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         while (next <= m0 + i) {
             ++lo;
-            next = lo + 1 < S ? row_offsets[lo + 1] : 0x7fffffff;
+            next = lo + 1 < S ? row_offsets[lo + 1] : NONE;
             id = ids[lo];
         }
         v[i] = id;
@@ -415,7 +417,7 @@ extern "C" moqe_status moqe_expand_ids(const int32_t* ids, const int32_t* row_of
     if (!ids || !row_offsets || !row_ids) return MOQE_ERR_NULL;
     if (S < 0 || M < 0 || (S == 0 && M != 0)) return MOQE_ERR_SHAPE;
     if (M == 0) return MOQE_OK;
-    const cudaError_t err = launch_chained(expand_ids_kernel, (M + 1023) / 1024, 256, (cudaStream_t)stream, ids, row_offsets, S, M, row_ids);
+    const cudaError_t err = launch_chained(expand_ids_kernel, (unsigned)(((long long)M + 1023) / 1024), 256, (cudaStream_t)stream, ids, row_offsets, S, M, row_ids);
     count_launch();
     return cuda_ok(err);
 }

@@ -49,3 +49,16 @@ def test_router_sample_groups(S, H, D):
     # fp32 sums of at most 70 + 512 terms of size ~1: 1e-6 relative, a hundredth of the bound
     assert np.all(np.abs(lg.cpu().numpy().astype(np.float64) - ref) <= 1e-4 * (1.0 + np.abs(ref)))
     assert np.array_equal(ids.cpu().numpy(), oracle.route(lg.cpu().numpy()))
+
+
+@pytest.mark.parametrize("M", [2 ** 31 - 1, 2 ** 31 - 300])
+def test_expand_ids_at_the_largest_row_counts(M):
+    """The last thread's four rows reach past row 2^31 - 1, which no 32-bit row offset marks as the end."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import dev
+    off = torch.tensor([0, 5, 5, 2 ** 30, M], dtype=torch.int32, device=dev())
+    ids = torch.tensor([3, 9, 1, 2], dtype=torch.int32, device=dev())
+    rows = moqe.moqe_expand_ids(ids, off, M)
+    assert moqe.moqe_async_status() == moqe.OK
+    for lo, hi, want in ((0, 5, 3), (5, 2 ** 30, 1), (2 ** 30, M, 2)):
+        assert int(rows[lo:hi].min()) == want and int(rows[lo:hi].max()) == want
