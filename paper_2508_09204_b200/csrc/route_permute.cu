@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(SORT_THREADS) sort_scatter_kernel(const int32_
     }
 }
 
-// launch with programmatic dependence on the kernel before (see chain_begin)
+// launch with programmatic dependence on the kernel before (see chain_begin); an error is returned, not left behind
 template <typename... KArgs, typename... Args>
 cudaError_t launch_chained(void (*kernel)(KArgs...), unsigned blocks, unsigned threads, cudaStream_t st, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -320,7 +320,9 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), unsigned blocks, unsigned t
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+    if (err != cudaSuccess) cudaGetLastError();
+    return err;
 }
 
 // (1) to (3) for M > 1024; block_tot: room for ceil(M / 1024) * (E + 1) counts
@@ -336,7 +338,7 @@ moqe_status launch_big_sort(const int32_t* row_ids, int M, int E, int32_t* block
         err = launch_chained(sort_scatter_kernel<false>, nblk, SORT_THREADS, st, row_ids, M, E, block_tot, perm, offsets, Y_zero_invalid, N);
         count_launch(3);
     }
-    if (err != cudaSuccess) { cudaGetLastError(); return MOQE_ERR_CUDA; }
+    if (err != cudaSuccess) return MOQE_ERR_CUDA;
     return cuda_ok(cudaGetLastError());
 }
 

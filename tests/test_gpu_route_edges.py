@@ -62,3 +62,33 @@ def test_expand_ids_at_the_largest_row_counts(M):
     assert moqe.moqe_async_status() == moqe.OK
     for lo, hi, want in ((0, 5, 3), (5, 2 ** 30, 1), (2 ** 30, M, 2)):
         assert int(rows[lo:hi].min()) == want and int(rows[lo:hi].max()) == want
+
+
+def test_a_refused_launch_leaves_no_error_for_the_next_call():
+    """Launches into a capture that has become invalid are refused by the runtime on the host; calls after that are not."""
+    import ctypes
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import dev
+    rt = ctypes.CDLL("libcudart.so.12")
+    L, side = moqe.lib(), torch.cuda.Stream()
+    st = ctypes.c_void_p(side.cuda_stream)
+    logits = torch.zeros((4, 3), device=dev())
+    ids = torch.zeros(4, dtype=torch.int32, device=dev())
+    off = torch.arange(5, dtype=torch.int32, device=dev())
+    rows, perm = torch.empty_like(ids), torch.empty_like(ids)
+    Y = torch.zeros((4, 8), dtype=torch.bfloat16, device=dev())
+    order = torch.arange(4, dtype=torch.int32, device=dev())
+    torch.cuda.synchronize()
+    calls = [lambda: L.moqe_route(logits.data_ptr(), 4, 3, ids.data_ptr(), st),
+             lambda: L.moqe_expand_ids(ids.data_ptr(), off.data_ptr(), 4, 4, rows.data_ptr(), st),
+             lambda: L.moqe_permute(None, ids.data_ptr(), 4, 0, 3, None, perm.data_ptr(), off.data_ptr(), None, 0, st)]
+    for call in calls:
+        assert rt.cudaStreamBeginCapture(st, 2) == 0            # (relaxed)
+        assert rt.cudaStreamSynchronize(st) != 0                # not allowed in a capture: it is invalid from here on
+        refused = call()
+        graph = ctypes.c_void_p()
+        assert rt.cudaStreamEndCapture(st, ctypes.byref(graph)) != 0
+        rt.cudaGetLastError()
+        assert refused == moqe.ERR_CUDA
+        assert moqe.lib().moqe_unpermute(Y.data_ptr(), order.data_ptr(), 4, 8, Y.data_ptr(), torch.cuda.current_stream().cuda_stream) == moqe.OK
+    torch.cuda.synchronize()
