@@ -1,0 +1,73 @@
+"""Where experts' device memory comes from and goes to: giving it back waits for the device and disturbs nobody's capture."""
+import ctypes
+import threading
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+THREAD_LOCAL, RELAXED = 1, 2                    # cudaStreamCaptureMode
+
+
+def _runtime():
+    return ctypes.CDLL("libcudart.so.12")
+
+
+class _Capture:
+    """A capture on a stream of its own; `graph` afterwards, `valid` whether it came to one."""
+
+    def __init__(self, mode):
+        self.mode, self.stream, self.graph = mode, torch.cuda.Stream(), ctypes.c_void_p()
+        self.handle = ctypes.c_void_p(self.stream.cuda_stream)
+
+    def __enter__(self):
+        torch.cuda.synchronize()
+        assert _runtime().cudaStreamBeginCapture(self.handle, self.mode) == 0
+        return self
+
+    def __exit__(self, *exc):
+        self.valid = _runtime().cudaStreamEndCapture(self.handle, ctypes.byref(self.graph)) == 0
+        _runtime().cudaGetLastError()
+
+
+def _elsewhere(call):
+    got = []
+
+    def run():
+        torch.cuda.set_device(0)
+        got.append(call())
+    t = threading.Thread(target=run)
+    t.start()
+    t.join()
+    return got[0]
+
+
+def _expert(N=512, K=512):
+    import paper_2508_09204_b200 as moqe
+    W = torch.randn((N, K), device="cuda", generator=torch.Generator("cuda").manual_seed(N + K))
+    return W, moqe.moqe_quantize_rtn(W, 4, 128, False)
+
+
+def test_destroy_waits_for_every_stream():
+    import paper_2508_09204_b200 as moqe
+    side = torch.cuda.Stream()
+    _, e = _expert()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(20_000_000)           # some 10 ms
+    assert not side.query()
+    e.close()
+    assert side.query()
+    assert moqe.moqe_async_status() == moqe.OK
+
+
+@pytest.mark.parametrize("mode,same_thread", [(THREAD_LOCAL, False), (RELAXED, False), (RELAXED, True)])
+def test_destroy_beside_a_capture(mode, same_thread):
+    import paper_2508_09204_b200 as moqe
+    _, e = _expert()
+    handle, e.handle = e.handle, None
+    with _Capture(mode) as c:
+        destroy = lambda: moqe.lib().moqe_expert_destroy(handle)
+        status = destroy() if same_thread else _elsewhere(destroy)
+    assert status == moqe.OK and c.valid
