@@ -80,8 +80,9 @@ typedef struct moqe_expert moqe_expert;
  *   s == 0 or non-finite after the fp16 rounding -> s = 1;   dequant = s*(c-z).
  * W: device fp32 [N][K], finite.  bits in {2,3,4,8}; group 0, 32, 64 or a multiple
  * of 128, dividing K.  On success *out owns new device buffers (from a memory
- * pool of the library, ordered on `stream`; the call is therefore not capturable in a CUDA graph) and must be
- * released with moqe_expert_destroy.  The kernels run on `stream`.
+ * pool of the library, ordered on `stream`) and must be released with moqe_expert_destroy.  The kernels run on `stream`.
+ * While `stream` is being captured the buffers come from cudaMalloc, which only a capture in relaxed mode or of another
+ * thread's allows (MOQE_ERR_ALLOC in the others, which are invalid afterwards); the graph then fills them when it runs.
  * ------------------------------------------------------------------------- */
 MOQE_API moqe_status moqe_quantize_rtn(const float* W, int N, int K, int bits, int group, int sym,
                               void* stream, moqe_expert** out);

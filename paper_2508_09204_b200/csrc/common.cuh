@@ -80,6 +80,7 @@ struct moqe_expert {
     int Np, Kp;                   // padded to multiples of 128
     int G;                        // real groups per row  (1 when group == 0)
     int device;
+    bool pooled;                  // its memory is the pool's (else cudaMalloc's)
     uint8_t* tiles;               // packed tiles with their meta
     __half* scales_pc;            // per-channel: [Np], else nullptr
     __nv_bfloat16* zeros_pc;      // per-channel asymmetric: [Np], else nullptr

@@ -521,14 +521,18 @@ cudaMemPool_t expert_pool(int device) {
     return g_pools[device];
 }
 
-// Memory for an expert that is filled on `st`.  nullptr: none to be had, or `st` is being captured (the memory would
-// belong to the graph).
-void* expert_malloc(size_t bytes, int device, cudaStream_t st) {
+// Memory for an expert that is filled on `st`, or nullptr.  A stream that is being captured gets memory from cudaMalloc, where the
+// capture's mode allows it: the pool's would belong to the graph.
+void* expert_malloc(size_t bytes, int device, cudaStream_t st, bool& pooled) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) { cudaGetLastError(); return nullptr; }
-    cudaMemPool_t pool = expert_pool(device);
     void* p = nullptr;
-    if (!pool || cudaMallocFromPoolAsync(&p, bytes, pool, st) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    pooled = cap == cudaStreamCaptureStatusNone;
+    cudaMemPool_t pool = pooled ? expert_pool(device) : nullptr;
+    if (pooled ? !pool || cudaMallocFromPoolAsync(&p, bytes, pool, st) != cudaSuccess : cudaMalloc(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
     return p;
 }
 // Waits until the current device has done all that was enqueued on it.  By giving back a small allocation, for which cudaFree
@@ -541,11 +545,11 @@ bool device_idle() {
     return cudaFree(p) == cudaSuccess;
 }
 // Gives it back once nothing on the device can be using it any more.
-bool expert_free(void* p, int device) {
+bool expert_free(void* p, bool pooled, int device) {
     int now = 0;
     if (cudaGetDevice(&now) != cudaSuccess) return false;
     bool ok = now == device || cudaSetDevice(device) == cudaSuccess;
-    ok = ok && device_idle() && cudaFreeAsync(p, nullptr) == cudaSuccess;
+    ok = ok && (pooled ? device_idle() && cudaFreeAsync(p, nullptr) == cudaSuccess : cudaFree(p) == cudaSuccess);
     if (!ok) cudaGetLastError();
     if (now != device) ok = cudaSetDevice(now) == cudaSuccess && ok;
     return ok;
@@ -578,7 +582,7 @@ moqe_status alloc_expert(int N, int K, int bits, int group, int sym, bool clear,
     e->pc_alloc = group == 0 ? (size_t)e->Np * 2 : 0;
     // one block: the tiles, then (per channel) scales and zero-points
     const size_t pc_total = e->pc_alloc * (e->sym ? 1 : 2);
-    e->tiles = (uint8_t*)expert_malloc(e->tiles_alloc + pc_total, e->device, st);
+    e->tiles = (uint8_t*)expert_malloc(e->tiles_alloc + pc_total, e->device, st, e->pooled);
     if (!e->tiles) { delete e; return MOQE_ERR_ALLOC; }
     if (group == 0) {
         e->scales_pc = (__half*)(e->tiles + e->tiles_alloc);
@@ -716,7 +720,7 @@ extern "C" moqe_status moqe_expert_info(const moqe_expert* e, int* N, int* K, in
 
 extern "C" moqe_status moqe_expert_destroy(moqe_expert* e) {
     if (!e) return MOQE_ERR_NULL;
-    const bool ok = expert_free(e->tiles, e->device);
+    const bool ok = expert_free(e->tiles, e->pooled, e->device);
     delete e;
     return ok ? MOQE_OK : MOQE_ERR_CUDA;
 }

@@ -71,3 +71,31 @@ def test_destroy_beside_a_capture(mode, same_thread):
         destroy = lambda: moqe.lib().moqe_expert_destroy(handle)
         status = destroy() if same_thread else _elsewhere(destroy)
     assert status == moqe.OK and c.valid
+
+
+@pytest.mark.parametrize("what", ["quantize", "prefetch"])
+@pytest.mark.parametrize("mode,same_thread", [(THREAD_LOCAL, False), (RELAXED, True)])
+def test_building_in_a_capture(mode, same_thread, what):
+    """The expert's memory exists at once, and the graph fills it when it runs."""
+    import paper_2508_09204_b200 as moqe
+    W, e = _expert()
+    host = moqe.moqe_expert_offload(e)
+    out = ctypes.c_void_p()
+    with _Capture(mode) as c:
+        if what == "quantize":
+            build = lambda: moqe.lib().moqe_quantize_rtn(W.data_ptr(), *W.shape, 4, 128, 0, c.handle, ctypes.byref(out))
+        else:
+            build = lambda: moqe.lib().moqe_expert_prefetch(host.handle, c.handle, ctypes.byref(out))
+        status = build() if same_thread else _elsewhere(build)
+    assert status == moqe.OK and c.valid
+    run = ctypes.c_void_p()
+    assert _runtime().cudaGraphInstantiate(ctypes.byref(run), c.graph, ctypes.c_ulonglong(0)) == 0
+    assert _runtime().cudaGraphLaunch(run, c.handle) == 0
+    torch.cuda.synchronize()
+    built = moqe.Expert(out.value)
+    for a, b in zip(moqe.moqe_expert_export(built), moqe.moqe_expert_export(e)):
+        assert torch.equal(a, b)
+    torch.cuda.synchronize()
+    _runtime().cudaGraphExecDestroy(run)
+    _runtime().cudaGraphDestroy(c.graph)
+    built.close()
