@@ -108,9 +108,14 @@ MOQE_API moqe_status moqe_expert_import(int N, int K, int bits, int group, int s
 MOQE_API moqe_status moqe_expert_info(const moqe_expert* e, int* N, int* K, int* bits, int* group, int* sym,
                              size_t* code_bytes, size_t* meta_bytes, size_t* alloc_bytes);
 
-/* Gives the expert's device buffers back (synchronises the device).  The library's pool keeps up to 1 GB of freed
- * expert memory per device for experts built later; the rest goes back to the device. */
+/* Gives the expert's device buffers back (waits for the device; not while this thread has a capture under way, unless it is
+ * relaxed).  The library's pool keeps up to 1 GB of freed expert memory per device for experts built later; the rest
+ * goes back to the device.  What is kept serves any allocation of this process that would fail without it. */
 MOQE_API moqe_status moqe_expert_destroy(moqe_expert* e);
+
+/* Gives freed expert memory of the current device back to the device until the pool holds at most keep_bytes (or what
+ * living experts occupy, if that is more); 0: all of it.  Synchronises the default stream. */
+MOQE_API moqe_status moqe_expert_pool_trim(size_t keep_bytes);
 
 /* ---------------------------------------------------------------------------
  * Expert residency (Section 4.4 and the appendix table "Router model and expert loading overhead": one expert

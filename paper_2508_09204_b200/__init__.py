@@ -24,7 +24,7 @@ MAX_EXPERTS = 32
 PATH_AUTO, PATH_STREAM, PATH_TCGEN05, PATH_DECODE, PATH_DENSE = 0, 1, 2, 5, 6
 
 EXPORTED = (
-    "moqe_quantize_rtn", "moqe_expert_export", "moqe_expert_import", "moqe_expert_info", "moqe_expert_destroy",
+    "moqe_quantize_rtn", "moqe_expert_export", "moqe_expert_import", "moqe_expert_info", "moqe_expert_destroy", "moqe_expert_pool_trim",
     "moqe_route", "moqe_expand_ids", "moqe_route_permute", "moqe_permute_workspace", "moqe_permute", "moqe_permute_static", "moqe_unpermute",
     "moqe_routed_qgemm_workspace", "moqe_routed_qgemm", "moqe_routed_qgemm_path", "moqe_routed_qgemm_sorted",
     "moqe_routed_qgemm_sorted_multi", "moqe_routed_qgemm_workspace_clear", "moqe_async_status",
@@ -60,6 +60,7 @@ def lib() -> C.CDLL:
         L.moqe_expert_import.argtypes = [i32, i32, i32, i32, i32, vp, vp, vp, vp, C.POINTER(vp)]
         L.moqe_expert_info.argtypes = [vp] + [C.POINTER(i32)] * 5 + [C.POINTER(sz)] * 3
         L.moqe_expert_destroy.argtypes = [vp]
+        L.moqe_expert_pool_trim.argtypes = [sz]
         L.moqe_route.argtypes = [vp, i32, i32, vp, vp]
         L.moqe_expand_ids.argtypes = [vp, vp, i32, i32, vp, vp]
         L.moqe_route_permute.argtypes = [vp, i32, i32, vp, i32, vp, vp, vp, vp, vp]
@@ -245,6 +246,11 @@ def moqe_expert_import(bits: int, group: int, sym: bool, codes: torch.Tensor, sc
     _check(lib().moqe_expert_import(N, K, int(bits), int(group), int(bool(sym)), _ptr(codes), _ptr(scales), _ptr(zeros),
                                     _stream(), C.byref(out)), "moqe_expert_import")
     return Expert(out.value)
+
+
+def moqe_expert_pool_trim(keep_bytes: int = 0) -> None:
+    """Gives the memory of destroyed experts back to the device, down to ``keep_bytes`` (the library keeps up to 1 GB)."""
+    _check(lib().moqe_expert_pool_trim(int(keep_bytes)), "moqe_expert_pool_trim")
 
 
 def moqe_route(logits: torch.Tensor) -> torch.Tensor:

@@ -99,3 +99,25 @@ def test_building_in_a_capture(mode, same_thread, what):
     _runtime().cudaGraphExecDestroy(run)
     _runtime().cudaGraphDestroy(c.graph)
     built.close()
+
+
+def test_trim_gives_freed_memory_back():
+    import paper_2508_09204_b200 as moqe
+    W = torch.randn((8192, 4096), device="cuda")
+    free = lambda: (torch.cuda.empty_cache(), torch.cuda.mem_get_info()[0])[1]         # (without what torch keeps)
+    moqe.moqe_expert_pool_trim()
+    before = free()
+    experts = [moqe.moqe_quantize_rtn(W, 8, 0, True) for _ in range(12)]
+    bytes_each = experts[0].alloc_bytes
+    assert before - free() >= 12 * bytes_each
+    for e in experts[1:]:
+        e.close()
+    assert free() < before - 12 * bytes_each + (1 << 20)          # kept for the next expert
+    moqe.moqe_expert_pool_trim(6 * bytes_each)
+    assert before - 7 * bytes_each <= free() <= before - bytes_each
+    moqe.moqe_expert_pool_trim()
+    assert before - 3 * bytes_each <= free() <= before - bytes_each  # (the living one, in the pool's own granularity)
+    assert torch.equal(moqe.moqe_expert_export(experts[0])[0], moqe.moqe_expert_export(moqe.moqe_quantize_rtn(W, 8, 0, True))[0])
+    experts[0].close()
+    moqe.moqe_expert_pool_trim()
+    assert free() == before
