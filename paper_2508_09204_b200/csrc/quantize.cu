@@ -273,7 +273,7 @@ __global__ void encode_pack_kernel(const float* __restrict__ W, const uint8_t* _
 
 // ---------------------------------------------------------------------------
 // K1: scales, zero-points, codes and packing in one kernel, for per-channel experts and groups within a k-block
-// (wider groups take K1a and K1b above).  Bound by the fp32 weights' bytes, which are read from HBM once: a warp holds
+// (others take K1a and K1b above, see one_kernel).  Bound by the fp32 weights' bytes, which are read from HBM once: a warp holds
 // the 16 channels x 128 k of a blob in registers between finding the groups' extremes and rounding.  A per-channel
 // expert's block goes over its 16 rows twice, the second time out of L2 (16 rows are 256 KB at K = 4096).  Every byte of
 // the tiles is written here, padding included.  11008 x 4096, 4-bit g128: 57 us (the two kernels: 92 + 60); three blocks
@@ -572,8 +572,12 @@ moqe_status check_format(int N, int K, int bits, int group) {
     return MOQE_OK;
 }
 
-// clear: zero the buffers on `st` (padded channels / padded k: codes 0, scale 0, zero-point 0); a caller that writes every
-// byte itself does without
+// zeroes the buffers: padded channels / padded k have codes 0, scale 0 and zero-point 0
+moqe_status clear_expert(const moqe_expert* e, cudaStream_t st) {
+    return cuda_ok(cudaMemsetAsync(e->tiles, 0, e->tiles_alloc + e->pc_alloc * (e->sym ? 1 : 2), st));
+}
+
+// clear: zero the buffers on `st`; a caller that writes every byte itself does without
 moqe_status alloc_expert(int N, int K, int bits, int group, int sym, bool clear, cudaStream_t st, moqe_expert** out) {
     moqe_expert* e = new (std::nothrow) moqe_expert();
     if (!e) return MOQE_ERR_ALLOC;
@@ -593,7 +597,7 @@ moqe_status alloc_expert(int N, int K, int bits, int group, int sym, bool clear,
         e->scales_pc = (__half*)(e->tiles + e->tiles_alloc);
         if (!e->sym) e->zeros_pc = (__nv_bfloat16*)(e->tiles + e->tiles_alloc + e->pc_alloc);
     }
-    if (clear && cudaMemsetAsync(e->tiles, 0, e->tiles_alloc + pc_total, st) != cudaSuccess) { moqe_expert_destroy(e); return MOQE_ERR_CUDA; }
+    if (clear && clear_expert(e, st) != MOQE_OK) { moqe_expert_destroy(e); return MOQE_ERR_CUDA; }
     *out = e;
     return MOQE_OK;
 }
@@ -612,6 +616,16 @@ moqe_status launch_quantize(const moqe_expert* e, const float* W, cudaStream_t s
 #undef MOQE_QP
     count_launch();
     return cuda_ok(cudaGetLastError());
+}
+
+// Whether an expert is built by quantize_pack_kernel, or by the two kernels before it.  Groups within a k-block are.  A per-channel
+// expert's strip of 16 rows belongs to one block there, which goes over it twice: that wants strips for every SM to the last
+// round, and short enough to be in L2 the second time.  Two kernels / one, device time in us, 8 bit: 11008 rows (688 strips on 148
+// SMs) x 4096 113 / 102, x 11008 267 / 296; 3072 rows (192 strips) x 4096 36 / 44; 128 rows x 11008 23 / 60.
+bool one_kernel(const moqe_expert* e) {
+    if (e->group != 0) return e->group <= 128;
+    const int strips = e->Np / 16, sms = device_sm_count(), rounds = (strips + sms - 1) / sms;
+    return e->K <= 5120 && strips * 10ll >= 9ll * sms * rounds;
 }
 
 template <bool FROM_CODES>
@@ -644,15 +658,16 @@ extern "C" moqe_status moqe_quantize_rtn(const float* W, int N, int K, int bits,
     if (reinterpret_cast<uintptr_t>(W) % 16 != 0) return MOQE_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)stream;
     moqe_expert* e = nullptr;
-    const bool one_pass = group <= 128;
-    s = alloc_expert(N, K, bits, group, sym, !one_pass, st, &e);
+    s = alloc_expert(N, K, bits, group, sym, false, st, &e);
     if (s != MOQE_OK) return s;
-    if (one_pass) {
+    if (one_kernel(e)) {                                 // (it writes every byte)
         s = launch_quantize(e, W, st);
         if (s != MOQE_OK) { moqe_expert_destroy(e); return s; }
         *out = e;
         return MOQE_OK;
     }
+    s = clear_expert(e, st);
+    if (s != MOQE_OK) { moqe_expert_destroy(e); return s; }
     long long warps = (long long)N * e->G;
     unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
     rtn_scales_kernel<<<blocks, 256, 0, st>>>(W, N, K, bits, group, e->G, e->sym, e->Kp / 128, e->tiles, e->scales_pc,

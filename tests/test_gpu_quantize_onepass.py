@@ -36,3 +36,22 @@ def test_halfway_weights_and_reused_memory(N, K, bits, group, sym):
     Y = moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), [e], path=moqe.PATH_TCGEN05)
     assert moqe.moqe_async_status() == moqe.OK
     assert_close(torch_to_bits(Y), oracle.routed_gemm(X, ids, [oracle.dequantize(c, s, z, group)]), "product")
+
+
+@pytest.mark.parametrize("bits,sym", [(8, True), (4, False), (3, False), (2, True)])
+@pytest.mark.parametrize("N,K", [(2296, 1088), (2368, 64), (2056, 1088), (2376, 5128), (2296, 5120)])
+def test_per_channel_by_one_kernel_and_by_two(N, K, bits, sym):
+    """144 and 148 strips of 16 rows are for one kernel on 148 SMs, up to K = 5120; 136 and 152 strips, and longer rows, for two.  The
+    memory is that of a larger expert before."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_close, assert_expert_matches, bf16_to_torch, dev, torch_to_bits
+    W = wl.weights_f32(f"pc/{N}/{K}", N, K)
+    moqe.moqe_quantize_rtn(torch.full((2 * N + 128, 2 * K), 3.0, device=dev()), 8, 0, False).close()
+    e = moqe.moqe_quantize_rtn(torch.from_numpy(W).to(dev()), bits, 0, sym)
+    canon = oracle.quantize_rtn(W, bits, 0, sym)
+    assert_expert_matches(e, canon)
+    X = wl.activations_bf16(f"pc/{K}", 40, K)
+    ids = np.zeros(40, np.int32)
+    Y = moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), [e], path=moqe.PATH_TCGEN05)
+    assert moqe.moqe_async_status() == moqe.OK
+    assert_close(torch_to_bits(Y), oracle.routed_gemm(X, ids, [oracle.dequantize(*canon, 0)]), "product")
