@@ -606,7 +606,7 @@ moqe_status launch_quantize(const moqe_expert* e, const float* W, cudaStream_t s
     const int KB = e->Kp / 128, strips = e->Np / 16;
     // a per-channel strip belongs to one block; grouped strips are cut along K as far as they go, a k-block to a warp (so many
     // small blocks leave no wave half empty: 63 -> 57 us for 688 strips)
-    const int cuts = e->group == 0 ? 1 : (KB + 7) / 8;
+    const int cuts = e->group == 0 ? 1 : (KB + 7) / 8 < 65535 ? (KB + 7) / 8 : 65535;      // (a grid has no more in y)
     const dim3 grid(strips, cuts);
 #define MOQE_QP(B) quantize_pack_kernel<B><<<grid, 256, 0, st>>>(W, e->N, e->K, e->group, e->sym, KB, e->tiles, e->scales_pc, e->zeros_pc)
     if (e->bits == 4) MOQE_QP(4);

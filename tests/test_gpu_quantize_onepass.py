@@ -55,3 +55,17 @@ def test_per_channel_by_one_kernel_and_by_two(N, K, bits, sym):
     Y = moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), [e], path=moqe.PATH_TCGEN05)
     assert moqe.moqe_async_status() == moqe.OK
     assert_close(torch_to_bits(Y), oracle.routed_gemm(X, ids, [oracle.dequantize(*canon, 0)]), "product")
+
+
+def test_rows_longer_than_a_grid_has_blocks():
+    """More than 65535 eights of k-blocks to a row."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import dev
+    N, K = 8, 65536 * 1024 + 128
+    W = torch.zeros((N, K), device=dev())
+    W[:, ::2] = 1.0
+    W[:, -128:] *= 2.0
+    codes, scales, zeros = moqe.moqe_expert_export(moqe.moqe_quantize_rtn(W, 8, 128, False))
+    assert bool((codes[:, ::2] == 255).all()) and not bool(codes[:, 1::2].any()) and not bool(zeros.any())
+    s = torch.tensor([1.0 / 255], dtype=torch.float32).half().to(dev())
+    assert bool((scales[:, :-1] == s).all()) and bool((scales[:, -1] == torch.tensor(2.0 / 255).half().to(dev())).all())
