@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(SORT_THREADS) route_sort_small_kernel(const fl
     if (live) perm[s_off[bucket] + rank_in_warp + s_warp[warp][bucket]] = t;
 }
 
-// M > 1024: two kernels, or three for more than FUSED_SCAN_BLOCKS blocks.  (1) per-block bucket totals, [bucket][block]
+// M > 1024: two kernels, or three where fused_scan says so.  (1) per-block bucket totals, [bucket][block]
 __global__ void __launch_bounds__(SORT_THREADS) sort_hist_kernel(const int32_t* __restrict__ row_ids, int M, int E,
                                                                  int32_t* __restrict__ block_tot, int* status) {
     __shared__ int s_warp[SORT_WARPS][MAXB];
@@ -255,8 +255,13 @@ __global__ void __launch_bounds__(1024) sort_scan_kernel(int32_t* __restrict__ b
 
 // (3) scatter row indices to their slots.  FUSED: `block_base` still holds the blocks' totals, and every block adds up those
 // before it by itself (a warp per bucket, coalesced; 784 blocks x 4 buckets are 12 KB out of L2): the scan's launch and its
-// 8 us on one SM go away (four 1x1 layers of 256 images with two sorts: 406 -> 372 us together with the chained launches).
+// 8 us on one SM go away (four 1x1 layers of 256 images with two sorts: 406 -> 372 us together with the chained launches).  All
+// blocks together read nblk^2 (E + 1) totals, which in the end costs more than the scan.  Three kernels / two: 2048 blocks, 8
+// experts (38 million totals) 43.2 / 42.0 us, 16 (71) 50.6 / 51.5, 24 (105) 57.5 / 61.1, 32 (138) 71.8 / 80.5; 1200 blocks, 32 experts
+// (48) 46.6 / 45.8, 1600 (84) 59.3 / 61.5.
 constexpr int FUSED_SCAN_BLOCKS = 2048;
+constexpr long long FUSED_SCAN_TOTALS = 60000000;
+bool fused_scan(int nblk, int E) { return nblk <= FUSED_SCAN_BLOCKS && (long long)nblk * nblk * (E + 1) <= FUSED_SCAN_TOTALS; }
 template <bool FUSED>
 __global__ void __launch_bounds__(SORT_THREADS) sort_scatter_kernel(const int32_t* __restrict__ row_ids, int M, int E,
                                                                     const int32_t* __restrict__ block_base,
@@ -330,7 +335,7 @@ moqe_status launch_big_sort(const int32_t* row_ids, int M, int E, int32_t* block
                             int* status, cudaStream_t st) {
     const int nblk = (M + SORT_THREADS - 1) / SORT_THREADS;
     cudaError_t err = launch_chained(sort_hist_kernel, nblk, SORT_THREADS, st, row_ids, M, E, block_tot, status);
-    if (err == cudaSuccess && nblk <= FUSED_SCAN_BLOCKS) {
+    if (err == cudaSuccess && fused_scan(nblk, E)) {
         err = launch_chained(sort_scatter_kernel<true>, nblk, SORT_THREADS, st, row_ids, M, E, block_tot, perm, offsets, Y_zero_invalid, N);
         count_launch(2);
     } else if (err == cudaSuccess) {

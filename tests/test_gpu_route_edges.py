@@ -92,3 +92,19 @@ def test_a_refused_launch_leaves_no_error_for_the_next_call():
         assert refused == moqe.ERR_CUDA
         assert moqe.lib().moqe_unpermute(Y.data_ptr(), order.data_ptr(), 4, 8, Y.data_ptr(), torch.cuda.current_stream().cuda_stream) == moqe.OK
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("blocks,E", [(1348, 32), (1349, 32), (2048, 13), (2048, 14)])
+def test_sort_either_side_of_the_fused_scan(blocks, E):
+    """nblk^2 (E + 1) up to 60 million totals: two kernels, above: three."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import dev
+    ids = torch.randint(-1, E + 1, (blocks * 1024 - 5,), device=dev(), dtype=torch.int32, generator=torch.Generator(dev()).manual_seed(blocks))
+    before = moqe.moqe_launch_count()
+    _, perm, offsets = moqe.moqe_permute(None, ids, E)
+    assert moqe.moqe_launch_count() - before == (2 if blocks * blocks * (E + 1) <= 60_000_000 else 3)
+    moqe.moqe_async_status()                                   # (invalid ids were latched)
+    bucket = torch.where((ids < 0) | (ids >= E), E, ids)
+    assert torch.equal(perm, torch.argsort(bucket, stable=True).to(torch.int32))
+    ends = torch.bincount(bucket, minlength=E + 1).cumsum(0)[:E]
+    assert torch.equal(offsets, torch.cat([ends.new_zeros(1), ends]).to(torch.int32))
