@@ -581,29 +581,34 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
         // latency; a super-tile takes 800.  (LLaMA block, 1 row: 73.3 -> 67.1 us; 16 rows: 107.7 -> 100.2.  16 rows x
         // 11008 x 4096, three experts: 32 super-tiles to a CTA instead of 28, 23.6 -> 21.5 us; with up to nine more,
         // 3584 x 18944 went from 30.1 to 31.5.)
+        // (This is in front of every launch whether it applies or not: quotients by multiplication -- x + 0.5 is at least 0.5 / d
+        // away from a multiple of d, and the approximate division is off by less up to 2^20 -- and votes for shuffles.)
         int aligned = 0;
+        const int wtop = __reduce_max_sync(0xffffffffu, TT > 0 ? wv : 1);
         {
-            const int nseg = __reduce_add_sync(0xffffffffu, segs);
-            const int kmax = __reduce_max_sync(0xffffffffu, TT > 0 ? KBv : 0), kmin = __reduce_min_sync(0xffffffffu, TT > 0 ? KBv : 0x7fffffff);
-            const int wtop = __reduce_max_sync(0xffffffffu, TT > 0 ? wv : 0), wlow = __reduce_min_sync(0xffffffffu, TT > 0 ? wv : 0x7fffffff);
+            const int nseg = __reduce_add_sync(0xffffffffu, segs), kmax = __reduce_max_sync(0xffffffffu, TT > 0 ? KBv : 0);
             const int grid = gridDim.x;
-            if (nseg > 0 && kmax == kmin && wtop * 8 <= wlow * 9) {
-                const int share = nseg <= grid ? grid / nseg : (nseg + grid - 1) / grid;      // CTAs to a segment, or the reverse
-                const int most = nseg <= grid ? (kmax + share - 1) / share : share * kmax;    // super-tiles of the fullest CTA
-                const int even = nseg * kmax / grid;
-                if (nseg <= grid) aligned = most <= even + GV_ALIGN && share <= kmax ? share * nseg : 0;
-                else aligned = most <= even + GV_ALIGN && nseg % share == 0 ? nseg / share : 0;
+            if (nseg > 0 && __all_sync(0xffffffffu, TT == 0 || (KBv == kmax && wtop * 8 <= wv * 9)) && max(nseg, kmax) < 1 << 20) {
+                auto quotient = [](int x, int d) { return (int)__fdividef((float)x + 0.5f, (float)d); };
+                const long long room = (long long)nseg * kmax + (long long)GV_ALIGN * grid;       // (GV_ALIGN more than an even share, times grid)
+                if (nseg <= grid) {
+                    const int share = quotient(grid, nseg);                            // CTAs to a segment ...
+                    const int most = quotient(kmax + share - 1, share);                // super-tiles of the fullest CTA
+                    if ((long long)most * grid <= room && share <= kmax) aligned = share * nseg;
+                } else {
+                    const int share = quotient(nseg + grid - 1, grid), ctas = quotient(nseg, share);     // ... or the reverse
+                    if ((long long)share * kmax * grid <= room && ctas * share == nseg) aligned = ctas;
+                }
             }
         }
         if (aligned) wv = 1;
         cost = (long long)TT * wv;
         long long incl = cost;
-        int wmax = TT > 0 ? wv : 1;
+        const int wmax = aligned ? 1 : wtop;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const long long o = __shfl_up_sync(0xffffffffu, incl, d);
             if (lane >= d) incl += o;
-            wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, d));
         }
         const long long C = __shfl_sync(0xffffffffu, incl, 31);
         const long long base = incl - cost;
@@ -634,8 +639,7 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
             if (te > tb) str = p.ps[v].stride;
         }
         // ring geometry: a stage holds two of the largest packed tiles this CTA will see
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) str = max(str, __shfl_xor_sync(0xffffffffu, str, d));
+        str = __reduce_max_sync(0xffffffffu, str);
         if (lane == 0) {
             const int stage_bytes = 2 * ((max(str, 128) + 127) & ~127);
             *s_C = C; *s_G = G;
