@@ -587,8 +587,12 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
         const int wtop = __reduce_max_sync(0xffffffffu, TT > 0 ? wv : 1);
         {
             const int nseg = __reduce_add_sync(0xffffffffu, segs), kmax = __reduce_max_sync(0xffffffffu, TT > 0 ? KBv : 0);
-            const int grid = gridDim.x;
-            if (nseg > 0 && __all_sync(0xffffffffu, TT == 0 || (KBv == kmax && wtop * 8 <= wv * 9)) && max(nseg, kmax) < 1 << 20) {
+            const int total = __reduce_add_sync(0xffffffffu, TT), grid = gridDim.x;
+            // No more super-tiles than CTAs: one each, whatever they cost.  (Shares by cost are as large as the dearest, so that
+            // a few CTAs would have two of the others, in two pieces that follow one another: 2304 x 256, three experts, 8 rows 9.9 ->
+            // 6.9 us; 2048 x 512, four experts of which one has groups of 64, 11.4 -> 8.7.)
+            if (total <= grid) aligned = total;
+            else if (nseg > 0 && __all_sync(0xffffffffu, TT == 0 || (KBv == kmax && wtop * 8 <= wv * 9)) && max(nseg, kmax) < 1 << 20) {
                 auto quotient = [](int x, int d) { return (int)__fdividef((float)x + 0.5f, (float)d); };
                 const long long room = (long long)nseg * kmax + (long long)GV_ALIGN * grid;       // (GV_ALIGN more than an even share, times grid)
                 if (nseg <= grid) {
