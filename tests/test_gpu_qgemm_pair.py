@@ -50,8 +50,11 @@ def test_pair_kernel_edges(M, N, K, kind):
 
 def test_pair_kernel_split_is_deterministic_and_clears_its_counters():
     """One token tile of one expert, 40 k-blocks deep: every cluster holds a part of it; the parts are added in a fixed
-    order (same bits every time) and the arrival counters come back to zero (the second call still completes)."""
-    from gpu_helpers import build_experts, assert_close
+    order (same bits every time) and the arrival counters come back to zero (calls on a sorted batch, whose workspace is
+    cleared once, still complete)."""
+    import torch
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import build_experts, assert_close, bf16_to_torch, dev, torch_to_bits
     M, N, K = 200, 256, 5120
     W = wl.weights_f32("pair/split", N, K)
     X = wl.activations_bf16("pair/split/X", M, K)
@@ -61,6 +64,15 @@ def test_pair_kernel_split_is_deterministic_and_clears_its_counters():
     assert_close(first, oracle.routed_gemm(X, ids, What), "split")
     for _ in range(3):
         assert np.array_equal(_run(X, ids, gpu, 2), first)
+    _, perm, offsets = moqe.moqe_permute(None, torch.from_numpy(ids).to(dev()), 1)
+    ws = moqe.alloc_workspace(moqe.moqe_routed_qgemm_workspace(M, N, K, 1))
+    ws.fill_(0xFF)
+    moqe.moqe_routed_qgemm_workspace_clear(ws, M, N, K, 1)
+    for _ in range(4):
+        Y = torch.full((M, N), float("nan"), dtype=torch.bfloat16, device=dev())
+        moqe.moqe_routed_qgemm_sorted(bf16_to_torch(X), perm, offsets, gpu, Y, ws, path=2)
+        assert moqe.moqe_async_status() == moqe.OK
+        assert np.array_equal(torch_to_bits(Y), first)
 
 
 @pytest.mark.parametrize("M,N,K", [(192, 19200, 64), (192, 19200, 128), (96, 9600, 640), (48, 6000, 1152)])
@@ -76,3 +88,32 @@ def test_steps_of_one_k_block(M, N, K):
     assert_close(first, oracle.routed_gemm(X, ids, What), f"odd steps M{M} N{N} K{K}")
     for _ in range(30):
         assert np.array_equal(_run(X, ids, gpu, 2), first)
+
+
+@pytest.mark.parametrize("M,N,K,specs", [(300, 6016, 1408, FORMATS), (700, 6016, 1408, FORMATS), (700, 6000, 1024, [(4, 128, False)]), (300, 9600, 640, [(4, 32, False), (8, 64, True)]),
+                                         (700, 6400, 384, [(8, 32, True)])])
+def test_wide_tiles_split(M, N, K, specs):
+    """Layers wide enough for the automatic choice to keep tiles of 128 and 256 tokens, and tiles left over that are split by k-blocks
+    (the last shape: one tile, whose cost is that of three units); an odd number of 128-channel tiles among them."""
+    from gpu_helpers import build_experts, assert_close
+    W = wl.weights_f32(f"pair/{N}/{K}", N, K)
+    X = wl.activations_bf16(f"pair/{M}/{K}", M, K)
+    specs = [f for f in specs if f[1] == 0 or K % f[1] == 0]
+    gpu, What, _ = build_experts(W, specs)
+    ids = _ids("short runs", M, len(specs))
+    first = _run(X, ids, gpu, 2)
+    assert_close(first, oracle.routed_gemm(X, ids, What), f"wide M{M} N{N} K{K}")
+    for _ in range(3):
+        assert np.array_equal(_run(X, ids, gpu, 2), first)
+
+
+@pytest.mark.parametrize("M,N,K", [(40, 384, 8192), (33, 128, 2048), (64, 256, 640)])
+def test_few_deep_tiles(M, N, K):
+    """One to three tiles over all clusters, from many units to a share down to fewer than one cluster's four."""
+    from gpu_helpers import build_experts, assert_close
+    W = wl.weights_f32(f"pair/{N}/{K}", N, K)
+    X = wl.activations_bf16(f"pair/{M}/{K}", M, K)
+    gpu, What, _ = build_experts(W, [(8, 0, True), (4, 128, False), (3, 64, False)])
+    for used in (1, 2, 3):
+        ids = (np.arange(M) % used).astype(np.int32)
+        assert_close(_run(X, ids, gpu, 2), oracle.routed_gemm(X, ids, What), f"deep M{M} N{N} K{K} {used}")
