@@ -492,10 +492,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, d));
         }
         const int C = __shfl_sync(0xffffffffu, cincl, 31), base = cincl - cost;
-        // Every cluster's share holds at least the start of four units: with two, few deep tiles had many short pieces, and the last
-        // arrival adds them up one after another (33 rows, three experts, 256 x 8192: 24.5 -> 17.6 us, where the streaming kernel
-        // takes 19.6; two experts, 256 x 11008: 31.5 -> 20.8; at worst 6 % more, 128 x 11008).
-        const int Gs = max(1, min(nclusters, C / (4 * wmax)));
+        // Every cluster's share holds at least the start of two units, and of four cheap ones: with two, few deep tiles had many
+        // short pieces, and the last arrival adds them up one after another (33 rows, three experts, 256 x 8192: 24.5 -> 17.6 us,
+        // where the streaming kernel takes 19.6; two experts, 256 x 11008: 31.5 -> 20.8; at worst 6 % more, 128 x 11008).  Four of
+        // the dearest, groups of 32 k, are too many (9408 rows, three experts, 256 x 1024: 30.7 -> 43.3).
+        const int Gs = max(1, min(nclusters, C / min(4 * wmax, max(2 * wmax, 100))));
         int ub = us, ue = us;
         if (cnt > 0 && cluster < Gs) {
             const int den = w * Gs, n0 = cluster * C - base * Gs, n1 = n0 + C;
