@@ -343,6 +343,11 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
                 const int b_lo = colhalf ? split : 0, b_hi = colhalf ? boxes : split;          // this warp's boxes of the chunk
                 if (!(ok = __all_sync(0xffffffffu, mbar_wait_short(bar_accfull + 8 * buf, acc_use[buf] & 1u, s_abort, p.status)))) break;
                 tc_fence_after();
+                auto hand_back = [&]() {                   // the accumulator, as soon as it has been read
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], 32;" ::"r"(bar_accempty + 8 * buf) : "memory");
+                };
                 for (int b = b_lo; b < b_hi; ++b) {
                     // The previous contents of this box have left shared memory: lane 0's own stores, a group to a box.  Of two before and
                     // two now, in turn, the one before last is this box's; in all other cases wait for all.
@@ -374,6 +379,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
                             asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(box + lane * 128 + (((half * 4 + j) ^ (lane & 7)) << 4)), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
                         }
                     }
+                    if (b + 1 == b_hi) hand_back();
                     if (run) {
                         fence_proxy_async();
                         __syncwarp();
@@ -383,10 +389,8 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
                         }
                     }
                 }
+                if (b_lo == b_hi) hand_back();
                 in_flight = run ? b_hi - b_lo : 0;
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], 32;" ::"r"(bar_accempty + 8 * buf) : "memory");
                 acc_use[buf]++;
                 buf ^= 1;
                 if (!run) {
