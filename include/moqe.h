@@ -248,8 +248,10 @@ MOQE_API moqe_status moqe_router_load_report(const float* logits, const int32_t*
  * invalid id are written as zeros).  M == 0 is valid.  workspace:
  * moqe_routed_qgemm_workspace(M, N, K, E) bytes, contents irrelevant on entry;
  * calls that share a workspace must not overlap on the device.
- * Decode batches (at most 32 rows) stream each touched expert's packed weights once through the decode kernel (bulk-copy ring, warp-level MMAs on fp16 operands,
- * stream-K split that follows the routing: experts without rows cost nothing).  That kernel converts the bf16
+ * Decode batches (at most 32 rows) stream each touched expert's packed weights once through the decode kernel (bulk-copy
+ * ring, warp-level MMAs on fp16 operands, stream-K split that follows the routing: experts without rows cost nothing).
+ * Codes enter its MMAs with an offset that is taken out of the fp32 sums: 1024 and less, or at most 128 (none for 8
+ * bits) if one of the call's experts has groups narrower than 128 k.  It converts the bf16
  * activations to fp16: values with |x| > 65504 are outside its domain (they become infinities), unless one of the
  * call's experts has groups narrower than 128 k (then rows are scaled block by block); every other kernel takes the
  * whole bf16 range.  33 to 48 rows with such an expert take the split-K mma.sync streaming kernel; all other
@@ -265,11 +267,17 @@ MOQE_API moqe_status moqe_routed_qgemm(const void* X_bf16, const int32_t* row_id
  * token tile), 3 / 4 = tcgen05 grouped GEMM with 128- / 256-token tiles, never split along K, 5 = decode kernel
  * (MOQE_ERR_UNSUPPORTED if the batch has more than 32 rows or an expert has groups narrower than 128 k),
  * 6 = dense-weights tcgen05 GEMM for large batches on small layers (more than 128 rows, K <= 1024, at most 1024
- * output channels; the automatic choice there: the layer is bound by its activations, so each expert's weights
- * are expanded to bf16 once per call and X / Y are streamed; MOQE_ERR_UNSUPPORTED otherwise). */
+ * output channels, MOQE_ERR_UNSUPPORTED otherwise: the layer is bound by its activations, so each expert's weights
+ * are expanded to bf16 once per call and X / Y are streamed).  The automatic choice takes it there for layers of at
+ * most 65536 weights, and for wider ones from 30000 rows on (12000 where an expert has groups of 32 k and K > N).
+ * Path 5 leaves groups narrower than 128 k to the automatic choice, which has an instantiation for them. */
 MOQE_API moqe_status moqe_routed_qgemm_path(const void* X_bf16, const int32_t* row_ids, int M,
                                    const moqe_expert* const* h_experts, int E, void* Y_bf16,
                                    void* workspace, size_t workspace_bytes, void* stream, int path);
+
+/* The name of the kernel that a call with these rows, experts and path takes (of a batch of several layers: that one of them
+ * alone takes), for reports; NULL where the arguments are refused.  A static string. */
+MOQE_API const char* moqe_routed_qgemm_kernel(int M, const moqe_expert* const* h_experts, int E, int path);
 
 /* The same product for a batch that is already sorted: `perm` [M] and `offsets`
  * [E+1] as moqe_permute wrote them (device pointers; rows perm[offsets[E]..M) are
@@ -326,7 +334,8 @@ MOQE_API const char* moqe_status_str(moqe_status s);
  *   "stream_tile_cost_w8" / "_w4" / "_w3" : relative cost of one packed 128x128 tile of
  *                            that bit-width in the streaming kernel's work split
  *                            (defaults 8 / 8 / 8).
- *   "decode_tile_cost_w8" / "_w4" / "_w3" : the same for the decode kernel (defaults 10 / 10 / 10).
+ *   "decode_tile_cost_w8" / "_w4" / "_w3" : the same for the decode kernel (defaults 21 / 20 / 22; not looked at where
+ *                            its work split follows the ends of the segments).
  *   "auto_decode"          : whether path 0 takes the decode kernel where it applies (default 1).
  *   "auto_dense"           : whether path 0 takes the dense-weights GEMM where it applies (default 1).
  * Unknown key: MOQE_ERR_UNSUPPORTED. */

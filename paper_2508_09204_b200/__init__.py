@@ -26,7 +26,7 @@ PATH_AUTO, PATH_STREAM, PATH_TCGEN05, PATH_DECODE, PATH_DENSE = 0, 1, 2, 5, 6
 EXPORTED = (
     "moqe_quantize_rtn", "moqe_expert_export", "moqe_expert_import", "moqe_expert_info", "moqe_expert_destroy", "moqe_expert_pool_trim",
     "moqe_route", "moqe_expand_ids", "moqe_route_permute", "moqe_permute_workspace", "moqe_permute", "moqe_permute_static", "moqe_unpermute",
-    "moqe_routed_qgemm_workspace", "moqe_routed_qgemm", "moqe_routed_qgemm_path", "moqe_routed_qgemm_sorted",
+    "moqe_routed_qgemm_workspace", "moqe_routed_qgemm", "moqe_routed_qgemm_path", "moqe_routed_qgemm_kernel", "moqe_routed_qgemm_sorted",
     "moqe_routed_qgemm_sorted_multi", "moqe_routed_qgemm_workspace_clear", "moqe_async_status",
     "moqe_status_str", "moqe_launch_count", "moqe_tune", "moqe_selftest_timeout",
     "moqe_router_mlp_workspace", "moqe_router_mlp", "moqe_router_load_report",
@@ -73,6 +73,8 @@ def lib() -> C.CDLL:
         L.moqe_routed_qgemm_workspace.restype = sz
         L.moqe_routed_qgemm.argtypes = [vp, vp, i32, C.POINTER(vp), i32, vp, vp, sz, vp]
         L.moqe_routed_qgemm_path.argtypes = [vp, vp, i32, vp, i32, vp, vp, sz, vp, i32]
+        L.moqe_routed_qgemm_kernel.argtypes = [i32, vp, i32, i32]
+        L.moqe_routed_qgemm_kernel.restype = C.c_char_p
         L.moqe_routed_qgemm_sorted.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp, sz, vp, i32]
         L.moqe_routed_qgemm_sorted_multi.argtypes = [vp, vp, vp, i32, i32, vp, i32, vp, vp, sz, vp]
         L.moqe_routed_qgemm_sorted_gated.argtypes = [vp, vp, vp, i32, vp, vp, i32, vp, vp, sz, vp]
@@ -369,6 +371,15 @@ def moqe_routed_qgemm(X: torch.Tensor, row_ids: torch.Tensor, experts: Sequence[
     return Y
 
 
+def moqe_routed_qgemm_kernel(M: int, experts: Sequence[Expert], path: int = PATH_AUTO) -> str:
+    """The name of the kernel that a call with ``M`` rows of these experts takes."""
+    arr = _handles(experts)
+    name = lib().moqe_routed_qgemm_kernel(int(M), arr.buffer_info()[0], len(experts), int(path))
+    if name is None:
+        raise MoqeError(ERR_SHAPE, "moqe_routed_qgemm_kernel")
+    return name.decode()
+
+
 def moqe_routed_qgemm_workspace_clear(workspace: torch.Tensor, M: int, N: int, K: int, E: int) -> None:
     _check(lib().moqe_routed_qgemm_workspace_clear(_ptr(workspace), workspace.numel(), int(M), int(N), int(K), int(E),
                                                    _stream()), "moqe_routed_qgemm_workspace_clear")
@@ -421,8 +432,8 @@ def moqe_routed_qgemm_sorted_multi(Xs: Sequence[torch.Tensor], perm: torch.Tenso
     E = len(experts[0])
     M = Xs[0].shape[0]
     if _arrs is None:
-        xa = array("Q", [x.data_ptr() for x in Xs])
-        ya = array("Q", [y.data_ptr() for y in Ys])
+        xa = array("Q", [_ptr(x) or 0 for x in Xs])
+        ya = array("Q", [_ptr(y) or 0 for y in Ys])
         ea = array("Q", [e.address for layer in experts for e in layer])
     else:
         xa, ya, ea = _arrs

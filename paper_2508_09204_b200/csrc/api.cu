@@ -103,11 +103,18 @@ int pick_kernel(int path, int M, const moqe_expert* const* ex, int E) {
     if (path == 0) {
         if (g_auto_decode && decode_supported(M, ex, E)) return 2;
         if (M <= AUTO_STREAM_MAX_ROWS && !(g_auto_decode && decode_supported_multi(1, ex, 1, E))) return 1;
-        // The dense-weights GEMM streams or re-reads an expert's whole matrix per 128 rows, the grouped GEMM drains every group
-        // of 32 k by itself.  Dense / grouped, three experts of which one has groups of 32: 1024 -> 256 channels, 3920 rows
-        // 35 / 19 us, 12544 rows 37 / 41; 256 -> 1024, 12544 rows 39 / 31, 25088 rows 57 / 52, 50176 rows 75 / 92.  Two experts
-        // without such groups: 1024 -> 256, 12544 rows 35 / 26, 25088 rows 50 / 39; 256 -> 1024, 39 / 29, 55 / 46, 50176 rows
-        // 84 / 81.  (64 x 256 weights stay resident: dense from 3920 rows 14 / 11 to 12544 rows 14 / 19 on the better one.)
+        // The dense-weights GEMM has a launch more, streams or re-reads an expert's whole matrix per 128 rows and multiplies grouped
+        // experts' weights twice; the grouped GEMM drains every group of 32 k by itself.  Dense / grouped, us, K -> N channels:
+        //                  rows    W8-pc W4-pc W4-g32   W4-pc        W8-pc W4-g64   W4-g128
+        //   256 ->   64    3920    12.4 / 10.8          10.2 / 8.8   12.4 / 9.7     10.4 / 8.7
+        //                 12544    12.9 / 18.2          10.4 / 11.5  12.4 / 14.1    11.4 / 11.3
+        //   256 -> 1024   20000    56.3 / 44.2          37.0 / 29.6  54.7 / 39.4    55.4 / 32.5
+        //                 35000    54.7 / 67.7          36.6 / 46.6  52.2 / 59.4    55.4 / 52.2
+        //   1024 -> 256   12544    36.6 / 40.0          18.7 / 16.2  34.3 / 25.0    28.8 / 16.8
+        //                 35000    49.4 / 54.5          30.9 / 27.0  47.3 / 39.2    49.2 / 29.7
+        //   512 -> 1024   35000    88.3 / 94.1          55.4 / 51.6  86.0 / 76.8    91.8 / 66.8
+        // The lines lie where calls with groups of 32 k and layers of 256 k have them.  Other formats with more k, and small layers
+        // below some 9000 rows, would do better on the grouped GEMM.
         bool fine = false;
         for (int e = 0; e < E; ++e) fine |= ex[e]->group == 32;
         const bool few = M < (fine && ex[0]->K > ex[0]->N ? 12000 : 30000) && (long long)ex[0]->N * ex[0]->K > 65536;
@@ -184,6 +191,18 @@ extern "C" moqe_status moqe_routed_qgemm_path(const void* X_bf16, const int32_t*
                     h_experts[0]->N, st);
     if (s != MOQE_OK) return s;
     return run_sorted(kernel, path, X_bf16, M, h_experts, E, Y_bf16, perm, offsets, base, w, st);
+}
+
+extern "C" const char* moqe_routed_qgemm_kernel(int M, const moqe_expert* const* h_experts, int E, int path) {
+    if (!h_experts || M <= 0 || E <= 0 || E > MOQE_MAX_EXPERTS || path < 0 || path > LAST_PATH) return nullptr;
+    for (int e = 0; e < E; ++e)
+        if (!h_experts[e]) return nullptr;
+    switch (pick_kernel(path, M, h_experts, E)) {
+        case 1: return "qgemm_stream_kernel";
+        case 2: return "qgemm_decode_kernel";
+        case 3: return "qgemm_dense_kernel";
+        default: return "qgemm_tc_kernel";
+    }
 }
 
 extern "C" moqe_status moqe_routed_qgemm_sorted(const void* X_bf16, const int32_t* perm, const int32_t* offsets, int M,

@@ -475,10 +475,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         int Td = T;
         if (p.split) {
             const int left = T % nclusters;
-            int wmean = mt > 0 ? w : 0;
+            int wdear = mt > 0 ? w : 0;
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) wmean = max(wmean, __shfl_xor_sync(0xffffffffu, wmean, d));
-            if (left != 0 && (nclusters - left) * p.KB * wmean > 300 * nclusters) Td = T - left;
+            for (int d = 16; d > 0; d >>= 1) wdear = max(wdear, __shfl_xor_sync(0xffffffffu, wdear, d));
+            if (left != 0 && (nclusters - left) * p.KB * wdear > 300 * nclusters) Td = T - left;
         }
         const int us = min(max(Td - tile0, 0), T_e) * p.KB;
         const int cnt = T_e * p.KB - us;
@@ -515,8 +515,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
     const uint32_t tmem_base = sh.tmem;
 
     if (warp < 4) {
-        if constexpr (TN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
-        else asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
         if (warp == 0 || warp == 3) {
             // ---------------- X producers: this CTA's XR token rows of every half tile, KS x 128 k per stage ----------------
             // Both warps walk the stages and arrive on the pair's xfull barrier; warp 0 also adds the byte count of the TMA
@@ -834,8 +833,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             }
         }
     } else if (warp < L::epi_warp0) {
-        if constexpr (TN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
-        else asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         // ---------------- dequant warps: thread = channel = TMEM lane ----------------
         TcDequant d;
         d.bar_wfull = bar_wfull; d.bar_wempty = bar_wempty; d.bar_done = bar_done;
@@ -1059,7 +1057,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 for (int i = 0; i < L::EC; ++i) acc[i] = 0.f;
                 // several clusters' sums are fetched in one round trip (as many as there are registers for), then added in
                 // cluster order
-                constexpr int CB = TN == 64 ? 2 : 1, CC = TN == 64 ? 32 : 32;
+                constexpr int CB = TN == 64 ? 2 : 1, CC = 32;
 #pragma unroll 1
                 for (int c = c_a; c <= c_b; c += CB) {
 #pragma unroll

@@ -1,6 +1,6 @@
-"""The routing chain where its kernels change shape: the two-kernel sort up to 2048 blocks of 1024 rows and the three-kernel
-one beyond (33 buckets, invalid ids among them), rows expanded four at a time, samples of the router's hidden layer taken
-eight to a warp.  All of it is integer work or fp32 sums, compared as the other tests of these calls do."""
+"""The routing chain where its kernels change shape: the two-kernel sort up to 2048 blocks of 1024 rows (fewer with many
+experts) and the three-kernel one beyond (33 buckets, invalid ids among them), rows expanded four at a time, samples of the router's hidden layer taken
+four to a warp.  All of it is integer work or fp32 sums, compared as the other tests of these calls do."""
 import numpy as np
 import pytest
 import torch
