@@ -621,11 +621,12 @@ moqe_status launch_quantize(const moqe_expert* e, const float* W, cudaStream_t s
 // Whether an expert is built by quantize_pack_kernel, or by the two kernels before it.  Groups within a k-block are.  A per-channel
 // expert's strip of 16 rows belongs to one block there, which goes over it twice: that wants strips for every SM to the last
 // round, and short enough to be in L2 the second time.  Two kernels / one, device time in us, 8 bit: 11008 rows (688 strips on 148
-// SMs) x 4096 113 / 102, x 11008 267 / 296; 3072 rows (192 strips) x 4096 36 / 44; 128 rows x 11008 23 / 60.
+// SMs) x 4096 113 / 102, x 11008 267 / 296; 3072 rows (192 strips) x 4096 36 / 44; 128 rows x 11008 23 / 60.  Rows of up to 1024
+// are over before the second launch would start (128 x 1024 18 / 12, 11008 x 1024 34 / 33).
 bool one_kernel(const moqe_expert* e) {
     if (e->group != 0) return e->group <= 128;
     const int strips = e->Np / 16, sms = device_sm_count(), rounds = (strips + sms - 1) / sms;
-    return e->K <= 5120 && strips * 10ll >= 9ll * sms * rounds;
+    return e->K <= 1024 || (e->K <= 5120 && strips * 10ll >= 9ll * sms * rounds);
 }
 
 template <bool FROM_CODES>
@@ -666,8 +667,10 @@ extern "C" moqe_status moqe_quantize_rtn(const float* W, int N, int K, int bits,
         *out = e;
         return MOQE_OK;
     }
-    s = clear_expert(e, st);
-    if (s != MOQE_OK) { moqe_expert_destroy(e); return s; }
+    if (e->N != e->Np || e->K != e->Kp) {                // (without padding the two kernels write every byte as well)
+        s = clear_expert(e, st);
+        if (s != MOQE_OK) { moqe_expert_destroy(e); return s; }
+    }
     long long warps = (long long)N * e->G;
     unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
     rtn_scales_kernel<<<blocks, 256, 0, st>>>(W, N, K, bits, group, e->G, e->sym, e->Kp / 128, e->tiles, e->scales_pc,
