@@ -32,6 +32,22 @@ int* device_status_word() {
     return g_status_words[dev].load(std::memory_order_relaxed);
 }
 
+int* device_status_word_if() {
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? g_status_words[dev].load(std::memory_order_acquire) : nullptr;
+}
+
+EncodeTiledFn encode_tiled_fn() {
+    static const EncodeTiledFn fn = []() -> EncodeTiledFn {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+            return (EncodeTiledFn)f;
+        return nullptr;
+    }();
+    return fn;
+}
+
 int device_sm_count() {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;

@@ -39,6 +39,7 @@
 // (the integer zero-point; symmetric experts use 2^(bits-1)).  Per-channel experts have no
 // per-tile meta: their scales / zero-points are plain [Np] arrays.
 #pragma once
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -97,10 +98,15 @@ namespace moqe {
 
 // first device-detected error of this device (0 = none); kernels latch with atomicCAS
 int* device_status_word();                 // allocates on first use for the current device
+int* device_status_word_if();              // ... nullptr if that has not happened yet (under a stream capture it may not)
 int device_sm_count();                     // of the current device (148 if it cannot be asked)
 // cudaFuncAttributeMaxDynamicSharedMemorySize of a kernel, set once per device: `done` is the kernel's own word of flags
 bool ensure_dynamic_smem(const void* kernel, int bytes, std::atomic<unsigned long long>& done);
 void count_launch(unsigned n = 1);
+// cuTensorMapEncodeTiled, nullptr if the driver has none
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn encode_tiled_fn();
 
 inline moqe_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? MOQE_OK : MOQE_ERR_CUDA; }
 

@@ -429,19 +429,6 @@ __global__ void __launch_bounds__(DN_THREADS, 1) qgemm_dense_kernel(const __grid
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn dn_encode_fn() {
-    static const EncodeTiledFn fn = []() -> EncodeTiledFn {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
-            return (EncodeTiledFn)f;
-        return nullptr;
-    }();
-    return fn;
-}
 bool dn_map(EncodeTiledFn enc, CUtensorMap* m, const void* base, size_t rows, size_t cols, unsigned box_rows = 64) {
     cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t gstride[1] = {(cuuint64_t)cols * 2};
@@ -473,7 +460,7 @@ moqe_status launch_qgemm_dense(const void* X, int M, int N, int K, const moqe_ex
     if (!dense_supported(M, N, K, ex, E)) return MOQE_ERR_UNSUPPORTED;
     const int Np = ex[0]->Np, Kp = ex[0]->Kp;
     if (!ws || ws_bytes < dense_workspace_bytes(M, K, E, Np, Kp)) return MOQE_ERR_WORKSPACE;
-    EncodeTiledFn enc = dn_encode_fn();
+    EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return MOQE_ERR_CUDA;
     char* base = (char*)ws;
     uint16_t* Wd = (uint16_t*)base;

@@ -1126,21 +1126,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-    static const EncodeTiledFn fn = []() -> EncodeTiledFn {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
-            return (EncodeTiledFn)f;
-        return nullptr;
-    }();
-    return fn;
-}
-
 // columns of a parked partial sum: no tile has more tokens than the batch
 int tc_cols(int M) { return M >= 256 ? 256 : (M + 31) / 32 * 32; }
 
@@ -1158,7 +1143,7 @@ moqe_status launch_qgemm_tc(const void* X, int M, int N, int K, const moqe_exper
                             cudaStream_t st) {
     if (M == 0) return MOQE_OK;
     if (!ws || ws_bytes < tc_workspace_bytes(M, K, E, ex[0]->Np)) return MOQE_ERR_WORKSPACE;
-    EncodeTiledFn enc = encode_fn();
+    EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return MOQE_ERR_CUDA;
     // Tile by batch size (the routing is not known here): LLaMA blocks, three experts, rows dealt evenly, 64 / 128 / 256
     // tokens: 192 rows 235 / 275 / 302 us, 256 rows 367 / 299 / 318, 384 rows 383 / 323 / 346, 512 rows 474 / 489 / 414.

@@ -3,15 +3,16 @@
 // Section 3.1 of the paper: the experts are quantized variants of one
 // full-precision model, built once and frozen.  The quantizer is affine
 // round-to-nearest per (output channel, group of input features); see moqe.h
-// for the exact arithmetic.  Every fp32 operation below is a single IEEE
-// operation (explicit __f*_rn intrinsics, no fused multiply-add, no fast
-// math), so codes, scales and zero-points are reproducible bit for bit.
+// for the exact arithmetic.  What decides a code, scale or zero-point is a single
+// IEEE operation (explicit __f*_rn intrinsics, no fast math; see round_chunk),
+// so they are reproducible bit for bit.
 #include <cstdio>
 #include <cstring>
 #include <mutex>
 #include <new>
 
 #include "dequant.cuh"
+#include "ptx.cuh"
 
 namespace moqe {
 namespace {
@@ -272,44 +273,207 @@ __global__ void encode_pack_kernel(const float* __restrict__ W, const uint8_t* _
 }
 
 // ---------------------------------------------------------------------------
-// K1: scales, zero-points, codes and packing in one kernel, for per-channel experts and groups within a k-block
-// (others take K1a and K1b above, see one_kernel).  Bound by the fp32 weights' bytes, which are read from HBM once: a warp holds
-// the 16 channels x 128 k of a blob in registers between finding the groups' extremes and rounding.  A per-channel
-// expert's block goes over its 16 rows twice, the second time out of L2 (16 rows are 256 KB at K = 4096).  Every byte of
-// the tiles is written here, padding included.  11008 x 4096, 4-bit g128: 57 us (the two kernels: 92 + 60); three blocks
-// to an SM (four: 54 us, but 3-bit g64 68 instead of 65; the loads through shared memory, a half piece ahead: 69).
+// K1: scales, zero-points, codes and packing in one kernel: quantize_group_kernel for groups within a k-block,
+// quantize_channel_kernel for per-channel experts (wider groups, and some of those, take K1a and K1b above, see one_kernel).
+// Every byte of the tiles is written here, padding included.
 // ---------------------------------------------------------------------------
-// rint(w / s) as IEEE division and rounding give it, from a multiplication by 1 / s.  The product is off by at most
-// 2^-22 of its size; only where it comes that close to the middle between two integers does the division decide.
-// Adding 1.5 * 2^23 rounds to the nearest even integer and leaves it in the low bits: no conversion instructions, which
-// run at a quarter of the rate.
+__device__ __forceinline__ uint64_t pack_f2(float lo, float hi) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; }
+__device__ __forceinline__ float2 unpack_f2(uint64_t v) { float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v)); return r; }
+__device__ __forceinline__ uint64_t fma_f2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+
+// what rounding a chunk of 8 weights needs of its group.  safe: no |w / s| of the group is large (see round_chunk)
+struct Rounding { float s, inv; int z; bool safe; };
 template <int BITS>
-__device__ __forceinline__ void round_chunk(const float (&w)[8], float s, float inv, int (&q)[8]) {
-    constexpr float SIZE = (float)(1 << (BITS + 1)), MAGIC = 12582912.f;
-    bool slow = false;
+__device__ __forceinline__ Rounding rounding(const GroupGrid& g, float top) {
+    const float inv = __frcp_rn(g.s);
+    return {g.s, inv, g.z, top * inv < (float)(1 << (BITS + 1))};
+}
+// Codes of a chunk, in pairs of 16 bits: clamp(rint(w / s) + z) as IEEE division and rounding give rint(w / s), from a
+// multiplication by 1 / s.  Adding 1.5 * 2^23 + z rounds w * inv to the nearest integer and leaves code and zero-point added up
+// in the low bits: no conversion instructions, which run at a quarter of the rate.  The product is off by at most 2^-22 of its
+// size; only where it comes that close to the middle between two integers (or is large) does the division decide.
+template <int BITS>
+__device__ __forceinline__ void round_chunk(const float* w, const Rounding& g, bool sym, uint32_t* pair) {
+    constexpr int L = (1 << BITS) - 1, half_code = 1 << (BITS - 1);
+    const float magic = 12582912.f + (float)g.z;                        // (a symmetric grid's z is half_code)
+    const uint64_t inv2 = pack_f2(g.inv, g.inv), magic2 = pack_f2(magic, magic), minus = pack_f2(-1.f, -1.f);
+    float worst = 0.f;
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        const float x = __fmul_rn(w[t], inv), y = __fadd_rn(x, MAGIC), d = __fsub_rn(x, __fsub_rn(y, MAGIC));
-        slow |= !(fabsf(d) < 0.5f - SIZE * 0x1p-21f) || !(fabsf(x) < SIZE);
-        q[t] = __float_as_int(y) - 0x4B400000;
+    for (int j = 0; j < 4; ++j) {
+        const uint64_t x = pack_f2(w[2 * j], w[2 * j + 1]), y = fma_f2(x, inv2, magic2);
+        const float2 yy = unpack_f2(y), d = unpack_f2(fma_f2(x, inv2, fma_f2(y, minus, magic2)));     // d: the product less its integer
+        worst = fmaxf(worst, fmaxf(fabsf(d.x), fabsf(d.y)));
+        pair[j] = __byte_perm(__float_as_uint(yy.x), __float_as_uint(yy.y), 0x5410u);
     }
-    if (slow) {
+    if (!g.safe || !(worst < 0.5f - (float)(1 << (BITS + 1)) * 0x1p-21f)) {
 #pragma unroll
-        for (int t = 0; t < 8; ++t) q[t] = (int)rintf(__fdiv_rn(w[t], s));
+        for (int j = 0; j < 4; ++j) {
+            const int a = (int)rintf(__fdiv_rn(w[2 * j], g.s)), b = (int)rintf(__fdiv_rn(w[2 * j + 1], g.s));
+            pair[j] = ((uint32_t)min(max(a + g.z, -1), L + 1) & 0xFFFFu) | (uint32_t)min(max(b + g.z, -1), L + 1) << 16;
+        }
+    }
+    constexpr uint32_t L2 = (uint32_t)L * 0x10001u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) pair[j] = sym ? __vmins2(__vmaxs2(pair[j], 0x10001u), L2) : __vimin_s16x2_relu(pair[j], L2);
+    static_assert(half_code >= 2, "a symmetric code is at least 1");
+}
+// the packed words of a piece from its codes in pairs (2 i, 2 i + 1): see encode_piece
+template <int BITS>
+__device__ __forceinline__ void encode_pairs(const uint32_t (&c)[16], uint32_t (&w)[PieceWords<BITS>::n]) {
+    if constexpr (BITS == 8) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[j] = __byte_perm(c[2 * j], c[2 * j + 1], 0x6420u);
+    } else if constexpr (BITS == 3) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            w[j] = c[5 * j];
+#pragma unroll
+            for (int f = 1; f < 5; ++f) w[j] |= c[5 * j + f] << (3 * f);
+            w[j] |= (c[15] >> j & 0x10001u) << 15;
+        }
+    } else {
+        constexpr int F = 16 / BITS;                                    // pairs to a word
+#pragma unroll
+        for (int j = 0; j < 16 / F; ++j) {
+            w[j] = c[F * j];
+#pragma unroll
+            for (int f = 1; f < F; ++f) w[j] |= c[F * j + f] << (BITS * f);
+        }
     }
 }
 
+// Groups of 32, 64 or 128 k.  Bound by the fp32 weights' bytes, read once.  A warp takes one blob, 16 channels x 128 k, after
+// another, an unrelated one each time; the next two are on their way into its own two stages of shared memory (four boxes of 32
+// k x 16 rows each: with the 128-byte swizzle a quarter-warp's eight rows fall on different banks), so that loads are always in
+// flight and take no registers.  One block of 12 warps to an SM: 192 KB of stages.  11008 x 4096, 4-bit g128, built and exported:
+// 90.7 -> 76.4 us against 24 warps an SM that load into registers and wait (of the 57 us that took, 31 are the weights' bytes).
+constexpr int QG_WARPS = 12, QG_STAGES = 2, QG_STAGE = 16 * 128 * 4;
+constexpr int QG_SMEM = 1024 + QG_WARPS * QG_STAGES * QG_STAGE;
 template <int BITS>
-__global__ void __launch_bounds__(256, 3) quantize_pack_kernel(const float* __restrict__ W, int N, int K, int group /* 0, 32, 64 or 128 */, int sym, int KB,
-                                                            uint8_t* __restrict__ tiles, __half* __restrict__ scales_pc,
-                                                            __nv_bfloat16* __restrict__ zeros_pc) {
-    constexpr int L = (1 << BITS) - 1, half_code = 1 << (BITS - 1), qmax = half_code - 1;
+__global__ void __launch_bounds__(QG_WARPS * 32, 1) quantize_group_kernel(const __grid_constant__ CUtensorMap wmap, int N, int K, int group, int sym, int KB,
+                                                                     long long blobs, uint8_t* __restrict__ tiles, int* status) {
+    extern __shared__ unsigned char q_smem[];
+    __shared__ unsigned long long bars[QG_WARPS * QG_STAGES];
+    __shared__ int s_abort;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t smem0 = (smem_u32(q_smem) + 1023u & ~1023u) + warp * (QG_STAGES * QG_STAGE), bar0 = smem_u32(bars) + warp * QG_STAGES * 8;
+    if (threadIdx.x == 0) s_abort = 0;
+    if (lane == 0)
+        for (int i = 0; i < QG_STAGES; ++i) mbar_init(bar0 + 8 * i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    __syncthreads();
+    const int q = lane >> 3, r = (lane & 7) ^ (2 * q);                  // this lane's slot: piece (q, r) of both halves
+    const int stride = moqe_tile_stride(BITS, group, !sym), per = moqe_groups_per_tile(group), meta_g = moqe_meta_group_bytes(!sym);
+    auto partner = [&](int d) { const int p = q ^ d; return p * 8 + (r ^ (2 * p)); };      // the lane that holds (q ^ d, r)
+    const long long step = (long long)gridDim.x * QG_WARPS;
+    auto fetch = [&](long long u, int stage) {                          // (by one lane)
+        const long long strip = u / KB;
+        const int k0 = (int)(u - strip * KB) * 128;
+        mbar_expect_tx(bar0 + 8 * stage, QG_STAGE);
+#pragma unroll
+        for (int G = 0; G < 4; ++G)
+            asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                         ::"r"(smem0 + stage * QG_STAGE + G * (QG_STAGE / 4)), "l"(&wmap), "r"(k0 + 32 * G), "r"((int)strip * 16), "r"(bar0 + 8 * stage) : "memory");
+    };
+    const long long u0 = (long long)warp * gridDim.x + blockIdx.x;
+    if (lane == 0)
+        for (int i = 0; i < QG_STAGES; ++i)
+            if (u0 + i * step < blobs) fetch(u0 + i * step, i);
+    __syncwarp();
+    int n = 0;
+#pragma unroll 1
+    for (long long u = u0; u < blobs; u += step, ++n) {
+        const int stage = n % QG_STAGES;
+        if (!__all_sync(0xffffffffu, mbar_wait_short(bar0 + 8 * stage, n / QG_STAGES & 1u, &s_abort, status))) break;
+        const long long strip = u / KB;
+        const int kb = (int)(u - strip * KB), nt = (int)(strip >> 3), nb = (int)(strip & 7);
+        uint8_t* tile = tiles + ((size_t)nt * KB + kb) * (size_t)stride;
+        const bool inside = nt * 128 + nb * 16 + 16 <= N && kb * 128 + 128 <= K;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int row = nt * 128 + nb * 16 + 8 * h + r;
+            float v[32];                                                // (zeros outside of W)
+#pragma unroll
+            for (int G = 0; G < 4; ++G)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const uint32_t at = smem0 + stage * QG_STAGE + G * (QG_STAGE / 4) + (8 * h + r) * 128 + (((2 * q + i) ^ r) << 4);
+                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                 : "=f"(v[8 * G + 4 * i]), "=f"(v[8 * G + 4 * i + 1]), "=f"(v[8 * G + 4 * i + 2]), "=f"(v[8 * G + 4 * i + 3]) : "r"(at));
+                }
+            float lo[4], hi[4];
+#pragma unroll
+            for (int G = 0; G < 4; ++G) {
+                lo[G] = hi[G] = 0.f;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) { lo[G] = fminf(lo[G], v[8 * G + t]); hi[G] = fmaxf(hi[G], v[8 * G + t]); }
+            }
+            if (per < 4) {
+                lo[0] = fminf(lo[0], lo[1]); hi[0] = fmaxf(hi[0], hi[1]);
+                lo[2] = fminf(lo[2], lo[3]); hi[2] = fmaxf(hi[2], hi[3]);
+            }
+            if (per == 1) { lo[0] = fminf(lo[0], lo[2]); hi[0] = fmaxf(hi[0], hi[2]); }
+            Rounding g[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (j < per) {
+                    float l = lo[0], t = hi[0];
+                    if (j > 0) {
+                        l = per == 2 ? lo[2] : (j == 1 ? lo[1] : (j == 2 ? lo[2] : lo[3]));
+                        t = per == 2 ? hi[2] : (j == 1 ? hi[1] : (j == 2 ? hi[2] : hi[3]));
+                    }
+#pragma unroll
+                    for (int d = 1; d < 4; d <<= 1) {
+                        l = fminf(l, __shfl_sync(0xffffffffu, l, partner(d)));
+                        t = fmaxf(t, __shfl_sync(0xffffffffu, t, partner(d)));
+                    }
+                    const float top = fmaxf(-l, t);                     // (max |w|)
+                    const GroupGrid gg = group_grid(l, t, top, BITS, sym);
+                    const Rounding rr = rounding<BITS>(gg, top);
+#pragma unroll
+                    for (int G = 0; G < 4; ++G)
+                        if (per == 1 || (per == 2 ? (G >> 1) == j : G == j)) g[G] = rr;
+                    if (q == 0) {
+                        const bool live = row < N && kb * 128 + j * (128 / per) < K;
+                        uint8_t* m = tile + moqe_tile_bytes(BITS) + j * meta_g + (nb * 16 + 8 * h + r) * 2;
+                        *reinterpret_cast<__half*>(m) = live ? gg.sh : __float2half_rn(0.f);
+                        if (!sym) *reinterpret_cast<__nv_bfloat16*>(m + 256) = __float2bfloat16_rn(live ? (float)gg.z : 0.f);
+                    }
+                }
+            }
+            // (every lane has its values of the second half: its extremes went through the exchange above)
+            if (h == 1 && lane == 0 && u + QG_STAGES * step < blobs) fetch(u + QG_STAGES * step, stage);
+            uint32_t c[16], w[PieceWords<BITS>::n];
+#pragma unroll
+            for (int G = 0; G < 4; ++G) round_chunk<BITS>(v + 8 * G, g[G], sym, c + 4 * G);
+            if (!inside) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    if (row >= N || kb * 128 + 32 * (i >> 2) + 8 * q >= K) c[i] = 0u;      // K % 8 == 0: a chunk is wholly inside or outside
+            }
+            encode_pairs<BITS>(c, w);
+            store_piece<BITS>(tile + nb * moqe_blob_bytes(BITS), h, lane, w);
+        }
+    }
+    if (s_abort) {
+        // let copies that may still be in flight land before the shared memory is released
+        const unsigned long long t0 = global_ns();
+        while (global_ns() - t0 < 200000ull) __nanosleep(1000);
+    }
+}
+
+// Per channel.  A block goes over its 16 rows twice, the second time out of L2 (16 rows are 256 KB at K = 4096); a warp holds the
+// 16 channels x 128 k of a blob in registers between loading and rounding.
+template <int BITS>
+__global__ void __launch_bounds__(256, 3) quantize_channel_kernel(const float* __restrict__ W, int N, int K, int sym, int KB,
+                                                               uint8_t* __restrict__ tiles, __half* __restrict__ scales_pc,
+                                                               __nv_bfloat16* __restrict__ zeros_pc) {
     __shared__ float s_ext[8][2][16];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nt = blockIdx.x >> 3, nb = blockIdx.x & 7;
     const int q = lane >> 3, r = (lane & 7) ^ (2 * q);                  // this lane's slot: piece (q, r) of both halves
     const int row0 = nt * 128 + nb * 16 + r;
-    const int stride = moqe_tile_stride(BITS, group, !sym);
+    const int stride = moqe_tile_stride(BITS, 0, !sym);
     // the lane that holds (q ^ d, r)
     auto partner = [&](int d) { const int p = q ^ d; return p * 8 + (r ^ (2 * p)); };
     auto load = [&](int n, int kb, float (&v)[32]) {
@@ -323,111 +487,53 @@ __global__ void __launch_bounds__(256, 3) quantize_pack_kernel(const float* __re
             v[8 * G + 4] = b.x; v[8 * G + 5] = b.y; v[8 * G + 6] = b.z; v[8 * G + 7] = b.w;
         }
     };
-    // (a symmetric grid needs max |w| only, an asymmetric one min and max; max |w| is the larger of -min and max)
-    GroupGrid pc[2];
-    if (group == 0) {
-        float lo[2] = {0.f, 0.f}, hi[2] = {0.f, 0.f};
-        for (int kb = warp; kb < KB; kb += 8) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float v[32];
-                load(row0 + 8 * h, kb, v);
-#pragma unroll
-                for (int i = 0; i < 32; ++i) { lo[h] = fminf(lo[h], v[i]); hi[h] = fmaxf(hi[h], v[i]); }
-            }
-        }
+    Rounding g[2];
+    float lo[2] = {0.f, 0.f}, hi[2] = {0.f, 0.f};
+    for (int kb = warp; kb < KB; kb += 8) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
+            float v[32];
+            load(row0 + 8 * h, kb, v);
 #pragma unroll
-            for (int d = 1; d < 4; d <<= 1) {
-                lo[h] = fminf(lo[h], __shfl_sync(0xffffffffu, lo[h], partner(d)));
-                hi[h] = fmaxf(hi[h], __shfl_sync(0xffffffffu, hi[h], partner(d)));
-            }
-            if (q == 0) { s_ext[warp][0][8 * h + r] = lo[h]; s_ext[warp][1][8 * h + r] = hi[h]; }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            for (int w = 0; w < 8; ++w) { lo[h] = fminf(lo[h], s_ext[w][0][8 * h + r]); hi[h] = fmaxf(hi[h], s_ext[w][1][8 * h + r]); }
-            pc[h] = group_grid(lo[h], hi[h], fmaxf(-lo[h], hi[h]), BITS, sym);
-            const int n = row0 + 8 * h;
-            if (warp == 0 && q == 0 && blockIdx.y == 0) {
-                scales_pc[n] = n < N ? pc[h].sh : __float2half_rn(0.f);
-                if (!sym) zeros_pc[n] = __float2bfloat16_rn(n < N ? (float)pc[h].z : 0.f);
-            }
+            for (int i = 0; i < 32; ++i) { lo[h] = fminf(lo[h], v[i]); hi[h] = fmaxf(hi[h], v[i]); }
         }
     }
-    const int per = moqe_groups_per_tile(group), meta_g = moqe_meta_group_bytes(!sym);
-    for (int kb = blockIdx.y * 8 + warp; kb < KB; kb += gridDim.y * 8) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int d = 1; d < 4; d <<= 1) {
+            lo[h] = fminf(lo[h], __shfl_sync(0xffffffffu, lo[h], partner(d)));
+            hi[h] = fmaxf(hi[h], __shfl_sync(0xffffffffu, hi[h], partner(d)));
+        }
+        if (q == 0) { s_ext[warp][0][8 * h + r] = lo[h]; s_ext[warp][1][8 * h + r] = hi[h]; }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        for (int w = 0; w < 8; ++w) { lo[h] = fminf(lo[h], s_ext[w][0][8 * h + r]); hi[h] = fmaxf(hi[h], s_ext[w][1][8 * h + r]); }
+        const float top = fmaxf(-lo[h], hi[h]);
+        const GroupGrid gg = group_grid(lo[h], hi[h], top, BITS, sym);
+        g[h] = rounding<BITS>(gg, top);
+        const int n = row0 + 8 * h;
+        if (warp == 0 && q == 0) {
+            scales_pc[n] = n < N ? gg.sh : __float2half_rn(0.f);
+            if (!sym) zeros_pc[n] = __float2bfloat16_rn(n < N ? (float)gg.z : 0.f);
+        }
+    }
+    for (int kb = warp; kb < KB; kb += 8) {
         uint8_t* tile = tiles + ((size_t)nt * KB + kb) * (size_t)stride;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int n = row0 + 8 * h;
             float v[32];
             load(n, kb, v);
-            float s[4], inv[4];
-            int z[4];
-            if (group == 0) {
-                const float iv = __frcp_rn(pc[h].s);
-#pragma unroll
-                for (int G = 0; G < 4; ++G) { s[G] = pc[h].s; inv[G] = iv; z[G] = pc[h].z; }
-            } else {
-                float lo[4], hi[4];
-#pragma unroll
-                for (int G = 0; G < 4; ++G) {
-                    lo[G] = hi[G] = 0.f;
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) { lo[G] = fminf(lo[G], v[8 * G + t]); hi[G] = fmaxf(hi[G], v[8 * G + t]); }
-                }
-                if (per < 4) {
-                    lo[0] = lo[1] = fminf(lo[0], lo[1]); hi[0] = hi[1] = fmaxf(hi[0], hi[1]);
-                    lo[2] = lo[3] = fminf(lo[2], lo[3]); hi[2] = hi[3] = fmaxf(hi[2], hi[3]);
-                }
-                if (per == 1) { lo[0] = fminf(lo[0], lo[2]); hi[0] = fmaxf(hi[0], hi[2]); }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (j < per) {
-                        const int G = per == 4 ? j : (per == 2 ? 2 * j : 0);
-                        float l = lo[0], u = hi[0];
-                        if (G == 1) { l = lo[1]; u = hi[1]; }
-                        if (G == 2) { l = lo[2]; u = hi[2]; }
-                        if (G == 3) { l = lo[3]; u = hi[3]; }
-#pragma unroll
-                        for (int d = 1; d < 4; d <<= 1) {
-                            l = fminf(l, __shfl_sync(0xffffffffu, l, partner(d)));
-                            u = fmaxf(u, __shfl_sync(0xffffffffu, u, partner(d)));
-                        }
-                        const GroupGrid g = group_grid(l, u, fmaxf(-l, u), BITS, sym);
-                        const float iv = __frcp_rn(g.s);
-#pragma unroll
-                        for (int G2 = 0; G2 < 4; ++G2)
-                            if (per == 1 || (per == 2 ? (G2 >> 1) == j : G2 == j)) { s[G2] = g.s; inv[G2] = iv; z[G2] = g.z; }
-                        if (q == 0) {
-                            const bool live = n < N && kb * 128 + j * (128 / per) < K;
-                            uint8_t* m = tile + moqe_tile_bytes(BITS) + j * meta_g + (nb * 16 + 8 * h + r) * 2;
-                            *reinterpret_cast<__half*>(m) = live ? g.sh : __float2half_rn(0.f);
-                            if (!sym) *reinterpret_cast<__nv_bfloat16*>(m + 256) = __float2bfloat16_rn(live ? (float)g.z : 0.f);
-                        }
-                    }
-                }
-            }
-            uint32_t c[32];
+            uint32_t c[16], w[PieceWords<BITS>::n];
 #pragma unroll
             for (int G = 0; G < 4; ++G) {
-                const bool live = n < N && kb * 128 + 32 * G + 8 * q < K;
-                float w8[8];
-                int qi[8];
-#pragma unroll
-                for (int t = 0; t < 8; ++t) w8[t] = v[8 * G + t];
-                round_chunk<BITS>(w8, s[G], inv[G], qi);
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const int code = sym ? max(-qmax, min(qmax, qi[t])) + half_code : max(0, min(L, qi[t] + z[G]));
-                    c[8 * G + t] = live ? (uint32_t)code : 0u;
-                }
+                round_chunk<BITS>(v + 8 * G, g[h], sym, c + 4 * G);
+                if (n >= N || kb * 128 + 32 * G + 8 * q >= K) c[4 * G] = c[4 * G + 1] = c[4 * G + 2] = c[4 * G + 3] = 0u;
             }
-            uint32_t w[PieceWords<BITS>::n];
-            encode_piece<BITS>(c, w);
+            encode_pairs<BITS>(c, w);
             store_piece<BITS>(tile + nb * moqe_blob_bytes(BITS), h, lane, w);
         }
     }
@@ -604,21 +710,47 @@ moqe_status alloc_expert(int N, int K, int bits, int group, int sym, bool clear,
 
 moqe_status launch_quantize(const moqe_expert* e, const float* W, cudaStream_t st) {
     const int KB = e->Kp / 128, strips = e->Np / 16;
-    // a per-channel strip belongs to one block; grouped strips are cut along K as far as they go, a k-block to a warp (so many
-    // small blocks leave no wave half empty: 63 -> 57 us for 688 strips)
-    const int cuts = e->group == 0 ? 1 : (KB + 7) / 8 < 65535 ? (KB + 7) / 8 : 65535;      // (a grid has no more in y)
-    const dim3 grid(strips, cuts);
-#define MOQE_QP(B) quantize_pack_kernel<B><<<grid, 256, 0, st>>>(W, e->N, e->K, e->group, e->sym, KB, e->tiles, e->scales_pc, e->zeros_pc)
-    if (e->bits == 4) MOQE_QP(4);
-    else if (e->bits == 8) MOQE_QP(8);
-    else if (e->bits == 2) MOQE_QP(2);
-    else MOQE_QP(3);
-#undef MOQE_QP
+    if (e->group == 0) {
+#define MOQE_QC(B) quantize_channel_kernel<B><<<strips, 256, 0, st>>>(W, e->N, e->K, e->sym, KB, e->tiles, e->scales_pc, e->zeros_pc)
+        if (e->bits == 4) MOQE_QC(4);
+        else if (e->bits == 8) MOQE_QC(8);
+        else if (e->bits == 2) MOQE_QC(2);
+        else MOQE_QC(3);
+#undef MOQE_QC
+        count_launch();
+        return cuda_ok(cudaGetLastError());
+    }
+    // W[N][K]: boxes of 32 k x 16 rows, 128-byte swizzle, zero fill outside
+    const EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc) return MOQE_ERR_CUDA;
+    int* status = device_status_word_if();
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (!status && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) status = device_status_word();
+    CUtensorMap map;
+    const cuuint64_t dim[2] = {(cuuint64_t)e->K, (cuuint64_t)e->N}, pitch[1] = {(cuuint64_t)e->K * 4};
+    const cuuint32_t box[2] = {32, 16}, es[2] = {1, 1};
+    if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(W), dim, pitch, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return MOQE_ERR_CUDA;
+    const long long blobs = (long long)strips * KB;
+    const int sms = device_sm_count();
+    const unsigned grid = (unsigned)(blobs < sms ? blobs : sms);
+    auto run = [&](auto kernel, std::atomic<unsigned long long>& attr) {
+        if (!ensure_dynamic_smem((const void*)kernel, QG_SMEM, attr)) return false;
+        kernel<<<grid, QG_WARPS * 32, QG_SMEM, st>>>(map, e->N, e->K, e->group, e->sym, KB, blobs, e->tiles, status);
+        return true;
+    };
+    static std::atomic<unsigned long long> attr[4] = {};
+    if (!(e->bits == 4 ? run(quantize_group_kernel<4>, attr[0]) : e->bits == 8 ? run(quantize_group_kernel<8>, attr[1])
+          : e->bits == 2 ? run(quantize_group_kernel<2>, attr[2]) : run(quantize_group_kernel<3>, attr[3]))) {
+        cudaGetLastError();
+        return MOQE_ERR_CUDA;
+    }
     count_launch();
     return cuda_ok(cudaGetLastError());
 }
 
-// Whether an expert is built by quantize_pack_kernel, or by the two kernels before it.  Groups within a k-block are.  A per-channel
+// Whether an expert is built by one kernel, or by the two before them.  Groups within a k-block are.  A per-channel
 // expert's strip of 16 rows belongs to one block there, which goes over it twice: that wants strips for every SM to the last
 // round, and short enough to be in L2 the second time.  Two kernels / one, device time in us, 8 bit: 11008 rows (688 strips on 148
 // SMs) x 4096 113 / 102, x 11008 267 / 296; 3072 rows (192 strips) x 4096 36 / 44; 128 rows x 11008 23 / 60.  Rows of up to 1024

@@ -38,6 +38,18 @@ def test_halfway_weights_and_reused_memory(N, K, bits, group, sym):
     assert_close(torch_to_bits(Y), oracle.routed_gemm(X, ids, [oracle.dequantize(c, s, z, group)]), "product")
 
 
+@pytest.mark.parametrize("bits,group,sym", [(4, 128, False), (3, 64, False), (8, 32, True), (2, 32, False)])
+@pytest.mark.parametrize("N,K", [(8, 128), (2368, 1536), (2360, 1664), (1192, 8192)])
+def test_blobs_to_a_warp(N, K, bits, group, sym):
+    """8 blobs of 16 channels x 128 k for 1776 warps (148 SMs); one each; for some two; two or three, so that stages are filled
+    again.  The channels' sizes go from scales that underflow in fp16 to large ones."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_expert_matches, dev
+    W = wl.weights_f32(f"blobs/{N}/{K}", N, K) * np.exp2(np.arange(N) % 43 - 30).astype(np.float32)[:, None]
+    e = moqe.moqe_quantize_rtn(torch.from_numpy(W).to(dev()), bits, group, sym)
+    assert_expert_matches(e, oracle.quantize_rtn(W, bits, group, sym))
+
+
 @pytest.mark.parametrize("bits,sym", [(8, True), (4, False), (3, False), (2, True)])
 @pytest.mark.parametrize("N,K", [(2296, 1088), (2368, 64), (2056, 1088), (2376, 5128), (2296, 5120), (2048, 1152), (264, 1024), (264, 1032)])
 def test_per_channel_by_one_kernel_and_by_two(N, K, bits, sym):
