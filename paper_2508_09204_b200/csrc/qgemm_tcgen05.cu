@@ -349,8 +349,6 @@ __device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, co
                     }
                 }
             }
-            __syncwarp();
-            mbar_arrive_if(lane == 0, d.bar_wempty + 8 * d.wring.stage);
             // the operand buffer is free once the step NA ago is done
             if (d.step >= L::NA) ok &= warp_wait(d.bar_done + 8 * ((d.step - L::NA) % L::nx), (d.step - L::NA) / L::nx & 1u, &sh.abort, status);
             tc_fence_after();
@@ -366,6 +364,10 @@ __device__ __forceinline__ bool dequant_piece(TcDequant& d, TcShared<TN>& sh, co
             chunk(std::integral_constant<int, 1>{});
             chunk(std::integral_constant<int, 2>{});
             chunk(std::integral_constant<int, 3>{});
+            // The packed tile is handed back only now that its codes have been used: an arrival right behind the loads can overtake
+            // them, and the next tile may land before they are done.
+            __syncwarp();
+            mbar_arrive_if(lane == 0, d.bar_wempty + 8 * d.wring.stage);
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
