@@ -790,43 +790,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                     const uint32_t done = bar_done + 8 * (step % NX);
                     const uint64_t xdesc = umma_desc_sw128(sbase + (step % NX) * L::xstage);
                     // sub-steps: the half tiles of the k-block, or the k-blocks of the step.  Sub-step u is drained by epilogue
-                    // group u (see there).
+                    // group u (see there), so they take turns group by group and both epilogue groups always have a buffer.
                     const int nu = KS == 2 ? nk : nh;
 #pragma unroll 1
-                    for (int u = 0; u < nu; ++u) {
-                        const int h = KS == 2 ? 0 : u, kk = KS == 2 ? u : 0;
-                        const uint32_t a_tmem = tmem_base + L::a_base + ((step % NA) * KS + kk) * TC_A_COLS;
-                        const uint32_t idesc = umma_idesc_pair(half_cols<L::HC>(pc.rows, h));
-                        const uint64_t bdesc = xdesc + u * (L::xhalf / 16);
-                        const bool last = u + 1 == nu;
-                        if (steps == 8) {
+                    for (int i0 = 0; i0 < 8; i0 += steps) {
+#pragma unroll 1
+                        for (int u = 0; u < nu; ++u) {
+                            const int h = KS == 2 ? 0 : u, kk = KS == 2 ? u : 0;
+                            const uint32_t a_tmem = tmem_base + L::a_base + ((step % NA) * KS + kk) * TC_A_COLS + 8 * i0;
+                            const uint32_t idesc = h ? idesc1 : idesc0;
+                            const uint64_t bd = xdesc + u * (L::xhalf / 16) + (i0 >> 2) * (L::XR * 8) + (i0 & 3) * 2;
+                            const uint32_t d = tmem_base + buf * L::HC;
+                            const uint32_t full = u + 1 == nu && i0 + steps == 8 ? done : bar_accfull + 8 * (u * NACC + buf);
                             ok &= warp_wait(bar_accempty + 8 * buf, buf_phase, s_abort, p.status);
                             tc_fence_after();
                             if (elect_one()) {
-                                mma_kblock(tmem_base + buf * L::HC, a_tmem, bdesc, idesc);
-                                umma_commit_pair(last ? done : bar_accfull + 8 * (u * NACC + buf));
+                                if (steps == 8) {
+                                    mma_kblock(d, a_tmem, bd, idesc);
+                                } else {
+                                    umma_pair_ts(d, a_tmem, bd, idesc, 0u);
+                                    umma_pair_ts(d, a_tmem + 8, bd + 2, idesc, 1u);
+                                    if (steps == 4) {
+                                        umma_pair_ts(d, a_tmem + 16, bd + 4, idesc, 1u);
+                                        umma_pair_ts(d, a_tmem + 24, bd + 6, idesc, 1u);
+                                    }
+                                }
+                                umma_commit_pair(full);
                             }
                             __syncwarp();
                             next_buf();
-                        } else {
-#pragma unroll 1
-                            for (int i0 = 0; i0 < 8; i0 += steps) {
-                                ok &= warp_wait(bar_accempty + 8 * buf, buf_phase, s_abort, p.status);
-                                tc_fence_after();
-                                const uint32_t d = tmem_base + buf * L::HC;
-                                const uint64_t bd = bdesc + (i0 >> 2) * (L::XR * 8) + (i0 & 3) * 2;
-                                if (elect_one()) {
-                                    umma_pair_ts(d, a_tmem + 8 * i0, bd, idesc, 0u);
-                                    umma_pair_ts(d, a_tmem + 8 * i0 + 8, bd + 2, idesc, 1u);
-                                    if (steps == 4) {
-                                        umma_pair_ts(d, a_tmem + 8 * i0 + 16, bd + 4, idesc, 1u);
-                                        umma_pair_ts(d, a_tmem + 8 * i0 + 24, bd + 6, idesc, 1u);
-                                    }
-                                    umma_commit_pair(last && i0 + steps == 8 ? done : bar_accfull + 8 * (u * NACC + buf));
-                                }
-                                __syncwarp();
-                                next_buf();
-                            }
                         }
                     }
                     ok = __all_sync(0xffffffffu, ok);
@@ -960,36 +952,53 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 remote_arrive_if(lane == 0, accempty0 + 8 * b, freed);
             };
             int left = nkb;
-            if (!keep && per == 1) {
-                // one buffer a step for this warp (the common formats): the loop is kept short, since a warp gets an
-                // instruction through every nine cycles or so and nothing else of the epilogue runs in parallel
-                const bool by_done = !alone || eg == 1;
+            if (!keep) {
+                // The loop is kept short, since a warp gets an instruction through every nine cycles or so and nothing else of
+                // the epilogue runs in parallel.
+                const bool by_done = !alone || eg == 1;            // announced by the step's own barrier if it is the last group
                 const int mine = alone ? eg : 0, uses = alone ? 2 : 1;
-                auto steps = [&](auto chunks) {
+                auto steps = [&](auto chunks, auto one) {
+                    constexpr bool ONE = decltype(one)::value;     // a group to a k-block (the common formats)
 #pragma unroll 1
                     for (; ok && left >= KS; left -= KS) {
-                        int ob = buf + mine;
-                        if (ob >= NACC) ob -= NACC;
-                        drain(chunks, true, by_done ? bar_done + 8 * (step % NX) : bar_accfull + 8 * ob, by_done ? step / NX & 1u : (full_phase >> ob) & 1u, ob);
-                        if (alone) full_phase ^= 1u << buf;
-                        buf += uses;
-                        if (buf >= NACC) buf -= NACC;
+#pragma unroll 1
+                        for (int g = 1; ; ++g) {
+                            const bool last = ONE || g == per;
+                            int ob = buf + mine;
+                            if (ob >= NACC) ob -= NACC;
+                            const bool dn = by_done && last;
+                            const int fb = ONE ? ob : (mine ? NACC : 0) + ob;
+                            drain(chunks, ONE, dn ? bar_done + 8 * (step % NX) : bar_accfull + 8 * fb, dn ? step / NX & 1u : (full_phase >> fb) & 1u, ob);
+                            if (alone) {
+                                full_phase ^= 1u << buf;
+                                if (!ONE && !last) full_phase ^= 1u << (NACC + (buf + 1 == NACC ? 0 : buf + 1));
+                            } else if (!last) {
+                                full_phase ^= 1u << buf;
+                            }
+                            buf += uses;
+                            if (buf >= NACC) buf -= NACC;
+                            if (last) break;
+                        }
                         ++step;
                         ok = __all_sync(0xffffffffu, ok);
                     }
                 };
-                if constexpr (TN == 256) {
-                    // The number of 32-column chunks is fixed at compile time: no branch between them, and the loads of a chunk
-                    // start before the sums of the last are done (16384 x 11008 x 4096, three LLaMA experts: 1430 -> 1395
-                    // us).  The smaller tiles, with one or two chunks, are faster with the branches (38.3 against 39.0).
-                    const int nch = (dcol + 31) >> 5;
-                    if (nch <= 1) steps(std::integral_constant<int, 1>{});
-                    else if (nch == 2) steps(std::integral_constant<int, 2>{});
-                    else if (nch == 3) steps(std::integral_constant<int, 3>{});
-                    else steps(std::integral_constant<int, 4>{});
-                } else {
-                    steps(std::integral_constant<int, 0>{});
-                }
+                auto run = [&](auto one) {
+                    if constexpr (TN == 256) {
+                        // The number of 32-column chunks is fixed at compile time: no branch between them, and the loads of a chunk
+                        // start before the sums of the last are done (16384 x 11008 x 4096, three LLaMA experts: 1430 -> 1395
+                        // us).  The smaller tiles, with one or two chunks, are faster with the branches (38.3 against 39.0).
+                        const int nch = (dcol + 31) >> 5;
+                        if (nch <= 1) steps(std::integral_constant<int, 1>{}, one);
+                        else if (nch == 2) steps(std::integral_constant<int, 2>{}, one);
+                        else if (nch == 3) steps(std::integral_constant<int, 3>{}, one);
+                        else steps(std::integral_constant<int, 4>{}, one);
+                    } else {
+                        steps(std::integral_constant<int, 0>{}, one);
+                    }
+                };
+                if (per == 1) run(std::true_type{});
+                else run(std::false_type{});
             }
             // The rest: one round per step (every group's buffer is drained, the last one of the step being announced by the
             // step's own barrier), or one for the whole piece (per channel).  The loops are kept rolled: unrolled over the
@@ -1000,7 +1009,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 const int nu = KS == 2 ? (keep ? 1 : min(KS, left)) : nh;
 #pragma unroll 1
                 for (int t = 0; t < nu * per; ++t) {
-                    const int u = t >= per ? 1 : 0;
+                    const int u = nu == 2 ? t & 1 : 0;
                     const bool by_done = !keep && t + 1 == nu * per;
                     const int fb = u * NACC + buf;
                     if (!alone || u == eg)
