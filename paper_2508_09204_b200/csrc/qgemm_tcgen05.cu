@@ -71,6 +71,11 @@ struct TcCfg {
     static constexpr int dq_arrive = KS == 2 ? 8 : 4;                        // dequant warps that fill one weight buffer
     static constexpr int epi_warp0 = 4 + dq_warps;
     static constexpr int threads = (epi_warp0 + TC_EPI) * 32;
+    // registers: what the producers and the dequant warps can do without goes to the epilogue, whose sums must not spill (300 rows in
+    // 128-token tiles, 4-bit g64: 34 us with this split, 39 with 48 / 80 / 136; 2048 rows in 256-token ones, 4-bit g128: 63, and 67 with 56 / 72 / 192)
+    static constexpr int regs_prod = TN == 256 ? 64 : (TN == 128 ? 56 : 48), regs_dq = 80, regs_epi = TN == 256 ? 184 : (TN == 128 ? 128 : 136);
+    static constexpr int regs_launch = TN == 256 ? 128 : 96;
+    static_assert(4 * regs_prod + dq_warps * regs_dq + TC_EPI * regs_epi <= threads / 32 * regs_launch, "setmaxnreg.inc draws on what the block was launched with");
     static constexpr int nx = 4;                                             // token stages: one step of the tile
     // (nx and NA are powers of two: stage and parity follow from the step's number)
     static_assert(NA <= nx, "the dequant warps wait for the step NA ago on its token stage's barrier");
@@ -130,14 +135,15 @@ __device__ __forceinline__ void remote_arrive_if(bool yes, uint32_t cluster_addr
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p mbarrier.arrive.shared::cluster.b64 _, [%0], %1;\n\t}"
                  ::"r"(cluster_addr), "r"(count), "r"((uint32_t)yes) : "memory");
 }
-__device__ __forceinline__ void remote_expect_tx_only(uint32_t cluster_addr, uint32_t bytes) {
-    asm volatile("mbarrier.expect_tx.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(cluster_addr), "r"(bytes) : "memory");
+__device__ __forceinline__ void remote_arrive_expect_tx(uint32_t cluster_addr, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_addr), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void tma_box_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t cluster_bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3}], [%4];"
         ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(cluster_bar) : "memory");
 }
+__device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) { asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory"); }
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t smem_dst, uint32_t cols) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
@@ -448,18 +454,56 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             for (int i = 0; i < 2 * TC_EPI; ++i) mbar_init(bar_xchg + 8 * i, 1);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        prefetch_tmap(&tmap);
     }
     // (the pair's barriers are initialised when both CTAs have arrived here; every role waits for that before it first touches
     // the other CTA, so the round trip hides behind the schedule)
     __syncwarp();
     cluster_arrive();
     if (warp == 1) tmem_alloc_pair(smem_u32(&sh.tmem), 512);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (warp == 0) {
-        // ---- the schedule: lane e works out expert e
+    // ---- the schedule.  Worked out from the offset table as it stands BEFORE the previous kernel is waited for (in a block's
+    // later layers it is final already), so that afterwards the table has only to be compared, while the rows of the first piece
+    // are being looked up; a table that has changed is gone through again.  (It took 1.6 us after the wait and the first rows' places
+    // another 1.0: 96 rows, seven layers of a LLaMA block, 206 -> 197 us with the weights' first tiles asked of L2.)
+    const bool x_warp = warp == 0 || warp == 3;
+    TcPiece x_pc;
+    TcWalk x_wk;
+    bool x_have = false;
+    int x_a[NH], x_b[NH];                                  // a producer lane's rows of X: lane and lane + 32 of each half tile
+    // real rows of this CTA in half tile h of a piece, and the first of them
+    auto x_rows = [&](const TcPiece& pc, int h, int& first_row) {
+        if (h > 0 && pc.rows <= L::HC) return 0;
+        const int per_cta = half_cols<L::HC>(pc.rows, h) >> 1;
+        first_row = h * half_split<L::HC>(pc.rows) + (int)rank * per_cta;
+        return max(min(per_cta, pc.rows - first_row), 0);
+    };
+    auto x_next = [&]() {
+        x_have = x_wk.next(sc, p, nclusters, x_pc);
+        if (!x_have) return;
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            int first_row = 0;
+            const int c = x_rows(x_pc, h, first_row);
+            x_a[h] = lane < c ? __ldcg(p.perm + x_pc.m0 + first_row + lane) : 0;
+            x_b[h] = lane + 32 < c ? __ldcg(p.perm + x_pc.m0 + first_row + lane + 32) : 0;
+        }
+    };
+    auto schedule = [&]() {
+        // lane e works out expert e
         const int e = lane;
-        const int o0 = e < p.E ? __ldcg(p.offsets + e) : 0, o1 = e < p.E ? __ldcg(p.offsets + e + 1) : 0;
+        // (a table that is still being written may hold anything: offsets are made to rise and to stay within the batch)
+        int o1 = e < p.E ? min(max(__ldcg(p.offsets + e + 1), 0), p.M) : 0;
+        int o0 = e == 0 ? min(max(__ldcg(p.offsets), 0), p.M) : 0;
+        o1 = max(o0, o1);
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, o1, d);
+            if (lane >= d) o1 = max(o1, o);
+        }
+        {
+            const int o = __shfl_up_sync(0xffffffffu, o1, 1);
+            if (lane > 0) o0 = o;
+        }
         const int R = o1 - o0;
         const int mt = (R + TN - 1) / TN;
         const int rpt = mt >= 4 ? TN : (mt > 0 ? ((R + mt - 1) / mt + 31) & ~31 : 32);
@@ -509,21 +553,53 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         if (e == p.E - 1) { sc.off[p.E] = o1; sc.tile0[p.E] = T; }
         sc.rpt[e] = rpt; sc.us[e] = us; sc.ub[e] = ub; sc.ue[e] = ue; sc.w[e] = w; sc.base[e] = base;
         if (lane == 0) { sc.Gs = Gs; sc.Td = Td; sc.C = C; }
+    };
+#pragma unroll 1
+    for (bool early = true;; early = false) {
+        if (warp == 0) schedule();
+        tc_fence_before();
+        __syncthreads();
+        bool changed = false;
+        if (early) {
+            if (warp == 2 && lane == 0) {
+                // the first packed tiles into L2 (a wrong guess costs prefetched lines only)
+                TcPiece pc;
+                TcWalk wk;
+                wk.start(cluster);
+                if (wk.next(sc, p, nclusters, pc) && 2 * pc.ntp + (int)rank < p.NT1) {
+                    const ExpertDev& ex = p.ex[pc.e];
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(ex.tiles + ((size_t)(2 * pc.ntp + (int)rank) * p.KB + pc.kb0) * ex.tile_stride),
+                                 "r"(min(p.nw, pc.kb1 - pc.kb0) * ex.tile_stride) : "memory");
+                }
+            }
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        }
+        if (x_warp) {
+            x_wk.start(cluster);
+            x_next();
+        } else if (early && warp == 2) {
+            changed = (lane < p.E && __ldcg(p.offsets + lane) != sc.off[lane]) || (lane == 0 && __ldcg(p.offsets + p.E) != sc.off[p.E]);
+        }
+        if (!early || !__syncthreads_or(changed)) break;
     }
-    tc_fence_before();
-    __syncthreads();
     if (warp != 2) cluster_wait();                         // (the weight producer touches its own CTA only)
     tc_fence_after();
     const uint32_t tmem_base = sh.tmem;
 
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(L::regs_prod));
         if (warp == 0 || warp == 3) {
             // ---------------- X producers: this CTA's XR token rows of every half tile, KS x 128 k per stage ----------------
-            // Both warps walk the stages and arrive on the pair's xfull barrier; warp 0 also adds the byte count of the TMA
-            // boxes.  A warp gathers every other pair of rows; its arrival for a stage follows once its copies have landed,
-            // LAG stages later (at once where nothing is gathered).
-            constexpr int LAG = 3;
+            // Both warps walk the stages and arrive on the pair's xfull barrier.  A piece whose rows all come in boxes has a lean
+            // loop: a warp fetches one 64-k sub-tile of every box, its arrival carries the byte count, and nothing is fenced or
+            // waited for (one loop for both kinds took the warp 1170 cycles a step, more than the tensor core's 1024: 2048 rows x
+            // 4096 x 4096, per channel, 57 -> 54 us).  Otherwise both warps gather, every other pair of rows each, with cp.async, and
+            // the arrival for a stage follows once its copies have landed, LAG stages later (2, and before the next piece's rows are
+            // waited for: 1024 rows in runs of 100, three experts, 4096 x 4096, 65 -> 62 us; with 3 67, with 1 also 67 and 300
+            // scattered rows 30 -> 36).  TMA's own gather, four rows to a request, takes an SM 45 cycles a request: those 300 rows
+            // 58 us.  Copies that arrive on a barrier, looked at between stages, cost the other warps their issue slots: 34 us.
+            constexpr int LAG = 2;
             const int gw = warp == 0 ? 0 : 1;
             int* s_xrow = sh.xrow[gw];
             const int hi = lane >> 4, c16 = lane & 15;
@@ -531,9 +607,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             const uint32_t r0 = 2 * gw + hi;
             const uint32_t sw0 = (c16 >> 3) * (L::XR * 128) + r0 * 128 + (((c16 & 7) ^ r0) << 4), sw1 = (c16 >> 3) * (L::XR * 128) + (r0 + 4) * 128 + (((c16 & 7) ^ (r0 + 4)) << 4);
             uint32_t step = 0, due = 0;                    // due: the step whose arrival comes next
-            TcPiece pc;
-            TcWalk wk;
-            wk.start(cluster);
             bool ok = true;
             int pending = 0;
             const uint32_t full0 = mapa(bar_xfull, 0), pitch = (uint32_t)p.K * 2;
@@ -543,88 +616,91 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 remote_arrive_if(lane == 0, full0 + 8 * (due % NX));
                 ++due;
             };
-            while (ok && wk.next(sc, p, nclusters, pc)) {
-                const int nh = NH == 1 ? 1 : (pc.rows > L::HC ? 2 : 1);
-                int src[NH], cnt[NH], bytes = 0;
+            auto arrive_all = [&]() {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                for (; pending > 0; --pending) arrive();
+            };
+            for (; ok && x_have; x_next()) {
+                const TcPiece pc = x_pc;
+                // (the last steps of the piece before: their arrivals must not wait for this one's rows, which are being looked up)
+                arrive_all();
+                int src[NH], cnt[NH], boxes = 0;
                 bool gathers = false;
                 __syncwarp();
 #pragma unroll
                 for (int h = 0; h < NH; ++h) {
-                    src[h] = -1; cnt[h] = 0;
-                    if (h < nh) {
-                        const int per_cta = half_cols<L::HC>(pc.rows, h) >> 1;
-                        const int first_row = h * half_split<L::HC>(pc.rows) + (int)rank * per_cta;
-                        const int c = max(min(per_cta, pc.rows - first_row), 0);         // real rows of this CTA
-                        const int a = lane < c ? __ldcg(p.perm + pc.m0 + first_row + lane) : 0;
-                        const int b = lane + 32 < c ? __ldcg(p.perm + pc.m0 + first_row + lane + 32) : 0;
-                        const int first = __shfl_sync(0xffffffffu, a, 0);
-                        const bool run = __all_sync(0xffffffffu, (lane >= c || a == first + lane) && (lane + 32 >= c || b == first + lane + 32));
-                        s_xrow[h * L::XR + (lane & 3) * (L::XR / 4) + (lane >> 2)] = a;
-                        if (L::XR > 32) s_xrow[h * L::XR + (lane & 3) * (L::XR / 4) + 8 + (lane >> 2)] = b;
-                        // (a box fetches XR rows whatever it needs; operand rows beyond the real ones yield columns that are
-                        // never stored, so they may hold anything)
-                        src[h] = run && 2 * c >= L::XR ? first : -1;
-                        cnt[h] = c;
-                        bytes += src[h] >= 0 ? L::xhalf : 0;
-                        gathers |= src[h] < 0 && c > 0;
-                    }
+                    int first_row = 0;
+                    const int c = x_rows(pc, h, first_row), a = x_a[h], b = x_b[h];
+                    const int first = __shfl_sync(0xffffffffu, a, 0);
+                    const bool run = __all_sync(0xffffffffu, (lane >= c || a == first + lane) && (lane + 32 >= c || b == first + lane + 32));
+                    s_xrow[h * L::XR + (lane & 3) * (L::XR / 4) + (lane >> 2)] = a;
+                    if (L::XR > 32) s_xrow[h * L::XR + (lane & 3) * (L::XR / 4) + 8 + (lane >> 2)] = b;
+                    // (a box fetches XR rows whatever it needs; operand rows beyond the real ones yield columns that are
+                    // never stored, so they may hold anything)
+                    src[h] = c > 0 ? first : -1;
+                    boxes += c > 0 ? 1 : 0;
+                    cnt[h] = c;
+                    gathers |= c > 0 && !(run && c > 8);
                 }
                 __syncwarp();
-                for (int kb0 = pc.kb0; kb0 < pc.kb1; kb0 += KS) {
-                    const int nk = min(KS, pc.kb1 - kb0);
-                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * (step % NX), (step / NX & 1u) ^ 1u, s_abort, p.status)))) break;
-                    const uint32_t full = full0 + 8 * (step % NX);
-                    if (gw == 0 && bytes > 0) {
-                        if (lane == 0) remote_expect_tx_only(full, bytes * nk);
-                        __syncwarp();
+                if (!gathers) {
+#pragma unroll 1
+                    for (int kb0 = pc.kb0; ok && kb0 < pc.kb1; kb0 += KS, ++step) {
+                        const int nk = min(KS, pc.kb1 - kb0);
+                        ok = warp_wait(bar_done + 8 * (step % NX), (step / NX & 1u) ^ 1u, s_abort, p.status);
+                        const uint32_t full = full0 + 8 * (step % NX);
+                        if (elect_one()) {
+                            remote_arrive_expect_tx(full, boxes * nk * (L::XR * 128));
+#pragma unroll
+                            for (int kk = 0; kk < KS; ++kk)
+#pragma unroll
+                                for (int h = 0; h < NH; ++h)
+                                    if (kk < nk && src[h] >= 0)
+                                        tma_box_pair(sbase + (step % NX) * L::xstage + (kk * NH + h) * L::xhalf + gw * (L::XR * 128), &tmap, (kb0 + kk) * 128 + gw * 64, src[h], full);
+                        }
+                        ok = __all_sync(0xffffffffu, ok);
                     }
+                    due = step;
+                    continue;
+                }
+#pragma unroll 1
+                for (int kb0 = pc.kb0; ok && kb0 < pc.kb1; kb0 += KS) {
+                    const int nk = min(KS, pc.kb1 - kb0);
+                    ok = warp_wait(bar_done + 8 * (step % NX), (step / NX & 1u) ^ 1u, s_abort, p.status);
 #pragma unroll
                     for (int kk = 0; kk < KS; ++kk) {
                         if (kk >= nk) break;
-                        const int kb = kb0 + kk;
-                        const uint32_t stage = sbase + (step % NX) * L::xstage + kk * (NH * L::xhalf);
-                        if (gw == 0 && bytes > 0) {
-#pragma unroll
-                            for (int h = 0; h < NH; ++h)
-                                if (src[h] >= 0 && lane < 2) tma_box_pair(stage + h * L::xhalf + lane * (L::XR * 128), &tmap, kb * 128 + lane * 64, src[h], full);
-                            __syncwarp();
-                        }
-                        const int k = kb * 128 + c16 * 8;
+                        const int k = (kb0 + kk) * 128 + c16 * 8;
                         const int real = k < p.K ? 16 : 0;
                         const char* xk = reinterpret_cast<const char*>(p.X) + (real ? (size_t)k * 2 : 0);
 #pragma unroll
                         for (int h = 0; h < NH; ++h) {
-                            if (src[h] < 0) {
-                                const uint32_t dst = stage + h * L::xhalf;
-                                const int4* list = reinterpret_cast<const int4*>(s_xrow + h * L::XR + r0 * (L::XR / 4));
-                                // (no branch per row: a list entry beyond the real rows is row 0, copied in vain)
-#pragma unroll 1
-                                for (int i = 0; 4 * i < cnt[h]; i += 4) {
-                                    const int4 r4 = list[i >> 2];
-                                    const uint32_t d = dst + (i >> 1) * 1024;
-                                    cp_async16(d + sw0, xk + (size_t)(uint32_t)r4.x * pitch, real);
-                                    cp_async16(d + sw1, xk + (size_t)(uint32_t)r4.y * pitch, real);
-                                    cp_async16(d + sw0 + 1024, xk + (size_t)(uint32_t)r4.z * pitch, real);
-                                    cp_async16(d + sw1 + 1024, xk + (size_t)(uint32_t)r4.w * pitch, real);
+                            const uint32_t dst = sbase + (step % NX) * L::xstage + (kk * NH + h) * L::xhalf;
+                            const int4* list = reinterpret_cast<const int4*>(s_xrow + h * L::XR + r0 * (L::XR / 4));
+                            // (no branch per row: a list entry beyond the real rows is row 0, copied in vain)
+#pragma unroll
+                            for (int i = 0; i < L::XR / 16; ++i)
+                                if (16 * i < cnt[h]) {
+                                    const int4 r4 = list[i];
+                                    cp_async16(dst + sw0 + i * 2048, xk + (size_t)(uint32_t)r4.x * pitch, real);
+                                    cp_async16(dst + sw1 + i * 2048, xk + (size_t)(uint32_t)r4.y * pitch, real);
+                                    cp_async16(dst + sw0 + i * 2048 + 1024, xk + (size_t)(uint32_t)r4.z * pitch, real);
+                                    cp_async16(dst + sw1 + i * 2048 + 1024, xk + (size_t)(uint32_t)r4.w * pitch, real);
                                 }
-                            }
                         }
                     }
                     asm volatile("cp.async.commit_group;" ::: "memory");
                     ++step;
-                    ++pending;
-                    if (!gathers) {
-                        asm volatile("cp.async.wait_group 0;" ::: "memory");
-                        for (; pending > 0; --pending) arrive();
-                    } else if (pending == LAG) {
+                    if (++pending == LAG) {
                         asm volatile("cp.async.wait_group %0;" ::"n"(LAG - 1) : "memory");
                         arrive();
                         --pending;
                     }
+                    ok = __all_sync(0xffffffffu, ok);
                 }
             }
+            if (ok) arrive_all();
             asm volatile("cp.async.wait_group 0;" ::: "memory");
-            for (; ok && pending > 0; --pending) arrive();
             // every stage handed back (the commits come from the leading CTA) before this CTA may exit
             for (int i = 0; ok && i < NX; ++i) {
                 ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * (step % NX), (step / NX & 1u) ^ 1u, s_abort, p.status));
@@ -827,7 +903,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             }
         }
     } else if (warp < L::epi_warp0) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(L::regs_dq));
         // ---------------- dequant warps: thread = channel = TMEM lane ----------------
         TcDequant d;
         d.bar_wfull = bar_wfull; d.bar_wempty = bar_wempty; d.bar_done = bar_done;
@@ -859,10 +935,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             }
         }
     } else {
-        if constexpr (TN == 256) asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
-        // (what the producers and the dequant warps can do without: with 120 the sums were spilled in every step; 96 rows x 4096 x
-        // 11008: 42 -> 38 us)
-        else asm volatile("setmaxnreg.inc.sync.aligned.u32 136;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(L::regs_epi));
         // ---------------- epilogue warps: scale-and-accumulate, then store ----------------
         // Two groups of four warps.  Of a tile with two half tiles each group drains one, of a step with two k-blocks each
         // drains one (an accumulator buffer then costs a warp one wait for all its columns); otherwise both drain every

@@ -1,8 +1,78 @@
-"""Grouped GEMM: the hand-over of packed tiles."""
+"""Grouped GEMM: token rows that come in boxes, that are gathered, or both in one tile; a routing that differs from the one whose
+offset table is still in the workspace; the hand-over of packed tiles."""
+import numpy as np
 import pytest
 import torch
 
+import oracle
+import moqe_workloads as wl
+
 pytestmark = pytest.mark.gpu
+
+
+def _rows(M):
+    return np.unique(np.concatenate([np.linspace(0, M - 1, 40).astype(int), [0, M - 1]]))
+
+
+@pytest.mark.parametrize("specs", [((8, 0, True), (4, 128, False), (3, 64, False)), ((4, 32, False), (2, 128, True))])
+@pytest.mark.parametrize("M", [70, 150, 300, 500, 780])
+@pytest.mark.parametrize("runs", [(1,), (8, 9), (100, 31, 5), (4000,)])
+def test_runs_of_rows(M, runs, specs):
+    """Runs of one row are gathered, runs that cover a half tile come in one box (of 9 rows and more), others leave tiles with
+    both; tiles of 64, 128 and 256 tokens."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_close, bf16_to_torch, build_experts, dev, torch_to_bits
+    N, K = 200, 384
+    W, X = wl.weights_f32(f"tcrows/{N}/{K}", N, K), wl.activations_bf16(f"tcrows/{M}/{K}", M, K)
+    experts, What, _ = build_experts(W, specs)
+    ids, e, i = np.zeros(M, np.int32), 0, 0
+    while i < M:
+        n = runs[e % len(runs)]
+        ids[i:i + n] = e % len(specs)
+        i, e = i + n, e + 1
+    Y = moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), experts, path=moqe.PATH_TCGEN05)
+    assert moqe.moqe_async_status() == moqe.OK
+    r = _rows(M)
+    assert_close(torch_to_bits(Y)[r], oracle.routed_gemm(X[r], ids[r], What), f"runs {runs}")
+
+
+@pytest.mark.parametrize("K", [72, 136, 328])
+@pytest.mark.parametrize("run", [1, 64])
+def test_ragged_k(K, run):
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_close, bf16_to_torch, build_experts, dev, torch_to_bits
+    M, N = 200, 136
+    W, X = wl.weights_f32(f"tcrows/{N}/{K}", N, K), wl.activations_bf16(f"tcrows/{M}/{K}", M, K)
+    experts, What, _ = build_experts(W, ((8, 0, True), (4, 0, False)))
+    ids = (np.arange(M) // run % 2).astype(np.int32)
+    Y = moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), experts, path=moqe.PATH_TCGEN05)
+    assert moqe.moqe_async_status() == moqe.OK
+    r = _rows(M)
+    assert_close(torch_to_bits(Y)[r], oracle.routed_gemm(X[r], ids[r], What), f"K {K}")
+
+
+def test_routing_changes_from_call_to_call():
+    """The schedule is worked out ahead from the table that the call before left behind: other counts, experts without rows, and
+    a smaller batch (whose table holds offsets beyond it)."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_close, bf16_to_torch, build_experts, dev, torch_to_bits
+    N, K, E = 520, 512, 3
+    W = wl.weights_f32(f"tcrows/{N}/{K}", N, K)
+    experts, What, _ = build_experts(W, ((8, 0, True), (4, 128, False), (3, 128, False)))
+    g = np.random.default_rng(7)
+    calls = []
+    for M, p in ((900, (1, 0, 0)), (900, (0, 0.5, 0.5)), (400, (0, 0, 1)), (900, (0.1, 0.8, 0.1)), (130, (0.4, 0.3, 0.3)), (880, (0.3, 0.3, 0.4))):
+        ids = g.choice(E, size=M, p=p).astype(np.int32)
+        X = wl.activations_bf16(f"tcrows/{M}/{K}", M, K)
+        calls.append((M, ids, X, bf16_to_torch(X), torch.from_numpy(ids).to(dev()), torch.full((M, N), float("nan"), dtype=torch.bfloat16, device=dev())))
+    ws = moqe.alloc_workspace(max(moqe.moqe_routed_qgemm_workspace(c[0], N, K, E) for c in calls))
+    for _ in range(3):
+        for c in calls:
+            moqe.moqe_routed_qgemm(c[3], c[4], experts, Y=c[5], workspace=ws, path=moqe.PATH_TCGEN05)
+    assert moqe.moqe_async_status() == moqe.OK
+    for M, ids, X, _, _, Y in calls:
+        r = _rows(M)
+        assert_close(torch_to_bits(Y)[r], oracle.routed_gemm(X[r], ids[r], What), f"{M} rows")
 
 
 @pytest.mark.parametrize("spec", [(8, 0, True), (4, 128, False), (3, 64, False)])
