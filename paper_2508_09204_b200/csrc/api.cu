@@ -129,11 +129,16 @@ int pick_kernel(int path, int M, const moqe_expert* const* ex, int E) {
         //   1024 -> 256   12544    36.6 / 40.0          18.7 / 16.2  34.3 / 25.0    28.8 / 16.8
         //                 35000    49.4 / 54.5          30.9 / 27.0  47.3 / 39.2    49.2 / 29.7
         //   512 -> 1024   35000    88.3 / 94.1          55.4 / 51.6  86.0 / 76.8    91.8 / 66.8
-        // The lines lie where calls with groups of 32 k and layers of 256 k have them.  Other formats with more k, and small layers
-        // below some 9000 rows, would do better on the grouped GEMM.
+        // and with more rows, W8-pc W4-g64 (256 images of a bottleneck's layer among them):
+        //   1024 -> 256    50176    69.2 / 53.6    100352 113 / 88
+        //   512 ->  512    50176    71.7 / 59.8    100352 118 / 103
+        //   256 -> 1024    50176    76.1 / 83.6    100352 127 / 156
+        // So rows of 512 k and more are the grouped GEMM's unless a group of 32 k is among the experts.  The other lines lie where
+        // calls with groups of 32 k and layers of 256 k have them.  Small layers below some 4000 rows would do better on the grouped
+        // GEMM (256 -> 64, 980 rows 12.4 / 8.5).
         bool fine = false;
         for (int e = 0; e < E; ++e) fine |= ex[e]->group == 32;
-        const bool few = M < (fine && ex[0]->K > ex[0]->N ? 12000 : 30000) && (long long)ex[0]->N * ex[0]->K > 65536;
+        const bool few = (M < (fine && ex[0]->K > ex[0]->N ? 12000 : 30000) || (!fine && ex[0]->K >= 512)) && (long long)ex[0]->N * ex[0]->K > 65536;
         return (g_auto_dense && !few && dense_supported(M, ex[0]->N, ex[0]->K, ex, E)) ? 3 : 0;
     }
     return 0;

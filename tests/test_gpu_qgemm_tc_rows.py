@@ -97,3 +97,19 @@ def test_repeats_bit_for_bit(spec):
         first = Y[0].clone() if first is None else first
         assert all(torch.equal(y, first) for y in Y)
     assert moqe.moqe_async_status() == moqe.OK
+
+
+@pytest.mark.parametrize("K,group,want", [(512, 64, "qgemm_tc_kernel"), (504, 0, "qgemm_dense_kernel"), (512, 32, "qgemm_dense_kernel")])
+def test_many_rows_of_512_k(K, group, want):
+    """31000 rows: 512 k without groups of 32 go to the grouped GEMM, 504 k and groups of 32 to the dense-weights one."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_close, bf16_to_torch, build_experts, dev, torch_to_bits
+    M, N = 31000, 256
+    W, X = wl.weights_f32(f"tcrows/{N}/{K}", N, K), wl.activations_bf16(f"tcrows/{M}/{K}", M, K)
+    experts, What, _ = build_experts(W, ((8, 0, True), (4, group, False)))
+    ids = (np.arange(M) // 196 % 2).astype(np.int32)
+    assert moqe.moqe_routed_qgemm_kernel(M, experts) == want
+    Y = moqe.moqe_routed_qgemm(bf16_to_torch(X), torch.from_numpy(ids).to(dev()), experts)
+    assert moqe.moqe_async_status() == moqe.OK
+    r = _rows(M)
+    assert_close(torch_to_bits(Y)[r], oracle.routed_gemm(X[r], ids[r], What), f"K {K}")
