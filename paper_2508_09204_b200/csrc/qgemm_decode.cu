@@ -556,21 +556,22 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
 
     // ---- prologue: nothing here depends on the previous kernel in the stream
     if (tid < p.P * 12) reinterpret_cast<int*>(smem + L::ps_off)[tid] = reinterpret_cast<const int*>(p.ps)[tid];
-    if (tid == 0) {
+    if (tid == 32) {                                       // (not by warp 0, whose work split every CTA waits for)
         for (int i = 0; i < GV_MAX_STAGES; ++i) { mbar_init(bar_wfull + 8 * i, 1); mbar_init(bar_wempty + 8 * i, GV_CONS); }
         for (int i = 0; i < 2; ++i) { mbar_init(bar_xfull + 8 * i, GV_SERV * 32); mbar_init(bar_xempty + 8 * i, GV_CONS); }
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // ---- the work split, by warp 0: lane v works out pair v from the offset table (read past L1: the table may be
-    // rewritten by the previous kernel between the two reads below)
-    auto work_split = [&]() {
+    // ---- the work split, by warp 0: lane v works out pair v from the offset table, entry l of it in lane l's `off`, entry 32 in
+    // `last` (read past L1: the table may be rewritten by the previous kernel between the two reads below)
+    auto work_split = [&](int off, int last) {
         const int v = lane;
         long long cost = 0;
         int TT = 0, wv = 1, segs = 0, KBv = 1;
         {
             const PairS q = p.ps[v < p.P ? v : 0];
-            const int rows = __ldcg(p.offsets + q.rexp + 1) - __ldcg(p.offsets + q.rexp);
+            const int from = __shfl_sync(0xffffffffu, off, q.rexp & 31), to = __shfl_sync(0xffffffffu, off, (q.rexp + 1) & 31);
+            const int rows = (q.rexp >= 31 ? last : to) - from;
             wv = q.w;
             segs = (v < p.P && rows > 0) ? ((FUSED && q.gated) ? q.NT1 : (q.NT1 + 1) >> 1) : 0;
             TT = segs * q.KB;
@@ -659,7 +660,7 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
     if (warp == 0) {
         guess_off = lane <= p.R ? __ldcg(p.offsets + lane) : 0;
         guess_last = p.R >= 32 ? __ldcg(p.offsets + p.R) : 0;
-        work_split();
+        work_split(guess_off, guess_last);
         __syncwarp();
         if (lane == 0) {
             GvWalk wk;
@@ -689,7 +690,7 @@ __global__ void __launch_bounds__(gv_threads(FINE), 1) qgemm_decode_kernel(const
     if (warp == 0) {
         const int my_off = lane <= p.R ? __ldcg(p.offsets + lane) : 0;
         const int my_last = p.R >= 32 ? __ldcg(p.offsets + p.R) : 0;
-        if (!__all_sync(0xffffffffu, my_off == guess_off && my_last == guess_last)) work_split();   // (else the guess was the split)
+        if (!__all_sync(0xffffffffu, my_off == guess_off && my_last == guess_last)) work_split(my_off, my_last);   // (else the guess was the split)
     }
     __syncthreads();
     const int nstg = s_geom[0], stage_bytes = s_geom[1];
