@@ -8,9 +8,9 @@
 //                  numbers (c - z) * 2^-13 in bf16 and stores them to its TMEM lane.  The unpacked weights never pass
 //                  through shared memory, whose bandwidth the token operand needs.
 //   B operand    : token rows, HC / 2 per CTA and half tile (each SM of the pair reads its own half and they share it).
-//                  Sorted rows that are consecutive in X come as one TMA box; any others are gathered through `perm` by
-//                  two warps' 16-byte cp.async copies into the same swizzled layout (the fused permutation: no gathered
-//                  copy of X exists).
+//                  Where all of a piece's rows are consecutive in X they come in TMA boxes, one per half tile; else they are
+//                  gathered through `perm` by two warps' 16-byte cp.async copies into the same swizzled layout (the fused
+//                  permutation: no gathered copy of X exists).
 //   accumulation : fp32 in three rotating TMEM buffers of HC tokens.  Grouped experts finish a buffer per (half tile,
 //                  quantization group, at most 128 k); eight "epilogue" warps drain it, multiply by the group's fp32
 //                  scale and add into register accumulators while the tensor core fills the next one:
