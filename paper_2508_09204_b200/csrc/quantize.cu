@@ -189,6 +189,10 @@ __device__ __forceinline__ GroupGrid group_grid(float lo, float hi, float a, int
     return g;
 }
 
+// rint(w / s) as a whole number, kept within 2^16 either way so that a zero-point can be added to it: a group whose scale would not
+// be finite in fp16 has scale 1, and then the quotient of a weight of 2^31 and more is beyond an int.
+__device__ __forceinline__ int quotient(float w, float s) { return min(max((int)rintf(__fdiv_rn(w, s)), -65536), 65536); }
+
 __global__ void rtn_scales_kernel(const float* __restrict__ W, int N, int K, int bits, int group, int G, int sym, int KB,
                                   uint8_t* __restrict__ tiles, __half* __restrict__ scales_pc,
                                   __nv_bfloat16* __restrict__ zeros_pc) {
@@ -259,7 +263,7 @@ __global__ void encode_pack_kernel(const float* __restrict__ W, const uint8_t* _
             float wv[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
-                int q = (int)rintf(__fdiv_rn(wv[t], s));
+                int q = quotient(wv[t], s);
                 if (sym) q = max(-qmax, min(qmax, q)) + half_code;
                 else     q = max(0, min(L, q + z));
                 c[8 * G + t] = (uint32_t)q;
@@ -308,8 +312,8 @@ __device__ __forceinline__ void round_chunk(const float* w, const Rounding& g, b
     if (!g.safe || !(worst < 0.5f - (float)(1 << (BITS + 1)) * 0x1p-21f)) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int a = (int)rintf(__fdiv_rn(w[2 * j], g.s)), b = (int)rintf(__fdiv_rn(w[2 * j + 1], g.s));
-            pair[j] = ((uint32_t)min(max(a + g.z, -1), L + 1) & 0xFFFFu) | (uint32_t)min(max(b + g.z, -1), L + 1) << 16;
+            const int a = quotient(w[2 * j], g.s) + g.z, b = quotient(w[2 * j + 1], g.s) + g.z;
+            pair[j] = ((uint32_t)min(max(a, -1), L + 1) & 0xFFFFu) | (uint32_t)min(max(b, -1), L + 1) << 16;
         }
     }
     constexpr uint32_t L2 = (uint32_t)L * 0x10001u;

@@ -38,6 +38,35 @@ def test_halfway_weights_and_reused_memory(N, K, bits, group, sym):
     assert_close(torch_to_bits(Y), oracle.routed_gemm(X, ids, [oracle.dequantize(c, s, z, group)]), "product")
 
 
+def _grid(W, bits, group, sym):
+    """Codes, scales and zero-points as the header states them, in fp32 and clamped before they become whole numbers."""
+    N, K = W.shape
+    w, L, qmax = W.reshape(N, -1, group or K), np.float32(2 ** bits - 1), np.float32(2 ** (bits - 1) - 1)
+    lo, hi = w.min(2, keepdims=True, initial=0), w.max(2, keepdims=True, initial=0)
+    with np.errstate(all="ignore"):
+        s16 = (np.maximum(-lo, hi) / qmax if sym else (hi - lo) / L).astype(np.float16)
+        s16 = np.where((s16 > 0) & np.isfinite(s16), s16, np.float16(1))
+        s = s16.astype(np.float32)
+        q = np.rint(w / s)
+        z = np.full_like(s, 2 ** (bits - 1)) if sym else np.clip(np.rint(-lo / s), 0, L) + np.float32(0)
+        c = np.clip(q, -qmax, qmax) + z if sym else np.clip(q + z, 0, L)
+    return c.reshape(N, K).astype(np.uint8), s16[..., 0].view(np.uint16), z[..., 0].astype(np.float16).view(np.uint16)
+
+
+@pytest.mark.parametrize("bits,group,sym", [(8, 0, True), (4, 0, False), (3, 32, True), (2, 64, True), (4, 128, True), (4, 128, False), (8, 256, True), (3, 256, False)])
+@pytest.mark.parametrize("N,K", [(16, 512), (16, 6144)])
+def test_weights_beyond_every_scale(N, K, bits, group, sym):
+    """Scale 1 where fp16 has none for the group, and quotients beyond 2^31: codes at the ends of the range, by one kernel (groups up to
+    128 k, short rows) and by two."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_expert_matches, dev
+    W = wl.weights_f32(f"beyond/{N}/{K}", N, K)
+    assert all(np.array_equal(a, b) for a, b in zip(_grid(W, bits, group, sym), oracle.quantize_rtn(W, bits, group, sym)))
+    W[1::2, ::7], W[1::2, 3::11], W[5::4, 5::13] = 3e9, -3e9, 3e38
+    e = moqe.moqe_quantize_rtn(torch.from_numpy(W).to(dev()), bits, group, sym)
+    assert_expert_matches(e, _grid(W, bits, group, sym))
+
+
 @pytest.mark.parametrize("bits,group,sym", [(4, 128, False), (3, 64, False), (8, 32, True), (2, 32, False)])
 @pytest.mark.parametrize("N,K", [(8, 128), (2368, 1536), (2360, 1664), (1192, 8192)])
 def test_blobs_to_a_warp(N, K, bits, group, sym):
