@@ -285,6 +285,9 @@ __device__ __forceinline__ uint64_t pack_f2(float lo, float hi) { uint64_t r; as
 __device__ __forceinline__ float2 unpack_f2(uint64_t v) { float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v)); return r; }
 __device__ __forceinline__ uint64_t fma_f2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 
+// (the larger one, and NaN if either is)
+__device__ __forceinline__ float max_or_nan(float a, float b) { float r; asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
+
 // what rounding a chunk of 8 weights needs of its group.  safe: no |w / s| of the group is large (see round_chunk)
 struct Rounding { float s, inv; int z; bool safe; };
 template <int BITS>
@@ -295,7 +298,7 @@ __device__ __forceinline__ Rounding rounding(const GroupGrid& g, float top) {
 // Codes of a chunk, in pairs of 16 bits: clamp(rint(w / s) + z) as IEEE division and rounding give rint(w / s), from a
 // multiplication by 1 / s.  Adding 1.5 * 2^23 + z rounds w * inv to the nearest integer and leaves code and zero-point added up
 // in the low bits: no conversion instructions, which run at a quarter of the rate.  The product is off by at most 2^-22 of its
-// size; only where it comes that close to the middle between two integers (or is large) does the division decide.
+// size; only where it comes that close to the middle between two integers (or is large, or no number) does the division decide.
 template <int BITS>
 __device__ __forceinline__ void round_chunk(const float* w, const Rounding& g, bool sym, uint32_t* pair) {
     constexpr int L = (1 << BITS) - 1, half_code = 1 << (BITS - 1);
@@ -306,7 +309,7 @@ __device__ __forceinline__ void round_chunk(const float* w, const Rounding& g, b
     for (int j = 0; j < 4; ++j) {
         const uint64_t x = pack_f2(w[2 * j], w[2 * j + 1]), y = fma_f2(x, inv2, magic2);
         const float2 yy = unpack_f2(y), d = unpack_f2(fma_f2(x, inv2, fma_f2(y, minus, magic2)));     // d: the product less its integer
-        worst = fmaxf(worst, fmaxf(fabsf(d.x), fabsf(d.y)));
+        worst = max_or_nan(worst, max_or_nan(fabsf(d.x), fabsf(d.y)));
         pair[j] = __byte_perm(__float_as_uint(yy.x), __float_as_uint(yy.y), 0x5410u);
     }
     if (!g.safe || !(worst < 0.5f - (float)(1 << (BITS + 1)) * 0x1p-21f)) {

@@ -67,6 +67,21 @@ def test_weights_beyond_every_scale(N, K, bits, group, sym):
     assert_expert_matches(e, _grid(W, bits, group, sym))
 
 
+@pytest.mark.parametrize("bits,group,sym", [(8, 0, True), (4, 0, False), (3, 32, True), (2, 64, False), (4, 128, True), (4, 128, False), (4, 256, False)])
+@pytest.mark.parametrize("N,K", [(16, 512), (16, 6144)])
+def test_weights_that_are_no_numbers(N, K, bits, group, sym):
+    """They have the zero-point's code and leave scales and the other codes alone, by one kernel and by two."""
+    import paper_2508_09204_b200 as moqe
+    from gpu_helpers import assert_expert_matches, dev
+    W = wl.weights_f32(f"nan/{N}/{K}", N, K)
+    gone = np.zeros((N, K), bool)
+    gone[1::2, ::5] = gone[1::2, 17:41] = gone[4] = True
+    W[gone] = 0.0                                                  # (the code of 0 is the zero-point)
+    canon = oracle.quantize_rtn(W, bits, group, sym)
+    W[gone] = np.nan
+    assert_expert_matches(moqe.moqe_quantize_rtn(torch.from_numpy(W).to(dev()), bits, group, sym), canon)
+
+
 @pytest.mark.parametrize("bits,group,sym", [(4, 128, False), (3, 64, False), (8, 32, True), (2, 32, False)])
 @pytest.mark.parametrize("N,K", [(8, 128), (2368, 1536), (2360, 1664), (1192, 8192)])
 def test_blobs_to_a_warp(N, K, bits, group, sym):
