@@ -83,6 +83,9 @@ typedef struct moqe_expert moqe_expert;
  * pool of the library, ordered on `stream`) and must be released with moqe_expert_destroy.  The kernels run on `stream`.
  * While `stream` is being captured the buffers come from cudaMalloc, which only a capture in relaxed mode or of another
  * thread's allows (MOQE_ERR_ALLOC in the others, which are invalid afterwards); the graph then fills them when it runs.
+ * Groups of 32, 64 and 128: the kernel waits for its copies of W, with a limit.  Should a wait run out, MOQE_ERR_TIMEOUT is
+ * latched (moqe_async_status; every run of a graph that holds the build latches its own) and the expert is only partly
+ * written: destroy it.
  * ------------------------------------------------------------------------- */
 MOQE_API moqe_status moqe_quantize_rtn(const float* W, int N, int K, int bits, int group, int sym,
                               void* stream, moqe_expert** out);

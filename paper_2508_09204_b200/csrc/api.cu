@@ -2,7 +2,6 @@
 // call, the device status word, status strings and the launch counter.
 #include <atomic>
 #include <cstring>
-#include <mutex>
 
 #include "common.cuh"
 #include "ptx.cuh"
@@ -11,7 +10,9 @@ namespace moqe {
 
 namespace {
 std::atomic<unsigned long long> g_launches{0};
-std::mutex g_status_mutex;
+// One a device, and zero, when the library's code is loaded there: nothing is allocated or cleared for it, which the first call
+// of a process could not do beside a capture (clearing it on the default stream made captures on blocking streams invalid).
+__device__ int g_status_word;
 std::atomic<int*> g_status_words[64] = {};
 std::atomic<int> g_sm_counts[64] = {};
 }  // namespace
@@ -21,20 +22,11 @@ void count_launch(unsigned n) { g_launches.fetch_add(n, std::memory_order_relaxe
 int* device_status_word() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    if (int* p = g_status_words[dev].load(std::memory_order_acquire)) return p;
-    std::lock_guard<std::mutex> lock(g_status_mutex);
-    if (!g_status_words[dev].load(std::memory_order_relaxed)) {
-        int* p = nullptr;
-        if (cudaMalloc(&p, sizeof(int)) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-        if (cudaMemset(p, 0, sizeof(int)) != cudaSuccess) { cudaFree(p); return nullptr; }
-        g_status_words[dev].store(p, std::memory_order_release);
-    }
-    return g_status_words[dev].load(std::memory_order_relaxed);
-}
-
-int* device_status_word_if() {
-    int dev = 0;
-    return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? g_status_words[dev].load(std::memory_order_acquire) : nullptr;
+    if (int* p = g_status_words[dev].load(std::memory_order_relaxed)) return p;
+    void* p = nullptr;
+    if (cudaGetSymbolAddress(&p, g_status_word) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    g_status_words[dev].store((int*)p, std::memory_order_relaxed);
+    return (int*)p;
 }
 
 EncodeTiledFn encode_tiled_fn() {

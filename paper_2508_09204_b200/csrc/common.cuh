@@ -97,8 +97,7 @@ struct moqe_expert {
 namespace moqe {
 
 // first device-detected error of this device (0 = none); kernels latch with atomicCAS
-int* device_status_word();                 // allocates on first use for the current device
-int* device_status_word_if();              // ... nullptr if that has not happened yet (under a stream capture it may not)
+int* device_status_word();                 // of the current device; under captures too
 int device_sm_count();                     // of the current device (148 if it cannot be asked)
 // cudaFuncAttributeMaxDynamicSharedMemorySize of a kernel, set once per device: `done` is the kernel's own word of flags
 bool ensure_dynamic_smem(const void* kernel, int bytes, std::atomic<unsigned long long>& done);

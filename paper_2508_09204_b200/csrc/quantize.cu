@@ -729,10 +729,8 @@ moqe_status launch_quantize(const moqe_expert* e, const float* W, cudaStream_t s
     }
     // W[N][K]: boxes of 32 k x 16 rows, 128-byte swizzle, zero fill outside
     const EncodeTiledFn enc = encode_tiled_fn();
-    if (!enc) return MOQE_ERR_CUDA;
-    int* status = device_status_word_if();
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (!status && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) status = device_status_word();
+    int* status = device_status_word();
+    if (!enc || !status) return MOQE_ERR_CUDA;
     CUtensorMap map;
     const cuuint64_t dim[2] = {(cuuint64_t)e->K, (cuuint64_t)e->N}, pitch[1] = {(cuuint64_t)e->K * 4};
     const cuuint32_t box[2] = {32, 16}, es[2] = {1, 1};

@@ -1,5 +1,8 @@
 """Where experts' device memory comes from and goes to: giving it back waits for the device and disturbs nobody's capture."""
 import ctypes
+import os
+import subprocess
+import sys
 import threading
 
 import pytest
@@ -99,6 +102,43 @@ def test_building_in_a_capture(mode, same_thread, what):
     _runtime().cudaGraphExecDestroy(run)
     _runtime().cudaGraphDestroy(c.graph)
     built.close()
+
+
+_FIRST_BUILD = """
+import ctypes, sys, threading, torch
+import paper_2508_09204_b200 as moqe
+mode, captured = int(sys.argv[1]), sys.argv[2] == "captured"
+rt = ctypes.CDLL("libcudart.so.12")
+W = torch.randn((512, 512), device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+side, blocking, graph, out = torch.cuda.Stream(), ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+assert rt.cudaStreamCreate(ctypes.byref(blocking)) == 0
+torch.cuda.synchronize()
+assert rt.cudaStreamBeginCapture(blocking, mode) == 0
+got = []
+def build():
+    torch.cuda.set_device(0)
+    got.append(moqe.lib().moqe_quantize_rtn(W.data_ptr(), 512, 512, 4, 128, 0, blocking if captured else side.cuda_stream, ctypes.byref(out)))
+t = threading.Thread(target=build)
+t.start()
+t.join()
+assert rt.cudaStreamEndCapture(blocking, ctypes.byref(graph)) == 0, "the capture is invalid"
+assert got == [moqe.OK], got
+if captured:
+    run = ctypes.c_void_p()
+    assert rt.cudaGraphInstantiate(ctypes.byref(run), graph, ctypes.c_ulonglong(0)) == 0 and rt.cudaGraphLaunch(run, blocking) == 0
+torch.cuda.synchronize()
+a, b = moqe.moqe_expert_export(moqe.Expert(out.value)), moqe.moqe_expert_export(moqe.moqe_quantize_rtn(W, 4, 128, False))
+assert all(torch.equal(x, y) for x, y in zip(a, b)) and moqe.moqe_async_status() == moqe.OK
+"""
+
+
+@pytest.mark.parametrize("mode,where", [(THREAD_LOCAL, "beside"), (RELAXED, "beside"), (THREAD_LOCAL, "captured")])
+def test_the_first_build_of_a_process(mode, where):
+    """A build by groups, the first thing a process has the library do, while a blocking stream is being captured by another thread: it
+    leaves the capture alone, and its status word exists in the captured stream too."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FIRST_BUILD, str(mode), where], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
 
 
 def test_trim_gives_freed_memory_back():
