@@ -189,10 +189,6 @@ __device__ __forceinline__ GroupGrid group_grid(float lo, float hi, float a, int
     return g;
 }
 
-// rint(w / s) as a whole number, kept within 2^16 either way so that a zero-point can be added to it: a group whose scale would not
-// be finite in fp16 has scale 1, and then the quotient of a weight of 2^31 and more is beyond an int.
-__device__ __forceinline__ int quotient(float w, float s) { return min(max((int)rintf(__fdiv_rn(w, s)), -65536), 65536); }
-
 __global__ void rtn_scales_kernel(const float* __restrict__ W, int N, int K, int bits, int group, int G, int sym, int KB,
                                   uint8_t* __restrict__ tiles, __half* __restrict__ scales_pc,
                                   __nv_bfloat16* __restrict__ zeros_pc) {
@@ -263,9 +259,9 @@ __global__ void encode_pack_kernel(const float* __restrict__ W, const uint8_t* _
             float wv[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
-                int q = quotient(wv[t], s);
+                int q = (int)rintf(__fdiv_rn(wv[t], s));   // (beyond an int where fp16 has no scale for the group: clamped before it is added to)
                 if (sym) q = max(-qmax, min(qmax, q)) + half_code;
-                else     q = max(0, min(L, q + z));
+                else     q = max(0, min(L, min(L, q) + z));
                 c[8 * G + t] = (uint32_t)q;
             }
         }
@@ -285,6 +281,9 @@ __device__ __forceinline__ uint64_t pack_f2(float lo, float hi) { uint64_t r; as
 __device__ __forceinline__ float2 unpack_f2(uint64_t v) { float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v)); return r; }
 __device__ __forceinline__ uint64_t fma_f2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 
+// the nearest whole number, within 16 bits, so that a zero-point can be added to it (where fp16 has no scale for a group its scale is 1,
+// and quotients may be beyond an int); 0 for NaN
+__device__ __forceinline__ int rounded16(float x) { short q; asm("cvt.rni.s16.f32 %0, %1;" : "=h"(q) : "f"(x)); return q; }
 // (the larger one, and NaN if either is)
 __device__ __forceinline__ float max_or_nan(float a, float b) { float r; asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
 
@@ -315,7 +314,7 @@ __device__ __forceinline__ void round_chunk(const float* w, const Rounding& g, b
     if (!g.safe || !(worst < 0.5f - (float)(1 << (BITS + 1)) * 0x1p-21f)) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int a = quotient(w[2 * j], g.s) + g.z, b = quotient(w[2 * j + 1], g.s) + g.z;
+            const int a = rounded16(__fdiv_rn(w[2 * j], g.s)) + g.z, b = rounded16(__fdiv_rn(w[2 * j + 1], g.s)) + g.z;
             pair[j] = ((uint32_t)min(max(a, -1), L + 1) & 0xFFFFu) | (uint32_t)min(max(b, -1), L + 1) << 16;
         }
     }
