@@ -1185,29 +1185,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
 #pragma unroll
             for (int i0 = 0; i0 < L::EC; i0 += 16)
                 if (i0 < ncol) {
-                    // (in phases, each over all 16 tokens: one group of four after another, every exchange waited for the last)
-                    uint32_t p01[4], p23[4], q01[4], q23[4];
-                    int to[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        p01[j] = pack_bf16x2(acc[i0 + 4 * j], acc[i0 + 4 * j + 1]);
-                        p23[j] = pack_bf16x2(acc[i0 + 4 * j + 2], acc[i0 + 4 * j + 3]);
-                        to[j] = to_list[i0 + 4 * j];
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) { q01[j] = __shfl_xor_sync(0xffffffffu, p01[j], 1); q23[j] = __shfl_xor_sync(0xffffffffu, p23[j], 1); }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        p01[j] = __byte_perm(p01[j], q01[j], sub & 1 ? 0x3276u : 0x5410u);       // two channels of token i + (sub & 1)
-                        p23[j] = __byte_perm(p23[j], q23[j], sub & 1 ? 0x3276u : 0x5410u);       // ... of token i + 2 + (sub & 1)
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) q01[j] = __shfl_xor_sync(0xffffffffu, sub & 2 ? p01[j] : p23[j], 2);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        uint16_t* at = y + (size_t)(uint32_t)max(to[j], 0) * (uint32_t)p.N;
+                    for (int i = i0; i < i0 + 16; i += 4) {
+                        const uint32_t p01 = pack_bf16x2(acc[i], acc[i + 1]), p23 = pack_bf16x2(acc[i + 2], acc[i + 3]);
+                        const uint32_t q01 = __shfl_xor_sync(0xffffffffu, p01, 1), q23 = __shfl_xor_sync(0xffffffffu, p23, 1);
+                        const uint32_t a = __byte_perm(p01, q01, sub & 1 ? 0x3276u : 0x5410u);       // two channels of token i + (sub & 1)
+                        const uint32_t b = __byte_perm(p23, q23, sub & 1 ? 0x3276u : 0x5410u);       // ... of token i + 2 + (sub & 1)
+                        const uint32_t other = __shfl_xor_sync(0xffffffffu, sub & 2 ? a : b, 2);
+                        const int to = to_list[i];
+                        uint16_t* at = y + (size_t)(uint32_t)max(to, 0) * (uint32_t)p.N;
                         asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %3, 0;\n\t@q st.global.v2.b32 [%0], {%1, %2};\n\t}"
-                                     ::"l"(at), "r"(sub & 2 ? q01[j] : p01[j]), "r"(sub & 2 ? p23[j] : q01[j]), "r"((int)(in_n && to[j] >= 0)) : "memory");
+                                     ::"l"(at), "r"(sub & 2 ? other : a), "r"(sub & 2 ? b : other), "r"((int)(in_n && to >= 0)) : "memory");
                     }
                 }
         }
