@@ -188,6 +188,7 @@ struct TcShared {
     TcSched sc;
     uint32_t tmem;
     int abort;
+    __align__(16) int walk[TC_EPI][12];     // per epilogue warp: what of the walk only the end of a piece asks for
     __align__(16) int perm[TC_EPI][L::EC];  // per epilogue warp: its columns' target rows
     __align__(16) int xrow[2][L::NH * L::XR];   // rows of X to gather, one list per gather warp: row 4 i + j at [j][i]
 };
@@ -411,6 +412,12 @@ __device__ __forceinline__ bool dequant_none(TcDequant& d, TcShared<TN>& sh, int
     return ok;
 }
 
+__device__ __forceinline__ void sts_v4(uint32_t at, int a, int b, int c, int d) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void lds_v4(uint32_t at, int& a, int& b, int& c, int& d) {
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(a), "=r"(b), "=r"(c), "=r"(d) : "r"(at) : "memory");
+}
 // acc[0..31] += s * v, two columns per instruction (each half rounds as a scalar fma does)
 __device__ __forceinline__ void fma_cols32(float* acc, const uint32_t (&v)[32], float s) {
 #pragma unroll
@@ -946,6 +953,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         const int row = quarter * 32 + lane;               // channel inside the 128-channel tile = TMEM lane
         const uint32_t accempty0 = mapa(bar_accempty, 0);
         const uint32_t lane_tmem = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        const uint32_t saved = smem_u32(sh.walk[ew]);
         int* my_perm = sh.perm[ew];                        // private to this warp: no cross-warp barrier
         TcPiece pc;
         TcWalk wk;
@@ -956,76 +964,109 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
         uint32_t step = 0, xphase = 0;                     // steps so far; parity of the exchange
         while (ok && wk.next(sc, p, nclusters, pc)) {
             const ExpertDev& ex = p.ex[pc.e];
-            const int nt = 2 * pc.ntp + (int)rank, n = nt * 128 + row;
-            const bool active = nt < p.NT1;
+            int nt = 2 * pc.ntp + (int)rank, n = nt * 128 + row;
+            bool active = nt < p.NT1;
             const int nh = NH == 1 ? 1 : (pc.rows > L::HC ? 2 : 1);
             // the columns this warp stores: ncol (may be <= 0) from token tok0 of the tile on
             const int hs = nh == 2 ? half_split<L::HC>(pc.rows) : L::HC / 2;
-            const int tok0 = eg * hs, ncol = min(hs, pc.rows - tok0);
+            int tok0 = eg * hs, ncol = min(hs, pc.rows - tok0);
             __syncwarp();
 #pragma unroll
             for (int i = 0; i < L::EC / 32; ++i) {
                 const int col = i * 32 + lane;
                 my_perm[col] = col < ncol ? __ldcg(p.perm + pc.m0 + tok0 + col) : -1;
             }
+            // What only the end of the piece asks for waits in shared memory: the drain loops have no registers for it, and the copies that
+            // the compiler spilled instead were loaded again inside them.
+            sts_v4(saved, pc.e, pc.ntp, pc.rows, pc.tile);
+            sts_v4(saved + 16, pc.kb0, pc.kb1, wk.t, wk.e);
+            sts_v4(saved + 32, wk.u, wk.ue, 0, 0);
             __syncwarp();
             float acc[L::DC];
 #pragma unroll
             for (int i = 0; i < L::DC; ++i) acc[i] = 0.f;
             const bool keep = ex.group == 0;
-            const int per = keep ? 1 : moqe_groups_per_tile(ex.group), nkb = pc.kb1 - pc.kb0;
+            const int per = moqe_groups_per_tile(ex.group), nkb = pc.kb1 - pc.kb0;
             const float s_pc = keep && active ? __half2float(ex.scales_pc[n]) * W8_PRESCALE : 0.f;   // (weights are unpacked as (c - z) * 2^-13)
             const bool alone = KS == 2 || nh == 2;             // a buffer is drained by one group
             const uint32_t freed = alone ? 2u : 1u;
             const int col0 = alone ? 0 : tok0;                 // first column drained, and how many hold a token
             const int dcol = KS == 2 ? pc.rows : ncol;
-            // Scales come straight from the tiles in global memory (the packed tile has just been fetched, so they are in L2),
-            // two drains ahead of their use.  Handed on by the dequant warps through shared memory and a barrier of their own,
-            // they cost both roles some 200 cycles a k-block.
-            const int mg = ex.has_zeros ? 512 : 256, round = KS * ex.tile_stride;
-            const unsigned char* meta = ex.tiles + ((size_t)(active ? nt : 0) * p.KB + pc.kb0) * ex.tile_stride + moqe_tile_bytes(ex.bits) + row * 2;
-            const int off_end = (nkb - 1) * ex.tile_stride + (per - 1) * mg;
-            int off = min(KS == 2 ? eg * ex.tile_stride : 0, (nkb - 1) * ex.tile_stride), oj = 0;
-            auto fetch_scale = [&]() { return keep ? (unsigned short)0 : __ldg(reinterpret_cast<const unsigned short*>(meta + off)); };
-            auto next_scale = [&](bool one) {                      // one: a group to a k-block
-                if (one) off = min(off + round, off_end);
-                else {
-                    const bool wrap = ++oj == per;
-                    off = min(off + (wrap ? round - (per - 1) * mg : mg), off_end);
-                    oj = wrap ? 0 : oj;
-                }
-            };
-            unsigned short s_now = fetch_scale();                  // (as loaded: converting waits for the load)
-            next_scale(per == 1);
-            unsigned short s_next = fetch_scale();
-            // waits for an accumulator buffer, adds it to the sums and hands it back
-            auto drain = [&](auto chunks, bool one, uint32_t bar, uint32_t phase, int b) {
-                ok &= warp_wait(bar, phase, s_abort, p.status);
-                tc_fence_after();
-                const uint32_t src = lane_tmem + b * L::HC + col0;
-                float sv = s_pc;
+            if (keep) {
+                // Per channel: a half tile's buffer is drained once.  (Apart from the groups' loops, whose scales and counts are then not
+                // alive here: 28224 rows of 256 -> 1024 channels 40.7 -> 34.9 us with the walk in shared memory, see below; as long as
+                // both shared one drain, a piece of two k-blocks paid for their spills.)
+                const int nu = KS == 2 ? 1 : nh;
+#pragma unroll 1
+                for (int u = 0; u < nu; ++u) {
+                    const int fb = u * NACC + buf;
+                    if (!alone || u == eg) {
+                        ok &= warp_wait(bar_accfull + 8 * fb, (full_phase >> fb) & 1u, s_abort, p.status);
+                        tc_fence_after();
 #pragma unroll
-                for (int c = 0; c < L::DC / 32; ++c) {
-                    if (decltype(chunks)::value > 0 ? c < decltype(chunks)::value : 32 * c < dcol) {
-                        uint32_t v[32];
-                        tmem_ld32(src + 32 * c, v);
-                        if (c == 0) {
-                            // (while the load is under way)
-                            if (one || !keep) sv = __half2float(__ushort_as_half(s_now)) * W8_PRESCALE;
-                            s_now = s_next;
-                            next_scale(one);
-                            s_next = fetch_scale();
-                        }
-                        tmem_ld_wait();
-                        fma_cols32(acc + 32 * c, v, sv);
+                        for (int c = 0; c < L::DC / 32; ++c)
+                            if (32 * c < dcol) {
+                                uint32_t v[32];
+                                tmem_ld32(lane_tmem + buf * L::HC + col0 + 32 * c, v);
+                                tmem_ld_wait();
+                                fma_cols32(acc + 32 * c, v, s_pc);
+                            }
+                        tc_fence_before();
+                        __syncwarp();
+                        remote_arrive_if(lane == 0, accempty0 + 8 * buf, freed);
                     }
+                    full_phase ^= 1u << fb;
+                    if (++buf == NACC) buf = 0;
                 }
-                tc_fence_before();
-                __syncwarp();
-                remote_arrive_if(lane == 0, accempty0 + 8 * b, freed);
-            };
-            int left = nkb;
-            if (!keep) {
+                step += (nkb + KS - 1) / KS;
+                ok = __all_sync(0xffffffffu, ok);
+            } else {
+                // Scales come straight from the tiles in global memory (the packed tile has just been fetched, so they are in L2),
+                // two drains ahead of their use.  Handed on by the dequant warps through shared memory and a barrier of their own,
+                // they cost both roles some 200 cycles a k-block.
+                const int mg = ex.has_zeros ? 512 : 256, round = KS * ex.tile_stride;
+                const unsigned char* meta = ex.tiles + ((size_t)(active ? nt : 0) * p.KB + pc.kb0) * ex.tile_stride + moqe_tile_bytes(ex.bits) + row * 2;
+                const int off_end = (nkb - 1) * ex.tile_stride + (per - 1) * mg;
+                int off = min(KS == 2 ? eg * ex.tile_stride : 0, (nkb - 1) * ex.tile_stride), oj = 0;
+                auto fetch_scale = [&]() { return __ldg(reinterpret_cast<const unsigned short*>(meta + off)); };
+                auto next_scale = [&](bool one) {                      // one: a group to a k-block
+                    if (one) off = min(off + round, off_end);
+                    else {
+                        const bool wrap = ++oj == per;
+                        off = min(off + (wrap ? round - (per - 1) * mg : mg), off_end);
+                        oj = wrap ? 0 : oj;
+                    }
+                };
+                unsigned short s_now = fetch_scale();                  // (as loaded: converting waits for the load)
+                next_scale(per == 1);
+                unsigned short s_next = fetch_scale();
+                // waits for an accumulator buffer, adds it to the sums and hands it back
+                auto drain = [&](auto chunks, bool one, uint32_t bar, uint32_t phase, int b) {
+                    ok &= warp_wait(bar, phase, s_abort, p.status);
+                    tc_fence_after();
+                    const uint32_t src = lane_tmem + b * L::HC + col0;
+                    float sv = 0.f;
+#pragma unroll
+                    for (int c = 0; c < L::DC / 32; ++c) {
+                        if (decltype(chunks)::value > 0 ? c < decltype(chunks)::value : 32 * c < dcol) {
+                            uint32_t v[32];
+                            tmem_ld32(src + 32 * c, v);
+                            if (c == 0) {
+                                // (while the load is under way)
+                                sv = __half2float(__ushort_as_half(s_now)) * W8_PRESCALE;
+                                s_now = s_next;
+                                next_scale(one);
+                                s_next = fetch_scale();
+                            }
+                            tmem_ld_wait();
+                            fma_cols32(acc + 32 * c, v, sv);
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    remote_arrive_if(lane == 0, accempty0 + 8 * b, freed);
+                };
+                int left = nkb;
                 // The loop is kept short, since a warp gets an instruction through every nine cycles or so and nothing else of
                 // the epilogue runs in parallel.
                 const bool by_done = !alone || eg == 1;            // announced by the step's own barrier if it is the last group
@@ -1057,42 +1098,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                     }
                 };
                 auto run = [&](auto one) {
-                    if constexpr (TN == 256) {
-                        // The number of 32-column chunks is fixed at compile time: no branch between them, and the loads of a chunk
-                        // start before the sums of the last are done (16384 x 11008 x 4096, three LLaMA experts: 1430 -> 1395
-                        // us).  The smaller tiles, with one or two chunks, are faster with the branches (38.3 against 39.0).
+                    // The number of 32-column chunks is fixed at compile time: no branch between them, and the loads of a chunk start before
+                    // the sums of the last are done.  128 tokens, two chunks, 18944 x 3584 in 4-bit g64 and g32: 32.6 and 51.3 us, with
+                    // the branches 36.4 and 58.2; a single chunk of narrow groups (50.8 against 57.4 in g32) and the smallest tile
+                    // (96 rows x 4096 x 11008: 38.3 against 39.0) are better with them.
+                    constexpr bool ONE = decltype(one)::value;
+                    if constexpr (TN == 64) {
+                        steps(std::integral_constant<int, 0>{}, one);
+                    } else if constexpr (TN == 128) {
+                        if (dcol > 32) steps(std::integral_constant<int, 2>{}, one);
+                        else steps(std::integral_constant<int, ONE ? 1 : 0>{}, one);
+                    } else {
                         const int nch = (dcol + 31) >> 5;
                         if (nch <= 1) steps(std::integral_constant<int, 1>{}, one);
                         else if (nch == 2) steps(std::integral_constant<int, 2>{}, one);
                         else if (nch == 3) steps(std::integral_constant<int, 3>{}, one);
                         else steps(std::integral_constant<int, 4>{}, one);
-                    } else {
-                        steps(std::integral_constant<int, 0>{}, one);
                     }
                 };
                 if (per == 1) run(std::true_type{});
                 else run(std::false_type{});
-            }
-            // The rest: one round per step (every group's buffer is drained, the last one of the step being announced by the
-            // step's own barrier), or one for the whole piece (per channel).  The loops are kept rolled: unrolled over the
-            // groups and the barriers' outcomes the kernel was 235 KB of code and spent a quarter of its warps' time fetching
-            // instructions.
+                if constexpr (KS == 2) {
+                    // The odd k-block of a piece: every group's buffer is drained, the last one being announced by the step's own barrier.
+                    // (The loop is kept rolled: the kernel is fetched as it runs.)
+                    if (ok && left > 0) {
 #pragma unroll 1
-            while (ok && left > 0) {
-                const int nu = KS == 2 ? (keep ? 1 : min(KS, left)) : nh;
-#pragma unroll 1
-                for (int t = 0; t < nu * per; ++t) {
-                    const int u = nu == 2 ? t & 1 : 0;
-                    const bool by_done = !keep && t + 1 == nu * per;
-                    const int fb = u * NACC + buf;
-                    if (!alone || u == eg)
-                        drain(std::integral_constant<int, 0>{}, false, by_done ? bar_done + 8 * (step % NX) : bar_accfull + 8 * fb, by_done ? step / NX & 1u : (full_phase >> fb) & 1u, buf);
-                    if (!by_done) full_phase ^= 1u << fb;
-                    if (++buf == NACC) buf = 0;
+                        for (int t = 0; t < per; ++t) {
+                            const bool by_done = t + 1 == per;
+                            if (eg == 0)
+                                drain(std::integral_constant<int, 0>{}, false, by_done ? bar_done + 8 * (step % NX) : bar_accfull + 8 * buf, by_done ? step / NX & 1u : (full_phase >> buf) & 1u, buf);
+                            if (!by_done) full_phase ^= 1u << buf;
+                            if (++buf == NACC) buf = 0;
+                        }
+                        ++step;
+                        ok = __all_sync(0xffffffffu, ok);
+                    }
                 }
-                step += keep ? (nkb + KS - 1) / KS : 1;
-                left = keep ? 0 : left - KS;
-                ok = __all_sync(0xffffffffu, ok);
             }
             if constexpr (KS == 2) {
                 // the two groups hold sums over different k-blocks: each takes half of the columns and hands over the others
@@ -1113,6 +1154,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 mbar_arrive_if(lane == 0, xempty + 8 * (ew ^ 4));
                 xphase ^= 1u;
                 ok = __all_sync(0xffffffffu, ok);
+            }
+            {
+                int unused;
+                lds_v4(saved, pc.e, pc.ntp, pc.rows, pc.tile);
+                lds_v4(saved + 16, pc.kb0, pc.kb1, wk.t, wk.e);
+                lds_v4(saved + 32, wk.u, wk.ue, unused, unused);
+                nt = 2 * pc.ntp + (int)rank; n = nt * 128 + row;
+                active = nt < p.NT1;
+                const int h0 = NH > 1 && pc.rows > L::HC ? half_split<L::HC>(pc.rows) : L::HC / 2;
+                tok0 = eg * h0; ncol = min(h0, pc.rows - tok0);
             }
             if (!ok) break;
             if (!active) continue;
