@@ -470,8 +470,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
     if (warp == 1) tmem_alloc_pair(smem_u32(&sh.tmem), 512);
     // ---- the schedule.  Worked out from the offset table as it stands BEFORE the previous kernel is waited for (in a block's
     // later layers it is final already), so that afterwards the table has only to be compared, while the rows of the first piece
-    // are being looked up; a table that has changed is gone through again.  (It took 1.6 us after the wait and the first rows' places
-    // another 1.0: 96 rows, seven layers of a LLaMA block, 206 -> 197 us with the weights' first tiles asked of L2.)
+    // are being looked up; a table that has changed is gone through again, from what the comparison has read.  (64 rows x 1024 x 1024
+    // through the one-call entry point, whose sort has just written the table: 10.9 us if it is the table of the call before, 11.95 if
+    // it is another; with the schedule after the wait 11.65 always.  96 rows x 4096 x 4096 on a sorted batch: 21.2, and 22.1.)
     const bool x_warp = warp == 0 || warp == 3;
     TcPiece x_pc;
     TcWalk x_wk;
@@ -495,12 +496,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             x_b[h] = lane + 32 < c ? __ldcg(p.perm + x_pc.m0 + first_row + lane + 32) : 0;
         }
     };
+    int t_first = 0, t_next = 0;                           // the table: its first entry, and lane e's entry e + 1
+    auto read_table = [&]() {
+        t_first = __ldcg(p.offsets);
+        t_next = lane < p.E ? __ldcg(p.offsets + lane + 1) : 0;
+    };
     auto schedule = [&]() {
         // lane e works out expert e
         const int e = lane;
         // (a table that is still being written may hold anything: offsets are made to rise and to stay within the batch)
-        int o1 = e < p.E ? min(max(__ldcg(p.offsets + e + 1), 0), p.M) : 0;
-        int o0 = e == 0 ? min(max(__ldcg(p.offsets), 0), p.M) : 0;
+        int o1 = min(max(t_next, 0), p.M);
+        int o0 = e == 0 ? min(max(t_first, 0), p.M) : 0;
         o1 = max(o0, o1);
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
@@ -563,13 +569,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
     };
 #pragma unroll 1
     for (bool early = true;; early = false) {
-        if (warp == 0) schedule();
+        if (warp == 0) {
+            if (early) read_table();
+            schedule();
+        }
         tc_fence_before();
         __syncthreads();
         bool changed = false;
+        const int g_first = t_first, g_next = t_next;
         if (early) {
-            if (warp == 2 && lane == 0) {
-                // the first packed tiles into L2 (a wrong guess costs prefetched lines only)
+            if (warp == 4 && lane == 0) {
+                // the first packed tiles into L2, by a warp that nobody waits for (a wrong guess costs prefetched lines only; without it 64 to
+                // 96 rows of a LLaMA layer take 1 % longer)
                 TcPiece pc;
                 TcWalk wk;
                 wk.start(cluster);
@@ -582,12 +593,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             asm volatile("griddepcontrol.wait;" ::: "memory");
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         }
+        if (early && warp == 0) read_table();              // (under way while the first rows are looked up)
         if (x_warp) {
             x_wk.start(cluster);
             x_next();
-        } else if (early && warp == 2) {
-            changed = (lane < p.E && __ldcg(p.offsets + lane) != sc.off[lane]) || (lane == 0 && __ldcg(p.offsets + p.E) != sc.off[p.E]);
         }
+        changed = t_first != g_first || t_next != g_next;
         if (!early || !__syncthreads_or(changed)) break;
     }
     if (warp != 2) cluster_wait();                         // (the weight producer touches its own CTA only)
