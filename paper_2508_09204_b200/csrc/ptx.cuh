@@ -21,6 +21,14 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 __device__ __forceinline__ void mbar_arrive_if(bool yes, uint32_t bar) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"((uint32_t)yes) : "memory");
 }
+// Arrives (one lane of a warp that has just been brought together) once `used` is there, which depends on what the warp has loaded
+// from a stage of shared memory that a bulk copy overwrites next.  Generic reads that are still under way are not ordered with the
+// asynchronous proxy's writes, and an arrival right behind them can overtake them.  (All lanes of a load come back together; where
+// plain stores follow, release and acquire are enough.)
+__device__ __forceinline__ void mbar_arrive_after(uint32_t used, bool yes, uint32_t bar) {
+    const uint32_t none = gridDim.y - 1u;                  // 0, which the compiler does not know
+    mbar_arrive_if(yes, bar | (used & none));
+}
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }

@@ -347,8 +347,21 @@ __device__ __noinline__ int mainloop_to_out(const StreamParams* pp, int e, int n
         if (!__all_sync(0xffffffffu, mbar_wait(bar_full + 8 * ring.stage, ring.phase, s_abort, p.status))) return -1;
         consume_stage<BITS, NT, NSETS, GM>(smem + ring.stage * stage_bytes, x_off, warp, gl, q, has_zeros, pc_zl, pc_zh, acc,
                                        part, xs);
+        // The stage's codes, scales and token rows have all been used where these sums are there (the k-block is one basic block, in
+        // which nothing else keeps their use in front of the arrival).
+        uint32_t used = 0;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+            if constexpr (GM == 0) {
+#pragma unroll
+                for (int c = 0; c < NSETS; ++c) used |= __float_as_uint(part[c][t][0]);
+                if (BITS != 8) used |= __float_as_uint(xs[t][0]);
+            } else {
+                used |= __float_as_uint(acc[t][0]) | __float_as_uint(acc[t][2]);
+            }
+        }
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_empty + 8 * ring.stage);
+        mbar_arrive_after(used, lane == 0, bar_empty + 8 * ring.stage);
         ring.advance(nstg);
     }
     if constexpr (GM == 0) {

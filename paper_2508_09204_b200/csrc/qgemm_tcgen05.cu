@@ -1162,7 +1162,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
 #pragma unroll
                 for (int i = 0; i < 32; ++i) acc[i] = (eg ? acc[i + 32] : acc[i]) + in[i * 32];
                 __syncwarp();
-                mbar_arrive_if(lane == 0, xempty + 8 * (ew ^ 4));
+                mbar_arrive_if(lane == 0, xempty + 8 * (ew ^ 4));   // (plain stores follow, which its release orders behind the reads)
                 xphase ^= 1u;
                 ok = __all_sync(0xffffffffu, ok);
             }
