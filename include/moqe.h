@@ -273,7 +273,7 @@ MOQE_API moqe_status moqe_routed_qgemm(const void* X_bf16, const int32_t* row_id
  * output channels, MOQE_ERR_UNSUPPORTED otherwise: the layer is bound by its activations, so each expert's weights
  * are expanded to bf16 once per call and X / Y are streamed).  The automatic choice takes it there for layers of at
  * most 65536 weights, and for wider ones from 30000 rows on (12000 where an expert has groups of 32 k and K > N), but not with
- * K >= 512 and no groups of 32 k.
+ * K >= 512 and no groups of 32 k (per-channel experts of 264 to 320 channels: K >= 576).
  * Path 5 leaves groups narrower than 128 k to the automatic choice, which has an instantiation for them. */
 MOQE_API moqe_status moqe_routed_qgemm_path(const void* X_bf16, const int32_t* row_ids, int M,
                                    const moqe_expert* const* h_experts, int E, void* Y_bf16,

@@ -113,25 +113,31 @@ int pick_kernel(int path, int M, const moqe_expert* const* ex, int E) {
         if (M <= AUTO_STREAM_MAX_ROWS && !(g_auto_decode && decode_supported_multi(1, ex, 1, E))) return 1;
         // The dense-weights GEMM has a launch more, streams or re-reads an expert's whole matrix per 128 rows and multiplies grouped
         // experts' weights twice; the grouped GEMM drains every group of 32 k by itself.  Dense / grouped, us, K -> N channels:
-        //                  rows    W8-pc W4-pc W4-g32   W4-pc        W8-pc W4-g64   W4-g128
-        //   256 ->   64    3920    12.4 / 10.8          10.2 / 8.8   12.4 / 9.7     10.4 / 8.7
-        //                 12544    12.9 / 18.2          10.4 / 11.5  12.4 / 14.1    11.4 / 11.3
-        //   256 -> 1024   20000    56.3 / 44.2          37.0 / 29.6  54.7 / 39.4    55.4 / 32.5
-        //                 35000    54.7 / 67.7          36.6 / 46.6  52.2 / 59.4    55.4 / 52.2
-        //   1024 -> 256   12544    36.6 / 40.0          18.7 / 16.2  34.3 / 25.0    28.8 / 16.8
-        //                 35000    49.4 / 54.5          30.9 / 27.0  47.3 / 39.2    49.2 / 29.7
-        //   512 -> 1024   35000    88.3 / 94.1          55.4 / 51.6  86.0 / 76.8    91.8 / 66.8
-        // and with more rows, W8-pc W4-g64 (256 images of a bottleneck's layer among them):
-        //   1024 -> 256    50176    69.2 / 53.6    100352 113 / 88
-        //   512 ->  512    50176    71.7 / 59.8    100352 118 / 103
-        //   256 -> 1024    50176    76.1 / 83.6    100352 127 / 156
-        // So rows of 512 k and more are the grouped GEMM's unless a group of 32 k is among the experts.  The other lines lie where
-        // calls with groups of 32 k and layers of 256 k have them.  Small layers below some 4000 rows would do better on the grouped
-        // GEMM (256 -> 64, 980 rows 12.4 / 8.5).
-        bool fine = false;
-        for (int e = 0; e < E; ++e) fine |= ex[e]->group == 32;
-        const bool few = (M < (fine && ex[0]->K > ex[0]->N ? 12000 : 30000) || (!fine && ex[0]->K >= 512)) && (long long)ex[0]->N * ex[0]->K > 65536;
-        return (g_auto_dense && !few && dense_supported(M, ex[0]->N, ex[0]->K, ex, E)) ? 3 : 0;
+        //                   rows    W8-pc W4-pc W4-g32   W4-pc        W8-pc W4-g64   W4-g128
+        //   256 ->   64      980    10.3 / 8.2           8.2 / 6.1    9.9 / 7.2      8.9 / 6.5
+        //                   3920    10.9 / 10.1          8.2 / 8.5    10.3 / 9.5     9.2 / 8.9
+        //                  12544    10.9 / 13.9          8.2 / 10.3   10.3 / 12.3    9.2 / 10.6
+        //   256 -> 1024    20000    48.1 / 39.0          33.3 / 27.6  45.7 / 36.9    51.5 / 32.6
+        //                  35000    52.4 / 60.5          35.3 / 42.5  49.8 / 56.0    53.3 / 50.7
+        //                 100352    120 / 148            90.1 / 109   125 / 138      144 / 128
+        //   1024 -> 256    12544    31.8 / 28.5          18.0 / 15.2  31.4 / 20.9    26.7 / 15.8
+        //                  50176    59.6 / 51.7          41.0 / 32.5  67.9 / 51.9    67.7 / 38.3
+        //                 100352    106 / 112            73.3 / 55.9  111 / 83.5     127 / 71.1
+        //   512 ->  512    35000    48.5 / 47.1          31.2 / 26.2  46.5 / 39.0    49.2 / 33.8
+        //                 100352    111 / 103            79.0 / 64.0  119 / 96.6     133 / 85.3
+        //   512 -> 1024    35000    86.1 / 77.9          53.9 / 45.2  84.0 / 69.6    89.6 / 63.0
+        // So rows of 512 k and more are the grouped GEMM's unless a group of 32 k is among the experts (no format, batch, number of
+        // experts or scattering of rows was found where it is behind, from 72 to 1024 channels), with one exception: per-channel
+        // experts of 512 k whose second pair of channel tiles is mostly padding (512 -> 264, W8-pc W4-pc: 50176 rows 39.2 / 41.0,
+        // 100352 71.1 / 73.5; 384 channels 42.6 / 42.1; 576 k 43.2 / 42.8).  The other lines lie where calls with groups of 32 k and
+        // layers of 256 k had them when the grouped GEMM drained such groups more slowly; it wins with 512 k and more at many sizes now,
+        // not at all (768 -> 384, 50176 rows: 79 / 96).  Small layers below some 3000 rows would do better on it.
+        bool fine = false, per_channel = true;
+        for (int e = 0; e < E; ++e) { fine |= ex[e]->group == 32; per_channel &= ex[e]->group == 0; }
+        const int N = ex[0]->N, K = ex[0]->K;
+        const bool padded = per_channel && K < 576 && N > 256 && N <= 320;
+        const bool few = (M < (fine && K > N ? 12000 : 30000) || (!fine && K >= 512 && !padded)) && (long long)N * K > 65536;
+        return (g_auto_dense && !few && dense_supported(M, N, K, ex, E)) ? 3 : 0;
     }
     return 0;
 }

@@ -34,3 +34,11 @@ def test_automatic_choice(M, N, K, specs, want, other):
         out.append(torch_to_bits(Y))
     assert np.array_equal(out[0], out[1])
     assert_close(out[2], out[0], f"M{M} N{N} K{K}")
+
+
+@pytest.mark.parametrize("M,N,K,specs,want,other", [
+    (30000, 264, 512, PC, DENSE, GROUPED), (30000, 320, 568, PC, DENSE, GROUPED), (30000, 328, 512, PC, GROUPED, DENSE), (30000, 264, 576, PC, GROUPED, DENSE),
+    (30000, 256, 512, PC, GROUPED, DENSE), (29999, 264, 512, PC, GROUPED, DENSE), (30000, 264, 512, G64, GROUPED, DENSE)])
+def test_padded_channels_of_512_k(M, N, K, specs, want, other):
+    """Per-channel experts of 512 k whose second pair of channel tiles is mostly padding."""
+    test_automatic_choice(M, N, K, specs, want, other)
