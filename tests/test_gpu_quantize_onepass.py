@@ -83,10 +83,11 @@ def test_weights_that_are_no_numbers(N, K, bits, group, sym):
 
 
 @pytest.mark.parametrize("bits,group,sym", [(4, 128, False), (3, 64, False), (8, 32, True), (2, 32, False)])
-@pytest.mark.parametrize("N,K", [(8, 128), (2368, 1536), (2360, 1664), (1192, 8192)])
+@pytest.mark.parametrize("N,K", [(8, 128), (2304, 1536), (2368, 1536), (2360, 1664), (1192, 8192), (2936, 6400)])
 def test_blobs_to_a_warp(N, K, bits, group, sym):
-    """8 blobs of 16 channels x 128 k for 1776 warps (148 SMs); one each; for some two; two or three, so that stages are filled
-    again.  The channels' sizes go from scales that underflow in fp16 to large ones."""
+    """Blobs of 16 channels x 128 k, N padded to 128, for the 12 warps of each of 148 SMs: 8; 1728, at most one each; 1824 and 1976, for
+    some two; 5120, two or three; 9200, five or six, so that both stages are filled twice again and their barriers' parity comes
+    round.  The channels' sizes go from scales that underflow in fp16 to large ones."""
     import paper_2508_09204_b200 as moqe
     from gpu_helpers import assert_expert_matches, dev
     W = wl.weights_f32(f"blobs/{N}/{K}", N, K) * np.exp2(np.arange(N) % 43 - 30).astype(np.float32)[:, None]
