@@ -71,8 +71,11 @@ struct TcCfg {
     static constexpr int dq_arrive = KS == 2 ? 8 : 4;                        // dequant warps that fill one weight buffer
     static constexpr int epi_warp0 = 4 + dq_warps;
     static constexpr int threads = (epi_warp0 + TC_EPI) * 32;
-    // registers: what the producers and the dequant warps can do without goes to the epilogue, whose sums must not spill (300 rows in
-    // 128-token tiles, 4-bit g64: 34 us with this split, 39 with 48 / 80 / 136; 2048 rows in 256-token ones, 4-bit g128: 63, and 67 with 56 / 72 / 192)
+    // registers: what the producers and the dequant warps can do without goes to the epilogue (300 rows in 128-token tiles, 4-bit g64:
+    // 34 us with this split, 39 with 48 / 80 / 136; 256 tokens: with 48 / 80 / 192 the gathering producers lose more than the
+    // epilogue gains, 500 scattered rows x 4096 x 4096 36.4 us and not 34.0).  The epilogue still spills, 150 bytes of the
+    // 256-token tile and 60 to 80 of the others: state of the walk and loop counters, no sums.  Fewer spills were not always faster:
+    // where they fall decides, and how they meet the gathers' copies, which go through the same pipe.
     static constexpr int regs_prod = TN == 256 ? 64 : (TN == 128 ? 56 : 48), regs_dq = 80, regs_epi = TN == 256 ? 184 : (TN == 128 ? 128 : 136);
     static constexpr int regs_launch = TN == 256 ? 128 : 96;
     static_assert(4 * regs_prod + dq_warps * regs_dq + TC_EPI * regs_epi <= threads / 32 * regs_launch, "setmaxnreg.inc draws on what the block was launched with");
@@ -241,8 +244,12 @@ __device__ __forceinline__ int half_cols(int rows, int h) {
     const int hs = half_split<HC>(rows);
     return (min(hs, rows - hs * h) + 31) & ~31;
 }
-// What a k-block of a tile costs, in units of 64 cycles (measured, every cluster busy): by tile size, rows of the tile and
-// quantization groups per k-block.  At most TC_COST_MAX.
+// What a k-block of a tile costs a cluster, in units of 64 cycles or so: by tile size, rows of the tile and quantization groups per
+// k-block.  At most TC_COST_MAX.  Decides the shares of clusters that split tiles of several formats, and what is worth splitting.
+// Taken with every cluster busy; whole tiles of one format, 4 bit, take now (pc, g128, g64, g32) 20, 22, 42, 71 with 256 rows, 12, 17,
+// 31, 53 with 128; 128 tokens 12, 16, 25, 48; 64 tokens 10, 12, 22, 33.  With those figures here mixed batches are as often slower
+// as faster (2926 rows x 512 x 3584, W8-pc W4-g64: 35.2 instead of 31.0 us; 250 rows x 4096 x 4096, W8-pc W4-g32 W4-g128: 2.6 % less):
+// shares are cut in whole k-blocks, and a gathered or parked k-block costs more than these.
 template <int TN>
 __device__ __forceinline__ int kblock_cost(int rows, int bits, int per) {
     const int wide = bits == 8 || bits == 3 ? 2 : 0;       // (the 8-bit tiles are larger, the 3-bit ones take longer to unpack)
@@ -611,12 +618,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             // ---------------- X producers: this CTA's XR token rows of every half tile, KS x 128 k per stage ----------------
             // Both warps walk the stages and arrive on the pair's xfull barrier.  A piece whose rows all come in boxes has a lean
             // loop: a warp fetches one 64-k sub-tile of every box, its arrival carries the byte count, and nothing is fenced or
-            // waited for (one loop for both kinds took the warp 1170 cycles a step, more than the tensor core's 1024: 2048 rows x
-            // 4096 x 4096, per channel, 57 -> 54 us).  Otherwise both warps gather, every other pair of rows each, with cp.async, and
-            // the arrival for a stage follows once its copies have landed, LAG stages later (2, and before the next piece's rows are
-            // waited for: 1024 rows in runs of 100, three experts, 4096 x 4096, 65 -> 62 us; with 3 67, with 1 also 67 and 300
-            // scattered rows 30 -> 36).  TMA's own gather, four rows to a request, takes an SM 45 cycles a request: those 300 rows
-            // 58 us.  Copies that arrive on a barrier, looked at between stages, cost the other warps their issue slots: 34 us.
+            // waited for (a loop for both kinds takes the warp 1170 cycles a step, more than the tensor core's 1024: 2048 rows x
+            // 4096 x 4096, per channel, 57 us instead of 54).  Otherwise both warps gather, every other pair of rows each, with cp.async,
+            // and the arrival for a stage follows once its copies have landed, LAG stages later, and before the next piece's rows are
+            // waited for (500 scattered rows, three experts, 4096 x 4096: 33.5 us, with LAG 1 43; 481 rows in runs of 10 to 90, 4096 x
+            // 11008: 67, with LAG 3 73; the stage's copies in a loop and not unrolled: 46 for the 500 rows).  TMA's own gather, four rows
+            // to a request, takes an SM 45 cycles a request: 300 scattered rows 58 us and not 29.  Copies that arrive on a barrier,
+            // looked at between stages, cost the other warps their issue slots: 34.
             constexpr int LAG = 2;
             const int gw = warp == 0 ? 0 : 1;
             int* s_xrow = sh.xrow[gw];
@@ -779,7 +787,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
                 };
                 // This warp's instructions are on the critical path of every step (the tensor core runs dry while it waits, votes
                 // and commits), so the loops of the common formats hold as few of them as can be (8192 rows x 4096 x 4096, per
-                // channel: 211 -> 194 us against one loop for every format).
+                // channel: 194 us, with one loop for every format 211).
                 const uint32_t xd0 = sbase, at0 = tmem_base + L::a_base;
                 if (keep) {
                     const int b1 = buf + 1 == NACC ? 0 : buf + 1;
@@ -1005,8 +1013,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TcCfg<TN>::threads, 
             const int dcol = KS == 2 ? pc.rows : ncol;
             if (keep) {
                 // Per channel: a half tile's buffer is drained once.  (Apart from the groups' loops, whose scales and counts are then not
-                // alive here: 28224 rows of 256 -> 1024 channels 40.7 -> 34.9 us with the walk in shared memory, see below; as long as
-                // both shared one drain, a piece of two k-blocks paid for their spills.)
+                // alive here: 28224 rows of 256 -> 1024 channels 34.6 us; 40.7 where both share one drain, and a piece of two k-blocks
+                // pays for its spills.)
                 const int nu = KS == 2 ? 1 : nh;
 #pragma unroll 1
                 for (int u = 0; u < nu; ++u) {

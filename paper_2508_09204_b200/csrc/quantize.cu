@@ -351,8 +351,8 @@ __device__ __forceinline__ void encode_pairs(const uint32_t (&c)[16], uint32_t (
 // Groups of 32, 64 or 128 k.  Bound by the fp32 weights' bytes, read once.  A warp takes one blob, 16 channels x 128 k, after
 // another, an unrelated one each time; the next two are on their way into its own two stages of shared memory (four boxes of 32
 // k x 16 rows each: with the 128-byte swizzle a quarter-warp's eight rows fall on different banks), so that loads are always in
-// flight and take no registers.  One block of 12 warps to an SM: 192 KB of stages.  11008 x 4096, 4-bit g128, built and exported:
-// 90.7 -> 76.4 us against 24 warps an SM that load into registers and wait (of the 57 us that took, 31 are the weights' bytes).
+// flight and take no registers.  One block of 12 warps to an SM: 192 KB of stages.  11008 x 4096, 4-bit g128: 42 us, of which 28 are
+// the weights' bytes at the copy rate; 57 with 24 warps an SM that load into registers and wait.  g32 74 (8 bit) and 70 (2 bit).
 constexpr int QG_WARPS = 12, QG_STAGES = 2, QG_STAGE = 16 * 128 * 4;
 constexpr int QG_SMEM = 1024 + QG_WARPS * QG_STAGES * QG_STAGE;
 template <int BITS>
