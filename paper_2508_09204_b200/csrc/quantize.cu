@@ -469,9 +469,10 @@ __global__ void __launch_bounds__(QG_WARPS * 32, 1) quantize_group_kernel(const 
 }
 
 // Per channel.  A block goes over its 16 rows twice, the second time out of L2 (16 rows are 256 KB at K = 4096); a warp holds the
-// 16 channels x 128 k of a blob in registers between loading and rounding.
-template <int BITS>
-__global__ void __launch_bounds__(256, 3) quantize_channel_kernel(const float* __restrict__ W, int N, int K, int sym, int KB,
+// 16 channels x 128 k of a blob in registers between loading and rounding.  BLOCKS: to an SM, see channel_blocks; with two a warp has
+// both halves of a blob under way before it rounds the first.
+template <int BITS, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS) quantize_channel_kernel(const float* __restrict__ W, int N, int K, int sym, int KB,
                                                                uint8_t* __restrict__ tiles, __half* __restrict__ scales_pc,
                                                                __nv_bfloat16* __restrict__ zeros_pc) {
     __shared__ float s_ext[8][2][16];
@@ -528,15 +529,16 @@ __global__ void __launch_bounds__(256, 3) quantize_channel_kernel(const float* _
     }
     for (int kb = warp; kb < KB; kb += 8) {
         uint8_t* tile = tiles + ((size_t)nt * KB + kb) * (size_t)stride;
+        float v[BLOCKS == 2 ? 2 : 1][32];
+        if constexpr (BLOCKS == 2) { load(row0, kb, v[0]); load(row0 + 8, kb, v[1]); }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int n = row0 + 8 * h;
-            float v[32];
-            load(n, kb, v);
+            const int n = row0 + 8 * h, at = BLOCKS == 2 ? h : 0;
+            if constexpr (BLOCKS != 2) load(n, kb, v[0]);
             uint32_t c[16], w[PieceWords<BITS>::n];
 #pragma unroll
             for (int G = 0; G < 4; ++G) {
-                round_chunk<BITS>(v + 8 * G, g[h], sym, c + 4 * G);
+                round_chunk<BITS>(v[at] + 8 * G, g[h], sym, c + 4 * G);
                 if (n >= N || kb * 128 + 32 * G + 8 * q >= K) c[4 * G] = c[4 * G + 1] = c[4 * G + 2] = c[4 * G + 3] = 0u;
             }
             encode_pairs<BITS>(c, w);
@@ -714,10 +716,23 @@ moqe_status alloc_expert(int N, int K, int bits, int group, int sym, bool clear,
     return MOQE_OK;
 }
 
+// Blocks of quantize_channel_kernel to an SM.  Three, unless their rows are too many for L2 (148 x 3 x 16 rows of K floats against 126
+// MB: beyond some 3800 k the second pass goes to HBM) and two have no more strips after one another on an SM, or as many and a last
+// round that is a good part empty either way.  Three / two, us, 8 bit and 3 bit: 11008 x 4096 111 / 105, 111 / 95; 10656 x 5120 129 / 120,
+// 132 / 115; 9472 x 4096 97 / 79; 18944 x 4096 165 / 151.  But 11008 x 3584 94 / 99, 13312 x 4096 112 / 113, 21312 x 4096 168 / 183,
+// 4736 x 4096 (one round) 40 / 42.
+int channel_blocks(int strips, int K) {
+    const int sms = device_sm_count();
+    auto rounds = [&](int b) { return (strips - sms / 8 + b * sms - 1) / (b * sms) * b; };      // (a few strips more make no round)
+    const int two = rounds(2), three = rounds(3);
+    return K > 3840 && strips > 2 * sms && (two < three || (two == three && strips * 20ll < 17ll * sms * three)) ? 2 : 3;
+}
+
 moqe_status launch_quantize(const moqe_expert* e, const float* W, cudaStream_t st) {
     const int KB = e->Kp / 128, strips = e->Np / 16;
     if (e->group == 0) {
-#define MOQE_QC(B) quantize_channel_kernel<B><<<strips, 256, 0, st>>>(W, e->N, e->K, e->sym, KB, e->tiles, e->scales_pc, e->zeros_pc)
+        const int blocks = channel_blocks(strips, e->K);
+#define MOQE_QC(B) (blocks == 2 ? quantize_channel_kernel<B, 2> : quantize_channel_kernel<B, 3>)<<<strips, 256, 0, st>>>(W, e->N, e->K, e->sym, KB, e->tiles, e->scales_pc, e->zeros_pc)
         if (e->bits == 4) MOQE_QC(4);
         else if (e->bits == 8) MOQE_QC(8);
         else if (e->bits == 2) MOQE_QC(2);
@@ -757,7 +772,7 @@ moqe_status launch_quantize(const moqe_expert* e, const float* W, cudaStream_t s
 // Whether an expert is built by one kernel, or by the two before them.  Groups within a k-block are.  A per-channel
 // expert's strip of 16 rows belongs to one block there, which goes over it twice: that wants strips for every SM to the last
 // round, and short enough to be in L2 the second time.  Two kernels / one, device time in us, 8 bit: 11008 rows (688 strips on 148
-// SMs) x 4096 113 / 102, x 11008 267 / 296; 3072 rows (192 strips) x 4096 36 / 44; 128 rows x 11008 23 / 60.  Rows of up to 1024
+// SMs) x 4096 113 / 105, x 11008 267 / 296; 3072 rows (192 strips) x 4096 36 / 44; 128 rows x 11008 23 / 60.  Rows of up to 1024
 // are over before the second launch would start (128 x 1024 18 / 12, 11008 x 1024 34 / 33).
 bool one_kernel(const moqe_expert* e) {
     if (e->group != 0) return e->group <= 128;

@@ -96,10 +96,11 @@ def test_blobs_to_a_warp(N, K, bits, group, sym):
 
 
 @pytest.mark.parametrize("bits,sym", [(8, True), (4, False), (3, False), (2, True)])
-@pytest.mark.parametrize("N,K", [(2296, 1088), (2368, 64), (2056, 1088), (2376, 5128), (2296, 5120), (2048, 1152), (264, 1024), (264, 1032)])
+@pytest.mark.parametrize("N,K", [(2296, 1088), (2368, 64), (2056, 1088), (2376, 5128), (2296, 5120), (2048, 1152), (264, 1024), (264, 1032), (9464, 3848), (9464, 3840)])
 def test_per_channel_by_one_kernel_and_by_two(N, K, bits, sym):
     """144 and 148 strips of 16 rows are for one kernel on 148 SMs, up to K = 5120; 136 and 152 strips, and longer rows, for two;
-    up to K = 1024 all are for one.  Without padding (2048 x 1152) nothing is cleared first.  The memory is that of a larger expert before."""
+    up to K = 1024 all are for one.  Without padding (2048 x 1152) nothing is cleared first.  Four strips to an SM go two at a time from
+    3848 k on, three at a time before.  The memory is that of a larger expert before."""
     import paper_2508_09204_b200 as moqe
     from gpu_helpers import assert_close, assert_expert_matches, bf16_to_torch, dev, torch_to_bits
     W = wl.weights_f32(f"pc/{N}/{K}", N, K)
